@@ -14,7 +14,7 @@
 // K-major operand layout) into the hi tiles of a stage; warps 0-3 write lo to
 // the lo tile at the same offset (the fp32 tile itself is the hi operand: a
 // kind::tf32 MMA reads only the upper 19 bits); lane 0 of warp 4 issues the
-// MMAs; warps 4-7 read the fp32 accumulator tile from TMEM. A thread-block
+// MMAs; warps 4-7 read the accumulators from TMEM. A thread-block
 // cluster of cs CTAs splits K; the members' partial tiles are summed into the
 // leader CTA over distributed shared memory (deterministic, no workspace)
 // before the leader writes S. With more tiles than SMs and short K (the blocked
@@ -42,12 +42,17 @@ struct GCfg {
     static constexpr uint32_t kABytes = kBM * kRowBytes;   // 16 KiB
     static constexpr uint32_t kBBytes = BN * kRowBytes;
     static constexpr uint32_t kStageBytes = 2 * kABytes + 2 * kBBytes;  // hi and lo of both operands
-    // K chunks rotate over kAcc accumulators (all 512 TMEM columns): each sees
-    // 1/kAcc of the additions, which bounds the tensor core's fp32 accumulation
-    // error; the epilogue sums them on CUDA cores with round-to-nearest.
+    // The tensor pipe's fp32 accumulation truncates (about a quarter ulp per addition,
+    // always toward zero). One pass: the K chunks rotate over kAcc accumulators (all 512
+    // TMEM columns), each sees 1/kAcc of the additions and the epilogue sums them with
+    // round-to-nearest. DRAIN: groups of kGroup chunks (24 additions) rotate, and the
+    // epilogue warps add every finished group into fp32 registers while the MMAs fill the
+    // next ones (a dot of 7168 features: 0.9e-6 off instead of 1.3e-5, 3 % more time).
     static constexpr int kAcc = 512 / BN < 8 ? 512 / BN : 8;
+    static constexpr int kGroup = 2;
     static constexpr uint32_t kTmemCols = 512;
-    static constexpr size_t kSmem = 1024 + (size_t)kStages * kStageBytes + 8 * (3 * kStages + 4) + 16;  // + barriers, TMEM slot, abort flag
+    static constexpr size_t kSmem =
+        1024 + (size_t)kStages * kStageBytes + 8 * (3 * kStages + 2 * kAcc + 3) + 16;  // + barriers, TMEM slot, abort flag
 };
 
 struct GParams {
@@ -110,8 +115,10 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm,
         : "memory");
 }
 
-template <int BN>
-__global__ void __launch_bounds__(kThreads, 1)
+// DRAIN: the epilogue warps work during the main loop, so warps 8 and 9 issue the MMAs and copies;
+// otherwise lane 0 of warps 4 and 5 does before their epilogue (two more warps cost 2.5 %).
+template <int BN, bool DRAIN>
+__global__ void __launch_bounds__(kThreads + (DRAIN ? 64 : 0), 1)
 score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GParams p) {
     using C = GCfg<BN>;
     extern __shared__ uint8_t smem_raw[];
@@ -119,12 +126,13 @@ score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     uint64_t* bars = (uint64_t*)(smem + (size_t)C::kStages * C::kStageBytes);
     uint64_t* full = bars;                   // count 4 (producer warps)
     uint64_t* empty = bars + C::kStages;     // count 1 (MMA commit)
-    uint64_t* tfull = empty + C::kStages;    // count 1
-    uint64_t* red_go = tfull + 1;            // count 1 (leader's remote arrive)
+    uint64_t* raw_full = empty + C::kStages; // [kStages] TMA bytes landed (count 1 + tx)
+    uint64_t* acc_full = raw_full + C::kStages;  // [kAcc] a group is in the accumulator (MMA commit)
+    uint64_t* acc_empty = acc_full + C::kAcc;    // [kAcc] the accumulator is drained (count 4)
+    uint64_t* red_go = acc_empty + C::kAcc;  // count 1 (leader's remote arrive)
     uint64_t* red_full = red_go + 1;         // count cs-1
     uint64_t* mma_done = red_full + 1;       // count 1
-    uint64_t* raw_full = mma_done + 1;       // [kStages] TMA bytes landed (count 1 + tx)
-    uint32_t* tmem_slot = (uint32_t*)(raw_full + C::kStages);
+    uint32_t* tmem_slot = (uint32_t*)(mma_done + 1);
     volatile int* abort = (volatile int*)(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -134,14 +142,18 @@ score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             mbar_init(smem_u32(&empty[s]), 1);
             mbar_init(smem_u32(&raw_full[s]), 1);
         }
-        mbar_init(smem_u32(tfull), 1);
+        for (int a = 0; a < C::kAcc; ++a) {
+            mbar_init(smem_u32(&acc_full[a]), 1);
+            mbar_init(smem_u32(&acc_empty[a]), 4);
+        }
         mbar_init(smem_u32(red_go), 1);
         mbar_init(smem_u32(red_full), p.cs > 1 ? p.cs - 1 : 1);
         mbar_init(smem_u32(mma_done), 1);
         *abort = 0;
         fence_mbar_init();
     }
-    if (warp == 4) {
+    constexpr int kMmaWarp = DRAIN ? 8 : 4, kTmaWarp = DRAIN ? 9 : 5;
+    if (warp == kMmaWarp) {
         tmem_alloc(smem_u32(tmem_slot), C::kTmemCols);
         tmem_relinquish();
     }
@@ -190,104 +202,108 @@ score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&full[s]));
         }
-    } else {
-        if (warp == 5 && lane == 0) {
-            // ---------------- TMA producer: fp32 chunks of Phi rows m0.. and Qhat rows n0..
-            // (features past the slice end belong to the next slice only when the slice
-            // is not the last; slices are multiples of 32 features, so no chunk crosses one)
-            uint32_t it = 0, last_par[C::kStages];
-            bool issued[C::kStages];
-            for (int s = 0; s < C::kStages; ++s) issued[s] = false;
-            for (int64_t kc = kc0; kc < kc1; ++kc, ++it) {
-                const int s = it % C::kStages;
-                const uint32_t ph = (it / C::kStages) & 1u;
-                if (!wait_bounded(smem_u32(&empty[s]), ph ^ 1u, abort, p.err)) break;
-                const uint32_t st = smem_u32(smem + (size_t)s * C::kStageBytes), bar = smem_u32(&raw_full[s]);
-                const int k = (int)(kbase + kc * kKC);
-                mbar_arrive_tx(bar, C::kABytes + C::kBBytes);
-                if (p.batched) {
-                    tma_load_3d(st, &tmA, k, (int)m0, zc, bar);
-                    tma_load_3d(st + 2 * C::kABytes, &tmB, k, (int)n0, zc, bar);
-                } else {
-                    tma_load_2d(st, &tmA, k, (int)m0, bar);
-                    tma_load_2d(st + 2 * C::kABytes, &tmB, k, (int)n0, bar);
-                }
-                issued[s] = true;
-                last_par[s] = ph;
+    }
+    if (warp == kTmaWarp && lane == 0) {
+        // ---------------- TMA producer: fp32 chunks of Phi rows m0.. and Qhat rows n0..
+        // (features past the slice end belong to the next slice only when the slice
+        // is not the last; slices are multiples of 32 features, so no chunk crosses one)
+        uint32_t it = 0, last_par[C::kStages];
+        bool issued[C::kStages];
+        for (int s = 0; s < C::kStages; ++s) issued[s] = false;
+        for (int64_t kc = kc0; kc < kc1; ++kc, ++it) {
+            const int s = it % C::kStages;
+            const uint32_t ph = (it / C::kStages) & 1u;
+            if (!wait_bounded(smem_u32(&empty[s]), ph ^ 1u, abort, p.err)) break;
+            const uint32_t st = smem_u32(smem + (size_t)s * C::kStageBytes), bar = smem_u32(&raw_full[s]);
+            const int k = (int)(kbase + kc * kKC);
+            mbar_arrive_tx(bar, C::kABytes + C::kBBytes);
+            if (p.batched) {
+                tma_load_3d(st, &tmA, k, (int)m0, zc, bar);
+                tma_load_3d(st + 2 * C::kABytes, &tmB, k, (int)n0, zc, bar);
+            } else {
+                tma_load_2d(st, &tmA, k, (int)m0, bar);
+                tma_load_2d(st + 2 * C::kABytes, &tmB, k, (int)n0, bar);
             }
-            // copies still in flight when the consumers stopped early land before the CTA exits
-            for (int s = 0; s < C::kStages; ++s)
-                if (issued[s]) {
-                    const uint64_t t0 = global_ns();
-                    while (!mbar_try_wait(smem_u32(&raw_full[s]), last_par[s]))
-                        if (global_ns() - t0 > kTimeoutNs) {
-                            atomicOr(p.err, kErrTimeout);
-                            break;
-                        }
-                }
+            issued[s] = true;
+            last_par[s] = ph;
         }
-        if (warp == 4 && lane == 0) {
-            // ---------------- MMA issuer
-            const uint32_t idesc = idesc_tf32(kBM, BN);
-            uint32_t it = 0;
-            bool ok = true;
-            for (int64_t kc = kc0; kc < kc1; ++kc, ++it) {
-                const int s = it % C::kStages;
-                const uint32_t ph = (it / C::kStages) & 1u;
-                if (!wait_bounded(smem_u32(&full[s]), ph, abort, p.err)) {
-                    ok = false;
-                    break;
-                }
-                tc_fence_after();
-                const uint32_t st = smem_u32(smem + (size_t)s * C::kStageBytes);
-                const uint64_t ahi = sw128_desc(st), alo = sw128_desc(st + C::kABytes);
-                const uint64_t bhi = sw128_desc(st + 2 * C::kABytes), blo = sw128_desc(st + 2 * C::kABytes + C::kBBytes);
+        // copies still in flight when the consumers stopped early land before the CTA exits
+        for (int s = 0; s < C::kStages; ++s)
+            if (issued[s]) {
+                const uint64_t t0 = global_ns();
+                while (!mbar_try_wait(smem_u32(&raw_full[s]), last_par[s]))
+                    if (global_ns() - t0 > kTimeoutNs) {
+                        atomicOr(p.err, kErrTimeout);
+                        break;
+                    }
+            }
+    }
+    if (warp == kMmaWarp && lane == 0) {
+        // ---------------- MMA issuer
+        const uint32_t idesc = idesc_tf32(kBM, BN);
+        uint32_t it = 0;
+        for (int64_t kc = kc0; kc < kc1; ++kc, ++it) {
+            const int s = it % C::kStages;
+            const uint32_t ph = (it / C::kStages) & 1u;
+            const uint32_t g = DRAIN ? it / C::kGroup : it, a = g % C::kAcc;  // group g goes to accumulator a
+            const bool start = DRAIN ? it % C::kGroup == 0 : it < (uint32_t)C::kAcc;
+            if (DRAIN && start && !wait_bounded(smem_u32(&acc_empty[a]), ((g / C::kAcc) & 1u) ^ 1u, abort, p.err)) break;
+            if (!wait_bounded(smem_u32(&full[s]), ph, abort, p.err)) break;
+            tc_fence_after();
+            const uint32_t st = smem_u32(smem + (size_t)s * C::kStageBytes);
+            const uint64_t ahi = sw128_desc(st), alo = sw128_desc(st + C::kABytes);
+            const uint64_t bhi = sw128_desc(st + 2 * C::kABytes), blo = sw128_desc(st + 2 * C::kABytes + C::kBBytes);
+            const uint32_t d = tmem + a * BN;
 #pragma unroll
-                for (int k = 0; k < kKC / 8; ++k) {  // K = 8 tf32 = 32 bytes per instruction
-                    const uint32_t d = tmem + (it % C::kAcc) * BN;
-                    const uint32_t first = (it < (uint32_t)C::kAcc && k == 0) ? 0u : 1u;
-                    mma_tf32(d, ahi + 2 * k, bhi + 2 * k, idesc, first);
-                    mma_tf32(d, ahi + 2 * k, blo + 2 * k, idesc, 1u);
-                    mma_tf32(d, alo + 2 * k, bhi + 2 * k, idesc, 1u);
-                }
-                mma_commit(smem_u32(&empty[s]));
+            for (int k = 0; k < kKC / 8; ++k) {  // K = 8 tf32 = 32 bytes per instruction
+                mma_tf32(d, ahi + 2 * k, bhi + 2 * k, idesc, start && k == 0 ? 0u : 1u);
+                mma_tf32(d, ahi + 2 * k, blo + 2 * k, idesc, 1u);
+                mma_tf32(d, alo + 2 * k, bhi + 2 * k, idesc, 1u);
             }
-            if (ok) mma_commit(smem_u32(tfull));
-            mma_commit(smem_u32(mma_done));
-            const uint64_t t0 = global_ns();
-            while (!mbar_try_wait(smem_u32(mma_done), 0))
-                if (global_ns() - t0 > kTimeoutNs) {
-                    atomicOr(p.err, kErrTimeout);
-                    break;
-                }
+            mma_commit(smem_u32(&empty[s]));
+            if (DRAIN ? (it % C::kGroup == C::kGroup - 1 || kc == kc1 - 1) : kc == kc1 - 1)
+                mma_commit(smem_u32(&acc_full[DRAIN ? a : 0u]));
         }
-        __syncwarp();
-        // ---------------- epilogue (warps 4-7): TMEM -> (cluster reduction) -> S
+        mma_commit(smem_u32(mma_done));
+        const uint64_t t0 = global_ns();
+        while (!mbar_try_wait(smem_u32(mma_done), 0))
+            if (global_ns() - t0 > kTimeoutNs) {
+                atomicOr(p.err, kErrTimeout);
+                break;
+            }
+    }
+    __syncwarp();
+    if (warp >= 4 && warp < 8) {
+        // ---------------- epilogue: TMEM groups -> registers -> (cluster reduction) -> S
         const int q = warp & 3;
         const int row = q * 32 + lane;  // Phi row within the tile
-        const bool empty_k = kc1 <= kc0;
-        bool got = true;
-        if (!empty_k) {
-            if (lane == 0) got = wait_bounded(smem_u32(tfull), 0, abort, p.err);
-            got = __shfl_sync(0xffffffffu, got, 0);
-        }
+        const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16);
+        const uint32_t nchunks = kc1 > kc0 ? (uint32_t)(kc1 - kc0) : 0u;
+        const uint32_t groups = DRAIN ? (nchunks + C::kGroup - 1) / C::kGroup : (nchunks > 0 ? 1u : 0u);
+        const uint32_t used = DRAIN ? 1u : (nchunks < (uint32_t)C::kAcc ? nchunks : (uint32_t)C::kAcc);
         float acc[BN];
-        if (!epi_any(!got)) {
+#pragma unroll
+        for (int c = 0; c < BN; ++c) acc[c] = 0.f;
+        bool got = true;
+        for (uint32_t g = 0; g < groups; ++g) {
+            const uint32_t a = g % C::kAcc;
+            if (lane == 0) got = wait_bounded(smem_u32(&acc_full[a]), (g / C::kAcc) & 1u, abort, p.err);
+            got = __shfl_sync(0xffffffffu, got, 0);
+            if (!got) break;
             tc_fence_after();
-            const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16);
-            const int used = (int)((kc1 - kc0) < C::kAcc ? (kc1 - kc0) : C::kAcc);  // accumulators written
 #pragma unroll
-            for (int c0 = 0; c0 < BN; c0 += 16) {
-#pragma unroll
-                for (int i = 0; i < 16; ++i) acc[c0 + i] = 0.f;
-                for (int a = 0; a < used; ++a) {
+            for (int c0 = 0; c0 < BN; c0 += 16)
+                for (uint32_t b = 0; b < used; ++b) {
                     float v[16];
-                    tmem_ld16(tbase + a * BN + c0, v);
+                    tmem_ld16(tbase + (a + b) * BN + c0, v);
 #pragma unroll
                     for (int i = 0; i < 16; ++i) acc[c0 + i] += v[i];
                 }
-            }
             tc_fence_before();
+            __syncwarp();
+            if (DRAIN && lane == 0) mbar_arrive(smem_u32(&acc_empty[a]));
+        }
+        if (!epi_any(!got)) {
             bool ok = true;
             if (p.cs > 1) {
                 // partial tiles of members 1..cs-1 land in the leader's stage buffers
@@ -338,18 +354,18 @@ score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                             if (n < p.n_q) Sz[n * p.ld_S + m] = p.alpha * acc[c];
                         }
                     } else {
-                        // the previous values of 32 columns are loaded before any is stored, so
+                        // the previous values of 16 columns are loaded before any is stored, so
                         // the loads are in flight together instead of one round trip per column
 #pragma unroll
-                        for (int c0 = 0; c0 < BN; c0 += 32) {
-                            float old[32];
+                        for (int c0 = 0; c0 < BN; c0 += 16) {
+                            float old[16];
 #pragma unroll
-                            for (int i = 0; i < 32; ++i) {
+                            for (int i = 0; i < 16; ++i) {
                                 const int64_t n = n0 + c0 + i;
                                 old[i] = n < p.n_q ? __ldcg(Sz + n * p.ld_S + m) : 0.f;
                             }
 #pragma unroll
-                            for (int i = 0; i < 32; ++i) {
+                            for (int i = 0; i < 16; ++i) {
                                 const int64_t n = n0 + c0 + i;
                                 if (n < p.n_q) Sz[n * p.ld_S + m] = p.beta * old[i] + p.alpha * acc[c0 + i];
                             }
@@ -362,7 +378,7 @@ score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 
     tc_fence_before();
     __syncthreads();
-    if (warp == 4) {
+    if (warp == kMmaWarp) {
         tc_fence_after();
         tmem_dealloc(tmem, C::kTmemCols);
     }
@@ -966,6 +982,30 @@ bool make_map_f32_3d(CUtensorMap* tm, const float* X, int64_t rows, int64_t K, i
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+template <int BN, bool DRAIN>
+cudaError_t launch_score3x(const CUtensorMap& tmA, const CUtensorMap& tmB, const GParams& p, int64_t tiles, int64_t nz,
+                           cudaStream_t s) {
+    using C = GCfg<BN>;
+    cudaError_t e = smem_attr_once<score3x_kernel<BN, DRAIN>>((int)C::kSmem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)p.cs;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)(tiles * p.cs), (unsigned)p.splits, (unsigned)nz);
+    cfg.blockDim = dim3(kThreads + (DRAIN ? 64 : 0));
+    cfg.dynamicSmemBytes = C::kSmem;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    note_launches(1);
+    e = cudaLaunchKernelEx(&cfg, score3x_kernel<BN, DRAIN>, tmA, tmB, p);
+    if (e != cudaSuccess) return e;
+    return cudaGetLastError();
+}
+
 template <int BN>
 cudaError_t launch_bn(GParams p, cudaStream_t s, int64_t nz = 1, size_t a_z_bytes = 0, size_t b_z_bytes = 0) {
     using C = GCfg<BN>;
@@ -1006,24 +1046,9 @@ cudaError_t launch_bn(GParams p, cudaStream_t s, int64_t nz = 1, size_t a_z_byte
         gemm3x_persist_kernel<BN><<<(unsigned)sms, kThreadsP, P::kSmem, s>>>(tmA, tmB, p);
         return cudaGetLastError();
     }
-    cudaError_t e = smem_attr_once<score3x_kernel<BN>>((int)C::kSmem);
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)cs;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3((unsigned)(tiles * cs), (unsigned)p.splits, (unsigned)nz);
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = C::kSmem;
-    cfg.stream = s;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    note_launches(1);
-    e = cudaLaunchKernelEx(&cfg, score3x_kernel<BN>, tmA, tmB, p);
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
+    // slices of materialised-gradient dots (thousands of features a slice) drain their accumulators
+    return p.kslice ? launch_score3x<BN, true>(tmA, tmB, p, tiles, nz, s)
+                    : launch_score3x<BN, false>(tmA, tmB, p, tiles, nz, s);
 }
 
 }  // namespace
