@@ -90,9 +90,9 @@ static RouteCounts route_counts(const tda_layer_desc& L, tda_op op, int64_t n1, 
     const double build = 2.0 * T * Ni * No;
     const double dense = 2.0 * No * Ni * ka + 2.0 * No * ka * kg;
     RouteCounts c;
-    // the unprojected Gram of bf16 factors runs on tensor cores when T is a power of two
-    c.gram_rate = (op == TDA_OP_SIMILARITY_EXACT && dt == TDA_BF16 && L.T > 0 && (L.T & (L.T - 1)) == 0 &&
-                   L.d_in % 8 == 0 && L.d_out % 8 == 0)
+    // the unprojected Gram of bf16 factors runs on tensor cores
+    c.gram_rate = ((op == TDA_OP_SIMILARITY_EXACT || op == TDA_OP_NORM_EXACT) && dt == TDA_BF16 && L.d_in % 8 == 0 &&
+                   L.d_out % 8 == 0)
                       ? 2
                       : 3;
     c.build = (op == TDA_OP_PROJECT || op == TDA_OP_NORM_PROJECTED || op == TDA_OP_NORM_EXACT ? B1 : B1 + B2) * build;
@@ -491,6 +491,11 @@ tda_status tda_norms(tda_op op, const tda_layer_desc* L, tda_dtype dtype, const 
     cudaStream_t s = (cudaStream_t)stream;
     if (N == 0) return TDA_OK;
     if (L->T == 0) return cuda_check(cudaMemsetAsync(out, 0, sizeof(float) * (size_t)N, s), "zero norms");
+    if (op == TDA_OP_NORM_EXACT && route == TDA_ROUTE_GRAM && gram_tc_supported(*L, dtype, A, B, A, B)) {
+        unsigned int* err = device_error_word();
+        if (!err) return fail(TDA_ERR_CUDA, "device error word unavailable");
+        return cuda_check(launch_gram_self_tc(*L, A, B, N, out, err, s), "norms (gram, tensor cores)");
+    }
     if (op == TDA_OP_NORM_EXACT && route == TDA_ROUTE_GRAM)
         return cuda_check(launch_gram_self(*L, dtype, A, B, N, L->d_in, L->d_out, 1.f, out, s), "norms (gram)");
     const size_t need = norms_ws(*L, op, 1, route);

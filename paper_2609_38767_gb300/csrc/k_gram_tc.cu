@@ -1,25 +1,54 @@
 // k_gram_tc.cu -- route (c), the factored Gram identity (Eq. 4), on the
-// tcgen05 tensor cores of sm_103a for bf16 factors:
+// tcgen05 tensor cores of sm_103a for bf16 factors, for any token count:
 //
-//   <DW_q, DW_i>_F = sum_{t,s} (A_q A_i^T)[t][s] * (B_q B_i^T)[t][s].
+//   <DW_q, DW_i>_F = sum_{t,s} (A_q A_i^T)[t][s] * (B_q B_i^T)[t][s],
+//
+// and the norms ||DW_i||^2 by the same identity with both sides example i.
 //
 // Both token Grams are dense contractions over the feature dimension, K-major
 // in memory (a token's activations are contiguous), so they map directly onto
 // tcgen05.mma: a 128-row tile of query tokens (M) against a 256-row tile of
-// train tokens (N), K = d_in for X = A_q A_i^T and then K = d_out for
-// Y = B_q B_i^T, both accumulators side by side in TMEM (2 x 256 columns). The
-// epilogue reads each token row of X and Y, forms sum_s X[t][s] Y[t][s] over the
-// columns of each train example and reduces over the rows of each query.
+// train tokens (N), first X = A_q A_i^T (K = d_in), then Y = B_q B_i^T
+// (K = d_out).
 //
-// Token tiles: for T <= 128 (a power of two) a query tile packs 128 / T query
-// examples and a train tile 256 / T train examples, so one tile pair yields a
-// whole block of S; for T >= 256 a (query, train) pair is a loop over its
-// (T/128) x (T/256) tile pairs, summed in a register.
+// Token tiles: for T <= 128 a query tile packs floor(128 / T) whole query
+// examples and a train tile floor(256 / T) train examples (their tokens are
+// consecutive rows), so one tile pair yields a whole block of S; rows past the
+// last whole example belong to the next tile's examples and are left out of
+// the sums. For T > 128 a (query, train) pair is a loop over its
+// ceil(T/128) x ceil(T/256) tile pairs (tokens past T read as zero rows).
 //
-// Warp roles (256 threads, one persistent CTA per SM): warp 0 TMA producer,
-// warp 1 TMEM allocator and MMA issuer (lane 0), warps 4-7 epilogue. Waits are
-// bounded (about 1 s) and set kErrTimeout on expiry, as in the projection
-// kernel.
+// Accuracy: the tensor pipe adds into its fp32 accumulators with truncation,
+// a loss of about a quarter ulp per addition that always points to zero (d =
+// 2048, 128 additions: 3.6e-6 low). So K goes in blocks of one to eight 64-feature
+// chunks, each into one of two 256-column TMEM buffers, and the epilogue adds
+// the blocks in registers with round-to-nearest: X's blocks are summed (128
+// registers a thread), and since the identity is bilinear every Y block is
+// multiplied into the sums as it arrives, sum_s X[t][s] Y_b[t][s], and need not
+// be kept. The buffers alternate, so the epilogue of one block overlaps the
+// MMAs of the next.
+//
+// What bounds it: each M = 128, N = 256, K = 16 MMA reads 12 KB of operands
+// from shared memory and the TMA writes as much, ~190 B/clock per SM against
+// ~128 B/clock of shared-memory bandwidth, so the tile tops out near two
+// thirds of the MMA rate. The epilogue (256 threads, 128 columns each) reads
+// 128 KB of TMEM per block, half the time of a two-chunk block's MMAs.
+//
+// Measured (similarity alone): 2048 -> 2048, T = 50, 16 x 512 pairs 34.9 ms on the
+// CUDA cores (T not a power of two), now 0.22 ms = 0.76 PFLOP/s useful (100 of 128
+// and 250 of 256 tile rows); 8192 -> 8192 at T = 8 / 32 / 128 / 512: 1.14 / 1.25 /
+// 1.27 / 0.99 PFLOP/s with one accumulation per tile and no overlap between tiles,
+// now 1.56 / 1.46 / 1.53 / 1.39.
+//
+// Norms (SELF): one 128-row tile of packed examples against itself needs one
+// 16 KB copy per chunk (A and B operand are the same tile) and is bound by
+// HBM (512 examples of 50 tokens, 2048 -> 2048: 3.9 ms on the CUDA cores, now
+// 78 us); T > 128 loops over the tile pairs i <= j, off-diagonal ones doubled.
+//
+// Warp roles (320 threads, one persistent CTA per SM): warp 0 TMA producer,
+// warp 1 TMEM allocator and MMA issuer (lane 0), warps 2-9 epilogue (two warps
+// per TMEM lane quadrant, each half of the columns). Waits are bounded (about
+// 1 s) and set kErrTimeout on expiry, as in the projection kernel.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -30,24 +59,33 @@
 namespace tda {
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kEpiWarps = 8;
+constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr int kTM = 128;                                 // query token rows per tile (MMA M)
-constexpr int kTN = 256;                                 // train token rows per tile (MMA N)
 constexpr int kChunkK = 64;                              // K elements per stage
 constexpr uint32_t kABytes = kTM * kChunkK * 2;          // 16 KiB
-constexpr uint32_t kBBytes = kTN * kChunkK * 2;          // 32 KiB
-constexpr uint32_t kStageBytes = kABytes + kBBytes;
-constexpr int kStages = 4;
-constexpr uint32_t kTmemCols = 512;                      // X: 0..255, Y: 256..511
-constexpr size_t kSmem = 1024 + (size_t)kStages * kStageBytes + 8 * 16 + 8 * (2 * kStages + 3) + 64;
-static_assert(kSmem <= 232448, "shared memory per CTA");
+constexpr uint32_t kTmemCols = 512;                      // two accumulator buffers of at most 256 columns
+constexpr int kMaxStages = 8;
+constexpr size_t kSmemMax = 232448;                      // 227 KiB of dynamic shared memory per CTA
+constexpr size_t kTailBytes = 16 * 8 + 8 * (2 * kMaxStages + 5) + 16;  // warp sums, barriers, TMEM slot, abort flag
+
+template <bool SELF>
+struct Cfg {
+    static constexpr int kTN = SELF ? 128 : 256;         // train token rows per tile (MMA N)
+    static constexpr int kCols = kTN / 2;                // columns per epilogue thread
+    static constexpr uint32_t kStageBytes = kABytes + kTN * kChunkK * 2;
+};
 
 struct GParams {
     int64_t n_q, n_t, T, ld_S;
-    int nk_in, nk_out;
-    int64_t n_units;      // tile pairs (T <= 128) or example pairs (T >= 256)
-    int64_t n_qtiles;     // packed query tiles (T <= 128)
-    int tiles_q, tiles_t; // token tiles per query / train example (T >= 256)
+    int nk_in, nk_out;      // K chunks per side
+    int kbx, kby;           // chunks per accumulation block of X and of Y
+    int stages;
+    int pq, pt;             // examples per query tile and per train tile (T <= 128), else 0
+    int ldr;                // floats per row of the per-example partial sums (packed)
+    int64_t n_units;        // tile pairs (packed) or example pairs (T > 128); SELF: tiles or examples
+    int64_t n_qtiles;       // packed query tiles
+    int tiles_q, tiles_t;   // token tiles per query / train example (T > 128)
     float alpha, beta;
     float* S;
     unsigned int* err;
@@ -60,40 +98,77 @@ __device__ __forceinline__ void emit(const GParams& p, int64_t q, int64_t i, flo
     *dst = p.beta == 0.f ? p.alpha * v : p.beta * (*dst) + p.alpha * v;
 }
 
-// sum over the rows of each query: lanes xor 1 .. R/2 (R <= 32) or the whole
-// warp (R > 32); result valid in the first lane of each row group
-__device__ __forceinline__ float row_reduce(float v, int R) {
-    const int w = R < 32 ? R : 32;
+// OR of v over the epilogue threads (named barrier 1).
+__device__ __forceinline__ bool epi_or(bool v) {
+    uint32_t r;
+    __syncwarp();
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.or.pred q, 1, %2, p;\n selp.u32 %0, 1, 0, q;\n}"
+        : "=r"(r)
+        : "r"((uint32_t)v), "n"(32 * kEpiWarps)
+        : "memory");
+    return r != 0;
+}
+
+__device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1)
-        if (o < w) v += __shfl_xor_sync(0xffffffffu, v, o);
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
 
+// One Y block of a packed tile for T = TS < 16: this thread's columns are kCols / TS whole train
+// examples, so every boundary is known when compiled (a run-time test per column cost 2.6 times
+// the MMAs' time at T = 8).
+template <int TS, int COLS>
+__device__ __forceinline__ void y_block_short(const float (&x)[COLS], uint32_t tb, float* myred, bool first) {
+    constexpr int kUse = COLS / TS * TS;
+    float s = 0.f;
+#pragma unroll
+    for (int c0 = 0; c0 < kUse; c0 += 16) {
+        float v[16];
+        tmem_ld16(tb + c0, v);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            if (c0 + i >= kUse) break;
+            s = (c0 + i) % TS == 0 ? x[c0 + i] * v[i] : fmaf(x[c0 + i], v[i], s);
+            if ((c0 + i + 1) % TS == 0) {
+                float* dst = myred + (c0 + i) / TS;
+                *dst = first ? s : *dst + s;
+            }
+        }
+    }
+}
+
+template <bool SELF>
 __global__ void __launch_bounds__(kThreads, 1)
 gram_tc_kernel(const __grid_constant__ CUtensorMap tmAq, const __grid_constant__ CUtensorMap tmAt,
                const __grid_constant__ CUtensorMap tmBq, const __grid_constant__ CUtensorMap tmBt,
                const GParams p) {
+    using C = Cfg<SELF>;
+    constexpr int kTN = C::kTN, kCols = C::kCols;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    float* red = (float*)(smem + (size_t)kStages * kStageBytes);   // [4 warps][4] cross-warp sums
-    uint64_t* bars = (uint64_t*)(red + 16);
-    uint64_t* full = bars;                 // stage landed (count 1 + tx)
-    uint64_t* empty = bars + kStages;      // MMAs done with the stage
-    uint64_t* tfull = bars + 2 * kStages;  // X, Y of a tile pair complete
-    uint64_t* tempty = tfull + 1;          // epilogue drained TMEM (count 4)
-    uint64_t* mma_done = tempty + 1;
+    float* wsum = (float*)(smem + (size_t)p.stages * C::kStageBytes);  // [8 warps] sums of a (query, train) pair
+    uint64_t* bars = (uint64_t*)(wsum + 32);
+    uint64_t* full = bars;                  // [stages] landed (count 1 + tx)
+    uint64_t* empty = bars + kMaxStages;    // [stages] MMAs done with the stage
+    uint64_t* tfull = bars + 2 * kMaxStages;  // [2] block accumulated
+    uint64_t* tempty = tfull + 2;           // [2] block drained (one arrive per epilogue warp)
+    uint64_t* mma_done = tempty + 2;
     uint32_t* tmem_slot = (uint32_t*)(mma_done + 1);
     volatile int* abort = (volatile int*)(tmem_slot + 1);
+    float* red = (float*)(tmem_slot + 4);   // packed: [2 column halves][128 rows][ldr examples] partial sums
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kStages; ++s) {
+        for (int s = 0; s < p.stages; ++s) {
             mbar_init(smem_u32(&full[s]), 1);
             mbar_init(smem_u32(&empty[s]), 1);
         }
-        mbar_init(smem_u32(tfull), 1);
-        mbar_init(smem_u32(tempty), 4);
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(smem_u32(&tfull[b]), 1);
+            mbar_init(smem_u32(&tempty[b]), kEpiWarps);
+        }
         mbar_init(smem_u32(mma_done), 1);
         *abort = 0;
         fence_mbar_init();
@@ -106,48 +181,55 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmAq, const __grid_constant__
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    const bool packed = p.T <= kTM;
+    const bool packed = p.pq > 0;
     const int nk_tot = p.nk_in + p.nk_out;
-    const int tpp = packed ? 1 : p.tiles_q * p.tiles_t;  // tile pairs per unit
+    const int nbx = (p.nk_in + p.kbx - 1) / p.kbx, nb = nbx + (p.nk_out + p.kby - 1) / p.kby;
+    // tile pairs per unit: SELF takes only i <= j
+    const int tpp = packed ? 1 : (SELF ? p.tiles_q * (p.tiles_q + 1) / 2 : p.tiles_q * p.tiles_t);
 
     if (warp == 0 && lane == 0) {
         // ---------------- TMA producer
-        uint32_t ring = 0, last_par[kStages];
-        bool issued[kStages], ok = true;
-        for (int s = 0; s < kStages; ++s) issued[s] = false;
-        for (int64_t u = blockIdx.x; ok && u < p.n_units; u += gridDim.x)
-            for (int tp = 0; ok && tp < tpp; ++tp)
-                for (int kc = 0; kc < nk_tot; ++kc, ++ring) {
-                    const int s = ring % kStages;
-                    const uint32_t ph = (ring / kStages) & 1u;
+        uint32_t s = 0, ph = 0, last_par[kMaxStages];
+        bool issued[kMaxStages], ok = true;
+        for (int i = 0; i < kMaxStages; ++i) issued[i] = false;
+        for (int64_t u = blockIdx.x; ok && u < p.n_units; u += gridDim.x) {
+            int ti = 0, tj = 0;
+            for (int tp = 0; ok && tp < tpp; ++tp) {
+                int rq, eq, rt, et;
+                if (packed) {  // rows of the [n*T][d] views
+                    rq = (int)((SELF ? u : u % p.n_qtiles) * p.pq * p.T);
+                    rt = SELF ? rq : (int)((u / p.n_qtiles) * p.pt * p.T);
+                    eq = et = 0;
+                } else {       // token tiles of one query and one train example
+                    eq = (int)(SELF ? u : u % p.n_q);
+                    et = SELF ? eq : (int)(u / p.n_q);
+                    rq = ti * kTM;
+                    rt = tj * kTN;
+                }
+                const bool one = SELF && ti == tj;  // both operands are the same tile
+                for (int kc = 0; kc < nk_tot; ++kc) {
                     if (!wait_bounded(smem_u32(&empty[s]), ph ^ 1u, abort, p.err)) {
                         ok = false;
                         break;
                     }
                     const bool side_b = kc >= p.nk_in;
                     const int d0 = (side_b ? kc - p.nk_in : kc) * kChunkK;
-                    int rq, eq, rt, et;
-                    if (packed) {  // rows of the [n*T][d] views
-                        rq = (int)((u % p.n_qtiles) * kTM);
-                        rt = (int)((u / p.n_qtiles) * kTN);
-                        eq = et = 0;
-                    } else {       // token tiles of one query and one train example
-                        eq = (int)(u % p.n_q);
-                        et = (int)(u / p.n_q);
-                        rq = (tp / p.tiles_t) * kTM;
-                        rt = (tp % p.tiles_t) * kTN;
-                    }
-                    uint8_t* st = smem + (size_t)s * kStageBytes;
-                    mbar_arrive_tx(smem_u32(&full[s]), kStageBytes);
+                    uint8_t* st = smem + (size_t)s * C::kStageBytes;
+                    mbar_arrive_tx(smem_u32(&full[s]), one ? kABytes : C::kStageBytes);
                     tma_load_3d(smem_u32(st), side_b ? &tmBq : &tmAq, d0, rq, eq, smem_u32(&full[s]));
-                    tma_load_3d(smem_u32(st + kABytes), side_b ? &tmBt : &tmAt, d0, rt, et, smem_u32(&full[s]));
+                    if (!one)
+                        tma_load_3d(smem_u32(st + kABytes), side_b ? &tmBt : &tmAt, d0, rt, et, smem_u32(&full[s]));
                     issued[s] = true;
                     last_par[s] = ph;
+                    if (++s == (uint32_t)p.stages) s = 0, ph ^= 1u;
                 }
-        for (int s = 0; s < kStages; ++s)
-            if (issued[s]) {
+                if (++tj == p.tiles_t) tj = SELF ? ++ti : (++ti, 0);
+            }
+        }
+        for (int i = 0; i < p.stages; ++i)
+            if (issued[i]) {
                 const uint64_t t0 = global_ns();
-                while (!mbar_try_wait(smem_u32(&full[s]), last_par[s]))
+                while (!mbar_try_wait(smem_u32(&full[i]), last_par[i]))
                     if (global_ns() - t0 > kTimeoutNs) {
                         atomicOr(p.err, kErrTimeout);
                         break;
@@ -155,37 +237,44 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmAq, const __grid_constant__
             }
     } else if (warp == 1 && lane == 0) {
         // ---------------- MMA issuer
-        uint32_t ring = 0, pair = 0;
+        uint32_t s = 0, ph = 0, cnt = 0;
         bool ok = true;
-        const uint32_t idesc = idesc_bf16(kTM, kTN);
-        for (int64_t u = blockIdx.x; ok && u < p.n_units; u += gridDim.x)
-            for (int tp = 0; ok && tp < tpp; ++tp, ++pair) {
-                if (!wait_bounded(smem_u32(tempty), (pair & 1u) ^ 1u, abort, p.err)) {
-                    ok = false;
-                    break;
-                }
-                tc_fence_after();
-                for (int kc = 0; kc < nk_tot; ++kc, ++ring) {
-                    const int s = ring % kStages;
-                    const uint32_t ph = (ring / kStages) & 1u;
-                    if (!wait_bounded(smem_u32(&full[s]), ph, abort, p.err)) {
+        constexpr uint32_t idesc = idesc_bf16(kTM, kTN);
+        for (int64_t u = blockIdx.x; ok && u < p.n_units; u += gridDim.x) {
+            int ti = 0, tj = 0;
+            for (int tp = 0; ok && tp < tpp; ++tp) {
+                const uint32_t boff = SELF && ti == tj ? 0u : kABytes;
+                for (int blk = 0; ok && blk < nb; ++blk, ++cnt) {
+                    const uint32_t b = cnt & 1u;
+                    if (!wait_bounded(smem_u32(&tempty[b]), ((cnt >> 1) & 1u) ^ 1u, abort, p.err)) {
                         ok = false;
                         break;
                     }
                     tc_fence_after();
-                    const bool side_b = kc >= p.nk_in;
-                    const int kk = side_b ? kc - p.nk_in : kc;
-                    uint8_t* st = smem + (size_t)s * kStageBytes;
-                    const uint64_t ad = sw128_desc(smem_u32(st)), bd = sw128_desc(smem_u32(st + kABytes));
-                    const uint32_t d_tmem = tmem + (side_b ? (uint32_t)kTN : 0u);
+                    const bool side_b = blk >= nbx;
+                    const int kb = side_b ? p.kby : p.kbx;
+                    const int left = side_b ? p.nk_out - (blk - nbx) * kb : p.nk_in - blk * kb;
+                    const int n = left < kb ? left : kb;
+                    for (int c = 0; c < n; ++c) {
+                        if (!wait_bounded(smem_u32(&full[s]), ph, abort, p.err)) {
+                            ok = false;
+                            break;
+                        }
+                        tc_fence_after();
+                        const uint32_t st = smem_u32(smem + (size_t)s * C::kStageBytes);
+                        const uint64_t ad = sw128_desc(st), bd = sw128_desc(st + boff);
 #pragma unroll
-                    for (int k = 0; k < kChunkK / 16; ++k)
-                        mma_bf16(d_tmem, ad + 2 * k, bd + 2 * k, idesc, (kk > 0 || k > 0) ? 1u : 0u);
-                    mma_commit(smem_u32(&empty[s]));
+                        for (int k = 0; k < kChunkK / 16; ++k)
+                            mma_bf16(tmem + b * 256u, ad + 2 * k, bd + 2 * k, idesc, (c > 0 || k > 0) ? 1u : 0u);
+                        mma_commit(smem_u32(&empty[s]));
+                        if (++s == (uint32_t)p.stages) s = 0, ph ^= 1u;
+                    }
+                    if (!ok) break;
+                    mma_commit(smem_u32(&tfull[b]));
                 }
-                if (!ok) break;
-                mma_commit(smem_u32(tfull));
+                if (++tj == p.tiles_t) tj = SELF ? ++ti : (++ti, 0);
             }
+        }
         mma_commit(smem_u32(mma_done));
         const uint64_t t0 = global_ns();
         while (!mbar_try_wait(smem_u32(mma_done), 0))
@@ -193,72 +282,167 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmAq, const __grid_constant__
                 atomicOr(p.err, kErrTimeout);
                 break;
             }
-    } else if (warp >= 4) {
-        // ---------------- epilogue
-        const int q4 = warp & 3, row = q4 * 32 + lane;
-        const int R = packed ? (int)p.T : kTM;   // rows per query in a tile
-        const int Cg = packed ? (int)p.T : kTN;  // columns per train example in a tile
-        const uint32_t lane_base = tmem + ((uint32_t)(q4 * 32) << 16);
-        uint32_t pair = 0;
-        bool stop = false;
+    } else if (warp >= 2) {
+        // ---------------- epilogue: warp ew covers TMEM lane quadrant warp % 4, column half h
+        const int ew = warp - 2, q4 = warp & 3, h = ew >> 2, row = q4 * 32 + lane;
+        const int et = threadIdx.x - 64, T = (int)p.T;
+        // this thread's columns [c_lo, c_lo + kCols): half the tile, or for packed T < 16 whole examples
+        const bool brief = packed && !SELF && T < 16;
+        const int c_lo = h * (brief ? kCols / T * T : kCols);
+        const int g_lo = packed && !SELF ? c_lo / T : 0;     // first train example among them
+        const uint32_t tbase = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)c_lo;
+        float* myred = red + (size_t)(h * kTM + row) * p.ldr;
+        // SELF packed: the columns of this row's own example
+        const int own = packed && SELF ? row / T * T : 0;
+        uint32_t cnt = 0;
+        bool ok = true, stop = false;
         for (int64_t u = blockIdx.x; !stop && u < p.n_units; u += gridDim.x) {
-            float pair_acc = 0.f;  // T >= 256: running sum of this (query, train) pair
-            for (int tp = 0; tp < tpp; ++tp, ++pair) {
-                bool got = true;
-                if (lane == 0) got = wait_bounded(smem_u32(tfull), pair & 1u, abort, p.err);
-                got = __shfl_sync(0xffffffffu, got, 0);
-                if (epi_any(!got)) {
-                    stop = true;
-                    break;
-                }
-                tc_fence_after();
-                float part = 0.f;
-                int g = 0;  // column group (train example within the tile)
-                for (int c0 = 0; c0 < kTN; c0 += 16) {
-                    float x[16], y[16];
-                    tmem_ld16(lane_base + c0, x);
-                    tmem_ld16(lane_base + kTN + c0, y);
+            float tot = 0.f;  // T > 128 and SELF: this thread's share of the sum
+            int ti = 0, tj = 0;
+            for (int tp = 0; tp < tpp; ++tp) {
+                float x[kCols], tile = 0.f;
 #pragma unroll
-                    for (int c = 0; c < 16; ++c) {
-                        part = fmaf(x[c], y[c], part);
-                        if (((c0 + c + 1) % Cg) == 0) {
-                            // one train example's columns done for this row
-                            if (packed) {
-                                float v = row_reduce(part, R);
-                                const int64_t qi = (u % p.n_qtiles) * (kTM / R) + row / R;
-                                const int64_t ti = (u / p.n_qtiles) * (kTN / Cg) + g;
-                                if (R <= 32) {
-                                    if ((lane & (R - 1)) == 0 && qi < p.n_q && ti < p.n_t) emit(p, qi, ti, v);
-                                } else {
-                                    // rows of one query span R / 32 warps
-                                    if (lane == 0) red[q4 * 4 + (g & 3)] = v;
-                                    epi_sync();
-                                    if (lane == 0 && (q4 % (R / 32)) == 0) {
-                                        float s = 0.f;
-                                        for (int w = 0; w < R / 32; ++w) s += red[(q4 + w) * 4 + (g & 3)];
-                                        if (qi < p.n_q && ti < p.n_t) emit(p, qi, ti, s);
-                                    }
-                                    epi_sync();
+                for (int c = 0; c < kCols; ++c) x[c] = 0.f;
+                for (int blk = 0; ok && blk < nb; ++blk, ++cnt) {
+                    const uint32_t b = cnt & 1u;
+                    if (lane == 0) ok = wait_bounded(smem_u32(&tfull[b]), (cnt >> 1) & 1u, abort, p.err);
+                    ok = __shfl_sync(0xffffffffu, ok, 0);
+                    if (!ok) break;  // the other roles see the abort flag; the barrier below ends the unit
+                    tc_fence_after();
+                    const uint32_t tb = tbase + b * 256u;
+                    if (blk < nbx) {
+#pragma unroll
+                        for (int c0 = 0; c0 < kCols; c0 += 16) {
+                            float v[16];
+                            tmem_ld16(tb + c0, v);
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) x[c0 + i] += v[i];
+                        }
+                    } else if (SELF || !packed) {
+                        // columns [c_first, c_last) of this thread's, relative to its first: the row's own
+                        // example (SELF, packed) or the tokens below T; a product left out, not
+                        // multiplied by zero, so that another example's infinity stays its own
+                        const int c_first = SELF && packed ? own - c_lo : 0;
+                        const int c_last = packed ? c_first + T : T - tj * kTN - c_lo;
+                        float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+                        for (int c0 = 0; c0 < kCols; c0 += 16) {
+                            float v[16];
+                            tmem_ld16(tb + c0, v);
+                            if (c_first <= c0 && c_last >= c0 + 16) {
+#pragma unroll
+                                for (int i = 0; i < 16; i += 2) {
+                                    s0 = fmaf(x[c0 + i], v[i], s0);
+                                    s1 = fmaf(x[c0 + i + 1], v[i + 1], s1);
                                 }
+                            } else {
+#pragma unroll
+                                for (int i = 0; i < 16; ++i)
+                                    if (c0 + i >= c_first && c0 + i < c_last) s0 = fmaf(x[c0 + i], v[i], s0);
                             }
-                            ++g;
-                            if (packed) part = 0.f;
+                        }
+                        if (packed || ti * kTM + row < T) tile += s0 + s1;
+                    } else if (brief) {
+                        const bool first = blk == nbx;
+                        switch (T) {
+#define TDA_SHORT(t) case t: y_block_short<t, kCols>(x, tb, myred, first); break;
+                            TDA_SHORT(1) TDA_SHORT(2) TDA_SHORT(3) TDA_SHORT(4) TDA_SHORT(5) TDA_SHORT(6) TDA_SHORT(7)
+                            TDA_SHORT(8) TDA_SHORT(9) TDA_SHORT(10) TDA_SHORT(11) TDA_SHORT(12) TDA_SHORT(13)
+                            TDA_SHORT(14) TDA_SHORT(15)
+#undef TDA_SHORT
+                        }
+                    } else {
+                        // packed, T >= 16: one sum per train example; left = columns to the end of the
+                        // current one, at most one end inside 16 columns
+                        const bool first = blk == nbx;
+                        float s0 = 0.f, s1 = 0.f;
+                        int left = (g_lo + 1) * T - c_lo;
+                        float* dst = myred;
+#pragma unroll
+                        for (int c0 = 0; c0 < kCols; c0 += 16) {
+                            float v[16];
+                            tmem_ld16(tb + c0, v);
+                            if (left > 16) {
+#pragma unroll
+                                for (int i = 0; i < 16; i += 2) {
+                                    s0 = fmaf(x[c0 + i], v[i], s0);
+                                    s1 = fmaf(x[c0 + i + 1], v[i + 1], s1);
+                                }
+                                left -= 16;
+                            } else {
+                                float n0 = 0.f;
+#pragma unroll
+                                for (int i = 0; i < 16; ++i) {
+                                    if (i < left)
+                                        s0 = fmaf(x[c0 + i], v[i], s0);
+                                    else
+                                        n0 = fmaf(x[c0 + i], v[i], n0);
+                                }
+                                *dst = first ? s0 + s1 : *dst + (s0 + s1);
+                                ++dst;
+                                s0 = n0;
+                                s1 = 0.f;
+                                left += T - 16;
+                            }
+                        }
+                        if (left < T) *dst = first ? s0 + s1 : *dst + (s0 + s1);  // ends in the next half
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&tempty[b]));
+                }
+                if (!ok) break;
+                tot = SELF && ti != tj ? fmaf(2.f, tile, tot) : tot + tile;  // (i, j) stands for (j, i) too
+                if (++tj == p.tiles_t) tj = SELF ? ++ti : (++ti, 0);
+            }
+            if (!packed) {
+                const float v = warp_sum(tot);
+                if (lane == 0) wsum[ew] = v;
+            } else if (SELF) {
+                myred[0] = tot;
+            }
+            stop = epi_or(!ok);
+            if (!stop) {
+                if (!packed) {
+                    if (et == 0) {
+                        float v = 0.f;
+                        for (int w = 0; w < kEpiWarps; ++w) v += wsum[w];
+                        if (SELF)
+                            emit(p, 0, u, v);
+                        else
+                            emit(p, u % p.n_q, u / p.n_q, v);
+                    }
+                } else {
+                    // output o = (query qi of the tile, train example g of the tile): T rows of partial
+                    // sums from the one or two column halves that hold the example's columns
+                    const int pt = SELF ? 1 : p.pt, nout = p.pq * pt;
+                    const int lanes = T >= 16 ? 32 : 1;  // long columns of partials: one warp each
+                    for (int o = et / lanes; o < nout; o += 32 * kEpiWarps / lanes) {
+                        const int qi = o / pt, g = o - qi * pt;
+                        // the column halves that hold example g, and the first example of each
+                        const int per = kCols / T;  // T < 16: examples per half
+                        const int h0 = SELF ? 0 : (brief ? g / per : g * T / kCols);
+                        const int h1 = SELF ? 1 : (brief ? h0 : (g * T + T - 1) / kCols);
+                        float v = 0.f;
+                        for (int hh = h0; hh <= h1; ++hh) {
+                            const int g0 = SELF ? 0 : (brief ? hh * per : hh * kCols / T);
+                            const float* r = red + (size_t)(hh * kTM + qi * T) * p.ldr + (SELF ? 0 : g - g0);
+                            for (int t = lanes > 1 ? lane : 0; t < T; t += lanes) v += r[(size_t)t * p.ldr];
+                        }
+                        if (lanes > 1) v = warp_sum(v);
+                        const int64_t qq = (SELF ? u : u % p.n_qtiles) * p.pq + qi;
+                        const int64_t ii = SELF ? 0 : (u / p.n_qtiles) * p.pt + g;
+                        if (lanes == 1 || lane == 0) {
+                            if (SELF) {
+                                if (qq < p.n_q) emit(p, 0, qq, v);
+                            } else if (qq < p.n_q && ii < p.n_t) {
+                                emit(p, qq, ii, v);
+                            }
                         }
                     }
                 }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(tempty));
-                if (!packed) {
-                    // the whole tile belongs to one (query, train) pair
-                    float v = row_reduce(part, 32);
-                    if (lane == 0) red[q4] = v;
-                    epi_sync();
-                    if (threadIdx.x == 128) pair_acc += red[0] + red[1] + red[2] + red[3];
-                    epi_sync();
-                }
             }
-            if (!stop && !packed && threadIdx.x == 128) emit(p, u % p.n_q, u / p.n_q, pair_acc);
+            epi_or(false);  // the partial sums are read: the next unit may write them
         }
     }
 
@@ -302,7 +486,77 @@ bool make_map(CUtensorMap* tm, const void* X, int64_t n, int64_t rows, int64_t d
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-bool is_pow2(int64_t v) { return v > 0 && (v & (v - 1)) == 0; }
+// Maps of one side's factors: packed rows [1][n*T][d], else [n][T][d].
+bool make_side(CUtensorMap* mA, CUtensorMap* mB, const tda_layer_desc& L, const void* A, const void* B, int64_t n,
+               bool packed, int box_rows) {
+    return packed ? make_map(mA, A, 1, n * L.T, L.d_in, box_rows) && make_map(mB, B, 1, n * L.T, L.d_out, box_rows)
+                  : make_map(mA, A, n, L.T, L.d_in, box_rows) && make_map(mB, B, n, L.T, L.d_out, box_rows);
+}
+
+// Most examples of one launch's side: 32-bit TMA row coordinates, strides below 2^40 bytes.
+int64_t max_examples(const tda_layer_desc& L, bool packed) {
+    const int64_t d_max = L.d_in > L.d_out ? L.d_in : L.d_out;
+    if (!packed) return ((int64_t)1 << 30);
+    const int64_t by_rows = ((int64_t)1 << 30) / L.T, by_stride = (((int64_t)1 << 40) - 1) / (L.T * d_max * 2);
+    return by_rows < by_stride ? by_rows : by_stride;
+}
+
+int sm_count() {
+    static std::atomic<int> sms{0};
+    int n = sms.load(std::memory_order_relaxed);
+    if (!n) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 1;
+        sms.store(n, std::memory_order_relaxed);
+    }
+    return n;
+}
+
+template <bool SELF>
+cudaError_t launch(const tda_layer_desc& L, const void* Aq, const void* Bq, int64_t n_q, const void* At,
+                   const void* Bt, int64_t n_t, GParams p, cudaStream_t s) {
+    using C = Cfg<SELF>;
+    const int64_t T = L.T;
+    const bool packed = T <= kTM;
+    CUtensorMap mAq, mAt, mBq, mBt;
+    if (!make_side(&mAq, &mBq, L, Aq, Bq, n_q, packed, kTM) ||
+        !make_side(&mAt, &mBt, L, At, Bt, n_t, packed, C::kTN))
+        return cudaErrorInvalidValue;
+    p.n_q = n_q;
+    p.n_t = n_t;
+    p.T = T;
+    p.nk_in = (int)((L.d_in + kChunkK - 1) / kChunkK);
+    p.nk_out = (int)((L.d_out + kChunkK - 1) / kChunkK);
+    // Block lengths that keep the accuracy of an fp32 FMA chain over d features (1.8e-7 at d = 256,
+    // 5.7e-7 at 2048, 8.9e-7 at 4096): 64, 128 or 256 features, whose truncation is 1.1e-7, 2.2e-7 or
+    // 4.5e-7. Short sequences (T < 16) pay the most per Y block and take it twice as long.
+    auto block = [](int nk) { return nk <= 8 ? 1 : (nk < 64 ? 2 : 4); };
+    p.kbx = block(p.nk_in);
+    p.kby = block(p.nk_out) * (packed && T < 16 ? 2 : 1);
+    p.pq = packed ? (int)(kTM / T) : 0;
+    p.pt = !packed ? 0 : (int)(T < 16 ? C::kCols / T * 2 : C::kTN / T);
+    p.tiles_q = packed ? 1 : (int)((T + kTM - 1) / kTM);
+    p.tiles_t = packed ? 1 : (int)((T + C::kTN - 1) / C::kTN);
+    p.n_qtiles = packed ? (n_q + p.pq - 1) / p.pq : 0;
+    if (SELF)
+        p.n_units = packed ? p.n_qtiles : n_q;
+    else
+        p.n_units = packed ? p.n_qtiles * ((n_t + p.pt - 1) / p.pt) : n_q * n_t;
+    // partial sums of a packed tile: rows of an odd stride (no bank conflicts)
+    p.ldr = !packed || SELF ? 1 : (int)(T < 16 ? C::kCols / T : (C::kCols - 1) / T + 2) | 1;
+    const size_t red = packed ? 2 * (size_t)kTM * p.ldr * sizeof(float) : 0;
+    const int64_t stages = ((int64_t)kSmemMax - 1024 - (int64_t)kTailBytes - (int64_t)red) / C::kStageBytes;
+    if (stages < 2) return cudaErrorInvalidValue;
+    p.stages = stages < kMaxStages ? (int)stages : kMaxStages;
+    const size_t smem = 1024 + (size_t)p.stages * C::kStageBytes + kTailBytes + red;
+    cudaError_t e = smem_attr_once<gram_tc_kernel<SELF>>((int)kSmemMax);
+    if (e != cudaSuccess) return e;
+    const int64_t grid = p.n_units < sm_count() ? p.n_units : sm_count();
+    note_launches(1);
+    gram_tc_kernel<SELF><<<(unsigned)grid, kThreads, smem, s>>>(mAq, mAt, mBq, mBt, p);
+    return cudaGetLastError();
+}
 
 }  // namespace
 
@@ -317,80 +571,53 @@ bool gram_tc_supported(const tda_layer_desc& L, tda_dtype dt, const void* Aq, co
         sm103 = (major == 10 && minor == 3) ? 1 : 0;
     }
     if (!sm103 || !encode_fn() || dt != TDA_BF16) return false;
-    if (!is_pow2(L.T) || L.T > (1 << 20) || L.d_in % 8 || L.d_out % 8) return false;
+    if (L.T < 1 || L.T > (1 << 20) || L.d_in % 8 || L.d_out % 8 || L.d_in > (1LL << 30) || L.d_out > (1LL << 30))
+        return false;
+    if (max_examples(L, L.T <= kTM) < kTM) return false;
     for (const void* x : {Aq, Bq, At, Bt})
         if ((uintptr_t)x & 15) return false;
     return true;
 }
 
-// S[q][i] = beta * S[q][i] + alpha * <DW_q, DW_i>_F for bf16 factors.
+// S[q][i] = beta * S[q][i] + alpha * <DW_q, DW_i>_F for bf16 factors. A side with more examples
+// than one launch addresses goes in pieces, each its own block of S.
 cudaError_t launch_gram_tc(const tda_layer_desc& L, const void* Aq, const void* Bq, int64_t n_q, const void* At,
                            const void* Bt, int64_t n_t, float* S, int64_t ld_S, float beta, float alpha,
                            unsigned int* err, cudaStream_t s) {
-    if (n_q == 0 || n_t == 0) return cudaSuccess;
-    const int64_t T = L.T;
-    const bool packed = T <= kTM;
-    const int64_t d_max = L.d_in > L.d_out ? L.d_in : L.d_out;
-    if (packed) {
-        // 32-bit TMA row coordinates and strides below 2^40 bytes: split the train side
-        int64_t max_t = ((int64_t)1 << 30) / T;
-        const int64_t by_stride = (((int64_t)1 << 40) - 1) / (T * d_max * 2);
-        if (by_stride < max_t) max_t = by_stride;
-        max_t = max_t / (kTN / T) * (kTN / T);
-        if (n_q * T >= ((int64_t)1 << 30) || n_q > by_stride || max_t < 1) return cudaErrorInvalidValue;
-        if (n_t > max_t) {
-            for (int64_t i0 = 0; i0 < n_t; i0 += max_t) {
-                const int64_t n = n_t - i0 < max_t ? n_t - i0 : max_t;
-                cudaError_t e = launch_gram_tc(L, Aq, Bq, n_q, (const char*)At + i0 * T * L.d_in * 2,
-                                               (const char*)Bt + i0 * T * L.d_out * 2, n, S + i0, ld_S, beta,
-                                               alpha, err, s);
-                if (e != cudaSuccess) return e;
-            }
-            return cudaSuccess;
-        }
-    }
-    CUtensorMap mAq, mAt, mBq, mBt;
-    bool ok;
-    if (packed)
-        ok = make_map(&mAq, Aq, 1, n_q * T, L.d_in, kTM) && make_map(&mAt, At, 1, n_t * T, L.d_in, kTN) &&
-             make_map(&mBq, Bq, 1, n_q * T, L.d_out, kTM) && make_map(&mBt, Bt, 1, n_t * T, L.d_out, kTN);
-    else
-        ok = make_map(&mAq, Aq, n_q, T, L.d_in, kTM) && make_map(&mAt, At, n_t, T, L.d_in, kTN) &&
-             make_map(&mBq, Bq, n_q, T, L.d_out, kTM) && make_map(&mBt, Bt, n_t, T, L.d_out, kTN);
-    if (!ok) return cudaErrorInvalidValue;
-    GParams p;
-    p.n_q = n_q;
-    p.n_t = n_t;
-    p.T = T;
-    p.ld_S = ld_S;
-    p.nk_in = (int)((L.d_in + kChunkK - 1) / kChunkK);
-    p.nk_out = (int)((L.d_out + kChunkK - 1) / kChunkK);
-    p.tiles_q = packed ? 1 : (int)(T / kTM);
-    p.tiles_t = packed ? 1 : (int)(T / kTN);
-    if (packed) {
-        p.n_qtiles = (n_q * T + kTM - 1) / kTM;
-        p.n_units = p.n_qtiles * ((n_t * T + kTN - 1) / kTN);
-    } else {
-        p.n_qtiles = 0;
-        p.n_units = n_q * n_t;
-    }
+    const int64_t most = max_examples(L, L.T <= kTM);
+    const size_t a_ex = (size_t)L.T * L.d_in * 2, b_ex = (size_t)L.T * L.d_out * 2;
+    GParams p = {};
     p.alpha = alpha;
     p.beta = beta;
-    p.S = S;
+    p.ld_S = ld_S;
     p.err = err;
-    static int sms = 0;
-    if (!sms) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (sms <= 0) sms = 1;
+    for (int64_t q0 = 0; q0 < n_q; q0 += most)
+        for (int64_t i0 = 0; i0 < n_t; i0 += most) {
+            p.S = S + q0 * ld_S + i0;
+            cudaError_t e = launch<false>(L, (const char*)Aq + q0 * a_ex, (const char*)Bq + q0 * b_ex,
+                                          n_q - q0 < most ? n_q - q0 : most, (const char*)At + i0 * a_ex,
+                                          (const char*)Bt + i0 * b_ex, n_t - i0 < most ? n_t - i0 : most, p, s);
+            if (e != cudaSuccess) return e;
+        }
+    return cudaSuccess;
+}
+
+// out[i] = ||DW_i||_F^2 for bf16 factors.
+cudaError_t launch_gram_self_tc(const tda_layer_desc& L, const void* A, const void* B, int64_t n, float* out,
+                                unsigned int* err, cudaStream_t s) {
+    const int64_t most = max_examples(L, L.T <= kTM);
+    const size_t a_ex = (size_t)L.T * L.d_in * 2, b_ex = (size_t)L.T * L.d_out * 2;
+    GParams p = {};
+    p.alpha = 1.f;
+    p.err = err;
+    for (int64_t i0 = 0; i0 < n; i0 += most) {
+        const char *a = (const char*)A + i0 * a_ex, *b = (const char*)B + i0 * b_ex;
+        const int64_t c = n - i0 < most ? n - i0 : most;
+        p.S = out + i0;
+        cudaError_t e = launch<true>(L, a, b, c, a, b, c, p, s);
+        if (e != cudaSuccess) return e;
     }
-    cudaError_t e = cudaFuncSetAttribute(gram_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
-    if (e != cudaSuccess) return e;
-    const int64_t grid = p.n_units < sms ? p.n_units : sms;
-    note_launches(1);
-    gram_tc_kernel<<<(unsigned)grid, kThreads, kSmem, s>>>(mAq, mAt, mBq, mBt, p);
-    return cudaGetLastError();
+    return cudaSuccess;
 }
 
 }  // namespace tda

@@ -138,12 +138,14 @@ cudaError_t launch_similarity_materialized(const tda_layer_desc& L, tda_dtype dt
                                            const void* Bq, int64_t n_q, const void* At,
                                            const void* Bt, int64_t n_t, float* S, int64_t ld_S,
                                            float beta, void* ws, size_t ws_bytes, cudaStream_t s);
-// Route (c) on tcgen05 for bf16 factors with T a power of two (k_gram_tc.cu).
+// Route (c) and exact norms on tcgen05 for bf16 factors (k_gram_tc.cu).
 bool gram_tc_supported(const tda_layer_desc& L, tda_dtype dt, const void* Aq, const void* Bq, const void* At,
                        const void* Bt);
 cudaError_t launch_gram_tc(const tda_layer_desc& L, const void* Aq, const void* Bq, int64_t n_q, const void* At,
                            const void* Bt, int64_t n_t, float* S, int64_t ld_S, float beta, float alpha,
                            unsigned int* err, cudaStream_t s);
+cudaError_t launch_gram_self_tc(const tda_layer_desc& L, const void* A, const void* B, int64_t n, float* out,
+                                unsigned int* err, cudaStream_t s);
 cudaError_t launch_similarity_gram(const tda_layer_desc& L, tda_dtype dt, const void* Aq,
                                    const void* Bq, int64_t n_q, const void* At, const void* Bt,
                                    int64_t n_t, float* S, int64_t ld_S, float beta, cudaStream_t s);
