@@ -132,6 +132,7 @@ struct Params {
     unsigned int* err;
     int n_ttiles;     // token tiles per slot
     int pack;         // examples per token tile (T <= 64), else 1
+    int k_in, k_out;  // projection sizes (ODD: below K or different per side)
     int nk_in, nk_out;
     int cs;           // CTAs per cluster sharing one example's token tiles (1, 2 or 4)
     float* cov;       // K-FAC: per-CTA partial sums of At^T At and Bt^T Bt ([grid][2][K*K])
@@ -219,12 +220,29 @@ __device__ __forceinline__ void write_sign_half(uint8_t* tile, int n, uint64_t w
     }
 }
 
+// This thread's rows rg*RB.. and columns cg*CB.. of an example's Phi, scaled. ODD: Phi is
+// k_out x k_in, smaller than the K x K block that the tiles are padded to.
+template <class C, bool ODD>
+__device__ __forceinline__ void write_phi(const float (&v)[C::RB][C::CB], float* out, int rg, int cg, const Params& p) {
+    constexpr int K = C::kK;
+#pragma unroll
+    for (int a = 0; a < C::RB; ++a)
+#pragma unroll
+        for (int c = 0; c < C::CB; ++c) {
+            const int i = rg * C::RB + a, j = cg * C::CB + c;
+            if (!ODD)
+                out[i * K + j] = v[a][c] * p.scale;
+            else if (i < p.k_out && j < p.k_in)
+                out[i * p.k_in + j] = v[a][c] * p.scale;
+        }
+}
+
 // Phi of example n (K x K partial sums in acc, thread et holding rows
 // rg*RB.. and columns cg*CB..) is complete in every CTA of the cluster: reduce
 // the members' blocks into the leader (rank 0) over distributed shared memory
 // and write it, scaled. The leader's staging rows (free between tiles) receive
 // member r's block at offset (r-1)*K*K floats, thread-major.
-template <class C>
+template <class C, bool ODD>
 __device__ __forceinline__ bool store_phi(float (&acc)[C::RB][C::CB], int64_t n, const Params& p, uint32_t crank,
                                           float* stage, uint64_t* red_go, uint64_t* red_full, uint32_t& red_use,
                                           volatile int* abort, int et, int lane) {
@@ -264,11 +282,7 @@ __device__ __forceinline__ bool store_phi(float (&acc)[C::RB][C::CB], int64_t n,
         ++red_use;
         if (crank != 0) return true;
     }
-    float* out = p.phi + n * p.ld_phi;
-#pragma unroll
-    for (int a = 0; a < C::RB; ++a)
-#pragma unroll
-        for (int c = 0; c < C::CB; ++c) out[(rg * C::RB + a) * K + cg * C::CB + c] = acc[a][c] * p.scale;
+    write_phi<C, ODD>(acc, p.phi + n * p.ld_phi, rg, cg, p);
     return true;
 }
 
@@ -367,7 +381,9 @@ __device__ __forceinline__ void store_sign_row(uint8_t* tile, int n, const uint4
 // factors At, Bt of every token instead of contracting them into Phi. SL: the
 // sign tiles come by TMA from a precomputed table (tmSA, tmSB: [K][d] bf16, a
 // side's S transposed) instead of the generator warps.
-template <int K, int G, bool KF, bool FO, bool SL = false, int SR = Cfg<K, G>::kStageRows, bool BAL = false>
+// ODD: k_in and k_out differ or are below K (the sign columns past them are computed and not written).
+template <int K, int G, bool KF, bool FO, bool SL = false, int SR = Cfg<K, G>::kStageRows, bool BAL = false,
+          bool ODD = false>
 __global__ void __launch_bounds__(kThreads, 1)
 project_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                   const __grid_constant__ CUtensorMap tmSA, const __grid_constant__ CUtensorMap tmSB,
@@ -629,7 +645,7 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             } while (ng > 0 && gx[u] == cur);
             if constexpr (BAL) {
                 if (ok) store_phi_bal<C>(acc, cur, p, et, abort + 1);
-            } else if (ok && !store_phi<C>(acc, cur, p, crank, stX, red_go, red_full, red_use, abort, et, lane)) {
+            } else if (ok && !store_phi<C, ODD>(acc, cur, p, crank, stX, red_go, red_full, red_use, abort, et, lane)) {
                 ok = false;
             }
         }
@@ -656,52 +672,9 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                 for (int c = 0; c < C::CB; ++c) ca[a][c] = cgm[a][c] = 0.f;
         }
 
-        // Phi of example `n` is complete in every cluster CTA: reduce the partial
-        // blocks into the leader (rank 0) over distributed shared memory and
-        // write it. The leader's staging buffer (free between tiles) receives
-        // member r's partial at offset (r-1)*K*K, thread-major.
+        // Phi of example `n` is complete in every cluster CTA
         auto flush = [&](int64_t n) -> bool {
-            if (p.cs > 1) {
-                constexpr int kPer = C::RB * C::CB;
-                const uint32_t slot = smem_u32(stX) + (uint32_t)(et * kPer) * 4u;
-                bool got = true;
-                if (crank == 0) {
-                    if (et == 0)
-                        for (int r = 1; r < p.cs; ++r) mbar_arrive_remote(smem_u32(red_go), (uint32_t)r);
-                    if (lane == 0) got = wait_bounded_cluster(smem_u32(red_full), red_use & 1u, abort, p.err);
-                    got = __shfl_sync(0xffffffffu, got, 0);
-                    if (epi_any(!got)) return false;
-                    for (int r = 1; r < p.cs; ++r) {
-                        const float* part = stX + (r - 1) * K * K + et * kPer;
-#pragma unroll
-                        for (int a = 0; a < C::RB; ++a)
-#pragma unroll
-                            for (int c = 0; c < C::CB; ++c) acc[a][c] += part[a * C::CB + c];
-                    }
-                    epi_sync();  // partials consumed; staging free for the next tile
-                } else {
-                    if (lane == 0) got = wait_bounded_cluster(smem_u32(red_go), red_use & 1u, abort, p.err);
-                    got = __shfl_sync(0xffffffffu, got, 0);
-                    if (epi_any(!got)) return false;
-                    const uint32_t dst = map_rank(slot, 0) + (crank - 1) * (uint32_t)(K * K) * 4u;
-#pragma unroll
-                    for (int a = 0; a < C::RB; ++a)
-#pragma unroll
-                        for (int c = 0; c < C::CB; ++c)
-                            st_cluster_f32(dst + (uint32_t)(a * C::CB + c) * 4u, acc[a][c]);
-                    fence_acq_rel_cluster();
-                    epi_sync();
-                    if (et == 0) mbar_arrive_remote(smem_u32(red_full), 0u);
-                }
-                ++red_use;
-                if (crank != 0) return true;
-            }
-            float* out = p.phi + n * p.ld_phi;
-#pragma unroll
-            for (int a = 0; a < C::RB; ++a)
-#pragma unroll
-                for (int c = 0; c < C::CB; ++c) out[(rg * C::RB + a) * K + cg * C::CB + c] = acc[a][c] * p.scale;
-            return true;
+            return store_phi<C, ODD>(acc, n, p, crank, stX, red_go, red_full, red_use, abort, et, lane);
         };
 
         for (int ng; !stop && (ng = it.take<G>(p, ncl, crank, gx, gt)) > 0; ++grp) {
@@ -830,12 +803,7 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 #pragma unroll
                                 for (int c = 0; c < C::CB; ++c) a2[a][c] = fmaf(y[a], x[c], a2[a][c]);
                         }
-                        float* out = p.phi + e * p.ld_phi;
-#pragma unroll
-                        for (int a = 0; a < C::RB; ++a)
-#pragma unroll
-                            for (int c = 0; c < C::CB; ++c)
-                                out[(rg * C::RB + a) * K + cg * C::CB + c] = a2[a][c] * p.scale;
+                        write_phi<C, ODD>(a2, p.phi + e * p.ld_phi, rg, cg, p);
                     }
                 }
                 epi_sync();
@@ -967,7 +935,8 @@ int sm_count() {
     return (b > 0 && b < sms) ? b : sms;
 }
 
-template <int K, int G, bool KF, bool FO, bool SL = false, int SR = Cfg<K, G>::kStageRows, bool BAL = false>
+template <int K, int G, bool KF, bool FO, bool SL = false, int SR = Cfg<K, G>::kStageRows, bool BAL = false,
+          bool ODD = false>
 cudaError_t launch_kg(const tda_layer_desc& L, const void* A, const void* B, int64_t N, float* phi,
                       int64_t ld_phi, unsigned int* err, cudaStream_t s, int pack, float* cov, int* grid_out,
                       float* fout, const void* signs = nullptr, void* bal_ws = nullptr) {
@@ -997,6 +966,8 @@ cudaError_t launch_kg(const tda_layer_desc& L, const void* A, const void* B, int
     p.ld_phi = ld_phi;
     p.pack = pack;
     p.n_slots = pack > 1 ? (N + pack - 1) / pack : N;
+    p.k_in = L.k_in;
+    p.k_out = L.k_out;
     p.key_in = side_key(L.seed, L.layer, 0);
     p.key_out = side_key(L.seed, L.layer, 1);
     p.scale = projection_scale(L);
@@ -1011,7 +982,7 @@ cudaError_t launch_kg(const tda_layer_desc& L, const void* A, const void* B, int
     p.part = nullptr;
     p.cnt = nullptr;
     const int sms = sm_count();
-    cudaError_t e = smem_attr_once<project_tc_kernel<K, G, KF, FO, SL, SR, BAL>>((int)C::kSmem);
+    cudaError_t e = smem_attr_once<project_tc_kernel<K, G, KF, FO, SL, SR, BAL, ODD>>((int)C::kSmem);
     if (e != cudaSuccess) return e;
     // Fewer examples than SMs: a cluster of cs CTAs shares each example's token
     // tiles and reduces the partial features through distributed shared memory.
@@ -1031,7 +1002,7 @@ cudaError_t launch_kg(const tda_layer_desc& L, const void* A, const void* B, int
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     cfg.gridDim = dim3((unsigned)(cs * (device_sms() / cs)));
-    int max_clusters = max_clusters_once<project_tc_kernel<K, G, KF, FO, SL, SR, BAL>>(cfg, cs, sms / cs);
+    int max_clusters = max_clusters_once<project_tc_kernel<K, G, KF, FO, SL, SR, BAL, ODD>>(cfg, cs, sms / cs);
     if (max_clusters > sms / cs) max_clusters = sms / cs;  // the SM budget (the occupancy query sees every SM)
     int64_t clusters = (FO || BAL) ? p.n_units : p.n_slots;
     if (clusters > max_clusters) clusters = max_clusters;
@@ -1045,14 +1016,14 @@ cudaError_t launch_kg(const tda_layer_desc& L, const void* A, const void* B, int
         if (e != cudaSuccess) return e;
     }
     note_launches(1);
-    e = cudaLaunchKernelEx(&cfg, project_tc_kernel<K, G, KF, FO, SL, SR, BAL>, tmA, tmB, tmSA, tmSB, p);
+    e = cudaLaunchKernelEx(&cfg, project_tc_kernel<K, G, KF, FO, SL, SR, BAL, ODD>, tmA, tmB, tmSA, tmSB, p);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 
 // Two tiles per stage once every CTA has at least two groups of work; fewer
 // units run one tile per stage so that they spread over all SMs.
-template <int K, bool KF, bool FO>
+template <int K, bool KF, bool FO, bool ODD = false>
 cudaError_t launch_k(const tda_layer_desc& L, const void* A, const void* B, int64_t N, float* phi,
                      int64_t ld_phi, unsigned int* err, cudaStream_t s, float* cov, int* grid_out, float* fout,
                      const void* signs = nullptr, void* bal_ws = nullptr) {
@@ -1072,7 +1043,7 @@ cudaError_t launch_k(const tda_layer_desc& L, const void* A, const void* B, int6
             const size_t a_ex = (size_t)L.T * L.d_in * 2, b_ex = (size_t)L.T * L.d_out * 2;
             for (int64_t e0 = 0; e0 < N; e0 += max_n) {
                 const int64_t n = N - e0 < max_n ? N - e0 : max_n;
-                cudaError_t e = launch_k<K, KF, FO>(L, (const char*)A + e0 * a_ex, (const char*)B + e0 * b_ex, n,
+                cudaError_t e = launch_k<K, KF, FO, ODD>(L, (const char*)A + e0 * a_ex, (const char*)B + e0 * b_ex, n,
                                                     phi + e0 * ld_phi, ld_phi, err, s, nullptr, nullptr, nullptr,
                                                     signs, bal_ws);
                 if (e != cudaSuccess) return e;
@@ -1086,6 +1057,14 @@ cudaError_t launch_k(const tda_layer_desc& L, const void* A, const void* B, int6
     // well for k >= 64 (k <= 32 measured faster with whole tiles: 7.1-7.3 against 6.9 TB/s on
     // the Llama-1B block); fewer examples keep the larger staging rows, which hold the cluster's
     // partial blocks.
+    if constexpr (ODD) {
+        if constexpr (K <= 64)
+            if ((pack > 1 ? (N + pack - 1) / pack : N * ((L.T + kTileM - 1) / kTileM)) >= 4 * (int64_t)sm_count())
+                return launch_kg<K, 2, false, false, false, Cfg<K, 2>::kStageRows, false, true>(
+                    L, A, B, N, phi, ld_phi, err, s, pack, cov, grid_out, fout);
+        return launch_kg<K, 1, false, false, false, Cfg<K, 1>::kStageRows, false, true>(L, A, B, N, phi, ld_phi, err, s,
+                                                                                       pack, cov, grid_out, fout);
+    }
     const bool bal = bal_ws && pack == 1;
     const bool narrow = K >= 64 && pack == 1 && N >= (int64_t)sm_count();
     if constexpr (K > 64) {
@@ -1142,15 +1121,19 @@ bool project_tc_supported(const tda_layer_desc& L, const void* A, const void* B)
     return true;
 }
 
-// The plain projection also runs k = 128 on the tensor cores (the fused K-FAC
-// covariances and the factor output stay at k <= 64).
+// The block edge K that a projection of k_in x k_out features is padded to.
+int padded_k(const tda_layer_desc& L) {
+    const int k = L.k_in > L.k_out ? L.k_in : L.k_out;
+    return k <= 16 ? 16 : (k <= 32 ? 32 : (k <= 64 ? 64 : 128));
+}
+
+// The plain projection runs every k_in, k_out up to 128 on the tensor cores (the fused
+// K-FAC covariances and the factor output stay at k_in = k_out in {16, 32, 64}).
 bool project_tc_plain_supported(const tda_layer_desc& L, const void* A, const void* B) {
-    if (L.k_in == 128 && L.k_out == 128) {
-        tda_layer_desc L64 = L;
-        L64.k_in = L64.k_out = 64;
-        return project_tc_supported(L64, A, B);
-    }
-    return project_tc_supported(L, A, B);
+    if (L.k_in < 1 || L.k_out < 1 || L.k_in > 128 || L.k_out > 128) return false;
+    tda_layer_desc L64 = L;
+    L64.k_in = L64.k_out = 64;
+    return project_tc_supported(L64, A, B);
 }
 
 size_t project_tc_sign_table_bytes(const tda_layer_desc& L) {
@@ -1176,6 +1159,17 @@ cudaError_t launch_project_tc(const tda_layer_desc& L, const void* A, const void
     if (ws && ((uintptr_t)ws & 255)) ws = nullptr;
     const size_t sign_b = (project_tc_sign_table_bytes(L) + 255) / 256 * 256;
     void* bal_ws = (ws && ws_bytes >= project_tc_ws_bytes(L)) ? (char*)ws + sign_b : nullptr;
+    // Unequal or other k: the kernel of the next block edge, which computes K columns per side and
+    // writes k_out x k_in of them. Streaming the factors stays the bound (1000 -> 2056, T = 130,
+    // 32 x 48, 96 examples: 1516 us on the CUDA cores, 80 us here).
+    if (L.k_in != L.k_out || L.k_in != padded_k(L)) {
+        switch (padded_k(L)) {
+            case 16: return launch_k<16, false, false, true>(L, A, B, N, phi, ld_phi, err, s, nullptr, nullptr, nullptr);
+            case 32: return launch_k<32, false, false, true>(L, A, B, N, phi, ld_phi, err, s, nullptr, nullptr, nullptr);
+            case 64: return launch_k<64, false, false, true>(L, A, B, N, phi, ld_phi, err, s, nullptr, nullptr, nullptr);
+            default: return launch_k<128, false, false, true>(L, A, B, N, phi, ld_phi, err, s, nullptr, nullptr, nullptr);
+        }
+    }
     switch (L.k_in) {
         case 16: return launch_k<16, false, false>(L, A, B, N, phi, ld_phi, err, s, nullptr, nullptr, nullptr, nullptr, bal_ws);
         case 32: return launch_k<32, false, false>(L, A, B, N, phi, ld_phi, err, s, nullptr, nullptr, nullptr, nullptr, bal_ws);

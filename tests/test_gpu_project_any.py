@@ -1,0 +1,61 @@
+"""The tensor-core projection at projection sizes that no tile edge matches (k_in != k_out, k below the padded block)
+and the shapes where its loops can go wrong: packed short sequences, tokens past a tile, widths past a K chunk, one
+example over a cluster, more units than SMs; and the factor output's work split (token scores) at few long examples.
+Tolerance: bf16 factors are exact in fp32 and both contractions accumulate in fp32, so the repository's fp32
+tolerance (1e-5 relative, per example) holds."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2609_38767_gb300 as tda
+from paper_2609_38767_gb300 import build as tbuild
+from paper_2609_38767_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-5
+TD = {"f32": tda.TDA_F32, "bf16": tda.TDA_BF16}
+
+
+@pytest.fixture(scope="module")
+def dev():
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    tbuild.build()
+    tda.load()
+    return torch.device("cuda:0")
+
+
+def factors(n, T, di, do, dtype, stream):
+    A = synth.factors(synth.SEED_A, stream, n, T, di, 1.0, 0, 0, dtype, 0.02)
+    B = synth.factors(synth.SEED_B, stream, n, T, do, 0.1, 0, 0, dtype, 0.02)
+    return A, B
+
+
+def up(x, dtype, dev):
+    if dtype == "bf16":
+        return torch.from_numpy(x.view(np.int16)).view(torch.bfloat16).to(dev)
+    return torch.from_numpy(x).to(dev)
+
+
+def rel(x, ref):
+    x = np.asarray(x, dtype=np.float64)
+    return float(np.linalg.norm(x - ref) / max(np.linalg.norm(ref), 1e-300))
+
+
+@pytest.mark.parametrize("N,T,di,do,ki,ko", [
+    (3, 7, 72, 64, 8, 8), (700, 5, 64, 72, 1, 5), (5, 45, 200, 136, 24, 24), (9, 130, 1000, 2056, 32, 48),
+    (2, 300, 64, 128, 16, 64), (3, 64, 136, 64, 100, 72), (160, 200, 72, 64, 48, 33), (1, 520, 64, 64, 64, 8),
+    (4, 129, 64, 200, 128, 96)])
+def test_tc_projection_any_k(dev, orc, N, T, di, do, ki, ko):
+    A, B = factors(N, T, di, do, "bf16", 61)
+    L = tda.LayerDesc(di, do, T, ki, ko, seed=7, layer=2)
+    Ad, Bd = up(A, "bf16", dev), up(B, "bf16", dev)
+    assert tda.tda_project_engine(L, tda.TDA_BF16, Ad, Bd) == 1
+    ld = ki * ko + 3
+    phi = torch.full((N, ld), 7.0, device=dev)
+    ws = torch.empty(64 << 20, dtype=torch.uint8, device=dev)  # offered, not needed
+    tda.tda_project(L, tda.TDA_BF16, Ad, Bd, N, phi, ld, tda.TDA_ROUTE_FACTORED, ws, 64 << 20)
+    tda.tda_device_status()
+    got = phi.cpu().numpy()
+    assert (got[:, ki * ko:] == 7.0).all()
+    ref = orc.project(synth.to_f64(A, "bf16"), synth.to_f64(B, "bf16"), ki, ko, 7, 2).reshape(N, -1)
+    assert max(rel(got[n, :ki * ko], ref[n]) for n in range(N)) <= TOL
