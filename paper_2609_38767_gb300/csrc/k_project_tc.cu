@@ -439,7 +439,10 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     const int nk_tot = p.nk_in + p.nk_out;
     int64_t gx[G];
     int gt[G];
-    typename std::conditional<BAL, TileRange, Units>::type it;
+    // FO writes every token's factors and needs no example whole: equal runs of token tiles, so that
+    // a few long examples fill the chip (16 examples of 1024 tokens, 4096 + 4096 wide, k = 64: 128 CTAs
+    // instead of 16, 525 -> 68 us)
+    typename std::conditional<BAL || FO, TileRange, Units>::type it;
     it.first(p, cid, crank);
 
     if (warp == 0 && lane == 0) {

@@ -59,3 +59,23 @@ def test_tc_projection_any_k(dev, orc, N, T, di, do, ki, ko):
     assert (got[:, ki * ko:] == 7.0).all()
     ref = orc.project(synth.to_f64(A, "bf16"), synth.to_f64(B, "bf16"), ki, ko, 7, 2).reshape(N, -1)
     assert max(rel(got[n, :ki * ko], ref[n]) for n in range(N)) <= TOL
+
+
+@pytest.mark.parametrize("N,T,di,do,k,nq", [(1, 1024, 64, 72, 64, 3), (16, 300, 136, 64, 32, 2), (200, 9, 64, 64, 16, 5),
+                                            (3, 130, 64, 64, 64, 1)])
+def test_token_scores_work_split(dev, orc, N, T, di, do, k, nq):
+    A, B = factors(N, T, di, do, "bf16", 62)
+    L = tda.LayerDesc(di, do, T, k, k, seed=7, layer=1)
+    R = np.random.default_rng(N).standard_normal((nq, k * k)).astype(np.float32)
+    wsb = tda.tda_token_scores_workspace_size(L) * N + (1 << 20)
+    ws = torch.empty(wsb, dtype=torch.uint8, device=dev)
+    out = torch.empty((nq, N * T), device=dev)
+    tda.tda_token_scores(L, tda.TDA_BF16, up(A, "bf16", dev), up(B, "bf16", dev), N, torch.from_numpy(R).to(dev), nq,
+                         k * k, out, N * T, 0.0, ws, wsb)
+    tda.tda_device_status()
+    # sum over a token's example gives <Phi_i, R_j>; the decomposition itself from the projected factors
+    Si = orc.proj_entries(7, 1, 0, di, k).astype(np.float64) / np.sqrt(k)
+    So = orc.proj_entries(7, 1, 1, do, k).astype(np.float64) / np.sqrt(k)
+    a, b = synth.to_f64(A, "bf16") @ Si, synth.to_f64(B, "bf16") @ So
+    ref = np.stack([np.einsum("ntr,rc,ntc->nt", b, R[j].reshape(k, k).astype(np.float64), a).ravel() for j in range(nq)])
+    assert rel(out.cpu().numpy(), ref) <= TOL
