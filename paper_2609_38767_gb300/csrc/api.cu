@@ -320,6 +320,16 @@ tda_status tda_project(const tda_layer_desc* L, tda_dtype dtype, const void* A, 
             if (!err) return fail(TDA_ERR_CUDA, "cannot resolve the device error word");
             return cuda_check(launch_project_tc(*L, A, B, N, phi, ld_phi, err, s, ws, ws_bytes), "project (tcgen05)");
         }
+        // fp32 factors: short jobs of narrow layers on the CUDA cores (one launch of a few us, against
+        // ten on the tensor cores), the rest on the tensor cores
+        if (dtype == TDA_F32 && project_small_supported(*L, A, B, N))
+            return cuda_check(launch_project_small(*L, A, B, N, phi, ld_phi, s), "project (small)");
+        if (dtype == TDA_F32 && project_f32_tc_supported(*L, A, B)) {
+            unsigned int* err = device_error_word();
+            if (!err) return fail(TDA_ERR_CUDA, "cannot resolve the device error word");
+            const cudaError_t e = launch_project_f32_tc(*L, A, B, N, phi, ld_phi, err, s);
+            if (e != cudaErrorNotSupported) return cuda_check(e, "project (tcgen05, fp32 factors)");
+        }
         return cuda_check(launch_project_simt(*L, dtype, A, B, N, phi, ld_phi, s), "project (simt)");
     }
     if (route == TDA_ROUTE_MATERIALIZE) {
@@ -336,7 +346,7 @@ tda_status tda_project(const tda_layer_desc* L, tda_dtype dtype, const void* A, 
 int32_t tda_project_engine(const tda_layer_desc* L, tda_dtype dtype, const void* A, const void* B) {
     g_msg[0] = 0;
     if (validate_layer(L, true) || validate_factors(L, dtype, A, B, 1, "tda_project_engine")) return -1;
-    return (dtype == TDA_BF16 && project_tc_plain_supported(*L, A, B)) ? 1 : 0;
+    return (dtype == TDA_BF16 ? project_tc_plain_supported(*L, A, B) : project_f32_tc_supported(*L, A, B)) ? 1 : 0;
 }
 
 tda_status tda_similarity_exact(const tda_layer_desc* L, tda_dtype dtype, const void* Aq,

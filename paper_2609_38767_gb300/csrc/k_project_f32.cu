@@ -1,0 +1,728 @@
+// k_project_f32.cu -- factored projection (Eq. 2) of fp32 factors on the
+// tcgen05 tensor cores, exact to fp32 rounding, for any k_in, k_out up to 64.
+//
+// Every fp32 value is cut into three bf16 pieces, x = h + m + l (8 significant
+// bits each, by truncation: h + m + l = x exactly), and the signs S are +-1, so
+// the products h S, m S, l S are exact and only sums round. At = A S_in keeps
+// two fp32 accumulators, sum h S and sum (m + l) S: within one, the terms are
+// so coarse against its ulp that the tensor pipe's truncating additions lose
+// almost nothing (2048 features: 1.2e-6 off with an fp32 chain on the CUDA
+// cores, 2e-7 here). The epilogue adds the two with round-to-nearest and
+// contracts Phi += Bt^T At over the tokens in fp32, as the bf16 kernel does.
+//
+// Pieces go to TMEM, not to shared memory: the MMA takes its A operand from
+// TMEM (a lane per token, two bf16 features per column), the split warps read
+// each TMA-written fp32 row once (a thread per token row: the 128-byte swizzle
+// makes its 16-byte loads conflict-free) and write three pieces with
+// tcgen05.st. Shared memory carries 8 bytes per value instead of 20 (write,
+// read, three pieces written and read), which at HBM speed (5.4 values a clock
+// and SM) would exceed its 128 bytes a clock.
+//
+// Measured: 64 examples of 512 tokens, 2048 -> 2048, k = 32 (537 MB): 7.6 ms on the
+// CUDA cores, 136 us here = 3.9 TB/s; 128 of 152 SMs have two tiles each.
+//
+// Token tiles of R = 128, 64 or 32 rows and clusters of 1 to 8 CTAs that share
+// an example's tiles, chosen by a model of the chunk time (plan()): few examples
+// fill the chip with smaller tiles and larger clusters. T <= R packs floor(R/T)
+// whole examples in a tile. The members' partial blocks are reduce-scattered
+// over distributed shared memory: every CTA sums and writes 1/cs of Phi.
+//
+// Warp roles (512 threads, one persistent CTA per SM): warp 0 TMA producer
+// (32-feature boxes of fp32, two per 64-feature chunk); warp 1 TMEM allocator
+// and MMA issuer; warps 2-3 sign generators (byte -> eight bf16 signs from a
+// table, as for k = 128 in the bf16 kernel); warps 4-7 epilogue; warps 8-15
+// split. Every wait is bounded (about 1 s); on expiry the kernel records
+// kErrTimeout, drains its copies, frees its TMEM and returns.
+#include <cuda.h>
+
+#include <mutex>
+
+#include "tda_internal.cuh"
+
+namespace tda {
+namespace {
+
+constexpr int kThreads = 512;
+constexpr int kTileM = 128;   // MMA M
+constexpr int kChunkK = 64;   // features per stage (two 32-feature fp32 boxes)
+constexpr uint32_t kBoxBytes = kTileM * 128;  // room of one 32-feature box
+constexpr size_t kSmemMax = 232448;
+constexpr int kMaxStages = 6;
+constexpr int kSR = 64;       // token rows staged at a time
+constexpr int kPieceCols = kChunkK / 2;       // TMEM columns of one piece of a chunk
+constexpr int kACols = 3 * kPieceCols;
+constexpr int kABufs = 2;
+constexpr size_t kLutBytes = 256 * 16;
+
+template <int K>
+struct Cfg {
+    static constexpr uint32_t kSignBytes = K * 128;
+    static constexpr uint32_t kStageBytes = 2 * kBoxBytes + kSignBytes;
+    static constexpr int kBufCols = 4 * K;                 // At: h, m+l; Bt: h, m+l
+    static constexpr int kBufs = K <= 32 ? 2 : 1;
+    static constexpr int kAOff = kBufs * kBufCols;         // first column of the A pieces
+    static constexpr int kStageLd = K + 4;
+    static constexpr size_t kStaging = 2ull * kSR * kStageLd * 4;
+    static constexpr size_t kTail = kLutBytes + 8 * (4 * kMaxStages + 2 * kABufs + 4 + 3) + 16;
+    static constexpr int kFit = (int)((kSmemMax - 1024 - kStaging - kTail) / kStageBytes);
+    static constexpr int kStages = kFit > kMaxStages ? kMaxStages : kFit;
+    static constexpr size_t kSmem = 1024 + (size_t)kStages * kStageBytes + kStaging + kTail;
+    static constexpr int RB = K / 16, CB = K / 8;          // 16 x 8 threads contract a K x K block
+    static constexpr int kPer = RB * CB;
+    static_assert(kAOff + kABufs * kACols <= 512, "TMEM columns");
+    static_assert(kStages >= 3 && kSmem <= kSmemMax && kStageBytes % 1024 == 0, "shared memory per CTA");
+    static_assert((size_t)K * K * 4 <= kStaging, "the other members' slices fit the staging rows");
+};
+
+struct Params {
+    int64_t N, T, ld_phi, n_slots;
+    uint64_t key_in, key_out;
+    float scale;
+    float* phi;
+    unsigned int* err;
+    int R;           // token rows per tile
+    int n_ttiles;    // token tiles per slot
+    int pack;        // examples per tile, or 1
+    int k_in, k_out, nk_in, nk_out;
+    int cs;          // CTAs per cluster sharing one example's tiles
+};
+
+#include "tc_ptx.cuh"
+
+__device__ __forceinline__ uint4 lds128(uint32_t a) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+    return v;
+}
+
+// D[tmem] (+)= A[tmem] * B[smem]^T, bf16 inputs, fp32 accumulation.
+__device__ __forceinline__ void mma_bf16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
+                                            uint32_t accumulate) {
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}" ::"r"(
+            d_tmem),
+        "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(
+            taddr),
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+        "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+        : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// The upper halves of two fp32 bit patterns: the truncated bf16 pair (lo in the low half).
+__device__ __forceinline__ uint32_t pack_hi(uint32_t lo, uint32_t hi) { return __byte_perm(lo, hi, 0x7632); }
+
+// x = h + m + l, each the upper half of its fp32 pattern. An infinite x has m = l = 0.
+__device__ __forceinline__ void split3(float x, uint32_t& h, uint32_t& m, uint32_t& l) {
+    h = __float_as_uint(x);
+    const float hf = __uint_as_float(h & 0xFFFF0000u);
+    float r = x - hf;
+    if (fabsf(x) == __int_as_float(0x7F800000)) r = 0.f;
+    m = __float_as_uint(r);
+    l = __float_as_uint(r - __uint_as_float(m & 0xFFFF0000u));
+}
+
+// The sequence of token tiles one CTA works on, identical for every warp role:
+// slots cid, cid + ncl, ... and, within a slot, the tiles crank, crank + cs, ...
+struct Units {
+    int64_t x;
+    int tt;
+    __device__ __forceinline__ void next(const Params& p, uint32_t ncl, uint32_t crank) {
+        tt += p.cs;
+        if (tt >= p.n_ttiles) {
+            tt = (int)crank;
+            x += ncl;
+        }
+    }
+};
+
+template <int K>
+__global__ void __launch_bounds__(kThreads, 1)
+project_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const Params p) {
+    using C = Cfg<K>;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    float* stX = (float*)(smem + (size_t)C::kStages * C::kStageBytes);  // [kSR][K+4] At rows
+    float* stY = stX + kSR * C::kStageLd;                               // [kSR][K+4] Bt rows
+    uint8_t* lut = smem + (size_t)C::kStages * C::kStageBytes + C::kStaging;
+    uint64_t* bars = (uint64_t*)(lut + kLutBytes);
+    uint64_t* full = bars;                     // [stages] fp32 boxes landed (count 1 + tx)
+    uint64_t* rempty = bars + kMaxStages;      // [stages] boxes read by the split warps (8)
+    uint64_t* sready = bars + 2 * kMaxStages;  // [stages] signs written (2)
+    uint64_t* sempty = bars + 3 * kMaxStages;  // [stages] MMAs done with the signs (1)
+    uint64_t* afull = bars + 4 * kMaxStages;   // [2] pieces in TMEM (8)
+    uint64_t* aempty = afull + kABufs;         // [2] MMAs done with the pieces (1)
+    uint64_t* tfull = aempty + kABufs;         // [2] accumulators ready (1)
+    uint64_t* tempty = tfull + 2;              // [2] accumulators drained (4)
+    uint64_t* mma_done = tempty + 2;
+    uint64_t* red_go = mma_done + 1;           // the other members' staging rows are free (cs - 1)
+    uint64_t* red_full = red_go + 1;           // the other members' slices have landed here (cs - 1)
+    uint32_t* tmem_slot = (uint32_t*)(red_full + 1);
+    volatile int* abort = (volatile int*)(tmem_slot + 1);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < C::kStages; ++s) {
+            mbar_init(smem_u32(&full[s]), 1);
+            mbar_init(smem_u32(&rempty[s]), 8);
+            mbar_init(smem_u32(&sready[s]), 2);
+            mbar_init(smem_u32(&sempty[s]), 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(smem_u32(&afull[b]), 8);
+            mbar_init(smem_u32(&aempty[b]), 1);
+            mbar_init(smem_u32(&tfull[b]), 1);
+            mbar_init(smem_u32(&tempty[b]), 4);
+        }
+        mbar_init(smem_u32(mma_done), 1);
+        mbar_init(smem_u32(red_go), p.cs > 1 ? p.cs - 1 : 1);
+        mbar_init(smem_u32(red_full), p.cs > 1 ? p.cs - 1 : 1);
+        *abort = 0;
+        fence_mbar_init();
+    }
+    if (threadIdx.x < 256) {  // entry e: bit j of e as the bf16 sign of element j
+        const uint32_t e = threadIdx.x;
+        uint32_t q[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            q[i] = (0x3F80u | (((e >> (2 * i)) & 1u) << 15)) | ((0x3F80u | (((e >> (2 * i + 1)) & 1u) << 15)) << 16);
+        *reinterpret_cast<uint4*>(lut + e * 16) = make_uint4(q[0], q[1], q[2], q[3]);
+    }
+    if (warp == 1) {
+        tmem_alloc(smem_u32(tmem_slot), 512);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();  // every CTA's barriers exist before any remote arrive
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    const uint32_t crank = cluster_rank(), cid = blockIdx.x / p.cs, ncl = gridDim.x / p.cs;
+    const int nk_tot = p.nk_in + p.nk_out;
+    Units it{(int64_t)cid, (int)crank};
+
+    if (warp == 0 && lane == 0) {
+        // ---------------- TMA producer
+        uint32_t s = 0, ph = 0, last_par[C::kStages];
+        bool issued[C::kStages], ok = true;
+        for (int i = 0; i < C::kStages; ++i) issued[i] = false;
+        const uint32_t box = (uint32_t)p.R * 128u;
+        for (; ok && it.x < p.n_slots; it.next(p, ncl, crank)) {
+            const int row = p.pack > 1 ? (int)(it.x * p.pack * p.T) : it.tt * p.R;
+            const int ex = p.pack > 1 ? 0 : (int)it.x;
+            for (int kc = 0; kc < nk_tot; ++kc) {
+                if (!wait_bounded(smem_u32(&rempty[s]), ph ^ 1u, abort, p.err)) {
+                    ok = false;
+                    break;
+                }
+                const bool side_b = kc >= p.nk_in;
+                const int d0 = (side_b ? kc - p.nk_in : kc) * kChunkK;
+                const uint32_t dst = smem_u32(smem + (size_t)s * C::kStageBytes), bar = smem_u32(&full[s]);
+                mbar_arrive_tx(bar, 2 * box);
+                tma_load_3d(dst, side_b ? &tmB : &tmA, d0, row, ex, bar);
+                tma_load_3d(dst + kBoxBytes, side_b ? &tmB : &tmA, d0 + 32, row, ex, bar);
+                issued[s] = true;
+                last_par[s] = ph;
+                if (++s == (uint32_t)C::kStages) s = 0, ph ^= 1u;
+            }
+        }
+        for (int i = 0; i < C::kStages; ++i)
+            if (issued[i]) {
+                const uint64_t t0 = global_ns();
+                while (!mbar_try_wait(smem_u32(&full[i]), last_par[i]))
+                    if (global_ns() - t0 > kTimeoutNs) {
+                        atomicOr(p.err, kErrTimeout);
+                        break;
+                    }
+            }
+    } else if (warp == 1 && lane == 0) {
+        // ---------------- MMA issuer
+        uint32_t s = 0, ph = 0, cnt = 0, tile = 0;
+        bool ok = true;
+        constexpr uint32_t idesc = idesc_bf16(kTileM, K);
+        for (; ok && it.x < p.n_slots; it.next(p, ncl, crank), ++tile) {
+            const uint32_t b = tile % C::kBufs, use = tile / C::kBufs;
+            if (!wait_bounded(smem_u32(&tempty[b]), (use & 1u) ^ 1u, abort, p.err)) break;
+            for (int kc = 0; kc < nk_tot; ++kc, ++cnt) {
+                const uint32_t a = cnt & 1u;
+                if (!wait_bounded(smem_u32(&sready[s]), ph, abort, p.err) ||
+                    !wait_bounded(smem_u32(&afull[a]), (cnt >> 1) & 1u, abort, p.err)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                const bool side_b = kc >= p.nk_in;
+                const bool start = kc == 0 || kc == p.nk_in;
+                const uint64_t bd = sw128_desc(smem_u32(smem + (size_t)s * C::kStageBytes + 2 * kBoxBytes));
+                const uint32_t dh = tmem + b * C::kBufCols + (side_b ? 2 * K : 0), dl = dh + K;
+                const uint32_t at = tmem + C::kAOff + a * kACols;
+#pragma unroll
+                for (int k = 0; k < kChunkK / 16; ++k) {  // K = 16: 8 columns of pieces, 32 bytes of signs
+                    const uint32_t acc = start && k == 0 ? 0u : 1u;
+                    mma_bf16_ta(dh, at + 8 * k, bd + 2 * k, idesc, acc);
+                    mma_bf16_ta(dl, at + kPieceCols + 8 * k, bd + 2 * k, idesc, acc);
+                    mma_bf16_ta(dl, at + 2 * kPieceCols + 8 * k, bd + 2 * k, idesc, 1u);
+                }
+                mma_commit(smem_u32(&aempty[a]));
+                mma_commit(smem_u32(&sempty[s]));
+                if (++s == (uint32_t)C::kStages) s = 0, ph ^= 1u;
+            }
+            if (!ok) break;
+            mma_commit(smem_u32(&tfull[b]));
+        }
+        mma_commit(smem_u32(mma_done));
+        const uint64_t t0 = global_ns();
+        while (!mbar_try_wait(smem_u32(mma_done), 0))
+            if (global_ns() - t0 > kTimeoutNs) {
+                atomicOr(p.err, kErrTimeout);
+                break;
+            }
+    } else if (warp == 2 || warp == 3) {
+        // ---------------- sign generators: the 64 threads share a tile's K rows, kParts threads per row
+        constexpr int kParts = 64 / K, kChunks = 8 / kParts;
+        const int g = (warp - 2) * 32 + lane, col = g / kParts, part = g % kParts;
+        const uint32_t lut_s = smem_u32(lut);
+        uint32_t s = 0, ph = 0;
+        bool ok = true;
+        for (; ok && it.x < p.n_slots; it.next(p, ncl, crank))
+            for (int kc = 0; kc < nk_tot; ++kc) {
+                const bool side_b = kc >= p.nk_in;
+                const uint64_t w = sign_word(side_b ? p.key_out : p.key_in, (uint32_t)col,
+                                             (uint64_t)(side_b ? kc - p.nk_in : kc));
+                uint4 q[kChunks];
+#pragma unroll
+                for (int c = 0; c < kChunks; ++c)
+                    q[c] = lds128(lut_s + ((((uint32_t)(w >> (8 * (part * kChunks + c)))) & 0xFFu) << 4));
+                bool got = true;
+                if (lane == 0) got = wait_bounded(smem_u32(&sempty[s]), ph ^ 1u, abort, p.err);
+                got = __shfl_sync(0xffffffffu, got, 0);
+                if (!got) {
+                    ok = false;
+                    break;
+                }
+                uint8_t* row = smem + (size_t)s * C::kStageBytes + 2 * kBoxBytes + (col >> 3) * 1024 + (col & 7) * 128;
+#pragma unroll
+                for (int c = 0; c < kChunks; ++c)
+                    *reinterpret_cast<uint4*>(row + (((part * kChunks + c) ^ (col & 7)) << 4)) = q[c];
+                fence_proxy_async();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&sready[s]));
+                if (++s == (uint32_t)C::kStages) s = 0, ph ^= 1u;
+            }
+    } else if (warp >= 8) {
+        // ---------------- split warps: a thread per token row, 32 features (one box) each
+        const int q4 = warp & 3, half = (warp - 8) >> 2, row = q4 * 32 + lane;
+        const bool active = q4 * 32 < p.R;
+        uint32_t s = 0, ph = 0, cnt = 0;
+        bool ok = true;
+        for (; ok && it.x < p.n_slots; it.next(p, ncl, crank))
+            for (int kc = 0; kc < nk_tot; ++kc, ++cnt) {
+                const uint32_t a = cnt & 1u;
+                bool got = true;
+                if (lane == 0) got = wait_bounded(smem_u32(&full[s]), ph, abort, p.err);
+                got = __shfl_sync(0xffffffffu, got, 0);
+                if (!got) {
+                    ok = false;
+                    break;
+                }
+                uint32_t h[16], m[16], l[16];
+                if (active) {
+                    const uint32_t src = smem_u32(smem + (size_t)s * C::kStageBytes) + (uint32_t)half * kBoxBytes +
+                                         (uint32_t)row * 128u;
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) {
+                        const uint4 v = lds128(src + (uint32_t)((c ^ (row & 7)) << 4));
+                        uint32_t hh[4], mm[4], ll[4];
+                        split3(__uint_as_float(v.x), hh[0], mm[0], ll[0]);
+                        split3(__uint_as_float(v.y), hh[1], mm[1], ll[1]);
+                        split3(__uint_as_float(v.z), hh[2], mm[2], ll[2]);
+                        split3(__uint_as_float(v.w), hh[3], mm[3], ll[3]);
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) {
+                            h[2 * c + i] = pack_hi(hh[2 * i], hh[2 * i + 1]);
+                            m[2 * c + i] = pack_hi(mm[2 * i], mm[2 * i + 1]);
+                            l[2 * c + i] = pack_hi(ll[2 * i], ll[2 * i + 1]);
+                        }
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(smem_u32(&rempty[s]));
+                    got = wait_bounded(smem_u32(&aempty[a]), ((cnt >> 1) & 1u) ^ 1u, abort, p.err);
+                }
+                got = __shfl_sync(0xffffffffu, got, 0);
+                if (!got) {
+                    ok = false;
+                    break;
+                }
+                if (active) {
+                    tc_fence_after();
+                    const uint32_t dst = tmem + ((uint32_t)(q4 * 32) << 16) + C::kAOff + a * kACols + half * 16;
+                    tmem_st16(dst, h);
+                    tmem_st16(dst + kPieceCols, m);
+                    tmem_st16(dst + 2 * kPieceCols, l);
+                    tmem_wait_st();
+                    tc_fence_before();
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&afull[a]));
+                if (++s == (uint32_t)C::kStages) s = 0, ph ^= 1u;
+            }
+    } else if (warp >= 4) {
+        // ---------------- epilogue: TMEM -> shared -> Phi += Bt^T At, kSR token rows at a time
+        const int q4 = warp & 3, et = threadIdx.x - 128, rg = et >> 3, cg = et & 7;
+        uint32_t tile = 0, red_use = 0;
+        bool ok = true;
+        float acc[C::RB][C::CB];
+        auto clear = [&]() {
+#pragma unroll
+            for (int i = 0; i < C::RB; ++i)
+#pragma unroll
+                for (int j = 0; j < C::CB; ++j) acc[i][j] = 0.f;
+        };
+        auto contract = [&](int t0, int t1) {  // staged rows [t0, t1)
+#pragma unroll 2
+            for (int t = t0; t < t1; ++t) {
+                float y[C::RB], x[C::CB];
+#pragma unroll
+                for (int i = 0; i < C::RB; ++i) y[i] = stY[t * C::kStageLd + rg * C::RB + i];
+#pragma unroll
+                for (int j = 0; j < C::CB; ++j) x[j] = stX[t * C::kStageLd + cg * C::CB + j];
+#pragma unroll
+                for (int i = 0; i < C::RB; ++i)
+#pragma unroll
+                    for (int j = 0; j < C::CB; ++j) acc[i][j] = fmaf(y[i], x[j], acc[i][j]);
+            }
+        };
+        auto write = [&](int64_t n) {
+            float* out = p.phi + n * p.ld_phi;
+#pragma unroll
+            for (int i = 0; i < C::RB; ++i)
+#pragma unroll
+                for (int j = 0; j < C::CB; ++j) {
+                    const int r = rg * C::RB + i, c = cg * C::CB + j;
+                    if (r < p.k_out && c < p.k_in) out[r * p.k_in + c] = acc[i][j] * p.scale;
+                }
+        };
+        // Phi of example n, summed over the cluster: thread et's elements belong to member
+        // et * cs / 128; every other member sends them there, in slots of 128 / cs threads each.
+        auto flush = [&](int64_t n) -> bool {
+            if (p.cs > 1) {
+                const int per = 128 / p.cs, own = et / per;
+                bool got = true;
+                epi_sync();  // this CTA's staged rows are read
+                if (et < p.cs && et != (int)crank) mbar_arrive_remote(smem_u32(red_go), (uint32_t)et);
+                if (lane == 0) got = wait_bounded_cluster(smem_u32(red_go), red_use & 1u, abort, p.err);
+                got = __shfl_sync(0xffffffffu, got, 0);
+                if (epi_any(!got)) return false;
+                if (own != (int)crank) {
+                    const uint32_t slot = crank < (uint32_t)own ? crank : crank - 1;  // senders in rank order
+                    const uint32_t dst = map_rank(smem_u32(stX) + (slot * per + (et - own * per)) * C::kPer * 4u, own);
+#pragma unroll
+                    for (int i = 0; i < C::RB; ++i)
+#pragma unroll
+                        for (int j = 0; j < C::CB; ++j) st_cluster_f32(dst + (i * C::CB + j) * 4u, acc[i][j]);
+                }
+                fence_acq_rel_cluster();
+                epi_sync();
+                if (et < p.cs && et != (int)crank) mbar_arrive_remote(smem_u32(red_full), (uint32_t)et);
+                if (lane == 0) got = wait_bounded_cluster(smem_u32(red_full), red_use & 1u, abort, p.err);
+                got = __shfl_sync(0xffffffffu, got, 0);
+                if (epi_any(!got)) return false;
+                ++red_use;
+                if (own == (int)crank) {
+                    for (int r = 0; r < p.cs - 1; ++r) {
+                        const float* part = stX + (size_t)(r * per + (et - own * per)) * C::kPer;
+#pragma unroll
+                        for (int i = 0; i < C::RB; ++i)
+#pragma unroll
+                            for (int j = 0; j < C::CB; ++j) acc[i][j] += part[i * C::CB + j];
+                    }
+                    write(n);
+                }
+                epi_sync();  // the slices are read: staging rows free for the next tile
+            } else {
+                write(n);
+            }
+            return true;
+        };
+        clear();
+        while (ok && it.x < p.n_slots) {
+            const int64_t cur = it.x;
+            const uint32_t b = tile % C::kBufs, use = tile / C::kBufs;
+            bool got = true;
+            if (lane == 0) got = wait_bounded(smem_u32(&tfull[b]), use & 1u, abort, p.err);
+            got = __shfl_sync(0xffffffffu, got, 0);
+            if (epi_any(!got)) break;
+            tc_fence_after();
+            const int rows = p.pack > 1 ? p.pack * (int)p.T : p.R;
+            int j = 0;  // packed: example of the tile whose rows come next
+            for (int r0 = 0; r0 < rows; r0 += kSR) {
+                const int srow = q4 * 32 + lane - r0;
+                if (srow >= 0 && srow < kSR) {
+                    const uint32_t tb = tmem + ((uint32_t)(q4 * 32) << 16) + b * C::kBufCols;
+#pragma unroll
+                    for (int side = 0; side < 2; ++side)
+#pragma unroll
+                        for (int c0 = 0; c0 < K; c0 += 16) {
+                            float hi[16], lo[16];
+                            tmem_ld16(tb + side * 2 * K + c0, hi);
+                            tmem_ld16(tb + side * 2 * K + K + c0, lo);
+                            float* dst = (side ? stY : stX) + srow * C::kStageLd + c0;
+#pragma unroll
+                            for (int i = 0; i < 16; i += 4)
+                                *reinterpret_cast<float4*>(dst + i) = make_float4(
+                                    hi[i] + lo[i], hi[i + 1] + lo[i + 1], hi[i + 2] + lo[i + 2], hi[i + 3] + lo[i + 3]);
+                        }
+                }
+                epi_sync();
+                const int end = rows - r0 < kSR ? rows - r0 : kSR;
+                if (p.pack == 1) {
+                    contract(0, end);
+                } else {
+                    // packed: example j's rows j*T .. may span two staged parts
+                    for (int t = 0; t < end;) {
+                        const int stop = (j + 1) * (int)p.T - r0 < end ? (j + 1) * (int)p.T - r0 : end;
+                        contract(t, stop);
+                        t = stop;
+                        if (stop + r0 == (j + 1) * (int)p.T) {
+                            const int64_t e = cur * p.pack + j;
+                            if (e < p.N) write(e);
+                            clear();
+                            ++j;
+                        }
+                    }
+                }
+                epi_sync();
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&tempty[b]));
+            it.next(p, ncl, crank);
+            ++tile;
+            if (p.pack == 1 && it.x != cur) {
+                ok = flush(cur);
+                clear();
+            }
+        }
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem, 512);
+    }
+    cluster_sync();  // no CTA leaves while a peer may still write to it
+}
+
+// ---------------------------------------------------------------- host side
+typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+EncodeTiledFn encode_fn() {
+    static EncodeTiledFn fn = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) ==
+                cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            fn = (EncodeTiledFn)f;
+    });
+    return fn;
+}
+
+// 3-D map over fp32 X[N][T][d]: box 32 (d) x rows x 1 (example), 128-byte swizzle, zero fill.
+bool make_map(CUtensorMap* tm, const void* X, int64_t N, int64_t T, int64_t d, int rows) {
+    EncodeTiledFn enc = encode_fn();
+    if (!enc) return false;
+    cuuint64_t dims[3] = {(cuuint64_t)d, (cuuint64_t)T, (cuuint64_t)N};
+    cuuint64_t strides[2] = {(cuuint64_t)(d * 4), (cuuint64_t)(T * d * 4)};
+    cuuint32_t box[3] = {32, (cuuint32_t)rows, 1};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return enc(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(X), dims, strides, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+int device_sms() {
+    static std::atomic<int> sms{0};
+    int n = sms.load(std::memory_order_relaxed);
+    if (!n) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 1;
+        sms.store(n, std::memory_order_relaxed);
+    }
+    return n;
+}
+
+template <int K>
+void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int cs, cudaStream_t s) {
+    cfg = {};
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)cs;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)(cs * (device_sms() / cs)));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = Cfg<K>::kSmem;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+}
+
+// Clusters of cs CTAs that fit the device at once (queried once per device and size).
+template <int K>
+int max_clusters(int cs) {
+    static std::atomic<int> cache[64][4];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) dev = -1;
+    const int slot = cs >= 8 ? 3 : (cs >= 4 ? 2 : cs - 1);
+    if (dev >= 0) {
+        const int v = cache[dev][slot].load(std::memory_order_relaxed);
+        if (v) return v;
+    }
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[1];
+    cluster_config<K>(cfg, attr, cs, nullptr);
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, project_f32_kernel<K>, &cfg) != cudaSuccess || n < 1) n = device_sms() / cs;
+    if (dev >= 0) cache[dev][slot].store(n, std::memory_order_relaxed);
+    return n;
+}
+
+struct Plan {
+    int R, cs, pack, n_ttiles;
+    int64_t slots, clusters;
+};
+
+// Tile rows and cluster size with the least time of the busiest CTA: its tiles times the time of a
+// 64-feature chunk, which the split and sign warps bound at about 750, 500 and 400 clocks for 128,
+// 64 and 32 rows, but at least what HBM takes (22 bytes a clock and SM); ties go to larger tiles
+// and smaller clusters. A tile's contraction and an example's reduction count as chunks.
+template <int K>
+Plan plan(const tda_layer_desc& L, int64_t N, int sms) {
+    Plan best{};
+    double best_cost = 0;
+    const double chunks = (double)((L.d_in + kChunkK - 1) / kChunkK + (L.d_out + kChunkK - 1) / kChunkK);
+    const double floor_clk = (double)N * L.T * (L.d_in + L.d_out) * 4.0 / (22.0 * sms);
+    for (int R = 128; R >= 32; R >>= 1) {
+        const double t = R == 128 ? 750 : (R == 64 ? 500 : 400);
+        const int pack = L.T <= R ? (int)(R / L.T) : 1;
+        const int64_t slots = (N + pack - 1) / pack;
+        const int nt = pack > 1 ? 1 : (int)((L.T + R - 1) / R);
+        for (int cs = 1; cs <= 8 && cs <= nt; cs *= 2) {
+            const int64_t fit = max_clusters<K>(cs) < sms / cs ? max_clusters<K>(cs) : sms / cs;
+            if (fit < 1) continue;
+            const int64_t clusters = slots < fit ? slots : fit;
+            const double tiles = (double)((slots + clusters - 1) / clusters) * ((nt + cs - 1) / cs);
+            const double flushes = (double)((slots + clusters - 1) / clusters);
+            double cost = tiles * (chunks * t + R * (K >= 64 ? 45.0 : 20.0)) + flushes * (cs > 1 ? 3000.0 : 500.0);
+            if (cost < floor_clk) cost = floor_clk;
+            if (best.R == 0 || cost < best_cost * 0.98) {
+                best = Plan{R, cs, pack, nt, slots, clusters};
+                best_cost = cost;
+            }
+        }
+    }
+    return best;
+}
+
+template <int K>
+cudaError_t launch_k(const tda_layer_desc& L, const void* A, const void* B, int64_t N, float* phi, int64_t ld_phi,
+                     unsigned int* err, cudaStream_t s) {
+    const int budget = sm_budget();
+    const int sms = budget > 0 && budget < device_sms() ? budget : device_sms();
+    cudaError_t e = smem_attr_once<project_f32_kernel<K>>((int)Cfg<K>::kSmem);  // before the occupancy queries
+    if (e != cudaSuccess) return e;
+    const Plan pl = plan<K>(L, N, sms);
+    // packed rows are one [1][N*T][d] view: 32-bit row coordinates, strides below 2^40 bytes
+    if (pl.pack > 1) {
+        const int64_t d_max = L.d_in > L.d_out ? L.d_in : L.d_out;
+        int64_t most = ((int64_t)1 << 30) / L.T;
+        const int64_t by_stride = (((int64_t)1 << 40) - 1) / (L.T * d_max * 4);
+        if (by_stride < most) most = by_stride;
+        most = most / 128 * 128;  // whole tiles of any packing
+        if (most < 128) return cudaErrorNotSupported;
+        if (N > most) {
+            for (int64_t e0 = 0; e0 < N; e0 += most) {
+                e = launch_k<K>(L, (const float*)A + e0 * L.T * L.d_in, (const float*)B + e0 * L.T * L.d_out,
+                                            N - e0 < most ? N - e0 : most, phi + e0 * ld_phi, ld_phi, err, s);
+                if (e != cudaSuccess) return e;
+            }
+            return cudaSuccess;
+        }
+    }
+    CUtensorMap mA, mB;
+    const bool flat = pl.pack > 1;
+    if (!make_map(&mA, A, flat ? 1 : N, flat ? N * L.T : L.T, L.d_in, pl.R) ||
+        !make_map(&mB, B, flat ? 1 : N, flat ? N * L.T : L.T, L.d_out, pl.R))
+        return cudaErrorNotSupported;
+    Params p;
+    p.N = N;
+    p.T = L.T;
+    p.ld_phi = ld_phi;
+    p.n_slots = pl.slots;
+    p.key_in = side_key(L.seed, L.layer, 0);
+    p.key_out = side_key(L.seed, L.layer, 1);
+    p.scale = projection_scale(L);
+    p.phi = phi;
+    p.err = err;
+    p.R = pl.R;
+    p.n_ttiles = pl.n_ttiles;
+    p.pack = pl.pack;
+    p.k_in = L.k_in;
+    p.k_out = L.k_out;
+    p.nk_in = (int)((L.d_in + kChunkK - 1) / kChunkK);
+    p.nk_out = (int)((L.d_out + kChunkK - 1) / kChunkK);
+    p.cs = pl.cs;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[1];
+    cluster_config<K>(cfg, attr, pl.cs, s);
+    cfg.gridDim = dim3((unsigned)(pl.clusters * pl.cs));
+    note_launches(1);
+    e = cudaLaunchKernelEx(&cfg, project_f32_kernel<K>, mA, mB, p);
+    if (e != cudaSuccess) return e;
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+bool project_f32_tc_supported(const tda_layer_desc& L, const void* A, const void* B) {
+    static int sm103 = -1;
+    if (sm103 < 0) {
+        int dev = 0, major = 0, minor = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
+        cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev);
+        sm103 = (major == 10 && minor == 3) ? 1 : 0;
+    }
+    if (!sm103 || !encode_fn() || L.kind != TDA_PROJ_RADEMACHER) return false;
+    if (L.k_in < 1 || L.k_out < 1 || L.k_in > 64 || L.k_out > 64) return false;
+    if (L.d_in % 4 || L.d_out % 4 || L.T < 1) return false;
+    if (((uintptr_t)A & 15) || ((uintptr_t)B & 15)) return false;
+    // TMA: 32-bit coordinates, an example's stride below 2^40 bytes
+    const int64_t d_max = L.d_in > L.d_out ? L.d_in : L.d_out;
+    if (L.T > (1LL << 30) || d_max > (1LL << 30) || L.T * d_max >= (1LL << 38)) return false;
+    return true;
+}
+
+cudaError_t launch_project_f32_tc(const tda_layer_desc& L, const void* A, const void* B, int64_t N, float* phi,
+                                  int64_t ld_phi, unsigned int* err, cudaStream_t s) {
+    if (N == 0) return cudaSuccess;
+    const int k = L.k_in > L.k_out ? L.k_in : L.k_out;
+    if (k <= 16) return launch_k<16>(L, A, B, N, phi, ld_phi, err, s);
+    if (k <= 32) return launch_k<32>(L, A, B, N, phi, ld_phi, err, s);
+    return launch_k<64>(L, A, B, N, phi, ld_phi, err, s);
+}
+
+}  // namespace tda

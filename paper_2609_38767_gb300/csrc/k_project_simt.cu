@@ -5,8 +5,9 @@
 //   At = A_n S_in (T x k_in), Bt = B_n S_out (T x k_out),
 //   Phi_n = scale * Bt^T At (k_out x k_in), scale = 1/sqrt(k_in k_out),
 // with S generated on chip from the counter hash (App. A.2) and never stored.
-// This kernel is the fp32 path (its 1e-5 tolerance excludes TF32 tensor
-// cores) and the fallback for shapes the tensor-core kernel does not cover.
+// The general kernel is the fallback for shapes the tensor-core kernels do not
+// cover (identity maps, k above their blocks); project_small_kernel takes short
+// fp32 jobs of narrow layers, with the general kernel's sums bit for bit.
 #include <cuda_bf16.h>
 
 #include "tda_internal.cuh"
@@ -130,7 +131,115 @@ project_simt_kernel(const T* __restrict__ A, const T* __restrict__ B, int64_t Tn
         }
 }
 
+// Few tokens of a narrow fp32 layer (T <= 64, d <= 512, k <= 16): one CTA per example, half its
+// threads on each side. Bound by latency: a (token, column) sum is a chain of d dependent adds.
+// A thread runs CPT such chains of one token (CPT = 4, 2, 1 for T <= 64, 32, 16, so that a side's
+// 256 threads cover T x 16 columns), with 64-feature chunks of the factors staged in shared
+// memory one chunk ahead in registers. The adds of a chain, and of an entry of Phi over the
+// tokens, run in the general kernel's order, so the features are the same bit for bit (an fp64
+// preconditioner state behind them sees no change). 64 examples, 256 -> 256, T = 32, k = 16:
+// 63 us in the general kernel, which computes 64 columns whatever k is, 16 tokens at a time;
+// about 25 us here.
+constexpr int kSmallT = 64, kSmallD = 512, kSmallK = 16;
+constexpr int kSmallLd = kDChunk + 4;  // padded row: 16-byte loads of different tokens miss each other's banks
+
+template <int CPT>
+__global__ void __launch_bounds__(512)
+project_small_kernel(const float* __restrict__ A, const float* __restrict__ B, int Tn, int d_in, int d_out, int k_in,
+                     int k_out, uint64_t key_in, uint64_t key_out, float scale, float* __restrict__ phi,
+                     int64_t ld_phi) {
+    constexpr int kTok = 16 * CPT;            // tokens the threads of a side cover
+    constexpr int kLoads = kTok * kDChunk / 4 / 256;  // 16-byte groups per thread and chunk
+    __shared__ __align__(16) float Vs[2][kTok][kSmallLd];
+    __shared__ float Xs[2][kTok][kSmallK + 1];
+    const int side = threadIdx.x >> 8, tid = threadIdx.x & 255;
+    const int d = side ? d_out : d_in;
+    const uint64_t key = side ? key_out : key_in;
+    const float* src = side ? B + (int64_t)blockIdx.x * Tn * d_out : A + (int64_t)blockIdx.x * Tn * d_in;
+    const int t = tid / (16 / CPT), c0 = tid % (16 / CPT) * CPT;
+    const int dmax = d_in > d_out ? d_in : d_out;
+    float4 next[kLoads];
+    auto load = [&](int dc) {
+#pragma unroll
+        for (int i = 0; i < kLoads; ++i) {
+            const int e = tid + 256 * i, tt = e / (kDChunk / 4), cc = dc + e % (kDChunk / 4) * 4;
+            next[i] = tt < Tn && cc < d ? __ldg(reinterpret_cast<const float4*>(src + (int64_t)tt * d + cc))
+                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    };
+    float o[CPT];
+#pragma unroll
+    for (int q = 0; q < CPT; ++q) o[q] = 0.f;
+    load(0);
+    for (int dc = 0; dc < dmax; dc += kDChunk) {
+        __syncthreads();  // the previous chunk is read
+#pragma unroll
+        for (int i = 0; i < kLoads; ++i) {
+            const int e = tid + 256 * i;
+            *reinterpret_cast<float4*>(&Vs[side][e / (kDChunk / 4)][e % (kDChunk / 4) * 4]) = next[i];
+        }
+        if (dc + kDChunk < dmax) load(dc + kDChunk);
+        uint32_t w[CPT][2];
+#pragma unroll
+        for (int q = 0; q < CPT; ++q) {
+            const uint64_t x = sign_word(key, (uint32_t)(c0 + q), (uint64_t)(dc >> 6));
+            w[q][0] = (uint32_t)x;
+            w[q][1] = (uint32_t)(x >> 32);
+        }
+        __syncthreads();
+        if (dc < d) {
+#pragma unroll
+            for (int half = 0; half < 2; ++half)
+#pragma unroll
+                for (int r = 0; r < 32; r += 4) {
+                    const float4 v4 = *reinterpret_cast<const float4*>(&Vs[side][t][32 * half + r]);
+                    const float v[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int q = 0; q < CPT; ++q)
+                            o[q] += __uint_as_float(__float_as_uint(v[i]) ^
+                                                    ((w[q][half] << (31 - r - i)) & 0x80000000u));
+                }
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < CPT; ++q) Xs[side][t][c0 + q] = o[q];
+    __syncthreads();
+    const int e = threadIdx.x, i = e / kSmallK, j = e % kSmallK;  // Phi entry (i, j): i < 16 for half the threads
+    if (i < k_out && j < k_in) {
+        float acc = 0.f;
+#pragma unroll 8
+        for (int tt = 0; tt < Tn; ++tt) acc = fmaf(Xs[1][tt][i], Xs[0][tt][j], acc);
+        phi[blockIdx.x * ld_phi + (int64_t)i * k_in + j] = acc * scale;
+    }
+}
+
 }  // namespace
+
+bool project_small_supported(const tda_layer_desc& L, const void* A, const void* B, int64_t N) {
+    return L.kind == TDA_PROJ_RADEMACHER && L.T >= 1 && L.T <= kSmallT && L.d_in <= kSmallD && L.d_out <= kSmallD &&
+           L.k_in <= kSmallK && L.k_out <= kSmallK && L.d_in % 4 == 0 && L.d_out % 4 == 0 && N <= 16384 / L.T &&
+           !((uintptr_t)A & 15) && !((uintptr_t)B & 15);
+}
+
+cudaError_t launch_project_small(const tda_layer_desc& L, const void* A, const void* B, int64_t N, float* phi,
+                                 int64_t ld_phi, cudaStream_t s) {
+    if (N == 0) return cudaSuccess;
+    const uint64_t key_in = side_key(L.seed, L.layer, 0), key_out = side_key(L.seed, L.layer, 1);
+    auto launch = [&](auto kernel) {
+        note_launches(1);
+        kernel<<<(unsigned)N, 512, 0, s>>>((const float*)A, (const float*)B, (int)L.T, (int)L.d_in, (int)L.d_out,
+                                           L.k_in, L.k_out, key_in, key_out, projection_scale(L), phi, ld_phi);
+    };
+    if (L.T > 32)
+        launch(project_small_kernel<4>);
+    else if (L.T > 16)
+        launch(project_small_kernel<2>);
+    else
+        launch(project_small_kernel<1>);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_proj_entries(uint64_t key, int kind, int64_t rows, int32_t cols, int8_t* out,
                                 cudaStream_t s) {

@@ -73,6 +73,11 @@ cudaError_t launch_proj_entries(uint64_t key, int kind, int64_t rows, int32_t co
 cudaError_t launch_project_simt(const tda_layer_desc& L, tda_dtype dt, const void* A, const void* B,
                                 int64_t N, float* phi, int64_t ld_phi, cudaStream_t s);
 
+// Short fp32 jobs of narrow layers, the generic kernel's sums bit for bit.
+bool project_small_supported(const tda_layer_desc& L, const void* A, const void* B, int64_t N);
+cudaError_t launch_project_small(const tda_layer_desc& L, const void* A, const void* B, int64_t N, float* phi,
+                                 int64_t ld_phi, cudaStream_t s);
+
 // tcgen05 / TMA projection for bf16 inputs. Returns cudaErrorNotSupported if
 // the shape has no tensor-core instantiation (caller falls back to SIMT).
 bool project_tc_supported(const tda_layer_desc& L, const void* A, const void* B);
@@ -125,6 +130,12 @@ size_t project_tc_ws_bytes(const tda_layer_desc& L);
 cudaError_t launch_project_tc(const tda_layer_desc& L, const void* A, const void* B, int64_t N,
                               float* phi, int64_t ld_phi, unsigned int* err, cudaStream_t s,
                               void* ws = nullptr, size_t ws_bytes = 0);
+
+// Factored projection of fp32 factors on tcgen05 (k_project_f32.cu), k_in and k_out up to 64;
+// cudaErrorNotSupported (nothing launched) for sizes its tensor maps cannot address.
+bool project_f32_tc_supported(const tda_layer_desc& L, const void* A, const void* B);
+cudaError_t launch_project_f32_tc(const tda_layer_desc& L, const void* A, const void* B, int64_t N, float* phi,
+                                  int64_t ld_phi, unsigned int* err, cudaStream_t s);
 
 // Route (b): materialise G = B^T A for nb examples into ws, then project it.
 size_t materialize_ws_bytes_per_example(const tda_layer_desc& L);

@@ -61,6 +61,77 @@ def test_tc_projection_any_k(dev, orc, N, T, di, do, ki, ko):
     assert max(rel(got[n, :ki * ko], ref[n]) for n in range(N)) <= TOL
 
 
+@pytest.mark.parametrize("N,T,di,do,ki,ko", [
+    (64, 32, 256, 256, 16, 16), (8, 32, 256, 256, 16, 16),  # packed, one and several examples a tile
+    (700, 5, 64, 72, 8, 5), (5, 45, 200, 136, 32, 48), (3, 33, 36, 100, 20, 12), (1, 1, 4, 4, 1, 1),
+    (2, 1024, 64, 72, 64, 64), (1, 300, 128, 64, 64, 16),   # clusters sharing an example, uneven tiles
+    (160, 200, 72, 64, 64, 64), (9, 130, 1000, 2056, 24, 24), (310, 70, 64, 68, 32, 32), (20, 257, 512, 136, 16, 16),
+    (40, 64, 132, 64, 64, 64), (153, 129, 64, 64, 48, 64)])
+def test_tc_projection_fp32(dev, orc, N, T, di, do, ki, ko):
+    # fp32 factors as three exact bf16 pieces: fp32 rounding of the sums only
+    A, B = factors(N, T, di, do, "f32", 63)
+    L = tda.LayerDesc(di, do, T, ki, ko, seed=7, layer=2)
+    Ad, Bd = up(A, "f32", dev), up(B, "f32", dev)
+    assert tda.tda_project_engine(L, tda.TDA_F32, Ad, Bd) == 1
+    ld = ki * ko + 3
+    outs = []
+    for _ in range(2):
+        phi = torch.full((N, ld), 7.0, device=dev)
+        tda.tda_project(L, tda.TDA_F32, Ad, Bd, N, phi, ld, tda.TDA_ROUTE_FACTORED)
+        tda.tda_device_status()
+        outs.append(phi.cpu().numpy())
+    np.testing.assert_array_equal(outs[0], outs[1])
+    got = outs[0]
+    assert (got[:, ki * ko:] == 7.0).all()
+    ref = orc.project(A.astype(np.float64), B.astype(np.float64), ki, ko, 7, 2).reshape(N, -1)
+    assert max(rel(got[n, :ki * ko], ref[n]) for n in range(N)) <= TOL
+
+
+def test_tc_projection_fp32_extremes(dev, orc):
+    # values whose pieces are subnormal, of the largest exponent, infinite or NaN stay in their example
+    N, T, d, k = 4, 3, 64, 16
+    A, B = factors(N, T, d, d, "f32", 64)
+    A[0] *= np.float32(1e-30)
+    B[0] *= np.float32(1e-3)
+    A[1] *= np.float32(1e36)
+    B[1] *= np.float32(1e-30)
+    A[2, 1, 5] = np.inf
+    B[3, 0, 7] = np.nan
+    L = tda.LayerDesc(d, d, T, k, k, seed=7, layer=2)
+    phi = torch.empty((N, k * k), device=dev)
+    tda.tda_project(L, tda.TDA_F32, up(A, "f32", dev), up(B, "f32", dev), N, phi, k * k, tda.TDA_ROUTE_FACTORED)
+    tda.tda_device_status()
+    got = phi.cpu().numpy()
+    ref = orc.project(A[:2].astype(np.float64), B[:2].astype(np.float64), k, k, 7, 2).reshape(2, -1)
+    assert max(rel(got[n], ref[n]) for n in range(2)) <= TOL
+    assert np.isinf(got[2]).all() and np.isnan(got[3]).all()
+
+
+@pytest.mark.parametrize("N,T,di,do,ki,ko", [(3, 64, 256, 512, 16, 16), (5, 33, 64, 100, 12, 7), (4, 32, 256, 256, 16, 16),
+                                             (9, 17, 36, 512, 1, 16), (7, 16, 128, 64, 8, 8), (300, 1, 4, 4, 3, 2)])
+def test_small_projection_is_the_serial_sum(dev, orc, N, T, di, do, ki, ko):
+    # short fp32 jobs of narrow layers: the sums of the definition taken in order in fp32 (features ascending, then
+    # fused multiply-adds over the tokens), reproduced bit for bit
+    A, B = factors(N, T, di, do, "f32", 65)
+    L = tda.LayerDesc(di, do, T, ki, ko, seed=7, layer=2)
+    phi = torch.empty((N, ki * ko), device=dev)
+    tda.tda_project(L, tda.TDA_F32, up(A, "f32", dev), up(B, "f32", dev), N, phi, ki * ko, tda.TDA_ROUTE_FACTORED)
+    tda.tda_device_status()
+
+    def chain(X, S):
+        o = np.zeros(X.shape[:2] + (S.shape[1],), np.float32)
+        for c in range(X.shape[2]):
+            o += X[:, :, c, None] * S[c].astype(np.float32)
+        return o
+
+    a, b = chain(A, orc.proj_entries(7, 2, 0, di, ki)), chain(B, orc.proj_entries(7, 2, 1, do, ko))
+    acc = np.zeros((N, ko, ki), np.float32)
+    for t in range(T):
+        acc = (b[:, t, :, None].astype(np.longdouble) * a[:, t, None, :] + acc).astype(np.float32)
+    ref = acc * np.float32(1.0 / (np.sqrt(float(ki)) * np.sqrt(float(ko))))
+    np.testing.assert_array_equal(phi.cpu().numpy(), ref.reshape(N, -1))
+
+
 @pytest.mark.parametrize("N,T,di,do,k,nq", [(1, 1024, 64, 72, 64, 3), (16, 300, 136, 64, 32, 2), (200, 9, 64, 64, 16, 5),
                                             (3, 130, 64, 64, 64, 1)])
 def test_token_scores_work_split(dev, orc, N, T, di, do, k, nq):
