@@ -141,10 +141,14 @@ fit_f32_kernel(St<float> st, const float* __restrict__ phi, int64_t n, int64_t l
 }
 
 // ---------------------------------------------------------------- FIT (fp64)
+// fp64 runs at two multiply-adds a clock and SM here, so what counts is that every SM has work:
+// T x T tiles with T = 64, or 16 when 64 would leave SMs idle (D = 256: 10 tiles, 75 us for 64
+// rows; 136 tiles of 16). An entry's sum runs over the rows in order whatever T is.
+template <int T>
 __global__ void __launch_bounds__(256)
 fit_f64_kernel(St<double> st, const float* __restrict__ phi, int64_t n, int64_t ld) {
     if (blockIdx.x > blockIdx.y) return;
-    constexpr int T = 64, K = 32;
+    constexpr int K = 32, R = T / 16;
     __shared__ double Xa[K][T + 1];
     __shared__ double Xb[K][T + 1];
     const int l = blockIdx.z;
@@ -152,7 +156,7 @@ fit_f64_kernel(St<double> st, const float* __restrict__ phi, int64_t n, int64_t 
     const float* ph = phi + (int64_t)l * D;
     const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16;
     const int64_t a0 = (int64_t)blockIdx.y * T, b0 = (int64_t)blockIdx.x * T;
-    double acc[4][4] = {};
+    double acc[R][R] = {};
     for (int64_t r0 = 0; r0 < n; r0 += K) {
         for (int e = tid; e < K * T; e += 256) {
             const int rr = e / T, cc = e % T;
@@ -163,15 +167,15 @@ fit_f64_kernel(St<double> st, const float* __restrict__ phi, int64_t n, int64_t 
         __syncthreads();
         for (int rr = 0; rr < K; ++rr)
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
+            for (int u = 0; u < R; ++u)
 #pragma unroll
-                for (int v = 0; v < 4; ++v) acc[u][v] += Xa[rr][ty * 4 + u] * Xb[rr][tx * 4 + v];
+                for (int v = 0; v < R; ++v) acc[u][v] += Xa[rr][ty * R + u] * Xb[rr][tx * R + v];
         __syncthreads();
     }
     double* M = st.M(l);
-    for (int u = 0; u < 4; ++u)
-        for (int v = 0; v < 4; ++v) {
-            const int64_t a = a0 + ty * 4 + u, b = b0 + tx * 4 + v;
+    for (int u = 0; u < R; ++u)
+        for (int v = 0; v < R; ++v) {
+            const int64_t a = a0 + ty * R + u, b = b0 + tx * R + v;
             if (a < D && b < D) M[a * D + b] += acc[u][v];
         }
 }
@@ -352,6 +356,164 @@ __global__ void __launch_bounds__(256) update_kernel(St<TS> st, int64_t k0) {
         }
 }
 
+// ---------------------------------------------------------------- FACTOR (fp64)
+// The same right-looking steps for an fp64 state, laid out for the fp64 pipe (two
+// multiply-adds a clock and SM, so a warp-wide one holds its pipe for tens of clocks): no
+// square root, division or triangular solve row by row on the serial path, work spread over
+// as many CTAs as there is, and nothing done twice but the 32 x 32 diagonal block.
+//
+// Panel step at k0, grid (row chunk, layer), 128 threads: a CTA eliminates the diagonal block
+// together with its 8 panel rows, A_ic -= (A_ij / p_j) A_cj with p_j = A_jj (one reciprocal per
+// column: an fp32 guess and one cubic Newton step, evaluated by every warp for itself), and
+// scales column j by 1/sqrt(p_j) at the end, all columns at once. Chunk 0 leaves L_kk in the
+// block's slot of Dinv; f64_inverse_kernel replaces it by its inverse after the last step.
+// D = 256: 150 us a step in panel_kernel (one CTA: two warps of serial chains).
+constexpr int kF64Rows = 8;
+
+// 1/p and 1/sqrt(p) for p > 0 to fp64 rounding: p = m 4^h with m in [1, 4); the fp32 guess for m
+// is within 2^-21, and one step of Householder's third-order iteration takes it past 2^-60.
+__device__ __forceinline__ double pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
+__device__ __forceinline__ double split_pow4(double p, int& h) {
+    int sub = 0;
+    if (p < 2.3e-308) p *= 18014398509481984.0, sub = 27;  // subnormal: times 2^54
+    const long long b = __double_as_longlong(p);
+    const int e = (int)(b >> 52) - 1023, odd = e & 1;
+    h = ((e - odd) >> 1) - sub;
+    return __longlong_as_double((b & 0xFFFFFFFFFFFFFll) | ((long long)(1023 + odd) << 52));
+}
+__device__ __forceinline__ double rcp_f64(double p) {
+    int h;
+    const double m = split_pow4(p, h), r = (double)__frcp_rn((float)m);
+    const double e = fma(-m, r, 1.0);
+    const bool wide = h > 510 || h < -510;
+    const double x = fma(r, fma(e, e, e), r) * pow2(wide ? -h : -2 * h);
+    return wide ? x * pow2(-h) : x;
+}
+__device__ __forceinline__ double rsqrt_f64(double p) {
+    int h;
+    const double m = split_pow4(p, h), r = (double)rsqrtf((float)m);
+    const double e = fma(-m * r, r, 1.0);
+    return fma(r * e, fma(0.375, e, 0.5), r) * pow2(-h);
+}
+
+__global__ void __launch_bounds__(128) panel_f64_kernel(St<double> st, int64_t k0) {
+    constexpr int R = kNB + kF64Rows;
+    __shared__ double A[R][kNB + 1];
+    __shared__ double inv[kNB];
+    const int l = blockIdx.y;
+    const int64_t D = st.D;
+    double* M = st.M(l);
+    const int nb = (int)((D - k0) < kNB ? (D - k0) : kNB);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t i0 = k0 + nb + (int64_t)blockIdx.x * kF64Rows;  // this CTA's panel rows
+    for (int e = tid; e < R * kNB; e += 128) {
+        const int i = e / kNB, j = e % kNB;
+        double v;
+        if (i < kNB)  // identity padding of a ragged last block
+            v = (i < nb && j < nb) ? (j <= i ? M[(k0 + i) * D + k0 + j] : 0.0) : (i == j ? 1.0 : 0.0);
+        else
+            v = (i0 + i - kNB < D && j < nb) ? M[(i0 + i - kNB) * D + k0 + j] : 0.0;
+        A[i][j] = v;
+    }
+    __syncthreads();
+    int bad = -1;
+    for (int j = 0; j < kNB - 1; ++j) {
+        const double p = A[j][j];
+        const bool ok = p > 0.0;
+        if (!ok && bad < 0) bad = j;
+        const double w = ok ? rcp_f64(p) : NAN;
+        // column c of the diagonal block's row `lane`, c = j + 1 + warp + 4 u <= lane
+        const double t = A[lane][j] * w;
+        for (int c = j + 1 + warp; c < kNB; c += 4)
+            if (c <= lane) A[lane][c] -= t * A[c][j];
+        // the panel rows: 8 rows x the columns after j, 16 columns at a time
+        const int pr = kNB + (tid & 7);
+        const double tp = A[pr][j] * w;
+        for (int c = j + 1 + (tid >> 3); c < kNB; c += 16) A[pr][c] -= tp * A[c][j];
+        __syncthreads();
+    }
+    if (warp == 0) {
+        const double p = A[lane][lane];
+        const bool ok = p > 0.0;
+        if (lane == kNB - 1 && !ok && bad < 0) bad = kNB - 1;
+        bad = __shfl_sync(0xffffffffu, bad, kNB - 1);
+        inv[lane] = ok ? rsqrt_f64(p) : NAN;
+        if (blockIdx.x == 0 && lane == 0 && bad >= 0 && bad < nb) {
+            double* h = st.header(l);
+            if (h[kPcFailedPivot] == 0.0) h[kPcFailedPivot] = (double)(k0 + bad + 1);
+        }
+    }
+    __syncthreads();
+    // the diagonal block of M is left as it is: other CTAs of this launch read it
+    if (blockIdx.x == 0) {
+        double* Lk = st.Dinv(l) + (k0 / kNB) * (kNB * kNB);
+        for (int e = tid; e < kNB * kNB; e += 128) {
+            const int i = e / kNB, j = e % kNB;
+            Lk[e] = j <= i ? A[i][j] * inv[j] : 0.0;
+        }
+    }
+    for (int e = tid; e < kF64Rows * kNB; e += 128) {
+        const int r = e / kNB, j = e % kNB;
+        if (i0 + r < D && j < nb) M[(i0 + r) * D + k0 + j] = A[kNB + r][j] * inv[j];
+    }
+}
+
+// Trailing update in 16 x 16 tiles, two entries a thread (D = 256: up to 105 tiles instead of 10).
+__global__ void __launch_bounds__(128) update_f64_kernel(St<double> st, int64_t k0) {
+    if (blockIdx.x > blockIdx.y) return;
+    constexpr int T = 16;
+    __shared__ double Pi[T][kNB + 1];
+    __shared__ double Pj[T][kNB + 1];
+    const int l = blockIdx.z;
+    const int64_t D = st.D;
+    double* M = st.M(l);
+    const int64_t s0 = k0 + kNB;
+    const int64_t i0 = s0 + (int64_t)blockIdx.y * T, j0 = s0 + (int64_t)blockIdx.x * T;
+    const int tid = threadIdx.x;
+    for (int e = tid; e < kNB * T; e += 128) {
+        const int r = e / kNB, m = e % kNB;
+        Pi[r][m] = i0 + r < D ? M[(i0 + r) * D + k0 + m] : 0.0;
+        Pj[r][m] = j0 + r < D ? M[(j0 + r) * D + k0 + m] : 0.0;
+    }
+    __syncthreads();
+    const int ty = tid / T, tx = tid % T;
+    double a0 = 0.0, a1 = 0.0;
+#pragma unroll 8
+    for (int m = 0; m < kNB; ++m) {
+        a0 += Pi[ty][m] * Pj[tx][m];
+        a1 += Pi[ty + 8][m] * Pj[tx][m];
+    }
+    const int64_t i = i0 + ty, j = j0 + tx;
+    if (i < D && j <= i) M[i * D + j] -= a0;
+    if (i + 8 < D && j <= i + 8) M[(i + 8) * D + j] -= a1;
+}
+
+// Dinv's slots from L_kk to its inverse, grid (block, layer): lane c of every warp holds column c
+// of X, L X = I, eliminated column by column; the four warps take every fourth row.
+__global__ void __launch_bounds__(128) f64_inverse_kernel(St<double> st) {
+    __shared__ double L[kNB][kNB + 1];
+    __shared__ double X[kNB][kNB + 1];
+    double* Di = st.Dinv(blockIdx.y) + (int64_t)blockIdx.x * (kNB * kNB);
+    const int tid = threadIdx.x, c = tid & 31, warp = tid >> 5;
+    for (int e = tid; e < kNB * kNB; e += 128) {
+        L[e / kNB][e % kNB] = Di[e];
+        X[e / kNB][e % kNB] = e / kNB == e % kNB ? 1.0 : 0.0;
+    }
+    __syncthreads();
+    __shared__ double inv[kNB];
+    if (tid < kNB) inv[tid] = 1.0 / L[tid][tid];
+    __syncthreads();
+    for (int i = 0; i < kNB; ++i) {
+        const double x = X[i][c] * inv[i];
+        for (int m = i + 1 + warp; m < kNB; m += 4) X[m][c] -= L[m][i] * x;
+        __syncthreads();
+    }
+    for (int e = tid; e < kNB * kNB; e += 128) {
+        const int i = e / kNB, j = e % kNB;
+        Di[e] = j <= i ? X[i][j] * inv[i] : 0.0;
+    }
+}
+
 // ---------------------------------------------------------------- APPLY
 // grid (query group, layer). G query rows per CTA; y[G][D] in shared memory.
 // Forward, block b:  r = q_b - L_{b,<b} y_<b ;  y_b = Dinv_b r
@@ -384,6 +546,47 @@ apply_kernel(St<TS> st, const float* __restrict__ q, int64_t n_q, int64_t ld_q, 
         const int64_t b0 = bi * kNB;
         const int nb = (int)((D - b0) < kNB ? (D - b0) : kNB);
         for (int e = tid; e < kNB * kNB; e += blockDim.x) Dsm[e / kNB][e % kNB] = Dv[bi * kNB * kNB + e];
+        if constexpr (sizeof(TS) == 8) {
+            // fp64: lane = row, the warps share the columns (an fp64 add per shuffle of a row sum
+            // would cost more than the row), partial sums meet in shared memory
+            TS acc[G];
+#pragma unroll
+            for (int g = 0; g < G; ++g) acc[g] = (TS)0;
+            if (lane < nb)
+#pragma unroll 4
+                for (int64_t m = warp; m < b0; m += 8) {
+                    const TS lv = L[(b0 + lane) * D + m];
+#pragma unroll
+                    for (int g = 0; g < G; ++g) acc[g] += lv * y[g * D + m];
+                }
+#pragma unroll
+            for (int g = 0; g < G; ++g) part[warp][g][lane] = acc[g];
+            __syncthreads();
+            for (int e = tid; e < G * kNB; e += blockDim.x) {
+                const int g = e / kNB, i = e % kNB;
+                TS t = (TS)0;
+                for (int w = 0; w < 8; ++w) t += part[w][g][i];
+                r[g][i] = (i < nb && g < gn) ? (TS)q[(g0 + g) * ld_q + (int64_t)l * D + b0 + i] - t : (TS)0;
+            }
+            __syncthreads();
+            // y_b = Dinv_b r: warp w takes columns 4w .. 4w + 3
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+                TS t = (TS)0;
+#pragma unroll
+                for (int j = 4 * warp; j < 4 * warp + 4; ++j) t += Dsm[lane][j] * r[g][j];
+                part[warp][g][lane] = t;
+            }
+            __syncthreads();
+            for (int e = tid; e < G * kNB; e += blockDim.x) {
+                const int g = e / kNB, i = e % kNB;
+                TS t = (TS)0;
+                for (int w = 0; w < 8; ++w) t += part[w][g][i];
+                if (i < nb) y[g * D + b0 + i] = t;
+            }
+            __syncthreads();
+            continue;
+        }
         for (int ii = warp; ii < kNB; ii += 8) {
             TS acc[G];
 #pragma unroll
@@ -438,10 +641,23 @@ apply_kernel(St<TS> st, const float* __restrict__ q, int64_t n_q, int64_t ld_q, 
             r[g][i] = (i < nb) ? y[g * D + b0 + i] - t : (TS)0;
         }
         __syncthreads();
+        if constexpr (sizeof(TS) == 8) {
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+                TS t = (TS)0;
+#pragma unroll
+                for (int j = 4 * warp; j < 4 * warp + 4; ++j) t += Dsm[j][lane] * r[g][j];
+                part[warp][g][lane] = t;
+            }
+            __syncthreads();
+        }
         for (int e = tid; e < G * kNB; e += blockDim.x) {
             const int g = e / kNB, i = e % kNB;
             TS s = (TS)0;
-            for (int j = i; j < kNB; ++j) s += Dsm[j][i] * r[g][j];
+            if constexpr (sizeof(TS) == 8)
+                for (int w = 0; w < 8; ++w) s += part[w][g][i];
+            else
+                for (int j = i; j < kNB; ++j) s += Dsm[j][i] * r[g][j];
             if (i < nb) y[g * D + b0 + i] = s;
         }
         __syncthreads();
@@ -1004,15 +1220,34 @@ cudaError_t factor_impl(int n_layers, int64_t D, void* state, int64_t n_total, d
     int64_t blocks = (D * D * n_layers + 255) / 256;
     if (blocks > 152 * 16) blocks = 152 * 16;
     scale_kernel<TS><<<(unsigned)blocks, 256, 0, s>>>(st, n_layers);
-    for (int64_t k0 = 0; k0 < D; k0 += kNB) {
-        const int64_t rest = D - k0 - kNB;
-        const unsigned chunks = (unsigned)(rest > 0 ? (rest + 255) / 256 : 1);
-        note_launches(1);
-        panel_kernel<TS><<<dim3(n_layers, chunks), 256, 0, s>>>(st, k0);
-        if (rest > 0) {
-            const unsigned t = (unsigned)((rest + 63) / 64);
+    if constexpr (sizeof(TS) == 8) {
+        for (int64_t k0 = 0; k0 < D; k0 += kNB) {
+            const int64_t rest = D - k0 - kNB;
             note_launches(1);
-            update_kernel<TS><<<dim3(t, t, n_layers), 256, 0, s>>>(st, k0);
+            panel_f64_kernel<<<dim3((unsigned)(rest > 0 ? (rest + kF64Rows - 1) / kF64Rows : 1), n_layers), 128, 0, s>>>(
+                st, k0);
+            if (rest <= 0) continue;
+            // 64 x 64 tiles (a quarter of the loads per entry) once they fill the chip
+            const unsigned t64 = (unsigned)((rest + 63) / 64), t16 = (unsigned)((rest + 15) / 16);
+            note_launches(1);
+            if ((int64_t)t64 * (t64 + 1) / 2 * n_layers >= 304)
+                update_kernel<TS><<<dim3(t64, t64, n_layers), 256, 0, s>>>(st, k0);
+            else
+                update_f64_kernel<<<dim3(t16, t16, n_layers), 128, 0, s>>>(st, k0);
+        }
+        note_launches(1);
+        f64_inverse_kernel<<<dim3((unsigned)((D + kNB - 1) / kNB), n_layers), 128, 0, s>>>(st);
+    } else {
+        for (int64_t k0 = 0; k0 < D; k0 += kNB) {
+            const int64_t rest = D - k0 - kNB;
+            const unsigned chunks = (unsigned)(rest > 0 ? (rest + 255) / 256 : 1);
+            note_launches(1);
+            panel_kernel<TS><<<dim3(n_layers, chunks), 256, 0, s>>>(st, k0);
+            if (rest > 0) {
+                const unsigned t = (unsigned)((rest + 63) / 64);
+                note_launches(1);
+                update_kernel<TS><<<dim3(t, t, n_layers), 256, 0, s>>>(st, k0);
+            }
         }
     }
     return cudaGetLastError();
@@ -1371,8 +1606,11 @@ cudaError_t launch_pc_fit(int n_layers, int64_t D, tda_dtype sdt, void* state, c
     }
     note_launches(1);
     if (sdt == TDA_F64) {
-        const unsigned t = (unsigned)((D + 63) / 64);
-        fit_f64_kernel<<<dim3(t, t, n_layers), 256, 0, s>>>(state_of<double>(state, D), phi, n, ld);
+        const unsigned t = (unsigned)((D + 63) / 64), t16 = (unsigned)((D + 15) / 16);
+        if ((int64_t)t * (t + 1) / 2 * n_layers >= 304)
+            fit_f64_kernel<64><<<dim3(t, t, n_layers), 256, 0, s>>>(state_of<double>(state, D), phi, n, ld);
+        else
+            fit_f64_kernel<16><<<dim3(t16, t16, n_layers), 256, 0, s>>>(state_of<double>(state, D), phi, n, ld);
     } else {
         const unsigned t = (unsigned)((D + kFT - 1) / kFT);
         fit_f32_kernel<<<dim3(t, t, n_layers), 256, 0, s>>>(state_of<float>(state, D), phi, n, ld);
@@ -1414,9 +1652,10 @@ cudaError_t launch_pc_apply(int n_layers, int64_t D, tda_dtype sdt, const void* 
     const size_t el = sdt == TDA_F64 ? 8 : 4;
     const size_t budget = 160 * 1024;
     if (sdt == TDA_F64) {
-        if ((size_t)D * el * 8 <= budget)
+        // fewer queries per CTA while CTAs are what is missing (the fp64 pipe is per SM)
+        if ((size_t)D * el * 8 <= budget && (n_q + 1) / 2 * n_layers >= 152)
             return apply_impl<double, 8>(n_layers, D, state, q, n_q, ld_q, qhat, ld_qhat, s);
-        if ((size_t)D * el * 2 <= budget)
+        if ((size_t)D * el * 2 <= budget && n_q * n_layers >= 152)
             return apply_impl<double, 2>(n_layers, D, state, q, n_q, ld_q, qhat, ld_qhat, s);
         return apply_impl<double, 1>(n_layers, D, state, q, n_q, ld_q, qhat, ld_qhat, s);
     }

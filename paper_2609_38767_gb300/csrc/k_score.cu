@@ -97,6 +97,29 @@ score_kernel(const TQ* __restrict__ Q, int64_t n_q, int64_t ld_q, const float* _
         }
 }
 
+// fp64 scores of few rows: one warp per (query, train) pair, lanes along the features. Two fp64
+// multiply-adds a clock and SM make idle SMs the cost: 8 x 64 scores of 256 features are one tile
+// of score_kernel (146 us on one SM) but 512 warps on 64.
+__global__ void __launch_bounds__(256)
+score_f64_pairs_kernel(const double* __restrict__ Q, int64_t n_q, int64_t ld_q, const float* __restrict__ P,
+                       int64_t n_t, int64_t ld_p, int64_t D, float* __restrict__ S, int64_t ld_S, float beta) {
+    const int64_t e = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (e >= n_q * n_t) return;
+    const int64_t q = e / n_t, i = e - q * n_t;
+    const double* a = Q + q * ld_q;
+    const float* b = P + i * ld_p;
+    double acc = 0.0;
+#pragma unroll 4
+    for (int64_t f = lane; f < D; f += 32) acc += a[f] * (double)b[f];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) {
+        float* dst = S + q * ld_S + i;
+        *dst = beta == 0.f ? (float)acc : (float)((double)beta * (double)(*dst) + acc);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Top-k. Each entry gets a 64-bit key whose descending order is "score
 // descending, then index ascending": the high word maps the float to an
@@ -210,7 +233,12 @@ cudaError_t launch_score(const void* Qhat, tda_dtype qdt, int64_t n_q, int64_t l
     if (n_q == 0 || n_t == 0) return cudaSuccess;
     dim3 grid((unsigned)((n_t + kTT - 1) / kTT), (unsigned)((n_q + kTQ - 1) / kTQ));
     note_launches(1);
-    if (qdt == TDA_F64)
+    // tiles for fewer than a quarter of the SMs: pairs (a tile does 2048 pairs' sums at once, a
+    // warp's own pays five adds and its share of idle lanes, about twice as much fp64 work)
+    if (qdt == TDA_F64 && (int64_t)grid.x * grid.y < 38)
+        score_f64_pairs_kernel<<<(unsigned)((n_q * n_t + 7) / 8), 256, 0, s>>>((const double*)Qhat, n_q, ld_q, Phi, n_t,
+                                                                              ld_phi, D, S, ld_S, beta);
+    else if (qdt == TDA_F64)
         score_kernel<double, double><<<grid, kSThreads, 0, s>>>(
             (const double*)Qhat, n_q, ld_q, Phi, n_t, ld_phi, D, S, ld_S, beta, D, 0);
     else

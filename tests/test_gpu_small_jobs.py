@@ -1,0 +1,79 @@
+"""The latency-bound small kernels at the sizes where they can go wrong: the fp64 preconditioner (ragged last blocks,
+one to several CTAs of panel rows, tile sizes, pivots far from one) and fp64 scores of few rows."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2609_38767_gb300 as tda
+from paper_2609_38767_gb300 import build as tbuild
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dev():
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    tbuild.build()
+    tda.load()
+    return torch.device("cuda:0")
+
+
+# fp64 state: backward error of a Cholesky solve is a few D eps of the condition number; with damping of a tenth of
+# the mean eigenvalue and more rows than features it is below 100, so 1e-11 (D = 600: 600 * 2.2e-16 * 100) holds.
+@pytest.mark.parametrize("D,nl,nq,scale", [(1, 1, 1, 1.0), (31, 2, 3, 1.0), (32, 1, 9, 1.0), (33, 1, 160, 1.0),
+                                           (144, 2, 5, 1.0), (256, 1, 8, 1e-17), (256, 1, 40, 3e17), (600, 1, 2, 1.0)])
+def test_fp64_preconditioner(dev, D, nl, nq, scale):
+    rng = np.random.default_rng(D + nq)
+    n = 2 * D + 5
+    phi = (rng.standard_normal((n, nl * D)) * scale).astype(np.float32)
+    q = rng.standard_normal((nq, nl * D)).astype(np.float32)
+    per = tda.tda_precondition_state_bytes(D, tda.TDA_F64)
+    state = torch.empty(nl * per, dtype=torch.uint8, device=dev)
+    ph, qd = torch.from_numpy(phi).to(dev), torch.from_numpy(q).to(dev)
+    out = torch.empty((nq, nl * D), dtype=torch.float64, device=dev)
+    args = (nl, D, tda.TDA_F64, state)
+    tda.tda_precondition(tda.TDA_PC_RESET, *args)
+    for a, b in ((0, n // 3), (n // 3, n)):
+        tda.tda_precondition(tda.TDA_PC_FIT_ACCUM, *args, phi=ph[a:], n=b - a, ld_phi=nl * D)
+    tda.tda_precondition(tda.TDA_PC_FACTOR, *args, n_total=n, lambda_rel_mean_eig=0.1)
+    tda.tda_precondition(tda.TDA_PC_APPLY, *args, q=qd, n_q=nq, ld_q=nl * D, qhat=out, ld_qhat=nl * D)
+    info = tda.tda_precondition_info(nl, D, tda.TDA_F64, state)
+    for l in range(nl):
+        x = phi[:, l * D:(l + 1) * D].astype(np.float64)
+        F = x.T @ x / n
+        lam = 0.1 * np.trace(F) / D
+        assert abs(info[4 * l] / lam - 1) < 1e-12 and info[4 * l + 2] == 0
+        ref = np.linalg.solve(F + lam * np.eye(D), q[:, l * D:(l + 1) * D].T.astype(np.float64)).T
+        got = out[:, l * D:(l + 1) * D].cpu().numpy()
+        assert np.linalg.norm(got - ref) <= 1e-11 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("D,bad", [(5, 0), (40, 31), (40, 33), (100, 70)])
+def test_fp64_failed_pivot_is_reported(dev, D, bad):
+    state = torch.empty(tda.tda_precondition_state_bytes(D, tda.TDA_F64), dtype=torch.uint8, device=dev)
+    tda.tda_precondition(tda.TDA_PC_RESET, 1, D, tda.TDA_F64, state)
+    m = state[64:64 + 8 * D * D].view(torch.float64).view(D, D)
+    m.copy_(torch.eye(D, dtype=torch.float64, device=dev))
+    m[bad, bad] = -50.0
+    out = torch.zeros((2, D), dtype=torch.float64, device=dev)
+    tda.tda_precondition(tda.TDA_PC_FACTOR_APPLY, 1, D, tda.TDA_F64, state, n_total=1, lambda_abs=1e-3,
+                         q=torch.ones((2, D), device=dev), n_q=2, ld_q=D, qhat=out, ld_qhat=D)
+    with pytest.raises(tda.TdaError) as e:
+        tda.tda_precondition_info(1, D, tda.TDA_F64, state)
+    assert e.value.status == tda.TDA_ERR_NOT_SPD and f"pivot {bad + 1}" in str(e.value)
+    assert torch.isnan(out).all()
+
+
+@pytest.mark.parametrize("nq,nt,D,beta", [(1, 1, 1, 0.0), (8, 64, 256, 0.0), (3, 77, 45, 1.0), (33, 1100, 40, 0.5),
+                                          (64, 1300, 31, 0.0)])
+def test_fp64_scores(dev, nq, nt, D, beta):
+    rng = np.random.default_rng(nt)
+    Q, P = rng.standard_normal((nq, D)), rng.standard_normal((nt, D)).astype(np.float32)
+    S = torch.full((nq, nt + 2), 2.0, device=dev)
+    tda.tda_score(torch.from_numpy(Q).to(dev), tda.TDA_F64, nq, D, torch.from_numpy(P).to(dev), nt, D, D, S, nt + 2,
+                  beta)
+    got = S.cpu().numpy()
+    ref = Q @ P.T.astype(np.float64) + 2.0 * beta
+    # one rounding to fp32 (half an ulp) of a sum that fp64 holds to far below it
+    assert (np.abs(got[:, :nt] - ref) <= 2.0 ** -23 * np.abs(ref) + 1e-12).all()
+    assert (got[:, nt:] == 2.0).all()
