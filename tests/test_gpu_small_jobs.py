@@ -1,5 +1,6 @@
 """The latency-bound small kernels at the sizes where they can go wrong: the fp64 preconditioner (ragged last blocks,
-one to several CTAs of panel rows, tile sizes, pivots far from one) and fp64 scores of few rows."""
+one to several CTAs of panel rows, tile sizes, pivots far from one), fp64 scores of few rows, and the top-k selection
+(row lengths around every kernel's limit, ties that need the index digits, non-finite scores)."""
 import numpy as np
 import pytest
 import torch
@@ -77,3 +78,29 @@ def test_fp64_scores(dev, nq, nt, D, beta):
     # one rounding to fp32 (half an ulp) of a sum that fp64 holds to far below it
     assert (np.abs(got[:, :nt] - ref) <= 2.0 ** -23 * np.abs(ref) + 1e-12).all()
     assert (got[:, nt:] == 2.0).all()
+
+
+@pytest.mark.parametrize("nt", [1, 31, 512, 513, 2048, 2049, 8192, 8193, 16384, 16385, 40000])
+@pytest.mark.parametrize("values", ["normal", "ties", "equal", "odd"])
+def test_topk_selection(dev, orc, nt, values):
+    rng = np.random.default_rng(nt)
+    nq = 3
+    if values == "normal":
+        S = rng.standard_normal((nq, nt))
+    elif values == "ties":
+        S = rng.integers(-3, 4, (nq, nt)) / 2.0
+    elif values == "equal":
+        S = np.full((nq, nt), -1.5)
+    else:
+        S = rng.choice([0.0, -0.0, np.inf, -np.inf, np.nan, 1e-40, -1e-40, 3.4e38, 1.0], (nq, nt))
+    S = S.astype(np.float32)
+    Sd = torch.zeros((nq, nt + 5), device=dev)
+    Sd[:, :nt] = torch.from_numpy(S).to(dev)
+    for k in sorted({1, min(nt, 100), min(nt, 257), min(nt, 1024)}):
+        idx = torch.full((nq, k), -7, dtype=torch.int32, device=dev)
+        val = torch.empty((nq, k), device=dev)
+        tda.tda_topk(Sd, nq, nt, nt + 5, k, idx, val)
+        oi, _ = orc.topk(S.astype(np.float64), k)
+        np.testing.assert_array_equal(idx.cpu().numpy(), oi)
+        np.testing.assert_array_equal(val.cpu().numpy().view(np.uint32),
+                                      np.take_along_axis(S, oi.astype(np.int64), 1).view(np.uint32))
