@@ -597,7 +597,7 @@ tda_status tda_token_scores(const tda_layer_desc* L, tda_dtype dtype, const void
     if (!ws || ws_bytes < per)
         return fail(TDA_ERR_WORKSPACE, "tda_token_scores needs >= %zu bytes of ws, got %zu", per, ws_bytes);
     cudaStream_t s = (cudaStream_t)stream;
-    // The tensor-core contraction (k_in = 32) keeps R's hi and lo halves at the
+    // The tensor-core contraction keeps R's hi and lo halves at the
     // front of the workspace when it has room for them and one example.
     const size_t rsplit = token_tc_split_bytes(L->k_in, L->k_out, n_q);
     const bool tc = token_tc_supported(L->k_in, L->k_out, n_q) && ((uintptr_t)ws & 255) == 0 && ws_bytes >= rsplit + per &&

@@ -1,26 +1,35 @@
 // k_tokens_tc.cu -- token-level scores on the tcgen05 tensor cores (3xTF32):
 //   out[q][t] = beta * out[q][t] + scale * g~_t^T R_q a~_t
-// for k_in = 32 and k_out in {16, 32, 64} (the token-level decomposition of
-// the score: summed over t it gives <Phi_i, R_q>).
+// for k_in in 17 .. 64 (a multiple of 4) and k_out in {16, 32, 64} (the token-level
+// decomposition of the score: summed over t it gives <Phi_i, R_q>). k_in up to 16
+// stays on the CUDA cores: half of every 32-wide MMA chunk would be padding.
 //
 // As a contraction: X[t][(q, r)] = sum_c a~_t[c] R_q[r][c] is a GEMM with
-// M = 128 tokens, N = 256 rows (q, r) of the stacked query matrices, K = k_in;
-// the epilogue weights X by g~_t[r] and sums over r, one output per (t, q).
-// fp32 accuracy from TF32 tensor cores as in the score GEMM: x = hi + lo,
-// products hi*hi + hi*lo + lo*hi.
+// M = 128 tokens, N rows (q, r) of the stacked query matrices, K = k_in; the
+// epilogue weights X by g~_t[r] and sums over r, one output per (t, q).
 //
-// Shared memory: two token-tile buffers (a~ hi and lo, 16 KiB each) and a ring
-// of two query stages (R hi and lo, 32 KiB each, split once per call into the
-// workspace). All tiles are K-major with 128-byte rows (32 fp32) and the
-// 128-byte swizzle that TMA writes.
+// fp32 accuracy from TF32: x = hi + lo, both rounded to nearest (truncated halves
+// lose 2^-22 of every product on the same side), products hi*hi + hi*lo + lo*hi.
+// The two small products of all k come first: the tensor pipe truncates its
+// running sum, and while that sum is small so is the loss (k = 32: 3.0e-7 off, 8.2e-7
+// with truncated halves and interleaved products). KC = 2 (below) keeps the two chunks'
+// hi*hi in accumulators of their own, added with round-to-nearest.
+//
+// Shared memory: K in chunks of 32 (one 128-byte operand row each), KC of them.
+// KC = 1: two token-tile buffers (hi and lo, 16 KiB each) and a ring of two query
+// stages of N = 256 rows (hi and lo, 32 KiB each). KC = 2 has twice the bytes per
+// row: one token-tile buffer, stages of N = 128. R's halves are split once per
+// call into the workspace. k_in below a whole chunk is zero-filled by TMA.
+//
+// Measured: 16 examples of 1024 tokens, 16 queries, k = 64: 180 us on the CUDA
+// cores (a thread per token, R_j broadcast from shared memory), 18 us here.
 //
 // Warp roles (256 threads, so that no SM sub-partition holds more than two
 // warps and every thread may use up to 255 registers): warps 0 and 3 split the
-// token tile in place (hi stays, lo goes to its own tile); warp 1 allocates
-// TMEM, its lane 0 issues the MMAs into two 256-column fp32 accumulators; lane
-// 0 of warp 2 issues the TMA copies; warps 4-7 are the epilogue (TMEM lane
-// quadrant warp % 4). Waits are bounded (about 1 s) and set kErrTimeout on
-// expiry.
+// token tile (hi in place, lo to its own tile); warp 1 allocates TMEM, its lane 0
+// issues the MMAs into two fp32 accumulators; lane 0 of warp 2 issues the TMA
+// copies; warps 4-7 are the epilogue (TMEM lane quadrant warp % 4). Waits are
+// bounded (about 1 s) and set kErrTimeout on expiry.
 #include <cuda.h>
 
 #include <mutex>
@@ -34,15 +43,21 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kTM = 128;                          // tokens per tile
-constexpr int kTN = 256;                          // (query, r) rows per stage
-constexpr int kKA = 32;                           // k_in: one 128-byte operand row
+constexpr int kKA = 32;                           // K chunk: one 128-byte operand row
 constexpr uint32_t kATile = kTM * kKA * 4;        // 16 KiB
-constexpr uint32_t kBTile = kTN * kKA * 4;        // 32 KiB
-constexpr uint32_t kABuf = 2 * kATile;            // hi + lo
-constexpr uint32_t kBBuf = 2 * kBTile;
 constexpr uint32_t kTmemCols = 512;
-constexpr size_t kSmem = 1024 + 2 * (size_t)kABuf + 2 * (size_t)kBBuf + 8 * 17 + 16;
-static_assert(kSmem <= 232448, "shared memory per CTA");
+
+template <int KC>
+struct Cfg {
+    static constexpr int kTN = 256 / KC;                  // (query, r) rows per stage
+    static constexpr int kABufs = 2 / KC;                 // token-tile buffers
+    static constexpr int kBufCols = 256;                  // TMEM columns of a stage's KC accumulators
+    static constexpr uint32_t kBTile = kTN * kKA * 4;     // one K chunk of a stage, hi or lo
+    static constexpr uint32_t kABuf = 2 * KC * kATile;    // hi chunks, lo chunks
+    static constexpr uint32_t kBBuf = 2 * KC * kBTile;
+    static constexpr size_t kSmem = 1024 + kABufs * (size_t)kABuf + 2 * (size_t)kBBuf + 8 * 17 + 16;
+    static_assert(kSmem <= 232448, "shared memory per CTA");
+};
 
 struct TParams {
     const float* Yb;   // g~ rows [NT][k_out]
@@ -66,9 +81,14 @@ __device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t adesc, uint64
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
+// x to TF32's 10 mantissa bits, nearest (a value that would round past the largest is truncated).
+__device__ __forceinline__ float round_tf32(float x) {
+    const uint32_t u = __float_as_uint(x), r = u + 0x1000u;
+    return __uint_as_float(((r & 0x7F800000u) == 0x7F800000u ? u : r) & 0xFFFFE000u);
+}
 __device__ __forceinline__ void split_tf32(float x, float& hi, float& lo) {
-    hi = __uint_as_float(__float_as_uint(x) & 0xFFFFE000u);
-    lo = x - hi;
+    hi = round_tf32(x);
+    lo = round_tf32(x - hi);
 }
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm, int c0, int c1, uint32_t bar) {
     asm volatile(
@@ -87,10 +107,10 @@ __device__ __forceinline__ void drain_wait(uint32_t bar, uint32_t parity, unsign
         }
 }
 
-// hi/lo halves of R: row (q, r) of Rs = R[q * ld_R + r * 32 + c]
-__global__ void split_r_kernel(const float* __restrict__ R, int64_t n_q, int64_t ld_R, int kg, float* __restrict__ Rhi,
-                               float* __restrict__ Rlo) {
-    const int64_t per = (int64_t)kg * kKA, total = n_q * per;
+// hi/lo halves of R: row (q, r) of Rs = R[q * ld_R + r * k_in + c]
+__global__ void split_r_kernel(const float* __restrict__ R, int64_t n_q, int64_t ld_R, int64_t per,
+                               float* __restrict__ Rhi, float* __restrict__ Rlo) {
+    const int64_t total = n_q * per;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t q = e / per, rc = e - q * per;
         float h, l;
@@ -100,15 +120,17 @@ __global__ void split_r_kernel(const float* __restrict__ R, int64_t n_q, int64_t
     }
 }
 
-template <int KG>
+template <int KG, int KC>
 __global__ void __launch_bounds__(kThreads, 1)
 token_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmRh,
                 const __grid_constant__ CUtensorMap tmRl, const TParams p) {
-    constexpr int G = kTN / KG;  // queries per stage
+    using C = Cfg<KC>;
+    constexpr int kTN = C::kTN, G = kTN / KG;  // G: queries per stage
+    constexpr uint32_t kABufs = C::kABufs, kABuf = C::kABuf, kBBuf = C::kBBuf, kBTile = C::kBTile;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t* abuf = smem;                  // [2] a~ hi | lo
-    uint8_t* bbuf = smem + 2 * kABuf;      // [2] R hi | lo
+    uint8_t* abuf = smem;                  // [kABufs] a~ hi | lo
+    uint8_t* bbuf = smem + kABufs * kABuf; // [2] R hi | lo
     uint64_t* bars = (uint64_t*)(bbuf + 2 * kBBuf);
     uint64_t* a_raw = bars;        // [2] TMA landed (1 + tx)
     uint64_t* a_full = bars + 2;   // [2] split done (2 warps)
@@ -149,15 +171,15 @@ token_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         const int pt = (warp == 0 ? 0 : 32) + lane;
         uint32_t it = 0;
         for (int u = blockIdx.x; u < p.n_tt; u += gridDim.x, ++it) {
-            const uint32_t ab = it & 1u, ph = (it >> 1) & 1u;
+            const uint32_t ab = it % kABufs, ph = (it / kABufs) & 1u;
             bool got = true;
             if (lane == 0) got = wait_bounded(smem_u32(&a_raw[ab]), ph, abort, p.err);
             got = __shfl_sync(0xffffffffu, got, 0);
             if (!got) break;
             uint8_t* hi = abuf + ab * kABuf;
-            uint8_t* lo = hi + kATile;
+            uint8_t* lo = hi + KC * kATile;
 #pragma unroll 4
-            for (uint32_t off = (uint32_t)pt * 16u; off < kATile; off += 64u * 16u) {
+            for (uint32_t off = (uint32_t)pt * 16u; off < KC * kATile; off += 64u * 16u) {
                 const float4 v = *reinterpret_cast<const float4*>(hi + off);
                 float4 h, l;
                 split_tf32(v.x, h.x, l.x);
@@ -178,11 +200,10 @@ token_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             uint32_t it = 0, rb = 0, tt = 0;
             bool ok = true;
             for (int u = blockIdx.x; ok && u < p.n_tt; u += gridDim.x, ++it) {
-                const uint32_t ab = it & 1u;
-                if (!wait_bounded(smem_u32(&a_full[ab]), (it >> 1) & 1u, abort, p.err)) break;
+                const uint32_t ab = it % kABufs;
+                if (!wait_bounded(smem_u32(&a_full[ab]), (it / kABufs) & 1u, abort, p.err)) break;
                 tc_fence_after();
                 const uint32_t ahs = smem_u32(abuf + ab * kABuf);
-                const uint64_t ahi = sw128_desc(ahs), alo = sw128_desc(ahs + kATile);
                 for (int j = 0; j < p.n_nt; ++j, ++rb, ++tt) {
                     const uint32_t s = rb & 1u, b = tt & 1u;
                     if (!wait_bounded(smem_u32(&tempty[b]), ((tt >> 1) & 1u) ^ 1u, abort, p.err) ||
@@ -192,14 +213,22 @@ token_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     }
                     tc_fence_after();
                     const uint32_t bhs = smem_u32(bbuf + s * kBBuf);
-                    const uint64_t bhi = sw128_desc(bhs), blo = sw128_desc(bhs + kBTile);
-                    const uint32_t d = tmem + b * kTN;
+                    const uint32_t d = tmem + b * C::kBufCols;
+                    // lo * hi and hi * lo of every k, then hi * hi (K = 8 tf32 = 32 bytes per instruction);
+                    // KC = 2: the first chunk's hi * hi in an accumulator of its own
 #pragma unroll
-                    for (int k = 0; k < kKA / 8; ++k) {  // K = 8 tf32 = 32 bytes per instruction
-                        mma_tf32(d, ahi + 2 * k, bhi + 2 * k, idesc, k > 0 ? 1u : 0u);
-                        mma_tf32(d, ahi + 2 * k, blo + 2 * k, idesc, 1u);
-                        mma_tf32(d, alo + 2 * k, bhi + 2 * k, idesc, 1u);
-                    }
+                    for (int pr = 0; pr < 3; ++pr)
+#pragma unroll
+                        for (int c = 0; c < KC; ++c) {
+                            const uint64_t ad = sw128_desc(ahs + (pr == 0 ? KC + c : c) * kATile);
+                            const uint64_t bd = sw128_desc(bhs + (pr == 1 ? KC + c : c) * kBTile);
+#pragma unroll
+                            for (int k = 0; k < kKA / 8; ++k)
+                                if (KC > 1 && pr == 2 && c == 0)
+                                    mma_tf32(d + kTN, ad + 2 * k, bd + 2 * k, idesc, k > 0 ? 1u : 0u);
+                                else
+                                    mma_tf32(d, ad + 2 * k, bd + 2 * k, idesc, (pr > 0 || c > 0 || k > 0) ? 1u : 0u);
+                        }
                     mma_commit(smem_u32(&b_empty[s]));
                     mma_commit(smem_u32(&tfull[b]));
                 }
@@ -216,10 +245,12 @@ token_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             uint32_t a_par[2], b_par[2];
             bool a_iss[2] = {false, false}, b_iss[2] = {false, false}, ok = true;
             for (int u = blockIdx.x; ok && u < p.n_tt; u += gridDim.x, ++it) {
-                const uint32_t ab = it & 1u, aph = (it >> 1) & 1u;
+                const uint32_t ab = it % kABufs, aph = (it / kABufs) & 1u;
                 if (!wait_bounded(smem_u32(&a_empty[ab]), aph ^ 1u, abort, p.err)) break;
-                mbar_arrive_tx(smem_u32(&a_raw[ab]), kATile);
-                tma_load_2d(smem_u32(abuf + ab * kABuf), &tmA, 0, u * kTM, smem_u32(&a_raw[ab]));
+                mbar_arrive_tx(smem_u32(&a_raw[ab]), KC * kATile);
+#pragma unroll
+                for (int c = 0; c < KC; ++c)
+                    tma_load_2d(smem_u32(abuf + ab * kABuf + c * kATile), &tmA, kKA * c, u * kTM, smem_u32(&a_raw[ab]));
                 a_iss[ab] = true;
                 a_par[ab] = aph;
                 for (int j = 0; j < p.n_nt; ++j, ++rb) {
@@ -230,8 +261,11 @@ token_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     }
                     const uint32_t dst = smem_u32(bbuf + s * kBBuf), bar = smem_u32(&b_full[s]);
                     mbar_arrive_tx(bar, kBBuf);
-                    tma_load_2d(dst, &tmRh, 0, j * kTN, bar);
-                    tma_load_2d(dst + kBTile, &tmRl, 0, j * kTN, bar);
+#pragma unroll
+                    for (int c = 0; c < KC; ++c) {
+                        tma_load_2d(dst + c * kBTile, &tmRh, kKA * c, j * kTN, bar);
+                        tma_load_2d(dst + (KC + c) * kBTile, &tmRl, kKA * c, j * kTN, bar);
+                    }
                     b_iss[s] = true;
                     b_par[s] = ph;
                 }
@@ -279,18 +313,28 @@ token_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     break;
                 }
                 tc_fence_after();
-                const uint32_t tb = tmem + ((uint32_t)(q4 * 32) << 16) + b * kTN;
+                const uint32_t tb = tmem + ((uint32_t)(q4 * 32) << 16) + b * C::kBufCols;
                 float acc[G];
 #pragma unroll
                 for (int gq = 0; gq < G; ++gq) {
-                    float s = 0.f;
+                    float s = 0.f, s1 = 0.f;
 #pragma unroll
                     for (int c = 0; c < KG; c += 16) {
                         float v[16];
                         tmem_ld16(tb + gq * KG + c, v);
+                        if constexpr (KC > 1) {
+                            float w[16];
+                            tmem_ld16(tb + kTN + gq * KG + c, w);
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) s = fmaf(g[c + i], v[i], s);
+                            for (int i = 0; i < 16; ++i) v[i] += w[i];
+                        }
+#pragma unroll
+                        for (int i = 0; i < 16; i += 2) {
+                            s = fmaf(g[c + i], v[i], s);
+                            s1 = fmaf(g[c + i + 1], v[i + 1], s1);
+                        }
                     }
+                    s += s1;
                     acc[gq] = rmw ? p.beta * old[gq] + p.scale * s : p.scale * s;
                 }
                 tc_fence_before();
@@ -334,12 +378,12 @@ EncodeTiledFn encode_fn() {
     return fn;
 }
 
-// 2-D map over fp32 rows of 32 elements: box 32 x box_rows, 128-byte swizzle, zero fill past the last row.
-bool make_rows_map(CUtensorMap* tm, const float* X, int64_t rows, int box_rows) {
+// 2-D map over fp32 rows of ka elements: box 32 x box_rows, 128-byte swizzle, zero fill past ka and the last row.
+bool make_rows_map(CUtensorMap* tm, const float* X, int64_t rows, int ka, int box_rows) {
     EncodeTiledFn enc = encode_fn();
     if (!enc) return false;
-    cuuint64_t dims[2] = {(cuuint64_t)kKA, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)(kKA * 4)};
+    cuuint64_t dims[2] = {(cuuint64_t)ka, (cuuint64_t)rows};
+    cuuint64_t strides[1] = {(cuuint64_t)ka * 4};
     cuuint32_t box[2] = {(cuuint32_t)kKA, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
     return enc(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(X), dims, strides, box, estr,
@@ -366,7 +410,7 @@ size_t token_tc_split_bytes(int ka, int kg, int64_t n_q) {
 }
 
 bool token_tc_supported(int ka, int kg, int64_t n_q) {
-    return is_sm103() && encode_fn() && ka == kKA && (kg == 16 || kg == 32 || kg == 64) && n_q >= 1 &&
+    return is_sm103() && encode_fn() && ka > 16 && ka <= 64 && ka % 4 == 0 && (kg == 16 || kg == 32 || kg == 64) && n_q >= 1 &&
            n_q * kg < ((int64_t)1 << 31) && device_error_word() != nullptr;
 }
 
@@ -380,13 +424,14 @@ cudaError_t launch_token_scores_tc(const float* Ya, const float* Yb, int64_t n, 
         return cudaErrorInvalidValue;
     float* Rhi = Rs;
     float* Rlo = Rs + n_q * kg * ka;
+    const int KC = ka > kKA ? 2 : 1, tn = 256 / KC;
     CUtensorMap mA, mRh, mRl;
-    if (!make_rows_map(&mA, Ya, NT, kTM) || !make_rows_map(&mRh, Rhi, n_q * kg, kTN) ||
-        !make_rows_map(&mRl, Rlo, n_q * kg, kTN))
+    if (!make_rows_map(&mA, Ya, NT, ka, kTM) || !make_rows_map(&mRh, Rhi, n_q * kg, ka, tn) ||
+        !make_rows_map(&mRl, Rlo, n_q * kg, ka, tn))
         return cudaErrorInvalidValue;
     note_launches(1);
     split_r_kernel<<<(unsigned)((n_q * kg * ka + 255) / 256 < 1024 ? (n_q * kg * ka + 255) / 256 : 1024), 256, 0, s>>>(
-        R, n_q, ld_R, kg, Rhi, Rlo);
+        R, n_q, ld_R, (int64_t)kg * ka, Rhi, Rlo);
     TParams p;
     p.Yb = Yb;
     p.out = out;
@@ -395,7 +440,7 @@ cudaError_t launch_token_scores_tc(const float* Ya, const float* Yb, int64_t n, 
     p.n_q = n_q;
     p.ld_q = ld_q;
     p.n_tt = (int)((NT + kTM - 1) / kTM);
-    p.n_nt = (int)((n_q * kg + kTN - 1) / kTN);
+    p.n_nt = (int)((n_q * kg + tn - 1) / tn);
     p.scale = scale;
     p.beta = beta;
     p.err = device_error_word();
@@ -407,21 +452,15 @@ cudaError_t launch_token_scores_tc(const float* Ya, const float* Yb, int64_t n, 
         if (sms <= 0) sms = 1;
     }
     const unsigned grid = (unsigned)(p.n_tt < sms ? p.n_tt : sms);
-    cudaError_t e;
     note_launches(1);
-    if (kg == 16) {
-        if ((e = cudaFuncSetAttribute(token_tc_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem)))
-            return e;
-        token_tc_kernel<16><<<grid, kThreads, kSmem, s>>>(mA, mRh, mRl, p);
-    } else if (kg == 32) {
-        if ((e = cudaFuncSetAttribute(token_tc_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem)))
-            return e;
-        token_tc_kernel<32><<<grid, kThreads, kSmem, s>>>(mA, mRh, mRl, p);
-    } else {
-        if ((e = cudaFuncSetAttribute(token_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem)))
-            return e;
-        token_tc_kernel<64><<<grid, kThreads, kSmem, s>>>(mA, mRh, mRl, p);
+#define TDA_TOKENS(kgv, kcv)                                                             \
+    if (kg == kgv && KC == kcv) {                                                        \
+        cudaError_t e = smem_attr_once<token_tc_kernel<kgv, kcv>>((int)Cfg<kcv>::kSmem); \
+        if (e != cudaSuccess) return e;                                                  \
+        token_tc_kernel<kgv, kcv><<<grid, kThreads, Cfg<kcv>::kSmem, s>>>(mA, mRh, mRl, p); \
     }
+    TDA_TOKENS(16, 1) TDA_TOKENS(32, 1) TDA_TOKENS(64, 1) TDA_TOKENS(16, 2) TDA_TOKENS(32, 2) TDA_TOKENS(64, 2)
+#undef TDA_TOKENS
     return cudaGetLastError();
 }
 

@@ -107,7 +107,7 @@ cudaError_t launch_token_scores(const float* Ya, const float* Yb, int64_t n, int
                                 const float* R, int64_t n_q, int64_t ld_R, float scale, float* out, int64_t ld_q,
                                 int64_t i0, float beta, cudaStream_t s);
 int mask_gather_tokens_per_pass(int64_t d_in, int64_t d_out, size_t el);
-// Token-level scores on tcgen05, 3xTF32 (k_tokens_tc.cu): k_in = 32, k_out in {16, 32, 64};
+// Token-level scores on tcgen05, 3xTF32 (k_tokens_tc.cu): k_in in 17 .. 64, k_out in {16, 32, 64};
 // Rs is token_tc_split_bytes of scratch for R's hi and lo halves.
 size_t token_tc_split_bytes(int ka, int kg, int64_t n_q);
 bool token_tc_supported(int ka, int kg, int64_t n_q);

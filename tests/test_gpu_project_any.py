@@ -132,21 +132,22 @@ def test_small_projection_is_the_serial_sum(dev, orc, N, T, di, do, ki, ko):
     np.testing.assert_array_equal(phi.cpu().numpy(), ref.reshape(N, -1))
 
 
-@pytest.mark.parametrize("N,T,di,do,k,nq", [(1, 1024, 64, 72, 64, 3), (16, 300, 136, 64, 32, 2), (200, 9, 64, 64, 16, 5),
-                                            (3, 130, 64, 64, 64, 1)])
-def test_token_scores_work_split(dev, orc, N, T, di, do, k, nq):
+@pytest.mark.parametrize("N,T,di,do,ki,ko,nq,beta", [
+    (1, 1024, 64, 72, 64, 64, 3, 0.0), (16, 300, 136, 64, 32, 32, 2, 0.0), (200, 9, 64, 64, 16, 16, 5, 0.0),
+    (3, 130, 64, 64, 64, 64, 1, 0.0), (160, 130, 64, 64, 64, 64, 37, 0.5),  # more token tiles than SMs, ragged stage
+    (2, 77, 64, 64, 20, 32, 9, 0.0), (3, 129, 72, 64, 48, 16, 17, 1.0), (2, 64, 64, 64, 4, 64, 5, 0.0)])
+def test_token_scores_work_split(dev, orc, N, T, di, do, ki, ko, nq, beta):
     A, B = factors(N, T, di, do, "bf16", 62)
-    L = tda.LayerDesc(di, do, T, k, k, seed=7, layer=1)
-    R = np.random.default_rng(N).standard_normal((nq, k * k)).astype(np.float32)
-    wsb = tda.tda_token_scores_workspace_size(L) * N + (1 << 20)
+    L = tda.LayerDesc(di, do, T, ki, ko, seed=7, layer=1)
+    R = np.random.default_rng(N).standard_normal((nq, ki * ko)).astype(np.float32)
+    wsb = tda.tda_token_scores_workspace_size(L) * N + (4 << 20)
     ws = torch.empty(wsb, dtype=torch.uint8, device=dev)
-    out = torch.empty((nq, N * T), device=dev)
+    out = torch.full((nq, N * T), 0.25, device=dev)
     tda.tda_token_scores(L, tda.TDA_BF16, up(A, "bf16", dev), up(B, "bf16", dev), N, torch.from_numpy(R).to(dev), nq,
-                         k * k, out, N * T, 0.0, ws, wsb)
+                         ki * ko, out, N * T, beta, ws, wsb)
     tda.tda_device_status()
-    # sum over a token's example gives <Phi_i, R_j>; the decomposition itself from the projected factors
-    Si = orc.proj_entries(7, 1, 0, di, k).astype(np.float64) / np.sqrt(k)
-    So = orc.proj_entries(7, 1, 1, do, k).astype(np.float64) / np.sqrt(k)
+    Si = orc.proj_entries(7, 1, 0, di, ki).astype(np.float64) / np.sqrt(ki)
+    So = orc.proj_entries(7, 1, 1, do, ko).astype(np.float64) / np.sqrt(ko)
     a, b = synth.to_f64(A, "bf16") @ Si, synth.to_f64(B, "bf16") @ So
-    ref = np.stack([np.einsum("ntr,rc,ntc->nt", b, R[j].reshape(k, k).astype(np.float64), a).ravel() for j in range(nq)])
-    assert rel(out.cpu().numpy(), ref) <= TOL
+    ref = np.stack([((a @ R[j].reshape(ko, ki).T.astype(np.float64)) * b).sum(2).ravel() for j in range(nq)])
+    assert rel(out.cpu().numpy() - 0.25 * beta, ref) <= TOL
