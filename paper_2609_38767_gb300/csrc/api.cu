@@ -766,13 +766,9 @@ tda_status tda_project_kfac(const tda_layer_desc* L, tda_dtype dtype, const void
     const int64_t k = L->k_in, kk = k * k;
     double* sd = (double*)state;
     const double sc = 1.0 / (double)k;
-    if ((st = cuda_check(launch_kfac_sum_partials(part, grid, 2 * kk, kk, sd + kfac_offset_sa(k, k), sc, sd, 0,
-                                                  (double)N * (double)L->T, s),
-                         "kfac sums a")))
-        return st;
-    return cuda_check(launch_kfac_sum_partials(part + kk, grid, 2 * kk, kk, sd + kfac_offset_sg(k, k), sc, nullptr, 0,
-                                               0.0, s),
-                      "kfac sums g");
+    return cuda_check(launch_kfac_sum_partials(part, grid, 2 * kk, 2 * kk, kk, sd + kfac_offset_sa(k, k),
+                                               sd + kfac_offset_sg(k, k), sc, sd, 0, (double)N * (double)L->T, s),
+                      "kfac sums");
 }
 
 tda_status tda_kfac_eigen(int32_t n_layers, int32_t k_in, int32_t k_out, void* state, void* stream) {

@@ -72,14 +72,28 @@ cov_partial_kernel(const float* __restrict__ Y, int64_t rows, int k, int64_t row
     }
 }
 
-// S[e] += scale * sum_b part[b * stride + e] in block order (fp64); header[slot] += add
-__global__ void sum_partials_kernel(const float* __restrict__ part, int nblk, int64_t stride, int64_t n,
-                                    double* __restrict__ S, double scale, double* __restrict__ header, int slot,
-                                    double add) {
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-        double v = 0.0;
-        for (int b = 0; b < nblk; ++b) v += (double)part[(int64_t)b * stride + e];
-        S[e] += scale * v;
+// S[e] += scale * sum_b part[b * stride + e] in fp64, n entries: the first n0 to S0, the others to
+// S1; header[slot] += add. A CTA has 32 entries: each of its 8 warps adds an eighth of the blocks in
+// order, then the eighths are added in order. (One thread per entry is a chain of loads and of fp64
+// adds on four SMs: 35 us for the 152 blocks of a k = 32 projection, twice per linear; 6 now.)
+__global__ void __launch_bounds__(256)
+sum_partials_kernel(const float* __restrict__ part, int nblk, int64_t stride, int64_t n, int64_t n0,
+                    double* __restrict__ S0, double* __restrict__ S1, double scale, double* __restrict__ header,
+                    int slot, double add) {
+    __shared__ double sub[8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int per = (nblk + 7) / 8, b0 = warp * per, b1 = b0 + per < nblk ? b0 + per : nblk;
+    const int64_t e = (int64_t)blockIdx.x * 32 + lane;
+    double v = 0.0;
+    if (e < n)
+#pragma unroll 8
+        for (int b = b0; b < b1; ++b) v += (double)part[(int64_t)b * stride + e];
+    sub[warp][lane] = v;
+    __syncthreads();
+    if (warp == 0 && e < n) {
+        for (int w = 1; w < 8; ++w) v += sub[w][lane];
+        double* dst = e < n0 ? S0 + e : S1 + (e - n0);
+        *dst += scale * v;
     }
     if (header && blockIdx.x == 0 && threadIdx.x == 0) header[slot] += add;
 }
@@ -423,85 +437,99 @@ ekfac_reg_kernel(const float* __restrict__ phi, int64_t n, int64_t ld, const dou
     for (int m = 0; m < RPT; ++m) out[(g + RG * m) * K + c] = acc[m];
 }
 
-// Le of every layer += its block partials (fixed order); N += n
-__global__ void ekfac_reduce_kernel(const float* __restrict__ part, int nblk, double* __restrict__ st0, int64_t stride,
-                                    int64_t ka, int64_t kg, double n) {
-    const int layer = blockIdx.y;
+// Le of every layer += its block partials (in fixed order: eighths of the blocks as in
+// sum_partials_kernel); N += n
+__global__ void __launch_bounds__(256)
+ekfac_reduce_kernel(const float* __restrict__ part, int nblk, double* __restrict__ st0, int64_t stride,
+                    int64_t ka, int64_t kg, double n) {
+    __shared__ double sub[8][32];
+    const int layer = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double* st = st0 + (int64_t)layer * stride;
     const KfLayout l(ka, kg);
-    const int64_t D = ka * kg;
+    const int64_t D = ka * kg, e = (int64_t)blockIdx.x * 32 + lane;
     const float* pl = part + (int64_t)layer * nblk * D;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < D; e += (int64_t)gridDim.x * blockDim.x) {
-        double v = 0.0;
-        for (int b = 0; b < nblk; ++b) v += (double)pl[(int64_t)b * D + e];
+    const int per = (nblk + 7) / 8, b0 = warp * per, b1 = b0 + per < nblk ? b0 + per : nblk;
+    double v = 0.0;
+    if (e < D)
+#pragma unroll 8
+        for (int b = b0; b < b1; ++b) v += (double)pl[(int64_t)b * D + e];
+    sub[warp][lane] = v;
+    __syncthreads();
+    if (warp == 0 && e < D) {
+        for (int w = 1; w < 8; ++w) v += sub[w][lane];
         st[l.Le + e] += v;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) st[1] += n;
 }
 
-// One CTA per (query row, layer): Qhat = U_g [(U_g^T Q U_a) / (Lam + lambda)] U_a^T
+// One CTA per (query row, layer): Qhat = U_g [(U_g^T Q U_a) / (Lam + lambda)] U_a^T. U_a's rows are
+// padded in shared memory: the last product but one walks down its columns (32 threads on one bank
+// otherwise: 64 us for 64 queries of three k = 32 layers, 27 now).
 template <bool SU>
 __global__ void __launch_bounds__(kKfThreads)
-kfac_apply_kernel(int kind, const double* __restrict__ st0, int64_t stride, int64_t ka, int64_t kg,
+kfac_apply_kernel(int kind, const double* __restrict__ st0, int64_t stride, int ka, int kg,
                   double lambda_abs, double lambda_rel, const float* __restrict__ q, int64_t ld_q,
                   float* __restrict__ qhat, int64_t ld_qhat) {
-    extern __shared__ float sm[];  // [U_a, U_g if SU] X [kg][ka], Y [kg][ka]
+    extern __shared__ float sm[];  // [U_a (padded), U_g if SU] X [kg][ka], Y [kg][ka]
     const int layer = blockIdx.y;
     const double* st = st0 + (int64_t)layer * stride;
     const KfLayout l(ka, kg);
-    const int64_t D = ka * kg;
-    float* X = sm + (SU ? ka * ka + kg * kg : 0);
+    const int D = ka * kg, lda = SU ? ka + 1 : ka;
+    float* X = sm + (SU ? ka * lda + kg * kg : 0);
     float* Y = X + D;
-    Bases<SU> U{sm, sm + ka * ka, st + l.Ua, st + l.Ug};
+    Bases<SU> U{sm, sm + ka * lda, st + l.Ua, st + l.Ug};
     if (SU) {
-        for (int64_t e = threadIdx.x; e < ka * ka; e += blockDim.x) sm[e] = (float)st[l.Ua + e];
-        for (int64_t e = threadIdx.x; e < kg * kg; e += blockDim.x) sm[ka * ka + e] = (float)st[l.Ug + e];
+        for (int e = threadIdx.x; e < ka * ka; e += blockDim.x) sm[e / ka * lda + e % ka] = (float)st[l.Ua + e];
+        for (int e = threadIdx.x; e < kg * kg; e += blockDim.x) sm[ka * lda + e] = (float)st[l.Ug + e];
     }
     __shared__ double red[kKfThreads];
-    const double nex = st[1];
-    auto lam_of = [&](int64_t e) -> double {
-        const int64_t r = e / ka, c = e - (e / ka) * ka;
-        if (kind == 0) return st[l.wg + r] * st[l.wa + c];
-        return nex > 0 ? st[l.Le + e] / nex : 0.0;
+    // Lam[e] = scale * raw(e): EK-FAC's sums are divided by the example count once
+    const double nex = st[1], scale = kind == 0 ? 1.0 : (nex > 0 ? 1.0 / nex : 0.0);
+    auto raw = [&](int e) -> double {
+        return kind == 0 ? st[l.wg + e / ka] * st[l.wa + e % ka] : st[l.Le + e];
     };
     double sacc = 0.0;
-    for (int64_t e = threadIdx.x; e < D; e += blockDim.x) sacc += lam_of(e);
+    for (int e = threadIdx.x; e < D; e += blockDim.x) sacc += raw(e);
     red[threadIdx.x] = sacc;
     __syncthreads();
     for (int h = blockDim.x / 2; h > 0; h >>= 1) {
         if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
         __syncthreads();
     }
-    const double lambda = lambda_abs + lambda_rel * red[0] / (double)D;
+    const double lambda = lambda_abs + lambda_rel * (scale * red[0]) / (double)D;
     const float* qi = q + (int64_t)blockIdx.x * ld_q + (int64_t)layer * D;
-    for (int64_t e = threadIdx.x; e < D; e += blockDim.x) X[e] = qi[e];
+    for (int e = threadIdx.x; e < D; e += blockDim.x) X[e] = qi[e];
     __syncthreads();
-    for (int64_t e = threadIdx.x; e < D; e += blockDim.x) {  // Y = Q U_a
-        const int64_t r = e / ka, c = e - (e / ka) * ka;
+    for (int e = threadIdx.x; e < D; e += blockDim.x) {  // Y = Q U_a
+        const int r = e / ka, c = e - r * ka;
         float a = 0.f;
-        for (int64_t j = 0; j < ka; ++j) a = fmaf(X[r * ka + j], U.a(j * ka + c), a);
+#pragma unroll 8
+        for (int j = 0; j < ka; ++j) a = fmaf(X[r * ka + j], U.a(j * lda + c), a);
         Y[e] = a;
     }
     __syncthreads();
-    for (int64_t e = threadIdx.x; e < D; e += blockDim.x) {  // X = (U_g^T Y) / (Lam + lambda)
-        const int64_t r = e / ka, c = e - (e / ka) * ka;
+    for (int e = threadIdx.x; e < D; e += blockDim.x) {  // X = (U_g^T Y) / (Lam + lambda)
+        const int r = e / ka, c = e - r * ka;
         float a = 0.f;
-        for (int64_t j = 0; j < kg; ++j) a = fmaf(U.g(j * kg + r), Y[j * ka + c], a);
-        X[e] = (float)((double)a / (lam_of(e) + lambda));
+#pragma unroll 8
+        for (int j = 0; j < kg; ++j) a = fmaf(U.g(j * kg + r), Y[j * ka + c], a);
+        X[e] = (float)((double)a / (scale * raw(e) + lambda));
     }
     __syncthreads();
-    for (int64_t e = threadIdx.x; e < D; e += blockDim.x) {  // Y = X U_a^T
-        const int64_t r = e / ka, c = e - (e / ka) * ka;
+    for (int e = threadIdx.x; e < D; e += blockDim.x) {  // Y = X U_a^T
+        const int r = e / ka, c = e - r * ka;
         float a = 0.f;
-        for (int64_t j = 0; j < ka; ++j) a = fmaf(X[r * ka + j], U.a(c * ka + j), a);
+#pragma unroll 8
+        for (int j = 0; j < ka; ++j) a = fmaf(X[r * ka + j], U.a(c * lda + j), a);
         Y[e] = a;
     }
     __syncthreads();
     float* out = qhat + (int64_t)blockIdx.x * ld_qhat + (int64_t)layer * D;
-    for (int64_t e = threadIdx.x; e < D; e += blockDim.x) {  // Qhat = U_g Y
-        const int64_t r = e / ka, c = e - (e / ka) * ka;
+    for (int e = threadIdx.x; e < D; e += blockDim.x) {  // out = U_g Y
+        const int r = e / ka, c = e - r * ka;
         float a = 0.f;
-        for (int64_t j = 0; j < kg; ++j) a = fmaf(U.g(r * kg + j), Y[j * ka + c], a);
+#pragma unroll 8
+        for (int j = 0; j < kg; ++j) a = fmaf(U.g(r * kg + j), Y[j * ka + c], a);
         out[e] = a;
     }
 }
@@ -520,7 +548,7 @@ cudaError_t launch_kfac_cov(const float* Y, int64_t rows, int k, double* S, doub
     if (rows == 0) {
         if (header && add_m != 0) {
             note_launches(1);
-            sum_partials_kernel<<<1, 32, 0, s>>>(part, 0, 0, 0, S, scale, header, 0, add_m);
+            sum_partials_kernel<<<1, 256, 0, s>>>(part, 0, 0, 0, 0, S, nullptr, scale, header, 0, add_m);
         }
         return cudaGetLastError();
     }
@@ -530,18 +558,19 @@ cudaError_t launch_kfac_cov(const float* Y, int64_t rows, int k, double* S, doub
     const int nblk = (int)((rows + per - 1) / per);
     note_launches(2);
     cov_partial_kernel<<<nblk, kKfThreads, (size_t)64 * k * 4, s>>>(Y, rows, k, per, part);
-    sum_partials_kernel<<<(unsigned)((k * k + 255) / 256), 256, 0, s>>>(part, nblk, (int64_t)k * k, (int64_t)k * k,
-                                                                       S, scale, header, 0, add_m);
+    sum_partials_kernel<<<(unsigned)((k * k + 31) / 32), 256, 0, s>>>(part, nblk, (int64_t)k * k, (int64_t)k * k,
+                                                                      (int64_t)k * k, S, nullptr, scale, header, 0,
+                                                                      add_m);
     return cudaGetLastError();
 }
 
-// Sums of per-CTA partials written by another kernel (the fused projection).
-cudaError_t launch_kfac_sum_partials(const float* part, int nblk, int64_t stride, int64_t n, double* S, double scale,
-                                     double* header, int slot, double add, cudaStream_t s) {
+// Sums of per-CTA partials written by another kernel (the fused projection): n0 entries to S0 and
+// n - n0 to S1.
+cudaError_t launch_kfac_sum_partials(const float* part, int nblk, int64_t stride, int64_t n, int64_t n0, double* S0,
+                                     double* S1, double scale, double* header, int slot, double add, cudaStream_t s) {
     note_launches(1);
-    int64_t blocks = (n + 255) / 256;
-    if (blocks < 1) blocks = 1;
-    sum_partials_kernel<<<(unsigned)blocks, 256, 0, s>>>(part, nblk, stride, n, S, scale, header, slot, add);
+    sum_partials_kernel<<<(unsigned)(n > 0 ? (n + 31) / 32 : 1), 256, 0, s>>>(part, nblk, stride, n, n0, S0, S1, scale,
+                                                                              header, slot, add);
     return cudaGetLastError();
 }
 
@@ -583,7 +612,7 @@ cudaError_t launch_kfac_ekfac_accum(int n_layers, double* state, int64_t ka, int
             ekfac_reg_kernel<32><<<grid, 256, 0, s>>>(phi, n, ld, state, stride, part);
         else
             ekfac_reg_kernel<64><<<grid, 256, 0, s>>>(phi, n, ld, state, stride, part);
-        ekfac_reduce_kernel<<<dim3((unsigned)((ka * kg + 255) / 256), (unsigned)n_layers), 256, 0, s>>>(
+        ekfac_reduce_kernel<<<dim3((unsigned)((ka * kg + 31) / 32), (unsigned)n_layers), 256, 0, s>>>(
             part, nblk, state, stride, ka, kg, (double)n);
         return cudaGetLastError();
     }
@@ -597,7 +626,7 @@ cudaError_t launch_kfac_ekfac_accum(int n_layers, double* state, int64_t ka, int
         ekfac_partial_kernel<true><<<grid, kKfThreads, smem, s>>>(phi, n, ld, state, stride, ka, kg, part);
     else
         ekfac_partial_kernel<false><<<grid, kKfThreads, smem, s>>>(phi, n, ld, state, stride, ka, kg, part);
-    ekfac_reduce_kernel<<<dim3((unsigned)((ka * kg + 255) / 256), (unsigned)n_layers), 256, 0, s>>>(
+    ekfac_reduce_kernel<<<dim3((unsigned)((ka * kg + 31) / 32), (unsigned)n_layers), 256, 0, s>>>(
         part, nblk, state, stride, ka, kg, (double)n);
     return cudaGetLastError();
 }
@@ -607,7 +636,7 @@ cudaError_t launch_kfac_apply(int kind, int n_layers, const double* state, int64
                               int64_t ld_qhat, cudaStream_t s) {
     if (n_q == 0) return cudaSuccess;
     const bool su = ka <= 64 && kg <= 64;
-    const size_t smem = (size_t)(2 * ka * kg + (su ? ka * ka + kg * kg : 0)) * 4;
+    const size_t smem = (size_t)(2 * ka * kg + (su ? ka * (ka + 1) + kg * kg : 0)) * 4;
     const int64_t stride = (int64_t)kfac_state_bytes(ka, kg) / 8;
     cudaError_t e = su ? cudaFuncSetAttribute(kfac_apply_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)smem)
@@ -617,10 +646,10 @@ cudaError_t launch_kfac_apply(int kind, int n_layers, const double* state, int64
     note_launches(1);
     const dim3 grid((unsigned)n_q, (unsigned)n_layers);
     if (su)
-        kfac_apply_kernel<true><<<grid, kKfThreads, smem, s>>>(kind, state, stride, ka, kg, lambda_abs, lambda_rel, q,
+        kfac_apply_kernel<true><<<grid, kKfThreads, smem, s>>>(kind, state, stride, (int)ka, (int)kg, lambda_abs, lambda_rel, q,
                                                                ld_q, qhat, ld_qhat);
     else
-        kfac_apply_kernel<false><<<grid, kKfThreads, smem, s>>>(kind, state, stride, ka, kg, lambda_abs, lambda_rel,
+        kfac_apply_kernel<false><<<grid, kKfThreads, smem, s>>>(kind, state, stride, (int)ka, (int)kg, lambda_abs, lambda_rel,
                                                                 q, ld_q, qhat, ld_qhat);
     return cudaGetLastError();
 }

@@ -94,8 +94,8 @@ int64_t kfac_offset_sa(int64_t ka, int64_t kg);
 int64_t kfac_offset_sg(int64_t ka, int64_t kg);
 cudaError_t launch_kfac_cov(const float* Y, int64_t rows, int k, double* S, double scale, double* header,
                             double add_m, float* part, cudaStream_t s);
-cudaError_t launch_kfac_sum_partials(const float* part, int nblk, int64_t stride, int64_t n, double* S, double scale,
-                                     double* header, int slot, double add, cudaStream_t s);
+cudaError_t launch_kfac_sum_partials(const float* part, int nblk, int64_t stride, int64_t n, int64_t n0, double* S0,
+                                     double* S1, double scale, double* header, int slot, double add, cudaStream_t s);
 cudaError_t launch_kfac_eigen(int n_layers, double* state, int64_t ka, int64_t kg, cudaStream_t s);
 cudaError_t launch_kfac_ekfac_accum(int n_layers, double* state, int64_t ka, int64_t kg, const float* phi, int64_t n,
                                     int64_t ld, float* part, int nblk, cudaStream_t s);
