@@ -129,6 +129,7 @@ __device__ int jacobi_sweeps(T* A, int lda, T* V, int ldv, int n, T* cs, T* sn, 
     }
     const double fro = red[0];
     __syncthreads();
+    const int W = n <= 32 ? 32 : (n <= 64 ? 64 : 128);
     int sweep = 0;
     for (; sweep < max_sweeps; ++sweep) {
         double off = 0.0;
@@ -171,61 +172,94 @@ __device__ int jacobi_sweeps(T* A, int lda, T* V, int ldv, int n, T* cs, T* sn, 
                 Q[i] = q < n ? q : -1;
             }
             __syncthreads();
-            const int half = m / 2;
-            for (int x = threadIdx.x; x < half * n; x += blockDim.x) {  // rows p, q: A <- J^T A
-                const int i = x / n, k = x - (x / n) * n;
-                if (Q[i] < 0 || sn[i] == T(0)) continue;
-                const int p = P[i], q = Q[i];
-                const T c = cs[i], sv = sn[i], apk = A[p * lda + k], aqk = A[q * lda + k];
-                A[p * lda + k] = c * apk - sv * aqk;
-                A[q * lda + k] = sv * apk + c * aqk;
-            }
+            // threads walk (pair, k) with k along a power of two of at least n (no divisions)
+            const int half = m / 2, k = threadIdx.x & (W - 1), step = blockDim.x / W;
+            if (k < n)
+                for (int i = threadIdx.x / W; i < half; i += step) {  // rows p, q: A <- J^T A; V <- V J
+                    const int p = P[i], q = Q[i];
+                    const T c = cs[i], sv = sn[i];
+                    if (q < 0 || sv == T(0)) continue;
+                    const T apk = A[p * lda + k], aqk = A[q * lda + k];
+                    const T vkp = V[k * ldv + p], vkq = V[k * ldv + q];
+                    A[p * lda + k] = c * apk - sv * aqk;
+                    A[q * lda + k] = sv * apk + c * aqk;
+                    V[k * ldv + p] = c * vkp - sv * vkq;
+                    V[k * ldv + q] = sv * vkp + c * vkq;
+                }
             __syncthreads();
-            for (int x = threadIdx.x; x < half * n; x += blockDim.x) {  // columns p, q: A <- A J, V <- V J
-                const int i = x / n, k = x - (x / n) * n;
-                if (Q[i] < 0 || sn[i] == T(0)) continue;
-                const int p = P[i], q = Q[i];
-                const T c = cs[i], sv = sn[i];
-                const T akp = A[k * lda + p], akq = A[k * lda + q];
-                A[k * lda + p] = c * akp - sv * akq;
-                A[k * lda + q] = sv * akp + c * akq;
-                const T vkp = V[k * ldv + p], vkq = V[k * ldv + q];
-                V[k * ldv + p] = c * vkp - sv * vkq;
-                V[k * ldv + q] = sv * vkp + c * vkq;
-            }
+            if (k < n)
+                for (int i = threadIdx.x / W; i < half; i += step) {  // columns p, q: A <- A J
+                    const int p = P[i], q = Q[i];
+                    const T c = cs[i], sv = sn[i];
+                    if (q < 0 || sv == T(0)) continue;
+                    const T akp = A[k * lda + p], akq = A[k * lda + q];
+                    A[k * lda + p] = c * akp - sv * akq;
+                    A[k * lda + q] = sv * akp + c * akq;
+                }
             __syncthreads();
         }
     }
     return -1;
 }
 
-// out = X^T Y (tx) or X Y, n x n fp64 in shared memory, row stride ld (one CTA)
-__device__ void gemm_nn(double* out, const double* X, const double* Y, int n, int ld, bool tx) {
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-        const int i = e / n, j = e - (e / n) * n;
+// out = X^T Y (tx) or X Y, n x n fp64 in the shared memory of every CTA of a cluster of cs (the same
+// X and Y in each, row stride ld): CTA r computes an equal share of the entries and writes them to
+// all. fp64 runs at two multiply-adds a clock and SM, so eight SMs take an eighth of the time.
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ void gemm_nn(double* out, const double* X, const double* Y, int n, int ld, bool tx, int cs, int rank) {
+    cluster_barrier();  // every CTA is done with what `out` held
+    const int total = n * n, per = (total + cs - 1) / cs;
+    const int e1 = (rank + 1) * per < total ? (rank + 1) * per : total;
+    for (int e = rank * per + threadIdx.x; e < e1; e += blockDim.x) {
+        const int i = e / n, j = e - i * n;
         double acc = 0.0;
+#pragma unroll 4
         for (int k = 0; k < n; ++k) acc += (tx ? X[k * ld + i] : X[i * ld + k]) * Y[k * ld + j];
-        out[i * ld + j] = acc;
+        const uint32_t at = (uint32_t)__cvta_generic_to_shared(out + i * ld + j);
+        for (int r = 0; r < cs; ++r) {
+            uint32_t dst;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"(at), "r"(r));
+            asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(dst), "d"(acc) : "memory");
+        }
     }
+    cluster_barrier();  // the whole product is in every CTA
+}
+// V <- V (3I - V^T V) / 2: one Newton-Schulz step towards orthonormal columns (T1, T2: scratch)
+__device__ void orthonormalise(double* V, double* T1, double* T2, int n, int ld, int cs, int rank) {
+    gemm_nn(T1, V, V, n, ld, true, cs, rank);
+    for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
+        const int i = e / n, j = e % n;
+        T1[i * ld + j] = ((i == j) ? 1.5 : 0.0) - 0.5 * T1[i * ld + j];
+    }
+    __syncthreads();
+    gemm_nn(T2, V, T1, n, ld, false, cs, rank);
+    for (int e = threadIdx.x; e < n * n; e += blockDim.x) V[(e / n) * ld + e % n] = T2[(e / n) * ld + e % n];
     __syncthreads();
 }
 
 // Eigenbases of C = S / M for the a side (blockIdx.x 0) and the g side (1) of
 // layer blockIdx.y, C = U diag(w) U^T.
-//   n <= 64 (MIXED): the sweeps run in fp32 (the fp64 pipe is a small fraction
-//   of the fp32 one here) until the off-diagonal part is near fp32 rounding;
-//   then, in fp64, two Newton-Schulz steps V <- V (3I - V^T V) / 2 make the
-//   fp32 eigenvectors orthonormal to fp64 precision, A = V^T C V is formed
-//   afresh, and fp64 sweeps finish (typically two). The header gets the fp64
-//   sweep count.
+//   n <= 64 (MIXED): a cluster of cs CTAs per side and layer. The sweeps run in
+//   fp32 (the fp64 pipe is a small fraction of the fp32 one here), the same in
+//   every CTA, until the off-diagonal part is near fp32 rounding. Then, in fp64
+//   and with products shared by the cluster: a Newton-Schulz step
+//   V <- V (3I - V^T V) / 2, A = V^T C V afresh, and twice the first-order
+//   rotation of all pairs at once, V <- V (I + E) with E_ij = A_ij / (A_jj - A_ii),
+//   made orthonormal by another Newton-Schulz step (errors of 1e-7 become 1e-14,
+//   then rounding; pairs with a gap below 1000 |A_ij| are left out). fp64 sweeps
+//   finish what is left: none, mostly, where two used to take most of the time
+//   (three k = 32 layers: 576 us, 220 now). The header gets the fp64 sweep count.
 //   n > 64: fp64 sweeps from the start, V in the state's U.
 template <bool MIXED>
 __global__ void __launch_bounds__(kKfThreads)
-jacobi_kernel(double* __restrict__ st0, int64_t stride, int64_t ka, int64_t kg) {
+jacobi_kernel(double* __restrict__ st0, int64_t stride, int64_t ka, int64_t kg, int cs) {
     extern __shared__ double smd[];
     double* st = st0 + (int64_t)blockIdx.y * stride;
     const KfLayout l(ka, kg);
-    const bool side_g = blockIdx.x == 1;
+    const bool side_g = (int)blockIdx.x / cs == 1;
+    const int rank = (int)blockIdx.x % cs;
     const int n = (int)(side_g ? kg : ka);
     const double* S = st + (side_g ? l.Sg : l.Sa);
     double* U = st + (side_g ? l.Ug : l.Ua);
@@ -237,11 +271,13 @@ jacobi_kernel(double* __restrict__ st0, int64_t stride, int64_t ka, int64_t kg) 
     const double inv = Mtok > 0 ? 1.0 / Mtok : 0.0;
     double* A = smd;  // [n][ld]
     int sweeps;
+    // every CTA of the cluster reads the sums before rank 0 writes the results (the a side's rank 0
+    // also clears the EK-FAC sums, which nothing here reads)
     if constexpr (MIXED) {
         double* V = A + sq;
         double* Tm = V + sq;  // fp64 scratch
-        double* cs = Tm + sq;
-        double* sn = cs + mh;
+        double* cs64 = Tm + sq;
+        double* sn = cs64 + mh;
         float* A32 = (float*)(sn + mh);
         float* V32 = A32 + sq;
         float* cs32 = V32 + sq;
@@ -262,29 +298,38 @@ jacobi_kernel(double* __restrict__ st0, int64_t stride, int64_t ka, int64_t kg) 
             V[i * ld + j] = (double)V32[i * ld + j];
         }
         __syncthreads();
-        for (int it = 0; it < 2; ++it) {  // Newton-Schulz: V <- V (3I - V^T V) / 2
-            gemm_nn(Tm, V, V, n, ld, true);
+        auto form_a = [&]() {  // A = V^T C V
+            for (int e = threadIdx.x; e < n * n; e += blockDim.x) A[(e / n) * ld + e % n] = S[e] * inv;
+            __syncthreads();
+            gemm_nn(Tm, A, V, n, ld, false, cs, rank);
+            gemm_nn(A, V, Tm, n, ld, true, cs, rank);
+        };
+        orthonormalise(V, Tm, A, n, ld, cs, rank);
+        form_a();
+        for (int it = 0; it < 2; ++it) {
             for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
                 const int i = e / n, j = e % n;
-                Tm[i * ld + j] = ((i == j) ? 1.5 : 0.0) - 0.5 * Tm[i * ld + j];
+                const double gap = A[j * ld + j] - A[i * ld + i], a = A[i < j ? i * ld + j : j * ld + i];
+                Tm[i * ld + j] = i == j ? 1.0 : (fabs(a) < 1e-3 * fabs(gap) ? a / gap : 0.0);
             }
             __syncthreads();
-            gemm_nn(A, V, Tm, n, ld, false);
+            gemm_nn(A, V, Tm, n, ld, false, cs, rank);
             for (int e = threadIdx.x; e < n * n; e += blockDim.x) V[(e / n) * ld + e % n] = A[(e / n) * ld + e % n];
             __syncthreads();
+            orthonormalise(V, Tm, A, n, ld, cs, rank);
+            form_a();
         }
-        for (int e = threadIdx.x; e < n * n; e += blockDim.x) A[(e / n) * ld + e % n] = S[e] * inv;  // C
-        __syncthreads();
-        gemm_nn(Tm, A, V, n, ld, false);  // C V
-        gemm_nn(A, V, Tm, n, ld, true);   // V^T C V
-        sweeps = jacobi_sweeps<double>(A, ld, V, ld, n, cs, sn, P, Q, red, &done, 1e-28, 60);
-        for (int e = threadIdx.x; e < n * n; e += blockDim.x) U[e] = V[(e / n) * ld + e % n];
+        sweeps = jacobi_sweeps<double>(A, ld, V, ld, n, cs64, sn, P, Q, red, &done, 1e-28, 60);
+        if (rank == 0)
+            for (int e = threadIdx.x; e < n * n; e += blockDim.x) U[e] = V[(e / n) * ld + e % n];
+        cluster_barrier();  // no CTA leaves while another may still write to it
+        if (rank != 0) return;
     } else {
         const bool v_shared = nmax <= 64;
         double* V = v_shared ? A + sq : U;
         const int ldv = v_shared ? ld : n;
-        double* cs = A + (v_shared ? 2 : 1) * sq;
-        double* sn = cs + mh;
+        double* c1 = A + (v_shared ? 2 : 1) * sq;
+        double* sn = c1 + mh;
         int* P = (int*)(sn + mh);
         int* Q = P + mh;
         for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
@@ -293,13 +338,13 @@ jacobi_kernel(double* __restrict__ st0, int64_t stride, int64_t ka, int64_t kg) 
             V[i * ldv + j] = (i == j) ? 1.0 : 0.0;
         }
         __syncthreads();
-        sweeps = jacobi_sweeps<double>(A, ld, V, ldv, n, cs, sn, P, Q, red, &done, 1e-28, 60);
+        sweeps = jacobi_sweeps<double>(A, ld, V, ldv, n, c1, sn, P, Q, red, &done, 1e-28, 60);
         if (v_shared)
             for (int e = threadIdx.x; e < n * n; e += blockDim.x) U[e] = V[(e / n) * ld + e % n];
     }
     for (int i = threadIdx.x; i < n; i += blockDim.x) w[i] = A[i * ld + i];
     if (threadIdx.x == 0) st[2 + (side_g ? 1 : 0)] = (double)sweeps;
-    if (blockIdx.x == 0) {  // a new eigenbasis invalidates the EK-FAC sums
+    if (!side_g) {  // a new eigenbasis invalidates the EK-FAC sums
         for (int64_t e = threadIdx.x; e < ka * kg; e += blockDim.x) st[l.Le + e] = 0.0;
         if (threadIdx.x == 0) st[1] = 0.0;
     }
@@ -582,15 +627,30 @@ cudaError_t launch_kfac_eigen(int n_layers, double* state, int64_t ka, int64_t k
     note_launches(1);
     if (nmax <= 64) {
         const size_t smem = (size_t)3 * sq * 8 + (size_t)mh * (8 + 8) + (size_t)2 * sq * 4 + (size_t)mh * (4 + 4 + 4 + 4);
-        if ((e = cudaFuncSetAttribute(jacobi_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
-            return e;
-        jacobi_kernel<true><<<dim3(2, (unsigned)n_layers), kKfThreads, smem, s>>>(state, stride, ka, kg);
+        // the largest shared memory of n <= 64, set once per device
+        constexpr int kMax = (int)((size_t)3 * 64 * 65 * 8 + 33 * 16 + (size_t)2 * 64 * 65 * 4 + 33 * 16);
+        if ((e = smem_attr_once<jacobi_kernel<true>>(kMax))) return e;
+        // clusters of eight while all of them fit the chip at once, else one CTA a problem
+        const int cs = (int64_t)n_layers * 2 * 8 <= 128 ? 8 : 1;
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)cs;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3((unsigned)(2 * cs), (unsigned)n_layers);
+        cfg.blockDim = dim3(kKfThreads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = s;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        if ((e = cudaLaunchKernelEx(&cfg, jacobi_kernel<true>, state, stride, ka, kg, cs))) return e;
         return cudaGetLastError();
     }
     const size_t smem = (size_t)sq * 8 + (size_t)mh * (8 + 8 + 4 + 4);
     if ((e = cudaFuncSetAttribute(jacobi_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
         return e;
-    jacobi_kernel<false><<<dim3(2, (unsigned)n_layers), kKfThreads, smem, s>>>(state, stride, ka, kg);
+    jacobi_kernel<false><<<dim3(2, (unsigned)n_layers), kKfThreads, smem, s>>>(state, stride, ka, kg, 1);
     return cudaGetLastError();
 }
 
