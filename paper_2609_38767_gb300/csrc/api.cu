@@ -315,20 +315,24 @@ tda_status tda_project(const tda_layer_desc* L, tda_dtype dtype, const void* A, 
     if (N == 0) return TDA_OK;
     if (L->T == 0) return cuda_check(cudaMemset2DAsync(phi, ld_phi * 4, 0, D * 4, N, s), "zero phi");
     if (route == TDA_ROUTE_FACTORED) {
-        if (dtype == TDA_BF16 && project_tc_plain_supported(*L, A, B)) {
-            unsigned int* err = device_error_word();
-            if (!err) return fail(TDA_ERR_CUDA, "cannot resolve the device error word");
-            return cuda_check(launch_project_tc(*L, A, B, N, phi, ld_phi, err, s, ws, ws_bytes), "project (tcgen05)");
-        }
         // fp32 factors: short jobs of narrow layers on the CUDA cores (one launch of a few us, against
         // ten on the tensor cores), the rest on the tensor cores
         if (dtype == TDA_F32 && project_small_supported(*L, A, B, N))
             return cuda_check(launch_project_small(*L, A, B, N, phi, ld_phi, s), "project (small)");
-        if (dtype == TDA_F32 && project_f32_tc_supported(*L, A, B)) {
+        const bool stream = dtype == TDA_BF16 && project_tc_plain_supported(*L, A, B);
+        const bool flex = project_flex_supported(*L, dtype, A, B);
+        if (stream || flex) {
             unsigned int* err = device_error_word();
             if (!err) return fail(TDA_ERR_CUDA, "cannot resolve the device error word");
-            const cudaError_t e = launch_project_f32_tc(*L, A, B, N, phi, ld_phi, err, s);
-            if (e != cudaErrorNotSupported) return cuda_check(e, "project (tcgen05, fp32 factors)");
+            if (flex) {
+                const bool bal = stream && ws && !((uintptr_t)ws & 255) && ws_bytes >= project_tc_ws_bytes(*L);
+                const cudaError_t e =
+                    launch_project_flex(*L, dtype, A, B, N, phi, ld_phi, err, s, !stream, bal);
+                if (e != cudaErrorNotSupported) return cuda_check(e, "project (tcgen05, flexible tiles)");
+            }
+            if (stream)
+                return cuda_check(launch_project_tc(*L, A, B, N, phi, ld_phi, err, s, ws, ws_bytes),
+                                  "project (tcgen05)");
         }
         return cuda_check(launch_project_simt(*L, dtype, A, B, N, phi, ld_phi, s), "project (simt)");
     }
@@ -346,7 +350,7 @@ tda_status tda_project(const tda_layer_desc* L, tda_dtype dtype, const void* A, 
 int32_t tda_project_engine(const tda_layer_desc* L, tda_dtype dtype, const void* A, const void* B) {
     g_msg[0] = 0;
     if (validate_layer(L, true) || validate_factors(L, dtype, A, B, 1, "tda_project_engine")) return -1;
-    return (dtype == TDA_BF16 ? project_tc_plain_supported(*L, A, B) : project_f32_tc_supported(*L, A, B)) ? 1 : 0;
+    return project_flex_supported(*L, dtype, A, B) || (dtype == TDA_BF16 && project_tc_plain_supported(*L, A, B)) ? 1 : 0;
 }
 
 tda_status tda_similarity_exact(const tda_layer_desc* L, tda_dtype dtype, const void* Aq,

@@ -1,16 +1,18 @@
-// k_project_f32.cu -- factored projection (Eq. 2) of fp32 factors on the
-// tcgen05 tensor cores, exact to fp32 rounding, for any k_in, k_out up to 64.
+// k_project_flex.cu -- factored projection (Eq. 2) on the tcgen05 tensor cores with
+// tiles and clusters cut to the batch, for any k_in, k_out up to 64: fp32 factors of
+// any batch, and bf16 factors where whole examples per SM would leave SMs idle.
 //
-// Every fp32 value is cut into three bf16 pieces, x = h + m + l (8 significant
-// bits each, by truncation: h + m + l = x exactly), and the signs S are +-1, so
-// the products h S, m S, l S are exact and only sums round. At = A S_in keeps
-// two fp32 accumulators, sum h S and sum (m + l) S: within one, the terms are
-// so coarse against its ulp that the tensor pipe's truncating additions lose
-// almost nothing (2048 features: 1.2e-6 off with an fp32 chain on the CUDA
-// cores, 2e-7 here). The epilogue adds the two with round-to-nearest and
-// contracts Phi += Bt^T At over the tokens in fp32, as the bf16 kernel does.
+// fp32 factors, exact to fp32 rounding: every value is cut into three bf16 pieces,
+// x = h + m + l (8 significant bits each, by truncation: h + m + l = x exactly), and
+// the signs S are +-1, so the products h S, m S, l S are exact and only sums round.
+// At = A S_in keeps two fp32 accumulators, sum h S and sum (m + l) S: within one,
+// the terms are so coarse against its ulp that the tensor pipe's truncating
+// additions lose almost nothing (2048 features: 1.2e-6 off with an fp32 chain on the
+// CUDA cores, 2e-7 here). The epilogue adds the two with round-to-nearest and
+// contracts Phi += Bt^T At over the tokens in fp32, as the other kernels do. bf16
+// factors are the MMA's A operand as TMA wrote them, one accumulator a side.
 //
-// Pieces go to TMEM, not to shared memory: the MMA takes its A operand from
+// The pieces go to TMEM, not to shared memory: the MMA takes its A operand from
 // TMEM (a lane per token, two bf16 features per column), the split warps read
 // each TMA-written fp32 row once (a thread per token row: the 128-byte swizzle
 // makes its 16-byte loads conflict-free) and write three pieces with
@@ -18,21 +20,24 @@
 // read, three pieces written and read), which at HBM speed (5.4 values a clock
 // and SM) would exceed its 128 bytes a clock.
 //
-// Measured: 64 examples of 512 tokens, 2048 -> 2048, k = 32 (537 MB): 7.6 ms on the
-// CUDA cores, 136 us here = 3.9 TB/s; 128 of 152 SMs have two tiles each.
+// Token tiles of R <= 128 rows and clusters of 1 to 8 CTAs that share an example's
+// tiles, chosen by a model of the chunk time (plan()): few examples fill the chip
+// with smaller tiles and larger clusters, and a token count just past a tile is
+// split evenly. T <= R packs floor(R/T) whole examples in a tile. The members'
+// partial blocks are reduce-scattered over distributed shared memory: every CTA
+// sums and writes 1/cs of Phi.
 //
-// Token tiles of R = 128, 64 or 32 rows and clusters of 1 to 8 CTAs that share
-// an example's tiles, chosen by a model of the chunk time (plan()): few examples
-// fill the chip with smaller tiles and larger clusters. T <= R packs floor(R/T)
-// whole examples in a tile. The members' partial blocks are reduce-scattered
-// over distributed shared memory: every CTA sums and writes 1/cs of Phi.
+// Signs: a byte of a sign word becomes eight bf16 signs by one table read (a second
+// pair of generator warps, each taking every other stage, measured 6 % slower).
 //
-// Warp roles (512 threads, one persistent CTA per SM): warp 0 TMA producer
-// (32-feature boxes of fp32, two per 64-feature chunk); warp 1 TMEM allocator
-// and MMA issuer; warps 2-3 sign generators (byte -> eight bf16 signs from a
-// table, as for k = 128 in the bf16 kernel); warps 4-7 epilogue; warps 8-15
-// split. Every wait is bounded (about 1 s); on expiry the kernel records
-// kErrTimeout, drains its copies, frees its TMEM and returns.
+// Measured, fp32: 64 examples of 512 tokens, 2048 -> 2048, k = 32 (537 MB): 7.6 ms
+// on the CUDA cores, 136 us here. bf16: see plan_bf16_flex().
+//
+// Warp roles (fp32 512, bf16 256 threads, one persistent CTA per SM): warp 0 TMA
+// producer; warp 1 TMEM allocator and MMA issuer; warps 2-3 sign generators;
+// warps 4-7 epilogue; fp32: warps 8-15 split. Every wait is bounded (about 1 s); on
+// expiry the kernel records kErrTimeout, drains its copies, frees its TMEM and
+// returns.
 #include <cuda.h>
 
 #include <mutex>
@@ -42,25 +47,27 @@
 namespace tda {
 namespace {
 
-constexpr int kThreads = 512;
 constexpr int kTileM = 128;   // MMA M
-constexpr int kChunkK = 64;   // features per stage (two 32-feature fp32 boxes)
-constexpr uint32_t kBoxBytes = kTileM * 128;  // room of one 32-feature box
+constexpr int kChunkK = 64;   // features per stage: one bf16 box or two 32-feature fp32 boxes
+constexpr uint32_t kBoxBytes = kTileM * 128;  // room of one box (a 128-byte row per token)
 constexpr size_t kSmemMax = 232448;
-constexpr int kMaxStages = 6;
+constexpr int kMaxStages = 8;
 constexpr int kSR = 64;       // token rows staged at a time
 constexpr int kPieceCols = kChunkK / 2;       // TMEM columns of one piece of a chunk
 constexpr int kACols = 3 * kPieceCols;
 constexpr int kABufs = 2;
 constexpr size_t kLutBytes = 256 * 16;
 
-template <int K>
+template <int K, bool F32>
 struct Cfg {
+    static constexpr int kThreads = F32 ? 512 : 256;
+    static constexpr uint32_t kTileBytes = (F32 ? 2 : 1) * kBoxBytes;
     static constexpr uint32_t kSignBytes = K * 128;
-    static constexpr uint32_t kStageBytes = 2 * kBoxBytes + kSignBytes;
-    static constexpr int kBufCols = 4 * K;                 // At: h, m+l; Bt: h, m+l
-    static constexpr int kBufs = K <= 32 ? 2 : 1;
-    static constexpr int kAOff = kBufs * kBufCols;         // first column of the A pieces
+    static constexpr uint32_t kStageBytes = kTileBytes + kSignBytes;
+    static constexpr int kSideCols = (F32 ? 2 : 1) * K;    // one side's accumulators (fp32: h, m+l)
+    static constexpr int kBufCols = 2 * kSideCols;         // At, Bt
+    static constexpr int kBufs = F32 && K > 32 ? 1 : 2;
+    static constexpr int kAOff = kBufs * kBufCols;         // first column of the A pieces (fp32)
     static constexpr int kStageLd = K + 4;
     static constexpr size_t kStaging = 2ull * kSR * kStageLd * 4;
     static constexpr size_t kTail = kLutBytes + 8 * (4 * kMaxStages + 2 * kABufs + 4 + 3) + 16;
@@ -69,7 +76,7 @@ struct Cfg {
     static constexpr size_t kSmem = 1024 + (size_t)kStages * kStageBytes + kStaging + kTail;
     static constexpr int RB = K / 16, CB = K / 8;          // 16 x 8 threads contract a K x K block
     static constexpr int kPer = RB * CB;
-    static_assert(kAOff + kABufs * kACols <= 512, "TMEM columns");
+    static_assert(kAOff + (F32 ? kABufs * kACols : 0) <= 512, "TMEM columns");
     static_assert(kStages >= 3 && kSmem <= kSmemMax && kStageBytes % 1024 == 0, "shared memory per CTA");
     static_assert((size_t)K * K * 4 <= kStaging, "the other members' slices fit the staging rows");
 };
@@ -141,20 +148,20 @@ struct Units {
     }
 };
 
-template <int K>
-__global__ void __launch_bounds__(kThreads, 1)
-project_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const Params p) {
-    using C = Cfg<K>;
+template <int K, bool F32>
+__global__ void __launch_bounds__(Cfg<K, F32>::kThreads, 1)
+project_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const Params p) {
+    using C = Cfg<K, F32>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     float* stX = (float*)(smem + (size_t)C::kStages * C::kStageBytes);  // [kSR][K+4] At rows
     float* stY = stX + kSR * C::kStageLd;                               // [kSR][K+4] Bt rows
     uint8_t* lut = smem + (size_t)C::kStages * C::kStageBytes + C::kStaging;
     uint64_t* bars = (uint64_t*)(lut + kLutBytes);
-    uint64_t* full = bars;                     // [stages] fp32 boxes landed (count 1 + tx)
-    uint64_t* rempty = bars + kMaxStages;      // [stages] boxes read by the split warps (8)
+    uint64_t* full = bars;                     // [stages] boxes landed (count 1 + tx)
+    uint64_t* rempty = bars + kMaxStages;      // [stages] fp32: boxes read by the split warps (8)
     uint64_t* sready = bars + 2 * kMaxStages;  // [stages] signs written (2)
-    uint64_t* sempty = bars + 3 * kMaxStages;  // [stages] MMAs done with the signs (1)
+    uint64_t* sempty = bars + 3 * kMaxStages;  // [stages] MMAs done with the signs, bf16: and the boxes (1)
     uint64_t* afull = bars + 4 * kMaxStages;   // [2] pieces in TMEM (8)
     uint64_t* aempty = afull + kABufs;         // [2] MMAs done with the pieces (1)
     uint64_t* tfull = aempty + kABufs;         // [2] accumulators ready (1)
@@ -212,20 +219,21 @@ project_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
         bool issued[C::kStages], ok = true;
         for (int i = 0; i < C::kStages; ++i) issued[i] = false;
         const uint32_t box = (uint32_t)p.R * 128u;
+        uint64_t* const free_bar = F32 ? rempty : sempty;
         for (; ok && it.x < p.n_slots; it.next(p, ncl, crank)) {
             const int row = p.pack > 1 ? (int)(it.x * p.pack * p.T) : it.tt * p.R;
             const int ex = p.pack > 1 ? 0 : (int)it.x;
             for (int kc = 0; kc < nk_tot; ++kc) {
-                if (!wait_bounded(smem_u32(&rempty[s]), ph ^ 1u, abort, p.err)) {
+                if (!wait_bounded(smem_u32(&free_bar[s]), ph ^ 1u, abort, p.err)) {
                     ok = false;
                     break;
                 }
                 const bool side_b = kc >= p.nk_in;
                 const int d0 = (side_b ? kc - p.nk_in : kc) * kChunkK;
                 const uint32_t dst = smem_u32(smem + (size_t)s * C::kStageBytes), bar = smem_u32(&full[s]);
-                mbar_arrive_tx(bar, 2 * box);
+                mbar_arrive_tx(bar, F32 ? 2 * box : box);
                 tma_load_3d(dst, side_b ? &tmB : &tmA, d0, row, ex, bar);
-                tma_load_3d(dst + kBoxBytes, side_b ? &tmB : &tmA, d0 + 32, row, ex, bar);
+                if constexpr (F32) tma_load_3d(dst + kBoxBytes, side_b ? &tmB : &tmA, d0 + 32, row, ex, bar);
                 issued[s] = true;
                 last_par[s] = ph;
                 if (++s == (uint32_t)C::kStages) s = 0, ph ^= 1u;
@@ -251,24 +259,30 @@ project_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
             for (int kc = 0; kc < nk_tot; ++kc, ++cnt) {
                 const uint32_t a = cnt & 1u;
                 if (!wait_bounded(smem_u32(&sready[s]), ph, abort, p.err) ||
-                    !wait_bounded(smem_u32(&afull[a]), (cnt >> 1) & 1u, abort, p.err)) {
+                    !(F32 ? wait_bounded(smem_u32(&afull[a]), (cnt >> 1) & 1u, abort, p.err)
+                          : wait_bounded(smem_u32(&full[s]), ph, abort, p.err))) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
                 const bool side_b = kc >= p.nk_in;
                 const bool start = kc == 0 || kc == p.nk_in;
-                const uint64_t bd = sw128_desc(smem_u32(smem + (size_t)s * C::kStageBytes + 2 * kBoxBytes));
-                const uint32_t dh = tmem + b * C::kBufCols + (side_b ? 2 * K : 0), dl = dh + K;
-                const uint32_t at = tmem + C::kAOff + a * kACols;
+                const uint32_t st = smem_u32(smem + (size_t)s * C::kStageBytes);
+                const uint64_t bd = sw128_desc(st + C::kTileBytes);
+                const uint32_t dh = tmem + b * C::kBufCols + (side_b ? C::kSideCols : 0), dl = dh + K;
 #pragma unroll
-                for (int k = 0; k < kChunkK / 16; ++k) {  // K = 16: 8 columns of pieces, 32 bytes of signs
+                for (int k = 0; k < kChunkK / 16; ++k) {  // K = 16: 32 bytes of bf16, 8 columns of pieces
                     const uint32_t acc = start && k == 0 ? 0u : 1u;
-                    mma_bf16_ta(dh, at + 8 * k, bd + 2 * k, idesc, acc);
-                    mma_bf16_ta(dl, at + kPieceCols + 8 * k, bd + 2 * k, idesc, acc);
-                    mma_bf16_ta(dl, at + 2 * kPieceCols + 8 * k, bd + 2 * k, idesc, 1u);
+                    if constexpr (F32) {
+                        const uint32_t at = tmem + C::kAOff + a * kACols;
+                        mma_bf16_ta(dh, at + 8 * k, bd + 2 * k, idesc, acc);
+                        mma_bf16_ta(dl, at + kPieceCols + 8 * k, bd + 2 * k, idesc, acc);
+                        mma_bf16_ta(dl, at + 2 * kPieceCols + 8 * k, bd + 2 * k, idesc, 1u);
+                    } else {
+                        mma_bf16(dh, sw128_desc(st) + 2 * k, bd + 2 * k, idesc, acc);
+                    }
                 }
-                mma_commit(smem_u32(&aempty[a]));
+                if constexpr (F32) mma_commit(smem_u32(&aempty[a]));
                 mma_commit(smem_u32(&sempty[s]));
                 if (++s == (uint32_t)C::kStages) s = 0, ph ^= 1u;
             }
@@ -285,7 +299,7 @@ project_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
     } else if (warp == 2 || warp == 3) {
         // ---------------- sign generators: the 64 threads share a tile's K rows, kParts threads per row
         constexpr int kParts = 64 / K, kChunks = 8 / kParts;
-        const int g = (warp - 2) * 32 + lane, col = g / kParts, part = g % kParts;
+        const int g = (warp & 1) * 32 + lane, col = g / kParts, part = g % kParts;
         const uint32_t lut_s = smem_u32(lut);
         uint32_t s = 0, ph = 0;
         bool ok = true;
@@ -305,7 +319,7 @@ project_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
                     ok = false;
                     break;
                 }
-                uint8_t* row = smem + (size_t)s * C::kStageBytes + 2 * kBoxBytes + (col >> 3) * 1024 + (col & 7) * 128;
+                uint8_t* row = smem + (size_t)s * C::kStageBytes + C::kTileBytes + (col >> 3) * 1024 + (col & 7) * 128;
 #pragma unroll
                 for (int c = 0; c < kChunks; ++c)
                     *reinterpret_cast<uint4*>(row + (((part * kChunks + c) ^ (col & 7)) << 4)) = q[c];
@@ -314,7 +328,7 @@ project_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
                 if (lane == 0) mbar_arrive(smem_u32(&sready[s]));
                 if (++s == (uint32_t)C::kStages) s = 0, ph ^= 1u;
             }
-    } else if (warp >= 8) {
+    } else if (F32 && warp >= 8) {
         // ---------------- split warps: a thread per token row, 32 features (one box) each
         const int q4 = warp & 3, half = (warp - 8) >> 2, row = q4 * 32 + lane;
         const bool active = q4 * 32 < p.R;
@@ -470,14 +484,18 @@ project_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
                     for (int side = 0; side < 2; ++side)
 #pragma unroll
                         for (int c0 = 0; c0 < K; c0 += 16) {
-                            float hi[16], lo[16];
-                            tmem_ld16(tb + side * 2 * K + c0, hi);
-                            tmem_ld16(tb + side * 2 * K + K + c0, lo);
+                            float v[16];
+                            tmem_ld16(tb + side * C::kSideCols + c0, v);
+                            if constexpr (F32) {
+                                float lo[16];
+                                tmem_ld16(tb + side * C::kSideCols + K + c0, lo);
+#pragma unroll
+                                for (int i = 0; i < 16; ++i) v[i] += lo[i];
+                            }
                             float* dst = (side ? stY : stX) + srow * C::kStageLd + c0;
 #pragma unroll
                             for (int i = 0; i < 16; i += 4)
-                                *reinterpret_cast<float4*>(dst + i) = make_float4(
-                                    hi[i] + lo[i], hi[i + 1] + lo[i + 1], hi[i + 2] + lo[i + 2], hi[i + 3] + lo[i + 3]);
+                                *reinterpret_cast<float4*>(dst + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
                         }
                 }
                 epi_sync();
@@ -540,17 +558,19 @@ EncodeTiledFn encode_fn() {
     return fn;
 }
 
-// 3-D map over fp32 X[N][T][d]: box 32 (d) x rows x 1 (example), 128-byte swizzle, zero fill.
-bool make_map(CUtensorMap* tm, const void* X, int64_t N, int64_t T, int64_t d, int rows) {
+// 3-D map over X[N][T][d]: box of one 128-byte row (32 fp32, 64 bf16) x rows x 1 (example),
+// 128-byte swizzle, zero fill.
+bool make_map(CUtensorMap* tm, const void* X, int64_t N, int64_t T, int64_t d, int rows, bool f32) {
     EncodeTiledFn enc = encode_fn();
     if (!enc) return false;
+    const int el = f32 ? 4 : 2;
     cuuint64_t dims[3] = {(cuuint64_t)d, (cuuint64_t)T, (cuuint64_t)N};
-    cuuint64_t strides[2] = {(cuuint64_t)(d * 4), (cuuint64_t)(T * d * 4)};
-    cuuint32_t box[3] = {32, (cuuint32_t)rows, 1};
+    cuuint64_t strides[2] = {(cuuint64_t)(d * el), (cuuint64_t)(T * d * el)};
+    cuuint32_t box[3] = {(cuuint32_t)(128 / el), (cuuint32_t)rows, 1};
     cuuint32_t estr[3] = {1, 1, 1};
-    return enc(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(X), dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    return enc(tm, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(X),
+               dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 int device_sms() {
@@ -565,7 +585,7 @@ int device_sms() {
     return n;
 }
 
-template <int K>
+template <int K, bool F32>
 void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int cs, cudaStream_t s) {
     cfg = {};
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -573,15 +593,15 @@ void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int cs, 
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3((unsigned)(cs * (device_sms() / cs)));
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = Cfg<K>::kSmem;
+    cfg.blockDim = dim3(Cfg<K, F32>::kThreads);
+    cfg.dynamicSmemBytes = Cfg<K, F32>::kSmem;
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
 }
 
 // Clusters of cs CTAs that fit the device at once (queried once per device and size).
-template <int K>
+template <int K, bool F32>
 int max_clusters(int cs) {
     static std::atomic<int> cache[64][4];
     int dev = 0;
@@ -593,70 +613,103 @@ int max_clusters(int cs) {
     }
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
-    cluster_config<K>(cfg, attr, cs, nullptr);
+    cluster_config<K, F32>(cfg, attr, cs, nullptr);
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, project_f32_kernel<K>, &cfg) != cudaSuccess || n < 1) n = device_sms() / cs;
+    if (cudaOccupancyMaxActiveClusters(&n, project_flex_kernel<K, F32>, &cfg) != cudaSuccess || n < 1) n = device_sms() / cs;
     if (dev >= 0) cache[dev][slot].store(n, std::memory_order_relaxed);
     return n;
+}
+
+// bf16 with k_in = k_out in {16, 32, 64}: whether this kernel's plan beats the streaming kernel of
+// k_project_tc.cu. That one takes 128-row tiles, whole examples per CTA, clusters of 2 or 4 below one
+// example per SM, or with the workspace (bal) equal runs of tiles; its chunk takes 960 clocks (as
+// above), at k = 64 1100, and 1350 without the workspace's smaller staging (the sign warps). 64
+// examples of 1024 tokens, 4096 -> 4096, k = 64 with the workspace: 302 us there, 224 us here; 16
+// of them: 97 us there, 120 us here. With two tiles a stage (four tiles per SM and more) and whole examples or equal runs for every SM it runs at HBM
+// speed and is kept.
+bool plan_bf16_flex(const tda_layer_desc& L, int64_t N, int sms, double cost, int K, bool bal) {
+    const int pack = L.T <= 64 ? (int)(kTileM / L.T) : 1;
+    const int64_t slots = (N + pack - 1) / pack, nt = pack > 1 ? 1 : (L.T + kTileM - 1) / kTileM;
+    const bool two = slots * nt >= 4 * (int64_t)sms;
+    bal = bal && pack == 1;
+    if (two && (pack > 1 || bal || N >= sms)) return false;
+    int cs = 1;
+    if (pack == 1 && N < sms) cs = 2 * N >= sms ? 2 : 4;
+    while (cs > nt) cs >>= 1;
+    const double chunks = (double)((L.d_in + kChunkK - 1) / kChunkK + (L.d_out + kChunkK - 1) / kChunkK);
+    const double t = K >= 64 ? (bal ? 1100.0 : 1350.0) : 960.0;
+    const int64_t room = sms / cs, rounds = (slots + room - 1) / room;
+    const double tile = chunks * t + kTileM * (K >= 64 ? 45.0 : 20.0);
+    if (bal) return cost < 0.95 * ((double)((slots * nt + sms - 1) / sms) * tile + 3000.0);
+    const double mine = (double)rounds * ((nt + cs - 1) / cs) * tile +
+                        rounds * (cs > 1 ? 3000.0 : 500.0);
+    return cost < 0.95 * mine;
 }
 
 struct Plan {
     int R, cs, pack, n_ttiles;
     int64_t slots, clusters;
+    double cost;  // clocks
 };
 
 // Tile rows and cluster size with the least time of the busiest CTA: its tiles times the time of a
-// 64-feature chunk, which the split and sign warps bound at about 750, 500 and 400 clocks for 128,
-// 64 and 32 rows, but at least what HBM takes (22 bytes a clock and SM); ties go to larger tiles
-// and smaller clusters. A tile's contraction and an example's reduction count as chunks.
-template <int K>
+// 64-feature chunk (one SM draws about 17 bytes a clock from HBM however few others do: 7.5 clocks a
+// bf16 row, 15 an fp32 row; at least 400 for the signs and the barriers), but at least what HBM
+// takes in all (22 bytes a clock and SM); ties go to fewer, larger tiles and smaller clusters. A
+// tile's contraction and an example's reduction count too. T past a multiple of the tile is cut into equal tiles (T = 130: two of 65 rows).
+template <int K, bool F32>
 Plan plan(const tda_layer_desc& L, int64_t N, int sms) {
     Plan best{};
-    double best_cost = 0;
     const double chunks = (double)((L.d_in + kChunkK - 1) / kChunkK + (L.d_out + kChunkK - 1) / kChunkK);
-    const double floor_clk = (double)N * L.T * (L.d_in + L.d_out) * 4.0 / (22.0 * sms);
-    for (int R = 128; R >= 32; R >>= 1) {
-        const double t = R == 128 ? 750 : (R == 64 ? 500 : 400);
-        const int pack = L.T <= R ? (int)(R / L.T) : 1;
+    const double floor_clk = (double)N * L.T * (L.d_in + L.d_out) * (F32 ? 4.0 : 2.0) / (22.0 * sms);
+    auto consider = [&](int R, int pack, int nt) {
+        const double t = R * (F32 ? 15.0 : 7.5) > 400.0 ? R * (F32 ? 15.0 : 7.5) : 400.0;
         const int64_t slots = (N + pack - 1) / pack;
-        const int nt = pack > 1 ? 1 : (int)((L.T + R - 1) / R);
         for (int cs = 1; cs <= 8 && cs <= nt; cs *= 2) {
-            const int64_t fit = max_clusters<K>(cs) < sms / cs ? max_clusters<K>(cs) : sms / cs;
+            const int64_t room = sms / cs, fit = max_clusters<K, F32>(cs) < room ? max_clusters<K, F32>(cs) : room;
             if (fit < 1) continue;
-            const int64_t clusters = slots < fit ? slots : fit;
-            const double tiles = (double)((slots + clusters - 1) / clusters) * ((nt + cs - 1) / cs);
-            const double flushes = (double)((slots + clusters - 1) / clusters);
-            double cost = tiles * (chunks * t + R * (K >= 64 ? 45.0 : 20.0)) + flushes * (cs > 1 ? 3000.0 : 500.0);
+            const int64_t clusters = slots < fit ? slots : fit, rounds = (slots + clusters - 1) / clusters;
+            const double tiles = (double)rounds * ((nt + cs - 1) / cs);
+            double cost = tiles * (chunks * t + R * (K >= 64 ? 45.0 : 20.0)) + rounds * (cs > 1 ? 3000.0 : 500.0);
             if (cost < floor_clk) cost = floor_clk;
-            if (best.R == 0 || cost < best_cost * 0.98) {
-                best = Plan{R, cs, pack, nt, slots, clusters};
-                best_cost = cost;
-            }
+            if (best.R == 0 || cost < best.cost * 0.98) best = Plan{R, cs, pack, nt, slots, clusters, cost};
         }
+    };
+    if (L.T <= kTileM)
+        for (int pack = (int)(kTileM / L.T); pack >= 1; pack >>= 1) {  // whole examples per tile
+            const int rows = (int)(pack * L.T);
+            consider((rows + 7) / 8 * 8, pack, 1);
+        }
+    const int64_t nt0 = (L.T + kTileM - 1) / kTileM;
+    for (int64_t nt = nt0; nt <= 4 * nt0 && nt < (1 << 24); nt = nt < 2 * nt0 ? nt + (nt0 + 3) / 4 : 2 * nt) {
+        const int R = (int)(((L.T + nt - 1) / nt + 7) / 8 * 8);
+        consider(R, 1, (int)((L.T + R - 1) / R));
     }
     return best;
 }
 
-template <int K>
+template <int K, bool F32>
 cudaError_t launch_k(const tda_layer_desc& L, const void* A, const void* B, int64_t N, float* phi, int64_t ld_phi,
-                     unsigned int* err, cudaStream_t s) {
+                     unsigned int* err, cudaStream_t s, bool force, bool bal) {
+    constexpr int el = F32 ? 4 : 2;
     const int budget = sm_budget();
     const int sms = budget > 0 && budget < device_sms() ? budget : device_sms();
-    cudaError_t e = smem_attr_once<project_f32_kernel<K>>((int)Cfg<K>::kSmem);  // before the occupancy queries
+    cudaError_t e = smem_attr_once<project_flex_kernel<K, F32>>((int)Cfg<K, F32>::kSmem);  // before occupancy queries
     if (e != cudaSuccess) return e;
-    const Plan pl = plan<K>(L, N, sms);
+    const Plan pl = plan<K, F32>(L, N, sms);
+    if (!force && !F32 && !plan_bf16_flex(L, N, sms, pl.cost, K, bal)) return cudaErrorNotSupported;
     // packed rows are one [1][N*T][d] view: 32-bit row coordinates, strides below 2^40 bytes
     if (pl.pack > 1) {
         const int64_t d_max = L.d_in > L.d_out ? L.d_in : L.d_out;
         int64_t most = ((int64_t)1 << 30) / L.T;
-        const int64_t by_stride = (((int64_t)1 << 40) - 1) / (L.T * d_max * 4);
+        const int64_t by_stride = (((int64_t)1 << 40) - 1) / (L.T * d_max * el);
         if (by_stride < most) most = by_stride;
-        most = most / 128 * 128;  // whole tiles of any packing
+        most = most / 128 * 128;
         if (most < 128) return cudaErrorNotSupported;
         if (N > most) {
             for (int64_t e0 = 0; e0 < N; e0 += most) {
-                e = launch_k<K>(L, (const float*)A + e0 * L.T * L.d_in, (const float*)B + e0 * L.T * L.d_out,
-                                            N - e0 < most ? N - e0 : most, phi + e0 * ld_phi, ld_phi, err, s);
+                e = launch_k<K, F32>(L, (const char*)A + e0 * L.T * L.d_in * el, (const char*)B + e0 * L.T * L.d_out * el,
+                                     N - e0 < most ? N - e0 : most, phi + e0 * ld_phi, ld_phi, err, s, true, bal);
                 if (e != cudaSuccess) return e;
             }
             return cudaSuccess;
@@ -664,8 +717,8 @@ cudaError_t launch_k(const tda_layer_desc& L, const void* A, const void* B, int6
     }
     CUtensorMap mA, mB;
     const bool flat = pl.pack > 1;
-    if (!make_map(&mA, A, flat ? 1 : N, flat ? N * L.T : L.T, L.d_in, pl.R) ||
-        !make_map(&mB, B, flat ? 1 : N, flat ? N * L.T : L.T, L.d_out, pl.R))
+    if (!make_map(&mA, A, flat ? 1 : N, flat ? N * L.T : L.T, L.d_in, pl.R, F32) ||
+        !make_map(&mB, B, flat ? 1 : N, flat ? N * L.T : L.T, L.d_out, pl.R, F32))
         return cudaErrorNotSupported;
     Params p;
     p.N = N;
@@ -687,17 +740,26 @@ cudaError_t launch_k(const tda_layer_desc& L, const void* A, const void* B, int6
     p.cs = pl.cs;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
-    cluster_config<K>(cfg, attr, pl.cs, s);
+    cluster_config<K, F32>(cfg, attr, pl.cs, s);
     cfg.gridDim = dim3((unsigned)(pl.clusters * pl.cs));
     note_launches(1);
-    e = cudaLaunchKernelEx(&cfg, project_f32_kernel<K>, mA, mB, p);
+    e = cudaLaunchKernelEx(&cfg, project_flex_kernel<K, F32>, mA, mB, p);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 
+template <bool F32>
+cudaError_t launch_any(const tda_layer_desc& L, const void* A, const void* B, int64_t N, float* phi, int64_t ld_phi,
+                       unsigned int* err, cudaStream_t s, bool force, bool bal) {
+    const int k = L.k_in > L.k_out ? L.k_in : L.k_out;
+    if (k <= 16) return launch_k<16, F32>(L, A, B, N, phi, ld_phi, err, s, force, bal);
+    if (k <= 32) return launch_k<32, F32>(L, A, B, N, phi, ld_phi, err, s, force, bal);
+    return launch_k<64, F32>(L, A, B, N, phi, ld_phi, err, s, force, bal);
+}
+
 }  // namespace
 
-bool project_f32_tc_supported(const tda_layer_desc& L, const void* A, const void* B) {
+bool project_flex_supported(const tda_layer_desc& L, tda_dtype dt, const void* A, const void* B) {
     static int sm103 = -1;
     if (sm103 < 0) {
         int dev = 0, major = 0, minor = 0;
@@ -708,7 +770,8 @@ bool project_f32_tc_supported(const tda_layer_desc& L, const void* A, const void
     }
     if (!sm103 || !encode_fn() || L.kind != TDA_PROJ_RADEMACHER) return false;
     if (L.k_in < 1 || L.k_out < 1 || L.k_in > 64 || L.k_out > 64) return false;
-    if (L.d_in % 4 || L.d_out % 4 || L.T < 1) return false;
+    const int q = dt == TDA_F32 ? 4 : 8;
+    if (L.d_in % q || L.d_out % q || L.T < 1) return false;
     if (((uintptr_t)A & 15) || ((uintptr_t)B & 15)) return false;
     // TMA: 32-bit coordinates, an example's stride below 2^40 bytes
     const int64_t d_max = L.d_in > L.d_out ? L.d_in : L.d_out;
@@ -716,13 +779,11 @@ bool project_f32_tc_supported(const tda_layer_desc& L, const void* A, const void
     return true;
 }
 
-cudaError_t launch_project_f32_tc(const tda_layer_desc& L, const void* A, const void* B, int64_t N, float* phi,
-                                  int64_t ld_phi, unsigned int* err, cudaStream_t s) {
+cudaError_t launch_project_flex(const tda_layer_desc& L, tda_dtype dt, const void* A, const void* B, int64_t N,
+                                float* phi, int64_t ld_phi, unsigned int* err, cudaStream_t s, bool force, bool bal) {
     if (N == 0) return cudaSuccess;
-    const int k = L.k_in > L.k_out ? L.k_in : L.k_out;
-    if (k <= 16) return launch_k<16>(L, A, B, N, phi, ld_phi, err, s);
-    if (k <= 32) return launch_k<32>(L, A, B, N, phi, ld_phi, err, s);
-    return launch_k<64>(L, A, B, N, phi, ld_phi, err, s);
+    return dt == TDA_F32 ? launch_any<true>(L, A, B, N, phi, ld_phi, err, s, force, bal)
+                         : launch_any<false>(L, A, B, N, phi, ld_phi, err, s, force, bal);
 }
 
 }  // namespace tda

@@ -1060,14 +1060,9 @@ cudaError_t launch_k(const tda_layer_desc& L, const void* A, const void* B, int6
     // well for k >= 64 (k <= 32 measured faster with whole tiles: 7.1-7.3 against 6.9 TB/s on
     // the Llama-1B block); fewer examples keep the larger staging rows, which hold the cluster's
     // partial blocks.
-    if constexpr (ODD) {
-        if constexpr (K <= 64)
-            if ((pack > 1 ? (N + pack - 1) / pack : N * ((L.T + kTileM - 1) / kTileM)) >= 4 * (int64_t)sm_count())
-                return launch_kg<K, 2, false, false, false, Cfg<K, 2>::kStageRows, false, true>(
-                    L, A, B, N, phi, ld_phi, err, s, pack, cov, grid_out, fout);
+    if constexpr (ODD)
         return launch_kg<K, 1, false, false, false, Cfg<K, 1>::kStageRows, false, true>(L, A, B, N, phi, ld_phi, err, s,
                                                                                        pack, cov, grid_out, fout);
-    }
     const bool bal = bal_ws && pack == 1;
     const bool narrow = K >= 64 && pack == 1 && N >= (int64_t)sm_count();
     if constexpr (K > 64) {
@@ -1130,10 +1125,11 @@ int padded_k(const tda_layer_desc& L) {
     return k <= 16 ? 16 : (k <= 32 ? 32 : (k <= 64 ? 64 : 128));
 }
 
-// The plain projection runs every k_in, k_out up to 128 on the tensor cores (the fused
-// K-FAC covariances and the factor output stay at k_in = k_out in {16, 32, 64}).
+// The plain projection runs k_in = k_out in {16, 32, 64} and every k_in, k_out with the larger
+// in 65 .. 128 (the fused K-FAC covariances and the factor output: {16, 32, 64} only).
 bool project_tc_plain_supported(const tda_layer_desc& L, const void* A, const void* B) {
-    if (L.k_in < 1 || L.k_out < 1 || L.k_in > 128 || L.k_out > 128) return false;
+    if (L.k_in < 1 || L.k_out < 1 || L.k_in > 128 || L.k_out > 128 || padded_k(L) < 128)
+        return project_tc_supported(L, A, B);
     tda_layer_desc L64 = L;
     L64.k_in = L64.k_out = 64;
     return project_tc_supported(L64, A, B);
@@ -1162,17 +1158,10 @@ cudaError_t launch_project_tc(const tda_layer_desc& L, const void* A, const void
     if (ws && ((uintptr_t)ws & 255)) ws = nullptr;
     const size_t sign_b = (project_tc_sign_table_bytes(L) + 255) / 256 * 256;
     void* bal_ws = (ws && ws_bytes >= project_tc_ws_bytes(L)) ? (char*)ws + sign_b : nullptr;
-    // Unequal or other k: the kernel of the next block edge, which computes K columns per side and
-    // writes k_out x k_in of them. Streaming the factors stays the bound (1000 -> 2056, T = 130,
-    // 32 x 48, 96 examples: 1516 us on the CUDA cores, 80 us here).
-    if (L.k_in != L.k_out || L.k_in != padded_k(L)) {
-        switch (padded_k(L)) {
-            case 16: return launch_k<16, false, false, true>(L, A, B, N, phi, ld_phi, err, s, nullptr, nullptr, nullptr);
-            case 32: return launch_k<32, false, false, true>(L, A, B, N, phi, ld_phi, err, s, nullptr, nullptr, nullptr);
-            case 64: return launch_k<64, false, false, true>(L, A, B, N, phi, ld_phi, err, s, nullptr, nullptr, nullptr);
-            default: return launch_k<128, false, false, true>(L, A, B, N, phi, ld_phi, err, s, nullptr, nullptr, nullptr);
-        }
-    }
+    // Unequal or other k above 64: the k = 128 kernel, which computes 128 columns per side and writes
+    // k_out x k_in of them (up to 64: k_project_flex.cu)
+    if (L.k_in != L.k_out || L.k_in != padded_k(L))
+        return launch_k<128, false, false, true>(L, A, B, N, phi, ld_phi, err, s, nullptr, nullptr, nullptr);
     switch (L.k_in) {
         case 16: return launch_k<16, false, false>(L, A, B, N, phi, ld_phi, err, s, nullptr, nullptr, nullptr, nullptr, bal_ws);
         case 32: return launch_k<32, false, false>(L, A, B, N, phi, ld_phi, err, s, nullptr, nullptr, nullptr, nullptr, bal_ws);

@@ -131,11 +131,13 @@ cudaError_t launch_project_tc(const tda_layer_desc& L, const void* A, const void
                               float* phi, int64_t ld_phi, unsigned int* err, cudaStream_t s,
                               void* ws = nullptr, size_t ws_bytes = 0);
 
-// Factored projection of fp32 factors on tcgen05 (k_project_f32.cu), k_in and k_out up to 64;
-// cudaErrorNotSupported (nothing launched) for sizes its tensor maps cannot address.
-bool project_f32_tc_supported(const tda_layer_desc& L, const void* A, const void* B);
-cudaError_t launch_project_f32_tc(const tda_layer_desc& L, const void* A, const void* B, int64_t N, float* phi,
-                                  int64_t ld_phi, unsigned int* err, cudaStream_t s);
+// Factored projection on tcgen05 with tiles cut to the batch (k_project_flex.cu), k_in and k_out up
+// to 64: fp32 factors, and bf16 factors. cudaErrorNotSupported (nothing launched) for sizes its
+// tensor maps cannot address and, without `force`, where the streaming kernel (with its balanced
+// ranges, if bal) is expected to be as fast.
+bool project_flex_supported(const tda_layer_desc& L, tda_dtype dt, const void* A, const void* B);
+cudaError_t launch_project_flex(const tda_layer_desc& L, tda_dtype dt, const void* A, const void* B, int64_t N,
+                                float* phi, int64_t ld_phi, unsigned int* err, cudaStream_t s, bool force, bool bal);
 
 // Route (b): materialise G = B^T A for nb examples into ws, then project it.
 size_t materialize_ws_bytes_per_example(const tda_layer_desc& L);
