@@ -363,11 +363,13 @@ __global__ void __launch_bounds__(256) update_kernel(St<TS> st, int64_t k0) {
 // as many CTAs as there is, and nothing done twice but the 32 x 32 diagonal block.
 //
 // Panel step at k0, grid (row chunk, layer), 128 threads: a CTA eliminates the diagonal block
-// together with its 8 panel rows, A_ic -= (A_ij / p_j) A_cj with p_j = A_jj (one reciprocal per
-// column: an fp32 guess and one cubic Newton step, evaluated by every warp for itself), and
-// scales column j by 1/sqrt(p_j) at the end, all columns at once. Chunk 0 leaves L_kk in the
-// block's slot of Dinv; f64_inverse_kernel replaces it by its inverse after the last step.
-// D = 256: 150 us a step in panel_kernel (one CTA: two warps of serial chains).
+// together with its 8 panel rows, A_ic -= (A_ij w_j) A_cj with w_j = 1 / A_jj, and scales column j
+// by 1/sqrt(A_jj) at the end, all columns at once. The serial chain is one pivot after the other,
+// so warp 0 does nothing else: it brings A_jj of the next column up to date and inverts it (an fp32
+// guess and one cubic step) while warps 1-3 update the rest with the current column; one barrier a
+// column. Chunk 0 leaves L_kk in the block's slot of Dinv; f64_inverse_kernel replaces it by its
+// inverse after the last step. D = 256: 150 us a step in panel_kernel (one CTA: two warps of
+// serial chains), 29 us with every warp inverting every pivot before its updates.
 constexpr int kF64Rows = 8;
 
 // 1/p and 1/sqrt(p) for p > 0 to fp64 rounding: p = m 4^h with m in [1, 4); the fp32 guess for m
@@ -416,28 +418,42 @@ __global__ void __launch_bounds__(128) panel_f64_kernel(St<double> st, int64_t k
         A[i][j] = v;
     }
     __syncthreads();
-    int bad = -1;
+    __shared__ double wj[2];  // 1 / A_jj of the current and the next column
+    int bad = -1;             // warp 0: first non-positive pivot
+    if (warp == 0) {
+        const double p = A[0][0];
+        if (!(p > 0.0)) bad = 0;
+        const double w = p > 0.0 ? rcp_f64(p) : NAN;
+        if (lane == 0) wj[0] = w;
+    }
+    __syncthreads();
     for (int j = 0; j < kNB - 1; ++j) {
-        const double p = A[j][j];
-        const bool ok = p > 0.0;
-        if (!ok && bad < 0) bad = j;
-        const double w = ok ? rcp_f64(p) : NAN;
-        // column c of the diagonal block's row `lane`, c = j + 1 + warp + 4 u <= lane
-        const double t = A[lane][j] * w;
-        for (int c = j + 1 + warp; c < kNB; c += 4)
-            if (c <= lane) A[lane][c] -= t * A[c][j];
-        // the panel rows: 8 rows x the columns after j, 16 columns at a time
-        const int pr = kNB + (tid & 7);
-        const double tp = A[pr][j] * w;
-        for (int c = j + 1 + (tid >> 3); c < kNB; c += 16) A[pr][c] -= tp * A[c][j];
+        const double w = wj[j & 1];
+        if (warp == 0) {
+            const double a = A[j + 1][j], p = A[j + 1][j + 1] - a * w * a;
+            if (!(p > 0.0) && bad < 0) bad = j + 1;
+            const double wn = p > 0.0 ? rcp_f64(p) : NAN;
+            if (lane == 0) {
+                A[j + 1][j + 1] = p;
+                wj[(j + 1) & 1] = wn;
+            }
+        } else {
+            const int u = warp - 1;
+            // the diagonal block's rows below j + 1: column c of row `lane`
+            if (lane > j + 1) {
+                const double t = A[lane][j] * w;
+                for (int c = j + 1 + u; c <= lane; c += 3) A[lane][c] -= t * A[c][j];
+            }
+            // the panel rows: 8 rows x the columns after j, 12 columns at a time
+            const int pr = kNB + (lane & 7);
+            const double tp = A[pr][j] * w;
+            for (int c = j + 1 + u * 4 + (lane >> 3); c < kNB; c += 12) A[pr][c] -= tp * A[c][j];
+        }
         __syncthreads();
     }
     if (warp == 0) {
         const double p = A[lane][lane];
-        const bool ok = p > 0.0;
-        if (lane == kNB - 1 && !ok && bad < 0) bad = kNB - 1;
-        bad = __shfl_sync(0xffffffffu, bad, kNB - 1);
-        inv[lane] = ok ? rsqrt_f64(p) : NAN;
+        inv[lane] = p > 0.0 ? rsqrt_f64(p) : NAN;
         if (blockIdx.x == 0 && lane == 0 && bad >= 0 && bad < nb) {
             double* h = st.header(l);
             if (h[kPcFailedPivot] == 0.0) h[kPcFailedPivot] = (double)(k0 + bad + 1);
@@ -518,6 +534,13 @@ __global__ void __launch_bounds__(128) f64_inverse_kernel(St<double> st) {
 // grid (query group, layer). G query rows per CTA; y[G][D] in shared memory.
 // Forward, block b:  r = q_b - L_{b,<b} y_<b ;  y_b = Dinv_b r
 // Backward, block b: r = y_b - L_{>b,b}^T x_>b ;  x_b = Dinv_b^T r
+// part[0..7][g][i] added in pairs: three dependent fp64 adds instead of eight
+template <typename TS, int G>
+__device__ __forceinline__ TS sum8(const TS (&part)[8][G][kNB], int g, int i) {
+    return ((part[0][g][i] + part[1][g][i]) + (part[2][g][i] + part[3][g][i])) +
+           ((part[4][g][i] + part[5][g][i]) + (part[6][g][i] + part[7][g][i]));
+}
+
 template <typename TS, int G>
 __global__ void __launch_bounds__(256)
 apply_kernel(St<TS> st, const float* __restrict__ q, int64_t n_q, int64_t ld_q, TS* __restrict__ out,
@@ -553,7 +576,7 @@ apply_kernel(St<TS> st, const float* __restrict__ q, int64_t n_q, int64_t ld_q, 
 #pragma unroll
             for (int g = 0; g < G; ++g) acc[g] = (TS)0;
             if (lane < nb)
-#pragma unroll 4
+#pragma unroll 8
                 for (int64_t m = warp; m < b0; m += 8) {
                     const TS lv = L[(b0 + lane) * D + m];
 #pragma unroll
@@ -564,8 +587,7 @@ apply_kernel(St<TS> st, const float* __restrict__ q, int64_t n_q, int64_t ld_q, 
             __syncthreads();
             for (int e = tid; e < G * kNB; e += blockDim.x) {
                 const int g = e / kNB, i = e % kNB;
-                TS t = (TS)0;
-                for (int w = 0; w < 8; ++w) t += part[w][g][i];
+                const TS t = sum8(part, g, i);
                 r[g][i] = (i < nb && g < gn) ? (TS)q[(g0 + g) * ld_q + (int64_t)l * D + b0 + i] - t : (TS)0;
             }
             __syncthreads();
@@ -580,8 +602,7 @@ apply_kernel(St<TS> st, const float* __restrict__ q, int64_t n_q, int64_t ld_q, 
             __syncthreads();
             for (int e = tid; e < G * kNB; e += blockDim.x) {
                 const int g = e / kNB, i = e % kNB;
-                TS t = (TS)0;
-                for (int w = 0; w < 8; ++w) t += part[w][g][i];
+                const TS t = sum8(part, g, i);
                 if (i < nb) y[g * D + b0 + i] = t;
             }
             __syncthreads();
@@ -637,7 +658,10 @@ apply_kernel(St<TS> st, const float* __restrict__ q, int64_t n_q, int64_t ld_q, 
         for (int e = tid; e < G * kNB; e += blockDim.x) {
             const int g = e / kNB, i = e % kNB;
             TS t = (TS)0;
-            for (int w = 0; w < 8; ++w) t += part[w][g][i];
+            if constexpr (sizeof(TS) == 8)
+                t = sum8(part, g, i);
+            else
+                for (int w = 0; w < 8; ++w) t += part[w][g][i];
             r[g][i] = (i < nb) ? y[g * D + b0 + i] - t : (TS)0;
         }
         __syncthreads();
@@ -655,7 +679,7 @@ apply_kernel(St<TS> st, const float* __restrict__ q, int64_t n_q, int64_t ld_q, 
             const int g = e / kNB, i = e % kNB;
             TS s = (TS)0;
             if constexpr (sizeof(TS) == 8)
-                for (int w = 0; w < 8; ++w) s += part[w][g][i];
+                s = sum8(part, g, i);
             else
                 for (int j = i; j < kNB; ++j) s += Dsm[j][i] * r[g][j];
             if (i < nb) y[g * D + b0 + i] = s;
