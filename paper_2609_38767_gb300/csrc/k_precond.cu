@@ -23,15 +23,13 @@
 // Every launch covers all layers of the call (grid z or y = layer).
 //
 // Blocked path (fp32 state, D a multiple of 128 and at least 2048): the same
-// right-looking Cholesky in 256-column panels of two 128-column halves. Per
-// half: the 128 x 128 diagonal block is factored in shared memory (column by
-// column, left-looking; Dinv of its four 32 x 32 blocks) and the rows below
-// it are solved against it (x L_BB^T = a); the second half's columns first take
-// the first half's update. The trailing lower triangle then takes the rank-256
-// update M -= P P^T on the tensor cores (3xTF32, launch_gemm_nt_tc). After the
-// last panel, L^T is copied into M's upper triangle. APPLY then solves the
-// query rows block by block: a 128-wide triangular solve per panel, and the
-// rest of every row updated by a tensor-core product with L's panel (forward)
+// right-looking Cholesky in 256-column panels. Per panel: the 256 x 256 diagonal
+// block is factored in shared memory by one CTA (diag_panel_kernel), the rows
+// below it are solved against it (solve_kernel, x L_BB^T = a), and the trailing
+// lower triangle takes the rank-256 update M -= P P^T on the tensor cores (3xTF32,
+// launch_gemm_nt_tc). After the last panel, L^T is copied into M's upper triangle.
+// APPLY then solves the query rows panel by panel: a 256-wide triangular solve, and
+// the rest of every row updated by a tensor-core product with L's panel (forward)
 // or with L^T's panel from the upper triangle (backward).
 #include <math.h>
 
@@ -1294,157 +1292,437 @@ cudaError_t apply_impl(int n_layers, int64_t D, const void* state, const float* 
 // ---------------------------------------------------------------- blocked path (fp32)
 constexpr int kBB = 128;                // panel width
 constexpr int64_t kBlockedMinD = 2048;  // smaller layers keep the one-launch cluster path
-constexpr int kTrsmWarps = 8;
-constexpr size_t kDiagSmem = sizeof(float) * (size_t)kBB * (kBB + 1);
-constexpr size_t kTrsmSmem =
-    sizeof(float) * ((size_t)kBB * (kBB + 1) + (size_t)(kBB / kNB) * kNB * (kNB + 1) + (size_t)kTrsmWarps * kBB);
 
-// Factor the 128 x 128 diagonal block at lo of every layer (grid = layer) in
-// shared memory by the left-looking (Cholesky-Crout) order, one column per
-// step: L_ij = (A_ij - sum_{m<j} L_im L_jm) / L_jj for every row i >= j at
-// once, two threads per row (each half of the dot product, four independent
-// partial sums). The serial chain is one short dot product, one rsqrt and two
-// barriers per column. L returns to M's lower triangle; the inverses of the
-// four 32 x 32 diagonal blocks go to Dinv (one warp each); a non-positive
-// pivot is recorded in the header and its column turns NaN.
-__global__ void __launch_bounds__(256) diag_block_kernel(St<float> st, int64_t lo) {
-    extern __shared__ __align__(16) float dsm[];
-    float(*A)[kBB + 1] = reinterpret_cast<float(*)[kBB + 1]>(dsm);
-    __shared__ float sinv[kBB];
-    const int l = blockIdx.x;
-    const int64_t D = st.D;
-    float* M = st.M(l);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int e = tid; e < kBB * kBB; e += 256) {
-        const int i = e / kBB, j = e % kBB;
-        A[i][j] = (j <= i) ? M[(lo + i) * D + lo + j] : 0.f;
-    }
-    __syncthreads();
-    const int i = tid >> 1, h = tid & 1;
-#pragma unroll 1
-    for (int j = 0; j < kBB; ++j) {
-        float s = 0.f;
-        if (i >= j) {
-            float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-            int m = h;
-            for (; m + 6 < j; m += 8) {
-                a0 = fmaf(A[i][m], A[j][m], a0);
-                a1 = fmaf(A[i][m + 2], A[j][m + 2], a1);
-                a2 = fmaf(A[i][m + 4], A[j][m + 4], a2);
-                a3 = fmaf(A[i][m + 6], A[j][m + 6], a3);
+// ---- diagonal panels. A panel is 256 columns (128 at the end of an odd D / 128): the rows and
+// columns [lo, lo + 256) of a layer, factored by one CTA with everything in shared memory, since
+// the pivots are a serial chain and the next panel waits for them. Per 128-column half:
+//   factor128   16 columns at a time: four warps, a thread per row with the 16 values in registers,
+//               one barrier per pivot (the pivot column's 16 entries pass through shared memory);
+//               then all 512 threads take the rank-16 update from the transposed columns;
+//   invert64    the inverse W of each 64 x 64 diagonal block (32 x 32 inverses by one warp each,
+//               then W10 = -W11 L10 W00), kept transposed in the block's strict upper triangle;
+// the second half's rows are solved against the first (64 columns at a time with W) and its
+// diagonal block takes L21 L21^T before its own factorisation. L goes to M's lower triangle, W^T
+// above the diagonal inside each 64 x 64 diagonal block (solve_kernel reads it), the 32 x 32
+// inverses to Dinv (APPLY's other path). D = 4096, seven layers: 85 us a 128-column block as a
+// column-by-column left-looking factorisation, plus 49 us and 33 us for the second half's solve
+// and update as launches of their own; 114 us the 256 columns here.
+constexpr int kDiagThreads = 512;
+constexpr int kLdS = kBB + 4;  // 16-byte rows, four banks apart
+struct DiagSmem {
+    float S11[kBB][kLdS];
+    float S21[kBB][kLdS];
+    float S22[kBB][kLdS];
+    float P[16][kLdS];      // a 16-column panel, transposed; invert64's scratch
+    float inv[2][kBB];      // 1 / L_jj of both halves
+    float col[2][16];       // the pivot column's entries in the panel's diagonal rows
+};
+static_assert(sizeof(DiagSmem) <= 232448 - 1024, "shared memory per CTA");
+static_assert(sizeof(float) * 2 * 32 * 33 <= sizeof(float) * 16 * kLdS, "invert64 scratch");
+
+__device__ __forceinline__ void bar_rows() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+
+__device__ void factor128(float (*S)[kLdS], DiagSmem& sm, float* inv, int64_t col0, double* h) {
+    const int tid = threadIdx.x;
+    for (int c0 = 0; c0 < kBB; c0 += 16) {
+        if (tid < kBB) {
+            const int r = tid;
+            float a[16];
+#pragma unroll
+            for (int c = 0; c < 16; c += 4) {
+                const float4 v = *reinterpret_cast<const float4*>(&S[r][c0 + c]);
+                a[c] = v.x, a[c + 1] = v.y, a[c + 2] = v.z, a[c + 3] = v.w;
             }
-            for (; m < j; m += 2) a0 = fmaf(A[i][m], A[j][m], a0);
-            s = (a0 + a1) + (a2 + a3);
-        }
-        s += __shfl_xor_sync(0xffffffffu, s, 1);
-        s = (i >= j) ? A[i][j] - s : 0.f;
-        if (i == j && h == 0) {
-            const bool ok = s > 0.f;
-            if (!ok) {
-                double* hd = st.header(l);
-                if (hd[kPcFailedPivot] == 0.0) hd[kPcFailedPivot] = (double)(lo + j + 1);
+            if (r >= c0 && r < c0 + 16) sm.col[0][r - c0] = a[0];
+            bar_rows();
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+                float cj[16];
+#pragma unroll
+                for (int c = 0; c < 16; c += 4) {
+                    const float4 v = *reinterpret_cast<const float4*>(&sm.col[j & 1][c]);
+                    cj[c] = v.x, cj[c + 1] = v.y, cj[c + 2] = v.z, cj[c + 3] = v.w;
+                }
+                const float p = cj[j], iv = p > 0.f ? rsqrtf(p) : NAN;
+                const float lr = a[j] * iv;  // L_rj (rows above the pivot: unused)
+                a[j] = lr;
+#pragma unroll
+                for (int c = j + 1; c < 16; ++c) a[c] -= lr * (cj[c] * iv);
+                if (r == c0 + j) {
+                    inv[c0 + j] = iv;
+                    if (!(p > 0.f) && h[kPcFailedPivot] == 0.0) h[kPcFailedPivot] = (double)(col0 + c0 + j + 1);
+                }
+                if (j < 15) {
+                    if (r >= c0 && r < c0 + 16) sm.col[(j + 1) & 1][r - c0] = a[j < 15 ? j + 1 : 15];
+                    bar_rows();
+                }
             }
-            // L_jj = s * rsqrt(s), 1 / L_jj = rsqrt(s)
-            const float inv = ok ? rsqrtf(s) : NAN;
-            sinv[j] = inv;
-            A[j][j] = s * inv;
+            if (r >= c0) {
+#pragma unroll
+                for (int c = 0; c < 16; c += 4)
+                    *reinterpret_cast<float4*>(&S[r][c0 + c]) = make_float4(a[c], a[c + 1], a[c + 2], a[c + 3]);
+            }
+#pragma unroll
+            for (int c = 0; c < 16; ++c) sm.P[c][r] = a[c];
         }
         __syncthreads();
-        if (i > j && h == 0) A[i][j] = s * sinv[j];
-        __syncthreads();
-    }
-    // inverses of the four diagonal blocks: warp w, lane c solves L X[:, c] = e_c
-    if (warp < kBB / kNB) {
-        const int b0 = warp * kNB, c = lane;
-        float x[kNB];
+        // rank-16 update of the 4 x 4 tiles on and below the diagonal, one tile a thread
+        const int s0 = c0 + 16, nt = (kBB - s0) / 4;
+        if (tid < nt * (nt + 1) / 2) {
+            int ti = (int)((sqrtf(8.f * (float)tid + 1.f) - 1.f) * 0.5f);
+            while (ti * (ti + 1) / 2 > tid) --ti;
+            while ((ti + 1) * (ti + 2) / 2 <= tid) ++ti;
+            const int i0 = s0 + 4 * ti, j0 = s0 + 4 * (tid - ti * (ti + 1) / 2);
+            float acc[4][4];
 #pragma unroll
-        for (int r = 0; r < kNB; ++r) x[r] = (r == c) ? 1.f : 0.f;
+            for (int u = 0; u < 4; ++u) {
+                const float4 v = *reinterpret_cast<const float4*>(&S[i0 + u][j0]);
+                acc[u][0] = v.x, acc[u][1] = v.y, acc[u][2] = v.z, acc[u][3] = v.w;
+            }
 #pragma unroll
-        for (int jj = 0; jj < kNB; ++jj) {
-            x[jj] = (jj < c) ? 0.f : x[jj] * sinv[b0 + jj];
+            for (int m = 0; m < 16; ++m) {
+                const float4 x = *reinterpret_cast<const float4*>(&sm.P[m][i0]);
+                const float4 y = *reinterpret_cast<const float4*>(&sm.P[m][j0]);
+                const float xa[4] = {x.x, x.y, x.z, x.w}, ya[4] = {y.x, y.y, y.z, y.w};
 #pragma unroll
-            for (int r = jj + 1; r < kNB; ++r) x[r] -= A[b0 + r][b0 + jj] * x[jj];
+                for (int u = 0; u < 4; ++u)
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) acc[u][v] -= xa[u] * ya[v];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                *reinterpret_cast<float4*>(&S[i0 + u][j0]) = make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]);
         }
-        float* Dg = st.Dinv(l) + ((lo + b0) / kNB) * (kNB * kNB);
-#pragma unroll
-        for (int r = 0; r < kNB; ++r) Dg[r * kNB + c] = x[r];
-    }
-    for (int e = tid; e < kBB * kBB; e += 256) {
-        const int r = e / kBB, c = e % kBB;
-        if (c <= r) M[(lo + r) * D + lo + c] = A[r][c];
+        __syncthreads();
     }
 }
 
-// Triangular solves of row vectors against the diagonal block B at lo of layer
-// l (grid y): FWD x <- L_BB^{-1} x, else x <- L_BB^{-T} x, for n_rows rows of
-// 128 values at column lo of X (row stride ldx, layer l's rows at byte offset
-// l * layer_bytes from base). One warp per row; the block's L and its four
-// diagonal inverses sit in shared memory. Used for the panel (rows of M below
-// the block, FWD) and for the query rows of APPLY (both directions).
-template <bool FWD>
-__global__ void __launch_bounds__(256) trsm_block_kernel(St<float> st, int64_t lo, char* base, size_t layer_bytes,
-                                                         int64_t ldx, int64_t n_rows) {
-    extern __shared__ __align__(16) float tsm[];
-    float(*Lb)[kBB + 1] = reinterpret_cast<float(*)[kBB + 1]>(tsm);
-    float(*Di)[kNB][kNB + 1] = reinterpret_cast<float(*)[kNB][kNB + 1]>(tsm + kBB * (kBB + 1));
-    float* Y = tsm + kBB * (kBB + 1) + (kBB / kNB) * kNB * (kNB + 1);
-    const int l = blockIdx.y;
-    const int64_t D = st.D;
-    const float* M = st.M(l);
-    const float* Dv = st.Dinv(l) + (lo / kNB) * (kNB * kNB);
+// W^T of both 64 x 64 diagonal blocks into their strict upper triangles (W's diagonal is inv).
+__device__ void invert64(float (*S)[kLdS], DiagSmem& sm, const float* inv) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int e = tid; e < kBB * kBB; e += 256) {
-        const int i = e / kBB, j = e % kBB;
-        Lb[i][j] = (j <= i) ? M[(lo + i) * D + lo + j] : 0.f;
-    }
-    for (int e = tid; e < (kBB / kNB) * kNB * kNB; e += 256) {
-        const int b = e / (kNB * kNB), i = (e / kNB) % kNB, j = e % kNB;
-        Di[b][i][j] = Dv[e];
-    }
-    __syncthreads();
-    float* y = Y + warp * kBB;
-    float* X = (float*)(base + (size_t)l * layer_bytes);
-    for (int64_t r = (int64_t)blockIdx.x * kTrsmWarps + warp; r < n_rows; r += (int64_t)gridDim.x * kTrsmWarps) {
-        float* x = X + r * ldx + lo;
+    if (warp < 4) {  // 32 x 32 block `warp`: lane c solves L X[:, c] = e_c, column order
+        const int b0 = warp * kNB, c = lane;
+        float x[kNB];
 #pragma unroll
-        for (int c = lane; c < kBB; c += 32) y[c] = x[c];
-        __syncwarp();
-        if (FWD) {
-#pragma unroll 1
-            for (int b = 0; b < kBB / kNB; ++b) {
-                const int c0 = b * kNB;
-                float acc = y[c0 + lane];
-                for (int m = 0; m < c0; ++m) acc -= Lb[c0 + lane][m] * y[m];
-                float out = 0.f;
+        for (int r = 0; r < kNB; ++r) x[r] = r == c ? 1.f : 0.f;
 #pragma unroll
-                for (int m = 0; m < kNB; ++m) {
-                    const float rm = __shfl_sync(0xffffffffu, acc, m);
-                    if (m <= lane) out += Di[b][lane][m] * rm;
-                }
-                __syncwarp();
-                y[c0 + lane] = out;
-                __syncwarp();
-            }
-        } else {
-#pragma unroll 1
-            for (int b = kBB / kNB - 1; b >= 0; --b) {
-                const int c0 = b * kNB;
-                float acc = y[c0 + lane];
-                for (int m = c0 + kNB; m < kBB; ++m) acc -= Lb[m][c0 + lane] * y[m];
-                float out = 0.f;
+        for (int j = 0; j < kNB; ++j) {
+            x[j] = j < c ? 0.f : x[j] * inv[b0 + j];
 #pragma unroll
-                for (int j = 0; j < kNB; ++j) {
-                    const float rj = __shfl_sync(0xffffffffu, acc, j);
-                    if (j >= lane) out += Di[b][j][lane] * rj;
-                }
-                __syncwarp();
-                y[c0 + lane] = out;
-                __syncwarp();
-            }
+            for (int r = j + 1; r < kNB; ++r) x[r] -= S[b0 + r][b0 + j] * x[j];
         }
 #pragma unroll
-        for (int c = lane; c < kBB; c += 32) x[c] = y[c];
-        __syncwarp();
+        for (int r = 1; r < kNB; ++r)
+            if (r > c) S[b0 + c][b0 + r] = x[r];
+    }
+    __syncthreads();
+    // W10 = -W11 (L10 W00) for the two 64-blocks: thread (block, row i, four columns)
+    float(*T)[kNB][kNB + 1] = reinterpret_cast<float(*)[kNB][kNB + 1]>(&sm.P[0][0]);
+    const int blk = tid >> 8, i = (tid >> 3) & 31, k0 = (tid & 7) * 4, lo = 64 * blk, hi = lo + kNB;
+    float t[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 8
+    for (int m = 0; m < kNB; ++m) {  // (L10 W00)[i][k] = sum_{m >= k} L10[i][m] W00[m][k]
+        const float l = S[hi + i][lo + m];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const int k = k0 + v;
+            const float w = m > k ? S[lo + k][lo + m] : (m == k ? inv[lo + k] : 0.f);
+            t[v] = fmaf(l, w, t[v]);
+        }
+    }
+#pragma unroll
+    for (int v = 0; v < 4; ++v) T[blk][i][k0 + v] = t[v];
+    __syncthreads();
+    float o[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 8
+    for (int m = 0; m < kNB; ++m) {  // W11[i][m], m <= i
+        const float w = m < i ? S[hi + m][hi + i] : (m == i ? inv[hi + i] : 0.f);
+#pragma unroll
+        for (int v = 0; v < 4; ++v) o[v] = fmaf(w, T[blk][m][k0 + v], o[v]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int v = 0; v < 4; ++v) S[lo + k0 + v][hi + i] = -o[v];
+    __syncthreads();
+}
+
+// Rows of S21 solved against S11: X L11^T = A, 64 columns at a time with W. 4 x 4 entries a thread.
+__device__ void solve_half(DiagSmem& sm) {
+    const int tid = threadIdx.x, r0 = (tid >> 4) * 4, i0 = (tid & 15) * 4;
+    for (int b = 0; b < 2; ++b) {
+        const int c0 = 64 * b;
+        float acc[4][4];
+        if (b == 1) {  // columns 64..127 less the solved columns' share
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v < 4; ++v) acc[u][v] = sm.S21[r0 + u][c0 + i0 + v];
+#pragma unroll 2
+            for (int k = 0; k < 64; k += 4) {
+                float4 x[4], y[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    x[u] = *reinterpret_cast<const float4*>(&sm.S21[r0 + u][k]);
+                    y[u] = *reinterpret_cast<const float4*>(&sm.S11[c0 + i0 + u][k]);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+#pragma unroll
+                    for (int v = 0; v < 4; ++v)
+                        acc[u][v] -= x[u].x * y[v].x + x[u].y * y[v].y + x[u].z * y[v].z + x[u].w * y[v].w;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                *reinterpret_cast<float4*>(&sm.S21[r0 + u][c0 + i0]) =
+                    make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]);
+            __syncthreads();
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int v = 0; v < 4; ++v) acc[u][v] = 0.f;
+        // out[r][i] = sum_{k <= i} x[r][k] W[i][k], W[i][k] = S11[c0 + k][c0 + i] for k < i
+        for (int k = 0; k < i0 + 4; ++k) {
+            float w[4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v)
+                w[v] = k < i0 + v ? sm.S11[c0 + k][c0 + i0 + v] : (k == i0 + v ? sm.inv[0][c0 + k] : 0.f);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float x = sm.S21[r0 + u][c0 + k];
+#pragma unroll
+                for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(x, w[v], acc[u][v]);
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            *reinterpret_cast<float4*>(&sm.S21[r0 + u][c0 + i0]) =
+                make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]);
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(kDiagThreads) diag_panel_kernel(St<float> st, int64_t lo) {
+    extern __shared__ __align__(16) unsigned char dsm[];
+    DiagSmem& sm = *reinterpret_cast<DiagSmem*>(dsm);
+    const int l = blockIdx.x;
+    const int64_t D = st.D;
+    float* M = st.M(l);
+    double* h = st.header(l);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool two = lo + kBB < D;
+    // a warp per row, 16 bytes a lane
+#pragma unroll 4
+    for (int r = warp; r < kBB; r += kDiagThreads / 32) {
+        const int c = 4 * lane;
+        float4 v = *reinterpret_cast<const float4*>(M + (lo + r) * D + lo + c);
+        float* d = &sm.S11[r][c];
+        d[0] = c <= r ? v.x : 0.f, d[1] = c + 1 <= r ? v.y : 0.f, d[2] = c + 2 <= r ? v.z : 0.f, d[3] = c + 3 <= r ? v.w : 0.f;
+        if (two) {
+            *reinterpret_cast<float4*>(&sm.S21[r][c]) =
+                *reinterpret_cast<const float4*>(M + (lo + kBB + r) * D + lo + c);
+            v = *reinterpret_cast<const float4*>(M + (lo + kBB + r) * D + lo + kBB + c);
+            d = &sm.S22[r][c];
+            d[0] = c <= r ? v.x : 0.f, d[1] = c + 1 <= r ? v.y : 0.f, d[2] = c + 2 <= r ? v.z : 0.f, d[3] = c + 3 <= r ? v.w : 0.f;
+        }
+    }
+    __syncthreads();
+    factor128(sm.S11, sm, sm.inv[0], lo, h);
+    invert64(sm.S11, sm, sm.inv[0]);
+    if (two) {
+        solve_half(sm);
+        // S22 -= L21 L21^T on and below the diagonal: 8 x 4 tiles
+        for (int u = tid; u < 16 * 17; u += kDiagThreads) {
+            // row pairs of 4-wide tiles: tile row ti has 2 (ti + 1) tiles
+            int ti = (int)((sqrtf(4.f * (float)u + 1.f) - 1.f) * 0.5f);
+            while (ti * (ti + 1) > u) --ti;
+            while ((ti + 1) * (ti + 2) <= u) ++ti;
+            const int i0 = 8 * ti, j0 = 4 * (u - ti * (ti + 1));
+            float acc[8][4];
+#pragma unroll
+            for (int a = 0; a < 8; ++a) {
+                const float4 v = *reinterpret_cast<const float4*>(&sm.S22[i0 + a][j0]);
+                acc[a][0] = v.x, acc[a][1] = v.y, acc[a][2] = v.z, acc[a][3] = v.w;
+            }
+            for (int k = 0; k < kBB; k += 4) {
+                float4 y[4];
+#pragma unroll
+                for (int v = 0; v < 4; ++v) y[v] = *reinterpret_cast<const float4*>(&sm.S21[j0 + v][k]);
+#pragma unroll
+                for (int a = 0; a < 8; ++a) {
+                    const float4 x = *reinterpret_cast<const float4*>(&sm.S21[i0 + a][k]);
+#pragma unroll
+                    for (int v = 0; v < 4; ++v)
+                        acc[a][v] -= x.x * y[v].x + x.y * y[v].y + x.z * y[v].z + x.w * y[v].w;
+                }
+            }
+#pragma unroll
+            for (int a = 0; a < 8; ++a)
+                *reinterpret_cast<float4*>(&sm.S22[i0 + a][j0]) = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
+        }
+        __syncthreads();
+        factor128(sm.S22, sm, sm.inv[1], lo + kBB, h);
+        invert64(sm.S22, sm, sm.inv[1]);
+    }
+    // L on and below the diagonal, W^T above it inside the 64 x 64 diagonal blocks (the rest of a
+    // half's upper triangle is the other 64-block's, written by upper_from_lower_kernel)
+    for (int r = warp; r < kBB; r += kDiagThreads / 32) {
+        const int c = 4 * lane;
+        for (int half = 0; half < (two ? 2 : 1); ++half) {
+            const float* src = half ? &sm.S22[r][c] : &sm.S11[r][c];
+            float* dst = M + (lo + half * kBB + r) * D + lo + half * kBB + c;
+            if (c / 64 <= r / 64) *reinterpret_cast<float4*>(dst) = *reinterpret_cast<const float4*>(src);
+        }
+        if (two)
+            *reinterpret_cast<float4*>(M + (lo + kBB + r) * D + lo + c) = *reinterpret_cast<const float4*>(&sm.S21[r][c]);
+    }
+    float* Dg = st.Dinv(l) + (lo / kNB) * (kNB * kNB);
+    for (int e = tid; e < (two ? 8 : 4) * kNB * kNB; e += kDiagThreads) {
+        const int b = e >> 10, r = (e >> 5) & 31, c = e & 31, half = b >> 2, o = (b & 3) * kNB;
+        const float(*S)[kLdS] = half ? sm.S22 : sm.S11;
+        Dg[e] = c < r ? S[o + c][o + r] : (c == r ? sm.inv[half][o + r] : 0.f);
+    }
+}
+
+// Row vectors solved against the panel's diagonal block B = [lo, lo + nb) of layer l (grid y),
+// nb = 256 or 128: FWD x <- L_BB^{-1} x, else x <- L_BB^{-T} x, for rows of nb values at column lo of
+// X (row stride ldx, layer l's rows at byte offset l * layer_bytes from base). Used for the rows of
+// M below a panel (FWD) and for the query rows of APPLY (both directions).
+// R rows a CTA, their nb values in shared memory; 64 columns at a time: the solved columns' share
+// is taken off with L, then the 64 x 64 inverse applied, both from one slab S[k][i] of
+// coefficients (k: solved or own column, i: column of the block). A thread has RT x 4 entries, so
+// a slab value read from shared memory serves RT products. R = 128 for many rows, 16 where few
+// rows would leave SMs idle. Seven layers, 256 columns: 3840 rows each 131 us as two 128-column
+// solves (a warp per row) and a product between them, 118 us here; 256 rows each 29 us.
+template <int R>
+struct SolveCfg {
+    static constexpr int RT = R / 16;                       // 16 row groups x 16 column groups
+    static constexpr int kLdX = 2 * kBB + 4;
+    static constexpr size_t kSmem = sizeof(float) * ((size_t)R * kLdX + (size_t)2 * kBB * 64 + 64);
+};
+template <int R, bool FWD>
+__global__ void __launch_bounds__(256) solve_kernel(St<float> st, int64_t lo, int nb, char* base, size_t layer_bytes,
+                                                    int64_t ldx, int64_t n_rows) {
+    using C = SolveCfg<R>;
+    constexpr int RT = C::RT;
+    extern __shared__ __align__(16) float ssm[];
+    float(*xs)[C::kLdX] = reinterpret_cast<float(*)[C::kLdX]>(ssm);
+    float(*S)[64] = reinterpret_cast<float(*)[64]>(ssm + R * C::kLdX);  // [k][i ^ 4 (k & 7)]
+    const int l = blockIdx.y;
+    const int64_t D = st.D;
+    const float* M = st.M(l) + lo * D + lo;
+    const int tid = threadIdx.x, rg = tid >> 4, i0 = (tid & 15) * 4;
+    const int64_t row0 = (int64_t)blockIdx.x * R;
+    float* X = (float*)(base + (size_t)l * layer_bytes) + lo;
+    // n 16-byte loads, eight of a thread's in flight together: ld(e) loads item e, st(e, value) stores it
+    auto copy = [&](int n, auto&& ld, auto&& st) {
+        for (int e0 = tid; e0 < n; e0 += 8 * 256) {
+            float4 v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (e0 + 256 * u < n) v[u] = ld(e0 + 256 * u);
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (e0 + 256 * u < n) st(e0 + 256 * u, v[u]);
+        }
+    };
+    const int q4 = nb / 4;
+    copy(R * q4,
+         [&](int e) {
+             const int r = e / q4, c = e % q4 * 4;
+             return row0 + r < n_rows ? *reinterpret_cast<const float4*>(X + (row0 + r) * ldx + c)
+                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+         },
+         [&](int e, const float4& v) { *reinterpret_cast<float4*>(&xs[e / q4][e % q4 * 4]) = v; });
+    const int nblk = nb / 64;
+    for (int s = 0; s < nblk; ++s) {
+        const int b = FWD ? s : nblk - 1 - s, c0 = 64 * b;   // this block's columns
+        const int k0 = FWD ? 0 : c0 + 64, nk = FWD ? c0 : nb - c0 - 64;  // the solved columns
+        __syncthreads();  // the previous block's slab is read
+        // slab rows 0 .. nk-1: L between the block's columns and the solved ones; rows nk .. nk+63: W
+        if (FWD)  // S[k][i] = L[c0 + i][k], a warp's lanes along i: every store hits 32 banks
+            copy(16 * nk, [&](int e) { return *reinterpret_cast<const float4*>(M + (int64_t)(c0 + e % 64) * D + e / 64 * 4); },
+                 [&](int e, const float4& v) {
+                     const int i = e % 64, k = e / 64 * 4;
+                     S[k][i ^ ((k & 7) << 2)] = v.x;
+                     S[k + 1][i ^ (((k + 1) & 7) << 2)] = v.y;
+                     S[k + 2][i ^ (((k + 2) & 7) << 2)] = v.z;
+                     S[k + 3][i ^ (((k + 3) & 7) << 2)] = v.w;
+                 });
+        else      // S[k][i] = L[k0 + k][c0 + i]
+            copy(16 * nk,
+                 [&](int e) { return *reinterpret_cast<const float4*>(M + (int64_t)(k0 + e / 16) * D + c0 + e % 16 * 4); },
+                 [&](int e, const float4& v) {
+                     const int k = e / 16;
+                     *reinterpret_cast<float4*>(&S[k][(e % 16 * 4) ^ ((k & 7) << 2)]) = v;
+                 });
+        // the block as stored: L left of the diagonal, W^T right of it. FWD: S[k][i] = W[i][k] =
+        // stored[k][i] for k < i; else S[k][i] = W[k][i] = stored[i][k] for k > i
+        copy(64 * 16, [&](int e) { return *reinterpret_cast<const float4*>(M + (int64_t)(c0 + e / 16) * D + c0 + e % 16 * 4); },
+             [&](int e, const float4& v4) {
+                 const int a = e / 16, c = e % 16 * 4;
+                 const float v[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+                 for (int t = 0; t < 4; ++t) {
+                     const int i = FWD ? c + t : a, k = FWD ? a : c + t, kr = nk + k;
+                     S[kr][i ^ ((kr & 7) << 2)] = (FWD ? k < i : k > i) ? v[t] : (k == i ? 1.f / v[t] : 0.f);
+                 }
+             });
+        __syncthreads();
+        float acc[RT][4];  // the solved columns' share less x, so that both products add
+#pragma unroll
+        for (int u = 0; u < RT; ++u) {
+            const float4 v = *reinterpret_cast<const float4*>(&xs[rg * RT + u][c0 + i0]);
+            acc[u][0] = -v.x, acc[u][1] = -v.y, acc[u][2] = -v.z, acc[u][3] = -v.w;
+        }
+        auto products = [&](int ks, int xc, int n) {  // acc += x[:, xc + k] S[ks + k][:]
+#pragma unroll 2
+            for (int k = 0; k < n; k += 4) {
+                float w[4][4];
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    const float4 v = *reinterpret_cast<const float4*>(&S[ks + k + t][i0 ^ (((ks + k + t) & 7) << 2)]);
+                    w[t][0] = v.x, w[t][1] = v.y, w[t][2] = v.z, w[t][3] = v.w;
+                }
+#pragma unroll
+                for (int u = 0; u < RT; ++u) {
+                    const float4 x = *reinterpret_cast<const float4*>(&xs[rg * RT + u][xc + k]);
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) {
+                        acc[u][v] = fmaf(x.x, w[0][v], acc[u][v]);
+                        acc[u][v] = fmaf(x.y, w[1][v], acc[u][v]);
+                        acc[u][v] = fmaf(x.z, w[2][v], acc[u][v]);
+                        acc[u][v] = fmaf(x.w, w[3][v], acc[u][v]);
+                    }
+                }
+            }
+        };
+        auto store = [&](float sign) {  // a row group's 16 threads are half a warp: they alone read its rows
+            __syncwarp();
+#pragma unroll
+            for (int u = 0; u < RT; ++u)
+                *reinterpret_cast<float4*>(&xs[rg * RT + u][c0 + i0]) =
+                    make_float4(sign * acc[u][0], sign * acc[u][1], sign * acc[u][2], sign * acc[u][3]);
+            __syncwarp();
+        };
+        if (nk > 0) {
+            products(0, k0, nk);
+            store(-1.f);
+        }
+#pragma unroll
+        for (int u = 0; u < RT; ++u)
+#pragma unroll
+            for (int v = 0; v < 4; ++v) acc[u][v] = 0.f;
+        products(nk, c0, 64);
+        store(1.f);
+    }
+    __syncthreads();
+    for (int e = tid; e < R * q4; e += 256) {
+        const int r = e / q4, c = e % q4 * 4;
+        if (row0 + r < n_rows)
+            *reinterpret_cast<float4*>(X + (row0 + r) * ldx + c) = *reinterpret_cast<const float4*>(&xs[r][c]);
     }
 }
 
@@ -1467,24 +1745,40 @@ __global__ void __launch_bounds__(256) scale_lower_kernel(St<float> st) {
     }
 }
 
-// M[i][j] = M[j][i] for every 32 x 32 block strictly above the diagonal blocks
-// (U = L^T, read by the backward solve's tensor-core products).
+// M[i][j] = M[j][i] for every 64 x 64 block strictly above the diagonal blocks (U = L^T, read by
+// the backward solve's tensor-core products; the diagonal blocks hold W^T there). Each thread has
+// four 16-byte loads in flight and the block index comes from an fp32 estimate corrected in
+// integers: with 32 x 32 blocks, scalar loads and an fp64 square root per block this took 417 us
+// for seven layers of D = 4096, 73056 us here.
 __global__ void __launch_bounds__(256) upper_from_lower_kernel(St<float> st, int n_layers) {
-    __shared__ float t[kNB][kNB + 1];
-    const int64_t D = st.D, nb = D / kNB, pairs = nb * (nb - 1) / 2;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    __shared__ float t[64][65];
+    const int64_t D = st.D, nb = D / 64, pairs = nb * (nb - 1) / 2;
+    const int r = threadIdx.x >> 4, c = (threadIdx.x & 15) * 4;
     for (int64_t w = blockIdx.x; w < pairs * n_layers; w += gridDim.x) {
         const int l = (int)(w / pairs);
         const int64_t p = w - (int64_t)l * pairs;
-        int64_t bj = (int64_t)((1.0 + sqrt(1.0 + 8.0 * (double)p)) * 0.5);  // p = bj(bj-1)/2 + bi, bi < bj
+        int64_t bj = (int64_t)((1.f + sqrtf(1.f + 8.f * (float)p)) * 0.5f);  // p = bj(bj-1)/2 + bi, bi < bj
         while (bj * (bj - 1) / 2 > p) --bj;
         while ((bj + 1) * bj / 2 <= p) ++bj;
         const int64_t bi = p - bj * (bj - 1) / 2;
         float* M = st.M(l);
-        for (int r = ty; r < kNB; r += 8) t[r][tx] = M[(bj * kNB + r) * D + bi * kNB + tx];
+        float4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            v[u] = *reinterpret_cast<const float4*>(M + (bj * 64 + r + 16 * u) * D + bi * 64 + c);
+        __syncthreads();  // the previous block is read
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            float* d = &t[r + 16 * u][c];
+            d[0] = v[u].x, d[1] = v[u].y, d[2] = v[u].z, d[3] = v[u].w;
+        }
         __syncthreads();
-        for (int r = ty; r < kNB; r += 8) M[(bi * kNB + r) * D + bj * kNB + tx] = t[tx][r];
-        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = r + 16 * u;
+            *reinterpret_cast<float4*>(M + (bi * 64 + i) * D + bj * 64 + c) =
+                make_float4(t[c][i], t[c + 1][i], t[c + 2][i], t[c + 3][i]);
+        }
     }
 }
 
@@ -1501,31 +1795,31 @@ bool blocked_pc(int64_t D, tda_dtype sdt) {
     return sdt == TDA_F32 && D % kBB == 0 && D >= kBlockedMinD && D < (1LL << 31) / kBB && gemm_tc_available();
 }
 
-cudaError_t blocked_attrs() {
-    static cudaError_t e = [] {
-        cudaError_t r = cudaFuncSetAttribute(diag_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)kDiagSmem);
-        if (r == cudaSuccess)
-            r = cudaFuncSetAttribute(trsm_block_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)kTrsmSmem);
-        if (r == cudaSuccess)
-            r = cudaFuncSetAttribute(trsm_block_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)kTrsmSmem);
-        return r;
-    }();
-    return e;
+template <int R, bool FWD>
+cudaError_t launch_solve_r(St<float> st, int n_layers, int64_t lo, int nb, char* base, size_t layer_bytes, int64_t ldx,
+                           int64_t n_rows, cudaStream_t s) {
+    cudaError_t e = smem_attr_once<solve_kernel<R, FWD>>((int)SolveCfg<R>::kSmem);
+    if (e != cudaSuccess) return e;
+    note_launches(1);
+    solve_kernel<R, FWD><<<dim3((unsigned)((n_rows + R - 1) / R), n_layers), 256, SolveCfg<R>::kSmem, s>>>(
+        st, lo, nb, base, layer_bytes, ldx, n_rows);
+    return cudaGetLastError();
 }
 
-unsigned trsm_grid(int64_t n_rows, int n_layers) {
-    int64_t g = (n_rows + kTrsmWarps - 1) / kTrsmWarps;
-    const int64_t cap = n_layers >= 304 ? 1 : 304 / n_layers;  // about two CTAs per SM over all layers
-    if (g > cap) g = cap;
-    return (unsigned)(g < 1 ? 1 : g);
+// 128 rows a CTA once those fill the chip, else 16 (a quarter of the products per slab value read)
+template <bool FWD>
+cudaError_t launch_solve(St<float> st, int n_layers, int64_t lo, int nb, char* base, size_t layer_bytes, int64_t ldx,
+                         int64_t n_rows, cudaStream_t s) {
+    return (n_rows + 127) / 128 * n_layers >= 114
+               ? launch_solve_r<128, FWD>(st, n_layers, lo, nb, base, layer_bytes, ldx, n_rows, s)
+               : ((n_rows + 31) / 32 * n_layers >= 114
+                      ? launch_solve_r<32, FWD>(st, n_layers, lo, nb, base, layer_bytes, ldx, n_rows, s)
+                      : launch_solve_r<16, FWD>(st, n_layers, lo, nb, base, layer_bytes, ldx, n_rows, s));
 }
 
 cudaError_t factor_blocked(int n_layers, int64_t D, void* state, int64_t n_total, double la, double lr,
                            cudaStream_t s) {
-    cudaError_t e = blocked_attrs();
+    cudaError_t e = smem_attr_once<diag_panel_kernel>((int)sizeof(DiagSmem));
     if (e != cudaSuccess) return e;
     unsigned int* err = device_error_word();
     if (!err) return cudaErrorUnknown;
@@ -1534,36 +1828,22 @@ cudaError_t factor_blocked(int n_layers, int64_t D, void* state, int64_t n_total
     prepare_kernel<float><<<n_layers, 256, 0, s>>>(st, n_total, la, lr);
     const unsigned rows_per = (unsigned)((D < 1024 ? D : 1024) * (n_layers < 8 ? 8 / n_layers : 1));
     scale_lower_kernel<<<dim3(rows_per < (unsigned)D ? rows_per : (unsigned)D, n_layers), 256, 0, s>>>(st);
-    // outer panels of 256 columns, each two 128-column sub-panels: the second sub-panel's
-    // columns take the first one's update alone (a 128-wide product), and the trailing
-    // matrix takes both at once (rank-256 update: twice the work per tile pass over M)
+    // panels of 256 columns: the diagonal block, the rows below it, then the trailing lower
+    // triangle of all layers in one launch: M -= P P^T, P = L[hi:D, lo:hi]
     float* M0 = (float*)((char*)state + 64);  // layer l's M is st.bytes further on
     const int64_t cz = (int64_t)(st.bytes / 4);
     for (int64_t lo = 0; lo < D; lo += 2 * kBB) {
-        const int64_t mid = lo + kBB;
         note_launches(1);
-        diag_block_kernel<<<n_layers, 256, kDiagSmem, s>>>(st, lo);
-        if (mid == D) break;
-        note_launches(1);
-        trsm_block_kernel<true><<<dim3(trsm_grid(D - mid, n_layers), n_layers), 256, kTrsmSmem, s>>>(
-            st, lo, (char*)M0 + (size_t)mid * D * 4, st.bytes, D, D - mid);
-        // rows [mid, D) of columns [mid, mid + 128) -= L[rows, lo:mid] L[mid:mid+128, lo:mid]^T
-        e = launch_gemm_nt_tc_batched(M0 + mid * D + lo, kBB, D, st.bytes, M0 + mid * D + lo, D - mid, D, st.bytes,
-                                      kBB, M0 + mid * D + mid, D, cz, n_layers, -1.f, 1.f, false, err, s);
+        diag_panel_kernel<<<n_layers, kDiagThreads, sizeof(DiagSmem), s>>>(st, lo);
+        const int64_t hi = lo + 2 * kBB, rest = D - hi;
+        if (rest <= 0) break;
+        e = launch_solve<true>(st, n_layers, lo, 2 * kBB, (char*)M0 + (size_t)hi * D * 4, st.bytes, D, rest, s);
         if (e != cudaSuccess) return e;
-        note_launches(1);
-        diag_block_kernel<<<n_layers, 256, kDiagSmem, s>>>(st, mid);
-        const int64_t hi = mid + kBB, rest = D - hi;
-        if (rest == 0) break;
-        note_launches(1);
-        trsm_block_kernel<true><<<dim3(trsm_grid(rest, n_layers), n_layers), 256, kTrsmSmem, s>>>(
-            st, mid, (char*)M0 + (size_t)hi * D * 4, st.bytes, D, rest);
-        // trailing lower triangle of all layers in one launch: M -= P P^T, P = L[hi:D, lo:hi]
         e = launch_gemm_nt_tc_batched(M0 + hi * D + lo, rest, D, st.bytes, M0 + hi * D + lo, rest, D, st.bytes,
                                       2 * kBB, M0 + hi * D + hi, D, cz, n_layers, -1.f, 1.f, true, err, s);
         if (e != cudaSuccess) return e;
     }
-    const int64_t nb = D / kNB;
+    const int64_t nb = D / 64;
     int64_t g = nb * (nb - 1) / 2 * n_layers;
     if (g > 152 * 8) g = 152 * 8;
     note_launches(1);
@@ -1577,8 +1857,7 @@ bool apply_blocked_ok(int64_t D, tda_dtype sdt, const void* qhat, int64_t ld_qha
 
 cudaError_t apply_blocked(int n_layers, int64_t D, const void* state, const float* q, int64_t n_q, int64_t ld_q,
                           float* qhat, int64_t ld_qhat, cudaStream_t s) {
-    cudaError_t e = blocked_attrs();
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
     unsigned int* err = device_error_word();
     if (!err) return cudaErrorUnknown;
     St<float> st = state_of<float>(const_cast<void*>(state), D);
@@ -1587,24 +1866,25 @@ cudaError_t apply_blocked(int n_layers, int64_t D, const void* state, const floa
                               cudaMemcpyDeviceToDevice, s);
         if (e != cudaSuccess) return e;
     }
-    const unsigned gx = trsm_grid(n_q, n_layers);
     const size_t lb = (size_t)D * 4;  // layer l's columns start l * D floats into each row
     const float* M0 = (const float*)((const char*)state + 64);  // layer l's M is st.bytes further on
-    for (int64_t lo = 0; lo < D; lo += kBB) {
-        note_launches(1);
-        trsm_block_kernel<true><<<dim3(gx, n_layers), 256, kTrsmSmem, s>>>(st, lo, (char*)qhat, lb, ld_qhat, n_q);
-        const int64_t hi = lo + kBB;
+    constexpr int64_t kPanel = 2 * kBB;
+    for (int64_t lo = 0; lo < D; lo += kPanel) {
+        const int64_t hi = lo + kPanel < D ? lo + kPanel : D;
+        e = launch_solve<true>(st, n_layers, lo, (int)(hi - lo), (char*)qhat, lb, ld_qhat, n_q, s);
+        if (e != cudaSuccess) return e;
         if (hi == D) break;
-        e = launch_gemm_nt_tc_batched(M0 + hi * D + lo, D - hi, D, st.bytes, qhat + lo, n_q, ld_qhat, lb, kBB,
+        e = launch_gemm_nt_tc_batched(M0 + hi * D + lo, D - hi, D, st.bytes, qhat + lo, n_q, ld_qhat, lb, kPanel,
                                       qhat + hi, ld_qhat, D, n_layers, -1.f, 1.f, false, err, s);
         if (e != cudaSuccess) return e;
     }
-    for (int64_t lo = D - kBB; lo >= 0; lo -= kBB) {
-        note_launches(1);
-        trsm_block_kernel<false><<<dim3(gx, n_layers), 256, kTrsmSmem, s>>>(st, lo, (char*)qhat, lb, ld_qhat, n_q);
+    for (int64_t lo = (D - 1) / kPanel * kPanel; lo >= 0; lo -= kPanel) {
+        const int64_t hi = lo + kPanel < D ? lo + kPanel : D;
+        e = launch_solve<false>(st, n_layers, lo, (int)(hi - lo), (char*)qhat, lb, ld_qhat, n_q, s);
+        if (e != cudaSuccess) return e;
         if (lo == 0) break;
-        // rows [0, lo) of U = L^T, columns [lo, lo + 128): U[i][j] = L[j][i]
-        e = launch_gemm_nt_tc_batched(M0 + lo, lo, D, st.bytes, qhat + lo, n_q, ld_qhat, lb, kBB, qhat, ld_qhat, D,
+        // rows [0, lo) of U = L^T, columns [lo, hi): U[i][j] = L[j][i]
+        e = launch_gemm_nt_tc_batched(M0 + lo, lo, D, st.bytes, qhat + lo, n_q, ld_qhat, lb, hi - lo, qhat, ld_qhat, D,
                                       n_layers, -1.f, 1.f, false, err, s);
         if (e != cudaSuccess) return e;
     }

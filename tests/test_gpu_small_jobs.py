@@ -104,3 +104,52 @@ def test_topk_selection(dev, orc, nt, values):
         np.testing.assert_array_equal(idx.cpu().numpy(), oi)
         np.testing.assert_array_equal(val.cpu().numpy().view(np.uint32),
                                       np.take_along_axis(S, oi.astype(np.int64), 1).view(np.uint32))
+
+
+# fp32 blocked path: rounding of a 3xTF32 / fp32 Cholesky solve, a few D eps of the condition number (below 50 with
+# damping of a tenth of the mean eigenvalue and four rows a feature): 2e-5 holds with room at D = 2432.
+@pytest.mark.parametrize("D,nl,nq,ld", [(2048, 1, 1, 0), (2176, 2, 17, 4), (2304, 1, 130, 0), (2432, 3, 300, 8)])
+def test_blocked_panels(dev, D, nl, nq, ld):
+    # panels of 256 columns, a last one of 128 or 256; few and many rows per solve launch; padded rows
+    rng = np.random.default_rng(D)
+    n, w = 4 * D, nl * D
+    ph = torch.from_numpy(rng.standard_normal((n, w)).astype(np.float32)).to(dev)
+    q = torch.from_numpy(rng.standard_normal((nq, w + ld)).astype(np.float32)).to(dev)
+    state = torch.empty(nl * tda.tda_precondition_state_bytes(D, tda.TDA_F32), dtype=torch.uint8, device=dev)
+    out = torch.full((nq, w + ld), 3.0, device=dev)
+    args = (nl, D, tda.TDA_F32, state)
+    tda.tda_precondition(tda.TDA_PC_RESET, *args)
+    tda.tda_precondition(tda.TDA_PC_FIT_ACCUM, *args, phi=ph, n=n, ld_phi=w)
+    tda.tda_precondition(tda.TDA_PC_FACTOR, *args, n_total=n, lambda_rel_mean_eig=0.1)
+    tda.tda_precondition(tda.TDA_PC_APPLY, *args, q=q, n_q=nq, ld_q=w + ld, qhat=out, ld_qhat=w + ld)
+    # the other substitution path, from the same state: rows that are not 16-byte aligned
+    out2 = torch.empty(nq * (w + 1) + 1, device=dev)[1:].view(nq, w + 1)
+    tda.tda_precondition(tda.TDA_PC_APPLY, *args, q=q, n_q=nq, ld_q=w + ld, qhat=out2, ld_qhat=w + 1)
+    tda.tda_device_status()
+    tda.tda_precondition_info(nl, D, tda.TDA_F32, state)
+    for l in range(nl):
+        x = ph[:, l * D:(l + 1) * D].double()
+        F = x.T @ x / n
+        F.diagonal().add_(0.1 * F.diagonal().mean())
+        ref = torch.linalg.solve(F, q[:, l * D:(l + 1) * D].double().T).T
+        for o in (out, out2):
+            got = o[:, l * D:(l + 1) * D].double()
+            assert float((got - ref).norm() / ref.norm()) <= 2e-5
+    assert (out[:, w:] == 3.0).all()
+
+
+@pytest.mark.parametrize("bad", [0, 130, 255, 256, 2047])
+def test_blocked_failed_pivot(dev, bad):
+    D = 2048
+    state = torch.empty(tda.tda_precondition_state_bytes(D, tda.TDA_F32), dtype=torch.uint8, device=dev)
+    tda.tda_precondition(tda.TDA_PC_RESET, 1, D, tda.TDA_F32, state)
+    m = state[64:64 + 4 * D * D].view(torch.float32).view(D, D)
+    m.copy_(torch.eye(D, device=dev))
+    m[bad, bad] = -50.0
+    out = torch.zeros((2, D), device=dev)
+    tda.tda_precondition(tda.TDA_PC_FACTOR_APPLY, 1, D, tda.TDA_F32, state, n_total=1, lambda_abs=1e-3,
+                         q=torch.ones((2, D), device=dev), n_q=2, ld_q=D, qhat=out, ld_qhat=D)
+    with pytest.raises(tda.TdaError) as e:
+        tda.tda_precondition_info(1, D, tda.TDA_F32, state)
+    assert e.value.status == tda.TDA_ERR_NOT_SPD and f"pivot {bad + 1}" in str(e.value)
+    assert torch.isnan(out).all()
