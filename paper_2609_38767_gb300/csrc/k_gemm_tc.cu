@@ -8,18 +8,15 @@
 // fp32); the product is hi*hi' + hi*lo' + lo*hi', dropping lo*lo' (relative
 // size ~2^-22). Each K=8 step therefore issues three tcgen05.mma.kind::tf32.
 //
-// CTA tile: 128 rows of Phi (MMA M, one TMEM lane each) x BN query columns
-// (MMA N). Lane 0 of warp 5 copies the fp32 chunks of both operands with TMA
-// (32 features = one 128-byte row per operand row, 128B swizzle: already the
-// K-major operand layout) into the hi tiles of a stage; warps 0-3 write lo to
-// the lo tile at the same offset (the fp32 tile itself is the hi operand: a
-// kind::tf32 MMA reads only the upper 19 bits); lane 0 of warp 4 issues the
-// MMAs; warps 4-7 read the accumulators from TMEM. A thread-block
-// cluster of cs CTAs splits K; the members' partial tiles are summed into the
-// leader CTA over distributed shared memory (deterministic, no workspace)
-// before the leader writes S. With more tiles than SMs and short K (the blocked
-// Cholesky's products) gemm3x_persist_kernel walks the tiles instead. All
-// waits are bounded (see tc_ptx.cuh).
+// gemm3t_kernel (below) is the general kernel: persistent, A operand in TMEM. score3x_kernel serves
+// products with too few tiles for the chip: a CTA tile of 128 rows of Phi (MMA M, one TMEM lane
+// each) x BN query columns (MMA N), a thread-block cluster of cs CTAs splitting K. There lane 0 of
+// warp 9 copies the fp32 chunks of both operands with TMA (32 features = one 128-byte row per
+// operand row, 128B swizzle: already the K-major operand layout) into the hi tiles of a stage;
+// warps 0-3 write lo to the lo tile at the same offset (the fp32 tile itself is the hi operand);
+// lane 0 of warp 8 issues the MMAs; warps 4-7 read the accumulators from TMEM. The members'
+// partial tiles are summed into the leader CTA over distributed shared memory (deterministic, no
+// workspace) before the leader writes S. All waits are bounded (see tc_ptx.cuh).
 #include <cuda.h>
 
 #include <mutex>
@@ -31,7 +28,7 @@ namespace {
 
 #include "tc_ptx.cuh"
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 320;  // score3x_kernel
 constexpr int kBM = 128;       // Phi rows per tile
 constexpr int kKC = 32;        // fp32 elements per K chunk (one 128-byte operand row)
 constexpr uint32_t kRowBytes = kKC * 4;
@@ -43,11 +40,9 @@ struct GCfg {
     static constexpr uint32_t kBBytes = BN * kRowBytes;
     static constexpr uint32_t kStageBytes = 2 * kABytes + 2 * kBBytes;  // hi and lo of both operands
     // The tensor pipe's fp32 accumulation truncates (about a quarter ulp per addition,
-    // always toward zero). One pass: the K chunks rotate over kAcc accumulators (all 512
-    // TMEM columns), each sees 1/kAcc of the additions and the epilogue sums them with
-    // round-to-nearest. DRAIN: groups of kGroup chunks (24 additions) rotate, and the
-    // epilogue warps add every finished group into fp32 registers while the MMAs fill the
-    // next ones (a dot of 7168 features: 0.9e-6 off instead of 1.3e-5, 3 % more time).
+    // always toward zero), so groups of kGroup K chunks (24 additions) rotate over kAcc
+    // accumulators (all 512 TMEM columns) and the epilogue warps add every finished group
+    // into round-to-nearest fp32 registers while the MMAs fill the next ones.
     static constexpr int kAcc = 512 / BN < 8 ? 512 / BN : 8;
     static constexpr int kGroup = 2;
     static constexpr uint32_t kTmemCols = 512;
@@ -115,10 +110,8 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm,
         : "memory");
 }
 
-// DRAIN: the epilogue warps work during the main loop, so warps 8 and 9 issue the MMAs and copies;
-// otherwise lane 0 of warps 4 and 5 does before their epilogue (two more warps cost 2.5 %).
-template <int BN, bool DRAIN>
-__global__ void __launch_bounds__(kThreads + (DRAIN ? 64 : 0), 1)
+template <int BN>
+__global__ void __launch_bounds__(kThreads, 1)
 score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GParams p) {
     using C = GCfg<BN>;
     extern __shared__ uint8_t smem_raw[];
@@ -152,7 +145,7 @@ score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         *abort = 0;
         fence_mbar_init();
     }
-    constexpr int kMmaWarp = DRAIN ? 8 : 4, kTmaWarp = DRAIN ? 9 : 5;
+    constexpr int kMmaWarp = 8, kTmaWarp = 9;
     if (warp == kMmaWarp) {
         tmem_alloc(smem_u32(tmem_slot), C::kTmemCols);
         tmem_relinquish();
@@ -245,9 +238,9 @@ score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         for (int64_t kc = kc0; kc < kc1; ++kc, ++it) {
             const int s = it % C::kStages;
             const uint32_t ph = (it / C::kStages) & 1u;
-            const uint32_t g = DRAIN ? it / C::kGroup : it, a = g % C::kAcc;  // group g goes to accumulator a
-            const bool start = DRAIN ? it % C::kGroup == 0 : it < (uint32_t)C::kAcc;
-            if (DRAIN && start && !wait_bounded(smem_u32(&acc_empty[a]), ((g / C::kAcc) & 1u) ^ 1u, abort, p.err)) break;
+            const uint32_t g = it / C::kGroup, a = g % C::kAcc;  // group g goes to accumulator a
+            const bool start = it % C::kGroup == 0;
+            if (start && !wait_bounded(smem_u32(&acc_empty[a]), ((g / C::kAcc) & 1u) ^ 1u, abort, p.err)) break;
             if (!wait_bounded(smem_u32(&full[s]), ph, abort, p.err)) break;
             tc_fence_after();
             const uint32_t st = smem_u32(smem + (size_t)s * C::kStageBytes);
@@ -261,8 +254,7 @@ score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 mma_tf32(d, alo + 2 * k, bhi + 2 * k, idesc, 1u);
             }
             mma_commit(smem_u32(&empty[s]));
-            if (DRAIN ? (it % C::kGroup == C::kGroup - 1 || kc == kc1 - 1) : kc == kc1 - 1)
-                mma_commit(smem_u32(&acc_full[DRAIN ? a : 0u]));
+            if (it % C::kGroup == C::kGroup - 1 || kc == kc1 - 1) mma_commit(smem_u32(&acc_full[a]));
         }
         mma_commit(smem_u32(mma_done));
         const uint64_t t0 = global_ns();
@@ -279,8 +271,7 @@ score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const int row = q * 32 + lane;  // Phi row within the tile
         const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16);
         const uint32_t nchunks = kc1 > kc0 ? (uint32_t)(kc1 - kc0) : 0u;
-        const uint32_t groups = DRAIN ? (nchunks + C::kGroup - 1) / C::kGroup : (nchunks > 0 ? 1u : 0u);
-        const uint32_t used = DRAIN ? 1u : (nchunks < (uint32_t)C::kAcc ? nchunks : (uint32_t)C::kAcc);
+        const uint32_t groups = (nchunks + C::kGroup - 1) / C::kGroup;
         float acc[BN];
 #pragma unroll
         for (int c = 0; c < BN; ++c) acc[c] = 0.f;
@@ -292,16 +283,15 @@ score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             if (!got) break;
             tc_fence_after();
 #pragma unroll
-            for (int c0 = 0; c0 < BN; c0 += 16)
-                for (uint32_t b = 0; b < used; ++b) {
-                    float v[16];
-                    tmem_ld16(tbase + (a + b) * BN + c0, v);
+            for (int c0 = 0; c0 < BN; c0 += 16) {
+                float v[16];
+                tmem_ld16(tbase + a * BN + c0, v);
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) acc[c0 + i] += v[i];
-                }
+                for (int i = 0; i < 16; ++i) acc[c0 + i] += v[i];
+            }
             tc_fence_before();
             __syncwarp();
-            if (DRAIN && lane == 0) mbar_arrive(smem_u32(&acc_empty[a]));
+            if (lane == 0) mbar_arrive(smem_u32(&acc_empty[a]));
         }
         if (!epi_any(!got)) {
             bool ok = true;
@@ -386,61 +376,104 @@ score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 }
 
 // ---------------------------------------------------------------------------
-// Persistent variant of the same product for many tiles with short K (the
-// blocked Cholesky's trailing updates and the substitutions' block products,
-// K = 128 or 256): each CTA walks tiles blockIdx.x, blockIdx.x + gridDim.x, ...
-// over all batch entries with one set of barriers and one TMEM allocation. The
-// accumulators are double-buffered (kAcc per buffer), so a tile's epilogue
-// (TMEM -> registers -> S) overlaps the next tile's loads, splits and MMAs.
-// Warps 0-3 split, warps 4-7 epilogue, lane 0 of warp 8 issues the TMA copies,
-// lane 0 of warp 9 the MMAs. Same arithmetic per tile as score3x_kernel (the
-// K chunks rotate over kAcc accumulators, summed on CUDA cores). No clusters,
-// no split-K. All waits are bounded. Ten warps share the register file's four
-// partitions unevenly (three warps on two of them), which caps a thread at 168
-// registers: the epilogue drains the accumulators 64 columns at a time.
-constexpr int kThreadsP = 320;
+// The same product without clusters, with the A operand in TMEM: one persistent CTA per SM walks
+// the tiles of all batch entries and feature slices.
+//
+// What bounds a 128 x 128 tile of three TF32 products per element pair is shared memory. With both
+// operands there, a 32-feature chunk (768 clocks of MMAs) costs 768 clocks of operand reads, 256 of
+// TMA writes and 512 of splitting at 128 bytes a clock. Here four warps read the rows of Phi once
+// (a thread per row: the 128-byte swizzle makes its 16-byte loads conflict-free) and put hi (the
+// fp32 value as it is: a kind::tf32 MMA reads its upper 19 bits) and lo into TMEM, a column per
+// feature, so only B's hi and lo are read by the MMAs: 1024 clocks.
+//
+// Accuracy: groups of kGroup chunks (24 truncating additions) alternate between two accumulators,
+// and eight epilogue warps (two per TMEM lane quadrant, half of the columns each) add every
+// finished group into round-to-nearest registers beside the next group's MMAs, then write the
+// tile beside the next tile's.
+//
+// Measured: scores of 256 x 8192, 7168 features: 205 us with both operands in shared memory and
+// one pass over the accumulators (1.3e-5 off), 188 us and 9e-7 off here.
+//
+// Warps: 0-3 A into TMEM, 4-7 B's lo, 8-15 epilogue, 16 MMA issuer, 17 TMA. All waits are bounded.
+constexpr int kThreadsT = 18 * 32;
 
 template <int BN>
-struct PCfg {
-    static constexpr int kStages = GCfg<BN>::kStages;
-    static constexpr uint32_t kABytes = GCfg<BN>::kABytes;
-    static constexpr uint32_t kBBytes = GCfg<BN>::kBBytes;
-    static constexpr uint32_t kStageBytes = GCfg<BN>::kStageBytes;
-    static constexpr int kAcc = 256 / BN;  // per buffer: two buffers fill the 512 TMEM columns
+struct TCfg {
+    static constexpr uint32_t kABytes = kBM * kRowBytes;  // 16 KiB
+    static constexpr uint32_t kBBytes = BN * kRowBytes;
+    static constexpr uint32_t kStageBytes = kABytes + 2 * kBBytes;  // A raw; B raw (hi) and lo
+    static constexpr int kStages = 4;                     // also TMEM slots of A
+    static constexpr int kGroup = 2;
+    static constexpr int kCols = BN / 2;                  // columns per epilogue thread
+    static constexpr int kAOff = 2 * BN;                  // first TMEM column of A: [stage][hi 32 | lo 32]
     static constexpr size_t kSmem = 1024 + (size_t)kStages * kStageBytes + 8 * (3 * kStages + 5) + 16;
+    static_assert(kAOff + kStages * 64 <= 512 && kSmem <= 232448, "TMEM columns, shared memory");
 };
 
-// Rows m0 (of A) and n0 (of B) and batch entry z of tile t.
+// D[tmem] (+)= A[tmem] * B[smem]^T, tf32 inputs.
+__device__ __forceinline__ void mma_tf32_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
+                                            uint32_t accumulate) {
+    asm volatile(
+        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}" ::"r"(
+            d_tmem),
+        "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(
+            taddr),
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+        "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+        : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// Tile t: rows m0 (of A) and n0 (of B), batch entry z, feature slice y.
+struct TileAt {
+    int64_t m0, n0;
+    int z, y;
+};
 template <int BN>
-__device__ __forceinline__ void tile_at(const GParams& p, int64_t t, int64_t& m0, int64_t& n0, int& z) {
-    z = (int)(t / p.tiles_z);
-    const int64_t tile = t - (int64_t)z * p.tiles_z;
+__device__ __forceinline__ TileAt tile_at(const GParams& p, int64_t t) {
+    TileAt a;
+    const int64_t per_z = p.tiles_z * p.splits;
+    a.z = (int)(t / per_z);
+    t -= (int64_t)a.z * per_z;
+    a.y = (int)(t / p.tiles_z);
+    const int64_t tile = t - (int64_t)a.y * p.tiles_z;
     if (p.lower) {
         int64_t i = (int64_t)((sqrt(8.0 * (double)tile + 1.0) - 1.0) * 0.5);
         while (i * (i + 1) / 2 > tile) --i;
         while ((i + 1) * (i + 2) / 2 <= tile) ++i;
-        n0 = i * BN;
-        m0 = (tile - i * (i + 1) / 2) * kBM;
+        a.n0 = i * BN;
+        a.m0 = (tile - i * (i + 1) / 2) * kBM;
     } else {
-        m0 = (tile / p.tiles_n) * kBM;
-        n0 = (tile % p.tiles_n) * BN;
+        a.m0 = (tile / p.tiles_n) * kBM;
+        a.n0 = (tile % p.tiles_n) * BN;
     }
+    return a;
+}
+// 32-feature chunks of slice y
+__device__ __forceinline__ int64_t chunks_of(const GParams& p, int y) {
+    const int64_t kbase = (int64_t)y * p.kslice;
+    const int64_t Kz = p.kslice ? ((p.K - kbase) < p.kslice ? (p.K - kbase) : p.kslice) : p.K;
+    return (Kz + kKC - 1) / kKC;
 }
 
 template <int BN>
-__global__ void __launch_bounds__(kThreadsP, 1)
-gemm3x_persist_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                      const GParams p) {
-    using C = PCfg<BN>;
+__global__ void __launch_bounds__(kThreadsT, 1)
+gemm3t_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GParams p) {
+    using C = TCfg<BN>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint64_t* bars = (uint64_t*)(smem + (size_t)C::kStages * C::kStageBytes);
-    uint64_t* raw_full = bars;                  // [kStages] TMA bytes landed (count 1 + tx)
-    uint64_t* full = raw_full + C::kStages;     // [kStages] split into hi/lo (count 4)
-    uint64_t* empty = full + C::kStages;        // [kStages] MMAs done reading (count 1)
-    uint64_t* tfull = empty + C::kStages;       // [2] accumulators ready (count 1)
-    uint64_t* tempty = tfull + 2;               // [2] accumulators drained (count 4)
-    uint64_t* mma_done = tempty + 2;            // count 1
+    uint64_t* raw_full = bars;               // [kStages] TMA bytes landed (count 1 + tx)
+    uint64_t* ready = raw_full + C::kStages; // [kStages] A in TMEM, B's lo written (8 warps)
+    uint64_t* empty = ready + C::kStages;    // [kStages] MMAs done reading (count 1)
+    uint64_t* acc_full = empty + C::kStages; // [2] a group is accumulated (count 1)
+    uint64_t* acc_empty = acc_full + 2;      // [2] the accumulator is drained (8 warps)
+    uint64_t* mma_done = acc_empty + 2;
     uint32_t* tmem_slot = (uint32_t*)(mma_done + 1);
     volatile int* abort = (volatile int*)(tmem_slot + 1);
 
@@ -448,18 +481,18 @@ gemm3x_persist_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::kStages; ++s) {
             mbar_init(smem_u32(&raw_full[s]), 1);
-            mbar_init(smem_u32(&full[s]), 4);
+            mbar_init(smem_u32(&ready[s]), 8);
             mbar_init(smem_u32(&empty[s]), 1);
         }
         for (int b = 0; b < 2; ++b) {
-            mbar_init(smem_u32(&tfull[b]), 1);
-            mbar_init(smem_u32(&tempty[b]), 4);
+            mbar_init(smem_u32(&acc_full[b]), 1);
+            mbar_init(smem_u32(&acc_empty[b]), 8);
         }
         mbar_init(smem_u32(mma_done), 1);
         *abort = 0;
         fence_mbar_init();
     }
-    if (warp == 9) {
+    if (warp == 16) {
         tmem_alloc(smem_u32(tmem_slot), 512);
         tmem_relinquish();
     }
@@ -467,119 +500,133 @@ gemm3x_persist_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    const int64_t total = p.tiles_z * p.nz;
-    const int64_t nkc = (p.K + kKC - 1) / kKC;
+    const int64_t total = p.tiles_z * p.splits * p.nz;
 
-    if (warp < 4) {
-        // ---------------- split warps: raw fp32 (TMA) -> hi in place + lo
-        const int pt = threadIdx.x;
+    if (warp < 8) {
+        // ---------------- split warps: 0-3 A's rows into TMEM, 4-7 B's lo into shared memory
         uint32_t it = 0;
         bool ok = true;
-        for (int64_t t = blockIdx.x; ok && t < total; t += gridDim.x)
+        for (int64_t t = blockIdx.x; ok && t < total; t += gridDim.x) {
+            const int64_t nkc = chunks_of(p, tile_at<BN>(p, t).y);
             for (int64_t kc = 0; kc < nkc; ++kc, ++it) {
-                const int s = it % C::kStages;
-                const uint32_t ph = (it / C::kStages) & 1u;
+                const uint32_t s = it % C::kStages, ph = (it / C::kStages) & 1u;
                 bool got = true;
                 if (lane == 0) got = wait_bounded(smem_u32(&raw_full[s]), ph, abort, p.err);
                 got = __shfl_sync(0xffffffffu, got, 0);
-                __syncwarp();
                 if (!got) {
                     ok = false;
                     break;
                 }
                 uint8_t* st = smem + (size_t)s * C::kStageBytes;
-                split_tile<C::kABytes>(st, st + C::kABytes, pt);
-                split_tile<C::kBBytes>(st + 2 * C::kABytes, st + 2 * C::kABytes + C::kBBytes, pt);
-                fence_proxy_async();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&full[s]));
-            }
-    } else if (warp < 8) {
-        // ---------------- epilogue: TMEM -> registers (buffer released) -> S
-        const int q = warp & 3;
-        const int row = q * 32 + lane;
-        const int used = (int)(nkc < C::kAcc ? nkc : C::kAcc);
-        uint32_t lt = 0;
-        for (int64_t t = blockIdx.x; t < total; t += gridDim.x, ++lt) {
-            const uint32_t b = lt & 1u, ph = (lt >> 1) & 1u;
-            bool got = true;
-            if (lane == 0) got = wait_bounded(smem_u32(&tfull[b]), ph, abort, p.err);
-            got = __shfl_sync(0xffffffffu, got, 0);
-            if (epi_any(!got)) break;
-            tc_fence_after();
-            const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + b * (uint32_t)(C::kAcc * BN);
-            int64_t m0, n0;
-            int z;
-            tile_at<BN>(p, t, m0, n0, z);
-            float* Sz = p.S + (int64_t)z * p.s_z;
-            const int64_t m = m0 + row;
-            // 64 columns at a time (register budget): the part's previous values are loaded first,
-            // so the 64 loads are in flight while the part's accumulators are read from TMEM; the
-            // buffer is released after the last read
-            constexpr int HW = BN < 64 ? BN : 64;
-            const bool rmw = p.beta != 0.f && m < p.n_t;
-#pragma unroll 1
-            for (int h0 = 0; h0 < BN; h0 += HW) {
-                float old[HW];
-                if (rmw) {
+                if (warp < 4) {
+                    // the stage's TMEM slot is free: its MMAs were done before TMA refilled the stage
+                    tc_fence_after();
+                    const int row = warp * 32 + lane;
+                    const uint8_t* src = st + (uint32_t)row * kRowBytes;
+                    const uint32_t dst = tmem + ((uint32_t)(warp * 32) << 16) + C::kAOff + s * 64u;
 #pragma unroll
-                    for (int i = 0; i < HW; ++i) {
-                        const int64_t n = n0 + h0 + i;
-                        old[i] = n < p.n_q ? __ldcg(Sz + n * p.ld_S + m) : 0.f;
+                    for (int h = 0; h < 2; ++h) {
+                        uint32_t hi[16], lo[16];
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            const float4 v =
+                                *reinterpret_cast<const float4*>(src + (((4 * h + c) ^ (row & 7)) << 4));
+                            const float x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                float hf, lf;
+                                split_tf32(x[i], hf, lf);
+                                hi[4 * c + i] = __float_as_uint(x[i]);
+                                lo[4 * c + i] = __float_as_uint(lf);
+                            }
+                        }
+                        tmem_st16(dst + 16 * h, hi);
+                        tmem_st16(dst + 32 + 16 * h, lo);
                     }
-                }
-                float acc[HW];
-#pragma unroll
-                for (int c0 = 0; c0 < HW; c0 += 16) {
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) acc[c0 + i] = 0.f;
-                    for (int a = 0; a < used; ++a) {
-                        float v[16];
-                        tmem_ld16(tbase + a * BN + h0 + c0, v);
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) acc[c0 + i] += v[i];
-                    }
-                }
-                if (h0 + HW >= BN) {
+                    tmem_wait_st();
                     tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&tempty[b]));
+                } else {
+                    split_tile<C::kBBytes>(st + C::kABytes, st + C::kABytes + C::kBBytes, threadIdx.x - 128);
+                    fence_proxy_async();
                 }
-                if (m < p.n_t) {
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&ready[s]));
+            }
+        }
+    } else if (warp < 16) {
+        // ---------------- epilogue: groups -> registers -> S
+        const int q4 = warp & 3, half = (warp - 8) >> 2, row = q4 * 32 + lane;
+        const uint32_t tbase = tmem + ((uint32_t)(q4 * 32) << 16) + half * C::kCols;
+        uint32_t cnt = 0;
+        bool got = true;
+        for (int64_t t = blockIdx.x; got && t < total; t += gridDim.x) {
+            const TileAt at = tile_at<BN>(p, t);
+            const uint32_t groups = (uint32_t)((chunks_of(p, at.y) + C::kGroup - 1) / C::kGroup);
+            float acc[C::kCols];
 #pragma unroll
-                    for (int i = 0; i < HW; ++i) {
-                        const int64_t n = n0 + h0 + i;
-                        if (n < p.n_q) Sz[n * p.ld_S + m] = rmw ? p.beta * old[i] + p.alpha * acc[i] : p.alpha * acc[i];
-                    }
+            for (int c = 0; c < C::kCols; ++c) acc[c] = 0.f;
+            for (uint32_t g = 0; g < groups; ++g, ++cnt) {
+                const uint32_t b = cnt & 1u;
+                if (lane == 0) got = wait_bounded(smem_u32(&acc_full[b]), (cnt >> 1) & 1u, abort, p.err);
+                got = __shfl_sync(0xffffffffu, got, 0);
+                if (!got) break;
+                tc_fence_after();
+#pragma unroll
+                for (int c0 = 0; c0 < C::kCols; c0 += 16) {
+                    float v[16];
+                    tmem_ld16(tbase + b * BN + c0, v);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) acc[c0 + i] += v[i];
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&acc_empty[b]));
+            }
+            const int64_t m = at.m0 + row, nb = at.n0 + half * C::kCols;
+            if (!got || m >= p.n_t) continue;
+            float* Sz = p.S + (int64_t)at.y * p.slab + (int64_t)at.z * p.s_z + m;
+            const int lim = (int)(p.n_q - nb < C::kCols ? p.n_q - nb : C::kCols);
+            if (p.beta == 0.f) {
+#pragma unroll
+                for (int c = 0; c < C::kCols; ++c)
+                    if (c < lim) Sz[(nb + c) * p.ld_S] = p.alpha * acc[c];
+            } else {
+                // 8 previous values are on their way together
+#pragma unroll
+                for (int c0 = 0; c0 < C::kCols; c0 += 8) {
+                    float old[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) old[i] = c0 + i < lim ? __ldcg(Sz + (nb + c0 + i) * p.ld_S) : 0.f;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                        if (c0 + i < lim) Sz[(nb + c0 + i) * p.ld_S] = p.beta * old[i] + p.alpha * acc[c0 + i];
                 }
             }
         }
-    } else if (warp == 8 && lane == 0) {
+    } else if (warp == 17 && lane == 0) {
         // ---------------- TMA producer
         uint32_t it = 0, last_par[C::kStages];
-        bool issued[C::kStages];
+        bool issued[C::kStages], ok = true;
         for (int s = 0; s < C::kStages; ++s) issued[s] = false;
-        bool ok = true;
         for (int64_t t = blockIdx.x; ok && t < total; t += gridDim.x) {
-            int64_t m0, n0;
-            int z;
-            tile_at<BN>(p, t, m0, n0, z);
+            const TileAt at = tile_at<BN>(p, t);
+            const int64_t nkc = chunks_of(p, at.y);
+            const int64_t kbase = (int64_t)at.y * p.kslice;
             for (int64_t kc = 0; kc < nkc; ++kc, ++it) {
-                const int s = it % C::kStages;
-                const uint32_t ph = (it / C::kStages) & 1u;
+                const uint32_t s = it % C::kStages, ph = (it / C::kStages) & 1u;
                 if (!wait_bounded(smem_u32(&empty[s]), ph ^ 1u, abort, p.err)) {
                     ok = false;
                     break;
                 }
                 const uint32_t st = smem_u32(smem + (size_t)s * C::kStageBytes), bar = smem_u32(&raw_full[s]);
-                const int k = (int)(kc * kKC);
+                const int k = (int)(kbase + kc * kKC);
                 mbar_arrive_tx(bar, C::kABytes + C::kBBytes);
                 if (p.batched) {
-                    tma_load_3d(st, &tmA, k, (int)m0, z, bar);
-                    tma_load_3d(st + 2 * C::kABytes, &tmB, k, (int)n0, z, bar);
+                    tma_load_3d(st, &tmA, k, (int)at.m0, at.z, bar);
+                    tma_load_3d(st + C::kABytes, &tmB, k, (int)at.n0, at.z, bar);
                 } else {
-                    tma_load_2d(st, &tmA, k, (int)m0, bar);
-                    tma_load_2d(st + 2 * C::kABytes, &tmB, k, (int)n0, bar);
+                    tma_load_2d(st, &tmA, k, (int)at.m0, bar);
+                    tma_load_2d(st + C::kABytes, &tmB, k, (int)at.n0, bar);
                 }
                 issued[s] = true;
                 last_par[s] = ph;
@@ -594,38 +641,37 @@ gemm3x_persist_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
                         break;
                     }
             }
-    } else if (warp == 9 && lane == 0) {
+    } else if (warp == 16 && lane == 0) {
         // ---------------- MMA issuer
-        const uint32_t idesc = idesc_tf32(kBM, BN);
-        uint32_t it = 0, lt = 0;
+        constexpr uint32_t idesc = idesc_tf32(kBM, BN);
+        uint32_t it = 0, cnt = 0;
         bool ok = true;
-        for (int64_t t = blockIdx.x; ok && t < total; t += gridDim.x, ++lt) {
-            const uint32_t b = lt & 1u, use = lt >> 1;
-            if (!wait_bounded(smem_u32(&tempty[b]), (use & 1u) ^ 1u, abort, p.err)) break;
-            tc_fence_after();
+        for (int64_t t = blockIdx.x; ok && t < total; t += gridDim.x) {
+            const int64_t nkc = chunks_of(p, tile_at<BN>(p, t).y);
             for (int64_t kc = 0; kc < nkc; ++kc, ++it) {
-                const int s = it % C::kStages;
-                const uint32_t ph = (it / C::kStages) & 1u;
-                if (!wait_bounded(smem_u32(&full[s]), ph, abort, p.err)) {
+                const uint32_t s = it % C::kStages, ph = (it / C::kStages) & 1u, b = cnt & 1u;
+                const bool start = kc % C::kGroup == 0, last = kc % C::kGroup == C::kGroup - 1 || kc == nkc - 1;
+                if ((start && !wait_bounded(smem_u32(&acc_empty[b]), ((cnt >> 1) & 1u) ^ 1u, abort, p.err)) ||
+                    !wait_bounded(smem_u32(&ready[s]), ph, abort, p.err)) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
                 const uint32_t st = smem_u32(smem + (size_t)s * C::kStageBytes);
-                const uint64_t ahi = sw128_desc(st), alo = sw128_desc(st + C::kABytes);
-                const uint64_t bhi = sw128_desc(st + 2 * C::kABytes), blo = sw128_desc(st + 2 * C::kABytes + C::kBBytes);
-                const uint32_t d = tmem + (b * C::kAcc + (uint32_t)(kc % C::kAcc)) * BN;
+                const uint32_t ahi = tmem + C::kAOff + s * 64u, alo = ahi + 32u, d = tmem + b * BN;
+                const uint64_t bhi = sw128_desc(st + C::kABytes), blo = sw128_desc(st + C::kABytes + C::kBBytes);
 #pragma unroll
-                for (int k = 0; k < kKC / 8; ++k) {
-                    const uint32_t first = (kc < C::kAcc && k == 0) ? 0u : 1u;
-                    mma_tf32(d, ahi + 2 * k, bhi + 2 * k, idesc, first);
-                    mma_tf32(d, ahi + 2 * k, blo + 2 * k, idesc, 1u);
-                    mma_tf32(d, alo + 2 * k, bhi + 2 * k, idesc, 1u);
+                for (int k = 0; k < kKC / 8; ++k) {  // K = 8 tf32: 8 TMEM columns, 32 bytes of shared memory
+                    mma_tf32_ta(d, ahi + 8 * k, bhi + 2 * k, idesc, start && k == 0 ? 0u : 1u);
+                    mma_tf32_ta(d, ahi + 8 * k, blo + 2 * k, idesc, 1u);
+                    mma_tf32_ta(d, alo + 8 * k, bhi + 2 * k, idesc, 1u);
                 }
                 mma_commit(smem_u32(&empty[s]));
+                if (last) {
+                    mma_commit(smem_u32(&acc_full[b]));
+                    ++cnt;
+                }
             }
-            if (!ok) break;
-            mma_commit(smem_u32(&tfull[b]));
         }
         mma_commit(smem_u32(mma_done));
         const uint64_t t0 = global_ns();
@@ -638,7 +684,7 @@ gemm3x_persist_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
 
     tc_fence_before();
     __syncthreads();
-    if (warp == 9) {
+    if (warp == 16) {
         tc_fence_after();
         tmem_dealloc(tmem, 512);
     }
@@ -982,30 +1028,6 @@ bool make_map_f32_3d(CUtensorMap* tm, const float* X, int64_t rows, int64_t K, i
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int BN, bool DRAIN>
-cudaError_t launch_score3x(const CUtensorMap& tmA, const CUtensorMap& tmB, const GParams& p, int64_t tiles, int64_t nz,
-                           cudaStream_t s) {
-    using C = GCfg<BN>;
-    cudaError_t e = smem_attr_once<score3x_kernel<BN, DRAIN>>((int)C::kSmem);
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)p.cs;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3((unsigned)(tiles * p.cs), (unsigned)p.splits, (unsigned)nz);
-    cfg.blockDim = dim3(kThreads + (DRAIN ? 64 : 0));
-    cfg.dynamicSmemBytes = C::kSmem;
-    cfg.stream = s;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    note_launches(1);
-    e = cudaLaunchKernelEx(&cfg, score3x_kernel<BN, DRAIN>, tmA, tmB, p);
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
-}
-
 template <int BN>
 cudaError_t launch_bn(GParams p, cudaStream_t s, int64_t nz = 1, size_t a_z_bytes = 0, size_t b_z_bytes = 0) {
     using C = GCfg<BN>;
@@ -1035,20 +1057,36 @@ cudaError_t launch_bn(GParams p, cudaStream_t s, int64_t nz = 1, size_t a_z_byte
     while (cs > 1 && (size_t)(cs - 1) * kBM * BN * 4 > (size_t)C::kStages * C::kStageBytes) cs >>= 1;
     p.cs = cs;
     p.tiles_n = (int)tiles_n;
-    if (cs == 1 && p.splits == 1 && !p.kslice && nkc <= 64 && tiles * nz > sms) {
-        // more tiles than SMs with short K: one persistent CTA per SM walks the tiles
-        using P = PCfg<BN>;
+    if (cs == 1) {
+        using T = TCfg<BN>;
         p.tiles_z = tiles;
         p.nz = (int)nz;
-        cudaError_t e = smem_attr_once<gemm3x_persist_kernel<BN>>((int)P::kSmem);
+        const int64_t total = tiles * p.splits * nz;
+        cudaError_t e = smem_attr_once<gemm3t_kernel<BN>>((int)T::kSmem);
         if (e != cudaSuccess) return e;
         note_launches(1);
-        gemm3x_persist_kernel<BN><<<(unsigned)sms, kThreadsP, P::kSmem, s>>>(tmA, tmB, p);
+        gemm3t_kernel<BN><<<(unsigned)(total < sms ? total : sms), kThreadsT, T::kSmem, s>>>(tmA, tmB, p);
         return cudaGetLastError();
     }
-    // slices of materialised-gradient dots (thousands of features a slice) drain their accumulators
-    return p.kslice ? launch_score3x<BN, true>(tmA, tmB, p, tiles, nz, s)
-                    : launch_score3x<BN, false>(tmA, tmB, p, tiles, nz, s);
+    // few tiles: a cluster of cs CTAs splits K
+    cudaError_t e = smem_attr_once<score3x_kernel<BN>>((int)C::kSmem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)cs;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)(tiles * cs), (unsigned)p.splits, (unsigned)nz);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = C::kSmem;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    note_launches(1);
+    e = cudaLaunchKernelEx(&cfg, score3x_kernel<BN>, tmA, tmB, p);
+    if (e != cudaSuccess) return e;
+    return cudaGetLastError();
 }
 
 }  // namespace
