@@ -161,7 +161,7 @@ score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     int64_t m0 = (tile / p.tiles_n) * kBM, n0 = (tile % p.tiles_n) * BN;
     if (p.lower) {
         // tile t of the lower triangle: row tile i (n), column tile j (m) <= i, t = i(i+1)/2 + j
-        int64_t i = (int64_t)((sqrt(8.0 * (double)tile + 1.0) - 1.0) * 0.5);
+        int64_t i = (int64_t)((sqrtf(8.f * (float)tile + 1.f) - 1.f) * 0.5f);  // fp64 is a slow pipe here
         while (i * (i + 1) / 2 > tile) --i;
         while ((i + 1) * (i + 2) / 2 <= tile) ++i;
         n0 = i * BN;
@@ -443,7 +443,7 @@ __device__ __forceinline__ TileAt tile_at(const GParams& p, int64_t t) {
     a.y = (int)(t / p.tiles_z);
     const int64_t tile = t - (int64_t)a.y * p.tiles_z;
     if (p.lower) {
-        int64_t i = (int64_t)((sqrt(8.0 * (double)tile + 1.0) - 1.0) * 0.5);
+        int64_t i = (int64_t)((sqrtf(8.f * (float)tile + 1.f) - 1.f) * 0.5f);  // fp64 is a slow pipe here
         while (i * (i + 1) / 2 > tile) --i;
         while ((i + 1) * (i + 2) / 2 <= tile) ++i;
         a.n0 = i * BN;
@@ -693,14 +693,20 @@ gemm3t_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
 // ---------------------------------------------------------------------------
 // Fisher fit on the tensor cores: M_l += Phi_l^T Phi_l for the lower 128 x 128
 // tiles of every layer l (layer l's features at column l*D of each row of Phi).
-// The MMA operand tiles are features x examples, K-major (32 examples per
-// chunk), but Phi holds examples x features. Lane 0 of warp 5 copies each chunk
-// raw with TMA (32 examples x 32 features per box, 128-byte swizzle, 4 boxes
-// per operand) into a ring of raw stages; warps 0-3 read it back transposed
-// (lane = example, 16 bytes of features per load: conflict-free thanks to the
-// swizzle), split every value to hi/lo and write both into the K-major swizzled
-// operand layout (conflict-free: the 32 lanes hit 32 distinct banks). A tile on
-// the diagonal has A = B and loads and splits one operand.
+// The MMA operands are features x examples, K-major (32 examples per chunk), but
+// Phi holds examples x features. Lane 0 of warp 17 copies each chunk raw with TMA
+// (32 examples x 32 features per box, 128-byte swizzle, 4 boxes per operand) into
+// a ring of raw stages. As in gemm3t_kernel the A operand goes to TMEM: warps 0-3
+// read the boxes with a lane per feature (32 lanes on one 128-byte row:
+// conflict-free), which is the TMEM lane, and write the 32 examples' hi and lo.
+// Warps 4-7 read B transposed (lane = example, 16 bytes of features per load:
+// conflict-free thanks to the swizzle), split every value to hi/lo and write both
+// into the K-major swizzled operand layout (conflict-free: the 32 lanes hit 32
+// distinct banks). A tile on the diagonal has A = B and loads one operand.
+// Shared memory bounds it: 1152 of a chunk's clocks at 128 bytes each, 1792 with
+// both operands there (seven layers of D = 4096, 8192 examples: 6.74 ms, 6.24 ms here).
+// A's features are the tile's columns of M, so that a warp's 32 lanes are 32
+// neighbouring entries of a row of M.
 template <int ROWS>
 __device__ __forceinline__ void store_split_t(const float4 (&vals)[ROWS / 16], uint8_t* hi, uint8_t* lo, int pt) {
     constexpr int kPer = ROWS / 16;
@@ -729,138 +735,234 @@ __device__ __forceinline__ void load_raw_t(const uint8_t* raw, float4 (&vals)[8]
 }
 
 struct FCfg {
-    static constexpr int kStages = 2;       // hi/lo operand stages
-    static constexpr int kRawStages = 3;    // raw TMA chunks
+    static constexpr int kStages = 3;                       // B hi/lo stages and TMEM slots of A
+    static constexpr int kRawStages = 4;                    // raw TMA chunks
     static constexpr uint32_t kABytes = kBM * kRowBytes;    // 16 KiB: one operand, hi or lo or raw
-    static constexpr uint32_t kStageBytes = 4 * kABytes;    // hi and lo of both operands
+    static constexpr uint32_t kStageBytes = 2 * kABytes;    // hi and lo of B
     static constexpr uint32_t kRawBytes = 2 * kABytes;      // raw chunk of both operands
     // The tensor pipe's fp32 accumulation rounds toward zero, so a long same-sign sum
-    // (a diagonal entry of M) drifts low by ~1 ulp per accumulate. Each accumulator
-    // therefore takes a group of kGroup consecutive chunks (48 accumulates) and the
-    // epilogue warps drain it into round-to-nearest fp32 registers while the MMAs
-    // move on to the next of the kAcc accumulators.
-    static constexpr int kAcc = 4;                          // 4 x 128 TMEM columns
-    static constexpr int kGroup = 4;                        // chunks per accumulator group
-    static constexpr uint32_t kTmemCols = 512;
+    // (a diagonal entry of M) drifts low by up to an ulp per accumulate. Groups of kGroup
+    // chunks (24 accumulates) alternate between two accumulators and the epilogue warps
+    // drain them into round-to-nearest fp32 registers while the MMAs move on.
+    static constexpr int kGroup = 2;
+    static constexpr int kAOff = 2 * 128;                   // first TMEM column of A
     static constexpr size_t kBarOff = (size_t)kStages * kStageBytes + (size_t)kRawStages * kRawBytes;
-    static constexpr size_t kSmem = 1024 + kBarOff + 8 * (2 * kStages + 2 * kRawStages + 2 * kAcc + 1) + 16;
+    static constexpr size_t kSmem = 1024 + kBarOff + 8 * (2 * kStages + 2 * kRawStages + 5) + 16;
+    static_assert(kSmem <= 232448 && kAOff + 64 * kStages <= 512, "fit3t shared memory, TMEM columns");
 };
-static_assert(FCfg::kSmem <= 232448, "fit3x shared memory");
-static_assert(128 * 129 * 4 <= FCfg::kStages * FCfg::kStageBytes, "fit3x staging tile");
 
 struct FParams {
     char* state;       // layer states, `bytes` apart; M at +64
     size_t bytes;
     int64_t D, n;
     int tiles;         // lower tiles per layer
+    int total;         // tiles of all layers
     unsigned int* err;
 };
 
-constexpr int kFitThreads = 320;  // warps 0-3 split, 4-7 epilogue, 8 MMA, 9 TMA
-__global__ void __launch_bounds__(kFitThreads, 1) fit3x_kernel(const __grid_constant__ CUtensorMap tm, const FParams p) {
+struct FTile {
+    int layer;
+    int64_t r0, c0;  // M's rows and columns
+    bool diag;
+};
+__device__ __forceinline__ FTile fit_tile(const FParams& p, int u) {
+    FTile f;
+    f.layer = u / p.tiles;
+    const int t = u - f.layer * p.tiles;
+    int by = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);  // lower-tile index -> (by, bx), bx <= by
+    while ((by + 1) * (by + 2) / 2 <= t) ++by;
+    while (by * (by + 1) / 2 > t) --by;
+    const int bx = t - by * (by + 1) / 2;
+    f.r0 = (int64_t)by * kBM;
+    f.c0 = (int64_t)bx * kBM;
+    f.diag = bx == by;
+    return f;
+}
+
+__global__ void __launch_bounds__(kThreadsT, 1) fit3t_kernel(const __grid_constant__ CUtensorMap tm, const FParams p) {
     constexpr int BN = 128;
     using C = FCfg;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t* raw0 = smem + (size_t)C::kStages * C::kStageBytes;
     uint64_t* bars = (uint64_t*)(smem + C::kBarOff);
-    uint64_t* full = bars;                          // count 4 (producer warps)
+    uint64_t* ready = bars;                         // operands split (8 warps)
     uint64_t* empty = bars + C::kStages;            // count 1 (MMA commit)
     uint64_t* raw_full = empty + C::kStages;        // count 1 + TMA bytes
-    uint64_t* raw_empty = raw_full + C::kRawStages; // count 4 (producer warps)
-    uint64_t* acc_full = raw_empty + C::kRawStages; // count 1 (MMA commit): a group is in accumulator a
-    uint64_t* acc_empty = acc_full + C::kAcc;       // count 4 (epilogue warps): accumulator a drained
-    uint64_t* mma_done = acc_empty + C::kAcc;
+    uint64_t* raw_empty = raw_full + C::kRawStages; // raw chunk read (8 warps)
+    uint64_t* acc_full = raw_empty + C::kRawStages; // [2] a group is accumulated (MMA commit)
+    uint64_t* acc_empty = acc_full + 2;             // [2] drained (8 warps)
+    uint64_t* mma_done = acc_empty + 2;
     uint32_t* tmem_slot = (uint32_t*)(mma_done + 1);
     volatile int* abort = (volatile int*)(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::kStages; ++s) {
-            mbar_init(smem_u32(&full[s]), 4);
+            mbar_init(smem_u32(&ready[s]), 8);
             mbar_init(smem_u32(&empty[s]), 1);
         }
         for (int r = 0; r < C::kRawStages; ++r) {
             mbar_init(smem_u32(&raw_full[r]), 1);
-            mbar_init(smem_u32(&raw_empty[r]), 4);
+            mbar_init(smem_u32(&raw_empty[r]), 8);
         }
-        for (int a = 0; a < C::kAcc; ++a) {
-            mbar_init(smem_u32(&acc_full[a]), 1);
-            mbar_init(smem_u32(&acc_empty[a]), 4);
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(smem_u32(&acc_full[b]), 1);
+            mbar_init(smem_u32(&acc_empty[b]), 8);
         }
         mbar_init(smem_u32(mma_done), 1);
         *abort = 0;
         fence_mbar_init();
     }
-    if (warp == 4) {
-        tmem_alloc(smem_u32(tmem_slot), C::kTmemCols);
+    if (warp == 16) {
+        tmem_alloc(smem_u32(tmem_slot), 512);
         tmem_relinquish();
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-
-    const int layer = blockIdx.x / p.tiles;
-    const int t = blockIdx.x - layer * p.tiles;
-    int by = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);  // lower-tile index -> (by, bx), bx <= by
-    while ((by + 1) * (by + 2) / 2 <= t) ++by;
-    while (by * (by + 1) / 2 > t) --by;
-    const int bx = t - by * (by + 1) / 2;
-    const bool diag = bx == by;
-    const int64_t a0 = (int64_t)by * kBM, b0 = (int64_t)bx * BN;
     const int64_t nkc = (p.n + kKC - 1) / kKC;
 
-    if (warp < 4) {
-        // ---------------- split warps: raw chunk (transposed reads) -> hi/lo operand stage
-        const int pt = threadIdx.x;
-        float4 va[8], vb[8];
-        for (int64_t kc = 0; kc < nkc; ++kc) {
-            const int r = (int)(kc % C::kRawStages), s = (int)(kc % C::kStages);
-            const uint32_t rph = (uint32_t)(kc / C::kRawStages) & 1u, ph = (uint32_t)(kc / C::kStages) & 1u;
-            bool got = true;
-            if (lane == 0) got = wait_bounded(smem_u32(&raw_full[r]), rph, abort, p.err);
-            got = __shfl_sync(0xffffffffu, got, 0);
-            __syncwarp();
-            if (!got) break;
-            const uint8_t* raw = raw0 + (size_t)r * C::kRawBytes;
-            load_raw_t(raw, va, pt);
-            if (!diag) load_raw_t(raw + C::kABytes, vb, pt);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&raw_empty[r]));
-            if (lane == 0) got = wait_bounded(smem_u32(&empty[s]), ph ^ 1u, abort, p.err);
-            got = __shfl_sync(0xffffffffu, got, 0);
-            __syncwarp();
-            if (!got) break;
-            uint8_t* st = smem + (size_t)s * C::kStageBytes;
-            store_split_t<kBM>(va, st, st + C::kABytes, pt);
-            if (!diag) store_split_t<BN>(vb, st + 2 * C::kABytes, st + 3 * C::kABytes, pt);
-            fence_proxy_async();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&full[s]));
+    if (warp < 8) {
+        // ---------------- split warps: raw chunk -> A in TMEM (0-3), B hi/lo in shared memory (4-7)
+        uint32_t it = 0;
+        bool ok = true;
+        for (int u = blockIdx.x; ok && u < p.total; u += gridDim.x) {
+            const bool diag = fit_tile(p, u).diag;
+            for (int64_t kc = 0; kc < nkc; ++kc, ++it) {
+                const uint32_t r = it % C::kRawStages, rph = (it / C::kRawStages) & 1u;
+                const uint32_t s = it % C::kStages, ph = (it / C::kStages) & 1u;
+                bool got = true;
+                if (lane == 0) got = wait_bounded(smem_u32(&raw_full[r]), rph, abort, p.err);
+                got = __shfl_sync(0xffffffffu, got, 0);
+                if (!got) {
+                    ok = false;
+                    break;
+                }
+                const uint8_t* raw = raw0 + (size_t)r * C::kRawBytes;
+                if (warp < 4) {
+                    const uint8_t* box = raw + (uint32_t)warp * 4096u + (lane & 3) * 4;
+                    uint32_t x[32];
+#pragma unroll
+                    for (int e = 0; e < 32; ++e)
+                        x[e] = *reinterpret_cast<const uint32_t*>(box + e * kRowBytes + (((lane >> 2) ^ (e & 7)) << 4));
+                    __syncwarp();
+                    if (lane == 0) {
+                        mbar_arrive(smem_u32(&raw_empty[r]));
+                        got = wait_bounded(smem_u32(&empty[s]), ph ^ 1u, abort, p.err);
+                    }
+                    got = __shfl_sync(0xffffffffu, got, 0);
+                    if (!got) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    const uint32_t dst = tmem + ((uint32_t)(warp * 32) << 16) + C::kAOff + s * 64u;
+                    tmem_st16(dst, x);
+                    tmem_st16(dst + 16, x + 16);
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) {
+                        float h, l;
+                        split_tf32(__uint_as_float(x[e]), h, l);
+                        x[e] = __float_as_uint(l);
+                    }
+                    tmem_st16(dst + 32, x);
+                    tmem_st16(dst + 48, x + 16);
+                    tmem_wait_st();
+                    tc_fence_before();
+                } else {
+                    const int pt = threadIdx.x - 128;
+                    float4 v[8];
+                    load_raw_t(raw + (diag ? 0u : C::kABytes), v, pt);
+                    __syncwarp();
+                    if (lane == 0) {
+                        mbar_arrive(smem_u32(&raw_empty[r]));
+                        got = wait_bounded(smem_u32(&empty[s]), ph ^ 1u, abort, p.err);
+                    }
+                    got = __shfl_sync(0xffffffffu, got, 0);
+                    if (!got) {
+                        ok = false;
+                        break;
+                    }
+                    uint8_t* st = smem + (size_t)s * C::kStageBytes;
+                    store_split_t<BN>(v, st, st + C::kABytes, pt);
+                    fence_proxy_async();
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&ready[s]));
+            }
         }
-    } else if (warp == 9) {
+    } else if (warp < 16) {
+        // ---------------- epilogue: groups -> registers -> M (lane: column of M, register: row)
+        const int q4 = warp & 3, half = (warp - 8) >> 2, row = q4 * 32 + lane;
+        const uint32_t tbase = tmem + ((uint32_t)(q4 * 32) << 16) + half * 64;
+        const uint32_t groups = (uint32_t)((nkc + C::kGroup - 1) / C::kGroup);
+        uint32_t cnt = 0;
+        bool got = true;
+        for (int u = blockIdx.x; got && u < p.total; u += gridDim.x) {
+            const FTile f = fit_tile(p, u);
+            float acc[64];
+#pragma unroll
+            for (int c = 0; c < 64; ++c) acc[c] = 0.f;
+            for (uint32_t g = 0; g < groups; ++g, ++cnt) {
+                const uint32_t b = cnt & 1u;
+                if (lane == 0) got = wait_bounded(smem_u32(&acc_full[b]), (cnt >> 1) & 1u, abort, p.err);
+                got = __shfl_sync(0xffffffffu, got, 0);
+                if (!got) break;
+                tc_fence_after();
+#pragma unroll
+                for (int c0 = 0; c0 < 64; c0 += 16) {
+                    float v[16];
+                    tmem_ld16(tbase + b * BN + c0, v);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) acc[c0 + i] += v[i];
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&acc_empty[b]));
+            }
+            const int64_t c = f.c0 + row, r0 = f.r0 + half * 64;
+            if (!got || c >= p.D) continue;
+            float* M = (float*)(p.state + (size_t)f.layer * p.bytes + 64) + c;
+            const int lim = (int)(p.D - r0 < 64 ? p.D - r0 : 64);
+#pragma unroll
+            for (int c0 = 0; c0 < 64; c0 += 8) {
+                float old[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) old[i] = c0 + i < lim ? M[(r0 + c0 + i) * p.D] : 0.f;
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (c0 + i < lim) M[(r0 + c0 + i) * p.D] = old[i] + acc[c0 + i];
+            }
+        }
+    } else if (warp == 17) {
         if (lane == 0) {
-            // ---------------- TMA producer: raw chunks of 32 examples, features a0.. (and b0..)
-            const int xa = (int)(layer * p.D + a0), xb = (int)(layer * p.D + b0);
-            const uint32_t bytes = diag ? C::kABytes : C::kRawBytes;
-            uint32_t last_par[C::kRawStages];
-            bool issued[C::kRawStages];
+            // ---------------- TMA producer: raw chunks of 32 examples, A: features c0.., B: r0..
+            uint32_t it = 0, last_par[C::kRawStages];
+            bool issued[C::kRawStages], ok = true;
             for (int r = 0; r < C::kRawStages; ++r) issued[r] = false;
-            for (int64_t kc = 0; kc < nkc; ++kc) {
-                const int r = (int)(kc % C::kRawStages);
-                const uint32_t rph = (uint32_t)(kc / C::kRawStages) & 1u;
-                if (!wait_bounded(smem_u32(&raw_empty[r]), rph ^ 1u, abort, p.err)) break;
-                const uint32_t dst = smem_u32(raw0 + (size_t)r * C::kRawBytes), bar = smem_u32(&raw_full[r]);
-                const int y = (int)(kc * kKC);
-                mbar_arrive_tx(bar, bytes);
+            for (int u = blockIdx.x; ok && u < p.total; u += gridDim.x) {
+                const FTile f = fit_tile(p, u);
+                const int xa = (int)(f.layer * p.D + f.c0), xb = (int)(f.layer * p.D + f.r0);
+                const uint32_t bytes = f.diag ? C::kABytes : C::kRawBytes;
+                for (int64_t kc = 0; kc < nkc; ++kc, ++it) {
+                    const uint32_t r = it % C::kRawStages, rph = (it / C::kRawStages) & 1u;
+                    if (!wait_bounded(smem_u32(&raw_empty[r]), rph ^ 1u, abort, p.err)) {
+                        ok = false;
+                        break;
+                    }
+                    const uint32_t dst = smem_u32(raw0 + (size_t)r * C::kRawBytes), bar = smem_u32(&raw_full[r]);
+                    const int y = (int)(kc * kKC);
+                    mbar_arrive_tx(bar, bytes);
 #pragma unroll
-                for (int b = 0; b < 4; ++b) tma_load_2d(dst + (uint32_t)b * 4096u, &tm, xa + 32 * b, y, bar);
-                if (!diag)
+                    for (int b = 0; b < 4; ++b) tma_load_2d(dst + (uint32_t)b * 4096u, &tm, xa + 32 * b, y, bar);
+                    if (!f.diag)
 #pragma unroll
-                    for (int b = 0; b < 4; ++b)
-                        tma_load_2d(dst + C::kABytes + (uint32_t)b * 4096u, &tm, xb + 32 * b, y, bar);
-                issued[r] = true;
-                last_par[r] = rph;
+                        for (int b = 0; b < 4; ++b)
+                            tma_load_2d(dst + C::kABytes + (uint32_t)b * 4096u, &tm, xb + 32 * b, y, bar);
+                    issued[r] = true;
+                    last_par[r] = rph;
+                }
             }
             // copies still in flight when the consumers stopped early land before the CTA exits
             for (int r = 0; r < C::kRawStages; ++r)
@@ -873,111 +975,50 @@ __global__ void __launch_bounds__(kFitThreads, 1) fit3x_kernel(const __grid_cons
                         }
                 }
         }
-    } else if (warp == 8) {
-        if (lane == 0) {
-            // ---------------- MMA issuer
-            const uint32_t idesc = idesc_tf32(kBM, BN);
-            for (int64_t kc = 0; kc < nkc; ++kc) {
-                const int s = (int)(kc % C::kStages);
-                const uint32_t ph = (uint32_t)(kc / C::kStages) & 1u;
-                const int64_t g = kc / C::kGroup;  // group g goes to accumulator g % kAcc, its use g / kAcc
-                const int a = (int)(g % C::kAcc);
-                const bool start = kc % C::kGroup == 0;
-                if (start && g >= C::kAcc &&
-                    !wait_bounded(smem_u32(&acc_empty[a]), (uint32_t)((g / C::kAcc) - 1) & 1u, abort, p.err))
+    } else if (lane == 0) {
+        // ---------------- MMA issuer
+        constexpr uint32_t idesc = idesc_tf32(kBM, BN);
+        uint32_t it = 0, cnt = 0;
+        bool ok = true;
+        for (int u = blockIdx.x; ok && u < p.total; u += gridDim.x)
+            for (int64_t kc = 0; kc < nkc; ++kc, ++it) {
+                const uint32_t s = it % C::kStages, ph = (it / C::kStages) & 1u, b = cnt & 1u;
+                const bool start = kc % C::kGroup == 0, last = kc % C::kGroup == C::kGroup - 1 || kc == nkc - 1;
+                if ((start && !wait_bounded(smem_u32(&acc_empty[b]), ((cnt >> 1) & 1u) ^ 1u, abort, p.err)) ||
+                    !wait_bounded(smem_u32(&ready[s]), ph, abort, p.err)) {
+                    ok = false;
                     break;
-                if (!wait_bounded(smem_u32(&full[s]), ph, abort, p.err)) break;
+                }
                 tc_fence_after();
                 const uint32_t st = smem_u32(smem + (size_t)s * C::kStageBytes);
-                const uint64_t ahi = sw128_desc(st), alo = sw128_desc(st + C::kABytes);
-                const uint64_t bhi = diag ? ahi : sw128_desc(st + 2 * C::kABytes);
-                const uint64_t blo = diag ? alo : sw128_desc(st + 3 * C::kABytes);
-                const uint32_t d = tmem + (uint32_t)a * BN;
+                const uint32_t ahi = tmem + C::kAOff + s * 64u, alo = ahi + 32u, d = tmem + b * BN;
+                const uint64_t bhi = sw128_desc(st), blo = sw128_desc(st + C::kABytes);
 #pragma unroll
                 for (int k = 0; k < kKC / 8; ++k) {
-                    mma_tf32(d, ahi + 2 * k, bhi + 2 * k, idesc, (start && k == 0) ? 0u : 1u);
-                    mma_tf32(d, ahi + 2 * k, blo + 2 * k, idesc, 1u);
-                    mma_tf32(d, alo + 2 * k, bhi + 2 * k, idesc, 1u);
+                    mma_tf32_ta(d, ahi + 8 * k, bhi + 2 * k, idesc, start && k == 0 ? 0u : 1u);
+                    mma_tf32_ta(d, ahi + 8 * k, blo + 2 * k, idesc, 1u);
+                    mma_tf32_ta(d, alo + 8 * k, bhi + 2 * k, idesc, 1u);
                 }
                 mma_commit(smem_u32(&empty[s]));
-                if (kc % C::kGroup == C::kGroup - 1 || kc == nkc - 1) mma_commit(smem_u32(&acc_full[a]));
-            }
-            mma_commit(smem_u32(mma_done));
-            const uint64_t t0 = global_ns();
-            while (!mbar_try_wait(smem_u32(mma_done), 0))
-                if (global_ns() - t0 > kTimeoutNs) {
-                    atomicOr(p.err, kErrTimeout);
-                    break;
+                if (last) {
+                    mma_commit(smem_u32(&acc_full[b]));
+                    ++cnt;
                 }
-        }
-    } else {
-        // ---------------- epilogue (warps 4-7): drain each group's accumulator into fp32
-        // registers (one row of the tile per thread), then M += the sum
-        const int q = warp & 3;
-        const int row = q * 32 + lane;
-        const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16);
-        const int64_t ngroups = (nkc + C::kGroup - 1) / C::kGroup;
-        float acc[BN];
-#pragma unroll
-        for (int c = 0; c < BN; ++c) acc[c] = 0.f;
-        bool ok = true;
-        for (int64_t g = 0; g < ngroups; ++g) {
-            const int a = (int)(g % C::kAcc);
-            bool got = true;
-            if (lane == 0) got = wait_bounded(smem_u32(&acc_full[a]), (uint32_t)(g / C::kAcc) & 1u, abort, p.err);
-            got = __shfl_sync(0xffffffffu, got, 0);
-            if (!got) {
-                ok = false;
+            }
+        mma_commit(smem_u32(mma_done));
+        const uint64_t t0 = global_ns();
+        while (!mbar_try_wait(smem_u32(mma_done), 0))
+            if (global_ns() - t0 > kTimeoutNs) {
+                atomicOr(p.err, kErrTimeout);
                 break;
             }
-            tc_fence_after();
-#pragma unroll
-            for (int c0 = 0; c0 < BN; c0 += 16) {
-                float v[16];
-                tmem_ld16(tbase + (uint32_t)(a * BN + c0), v);
-#pragma unroll
-                for (int i = 0; i < 16; ++i) acc[c0 + i] += v[i];
-            }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&acc_empty[a]));
-        }
-        // the tile's sums to shared memory (the operand stages are free once the last group
-        // has landed: every stage was consumed by its MMAs), row stride 129: conflict-free
-        if (ok) {
-            float* stg = (float*)smem;
-#pragma unroll
-            for (int c = 0; c < BN; ++c) stg[row * (BN + 1) + c] = acc[c];
-        }
     }
+
     tc_fence_before();
     __syncthreads();
-    if (!*abort) {
-        // M += tile, coalesced: warp w takes rows 4j..4j+3 for j = w, w + 10, ..., lane the
-        // columns lane + 32i; all 16 old values of a batch are loaded before any store
-        const float* stg = (const float*)smem;
-        float* M = (float*)(p.state + (size_t)layer * p.bytes + 64);
-        for (int j = warp; j < kBM / 4; j += kFitThreads / 32) {
-            float old[4][BN / 32];
-#pragma unroll
-            for (int r = 0; r < 4; ++r)
-#pragma unroll
-                for (int i = 0; i < BN / 32; ++i) {
-                    const int64_t a = a0 + 4 * j + r, b = b0 + lane + 32 * i;
-                    old[r][i] = (a < p.D && b < p.D) ? M[a * p.D + b] : 0.f;
-                }
-#pragma unroll
-            for (int r = 0; r < 4; ++r)
-#pragma unroll
-                for (int i = 0; i < BN / 32; ++i) {
-                    const int64_t a = a0 + 4 * j + r, b = b0 + lane + 32 * i;
-                    if (a < p.D && b < p.D) M[a * p.D + b] = old[r][i] + stg[(4 * j + r) * (BN + 1) + lane + 32 * i];
-                }
-        }
-    }
-    if (warp == 4) {
+    if (warp == 16) {
         tc_fence_after();
-        tmem_dealloc(tmem, C::kTmemCols);
+        tmem_dealloc(tmem, 512);
     }
 }
 
@@ -1251,11 +1292,20 @@ cudaError_t launch_fit_tc(int n_layers, int64_t D, void* state, size_t state_byt
     p.D = D;
     p.n = n;
     p.tiles = (int)(nt * (nt + 1) / 2);
+    p.total = p.tiles * n_layers;
     p.err = err;
-    cudaError_t e = smem_attr_once<fit3x_kernel>((int)C::kSmem);
+    static std::atomic<int> sms_cache{0};
+    int sms = sms_cache.load(std::memory_order_relaxed);
+    if (!sms) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 1;
+        sms_cache.store(sms, std::memory_order_relaxed);
+    }
+    cudaError_t e = smem_attr_once<fit3t_kernel>((int)C::kSmem);
     if (e != cudaSuccess) return e;
     note_launches(1);
-    fit3x_kernel<<<(unsigned)(p.tiles * n_layers), kFitThreads, C::kSmem, s>>>(tm, p);
+    fit3t_kernel<<<(unsigned)(p.total < sms ? p.total : sms), kThreadsT, C::kSmem, s>>>(tm, p);
     return cudaGetLastError();
 }
 
