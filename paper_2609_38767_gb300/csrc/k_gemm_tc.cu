@@ -376,48 +376,108 @@ score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 }
 
 // ---------------------------------------------------------------------------
-// The same product without clusters, with the A operand in TMEM: one persistent CTA per SM walks
-// the tiles of all batch entries and feature slices.
+// The same product without a split of K, and the Fisher fit, with the A operand in TMEM: persistent
+// CTAs, one per SM, walk the tiles of all batch entries and feature slices. With PAIR the two CTAs
+// of a cluster share a tile of 256 rows of A x BN rows of B (cta_group::2): each has its own 128
+// rows of A and of the accumulators, and half of B.
 //
-// What bounds a 128 x 128 tile of three TF32 products per element pair is shared memory. With both
-// operands there, a 32-feature chunk (768 clocks of MMAs) costs 768 clocks of operand reads, 256 of
-// TMA writes and 512 of splitting at 128 bytes a clock. Here four warps read the rows of Phi once
-// (a thread per row: the 128-byte swizzle makes its 16-byte loads conflict-free) and put hi (the
-// fp32 value as it is: a kind::tf32 MMA reads its upper 19 bits) and lo into TMEM, a column per
-// feature, so only B's hi and lo are read by the MMAs: 1024 clocks.
+// What bounds a tile: three TF32 products of 32 features take 768 clocks (BN = 128). At 128 bytes a
+// clock, shared memory with both operands there takes 1536 (768 of operand reads, 256 of TMA
+// writes, 512 of splitting), with A in TMEM and one CTA 1152, and a pair needs 700. The rest is
+// latency, a chain of waits per chunk in every role. One lane polling and then a shuffle took about
+// 250 clocks a wait, and MMAs issued behind `lane == 0` about 80 clocks each (1000 a chunk, the
+// bound of the whole kernel), so whole warps poll and an elected lane issues. A chunk now takes
+// 980 clocks (scores) to 1040 (fit), one CTA a tile 1290 and 1080.
 //
-// Accuracy: groups of kGroup chunks (24 truncating additions) alternate between two accumulators,
-// and eight epilogue warps (two per TMEM lane quadrant, half of the columns each) add every
-// finished group into round-to-nearest registers beside the next group's MMAs, then write the
-// tile beside the next tile's.
+// FIT: M_l += Phi_l^T Phi_l, lower triangle, layer l's features at column l*D of each row of Phi.
+// The operands are features x examples, K-major, but Phi holds examples x features, so a chunk
+// is 32 examples in boxes of 32 features (128-byte swizzle). A: a lane per feature, 32 lanes on one
+// 128-byte row. B: a lane per example, 16 bytes of features a load, 4-byte stores of 32 lanes into
+// one row of the operand. All of these are free of bank conflicts. A's rows are columns of
+// M, so that a warp's 32 lanes are 32 neighbouring entries of a row of M.
 //
-// Measured: scores of 256 x 8192, 7168 features: 205 us with both operands in shared memory and
-// one pass over the accumulators (1.3e-5 off), 188 us and 9e-7 off here.
+// A's hi is the fp32 value as it is (a kind::tf32 MMA reads its upper 19 bits).
 //
-// Warps: 0-3 A into TMEM, 4-7 B's lo, 8-15 epilogue, 16 MMA issuer, 17 TMA. All waits are bounded.
+// Accuracy: the tensor pipe's fp32 accumulation rounds toward zero, so a long same-sign sum (a
+// diagonal entry of M) drifts low by up to an ulp per accumulate. Groups of kGroup chunks (24
+// accumulates) alternate between two accumulators, and eight epilogue warps (two per TMEM lane
+// quadrant, half of the columns each) add every finished group into round-to-nearest registers
+// beside the next group's MMAs, then write the tile beside the next tile's.
+//
+// Measured: scores of 256 x 8192, 7168 features: 205 us with both operands in shared memory and one
+// pass over the accumulators (1.3e-5 off), 188 us with A in TMEM (9e-7 off), 114 us in pairs.
+// Fit of seven layers of D = 4096, 8192 examples: 6.74 ms, 6.24 ms, 3.61 ms.
+//
+// Warps: 0-3 A into TMEM, 4-7 B's hi and lo into the operand slots, 8-15 epilogue, 16 MMA issuer (of
+// the pair: in CTA 0), 17 TMA. Every wait is bounded.
 constexpr int kThreadsT = 18 * 32;
 
-template <int BN>
+template <int BN, bool PAIR>
 struct TCfg {
+    static constexpr int kCtas = PAIR ? 2 : 1;
+    static constexpr int kBRows = BN / kCtas;             // rows of B in this CTA
     static constexpr uint32_t kABytes = kBM * kRowBytes;  // 16 KiB
-    static constexpr uint32_t kBBytes = BN * kRowBytes;
-    static constexpr uint32_t kStageBytes = kABytes + 2 * kBBytes;  // A raw; B raw (hi) and lo
-    static constexpr int kStages = 4;                     // also TMEM slots of A
+    static constexpr uint32_t kBBytes = kBRows * kRowBytes;
+    static constexpr uint32_t kRawBytes = kABytes + kBBytes;
+    static constexpr int kRaw = PAIR ? 6 : 4;             // raw chunks
+    static constexpr int kSlots = PAIR ? 4 : 3;           // A in TMEM, B's hi and lo in shared memory
+    static constexpr uint32_t kSlotBytes = 2 * kBBytes;
     static constexpr int kGroup = 2;
     static constexpr int kCols = BN / 2;                  // columns per epilogue thread
-    static constexpr int kAOff = 2 * BN;                  // first TMEM column of A: [stage][hi 32 | lo 32]
-    static constexpr size_t kSmem = 1024 + (size_t)kStages * kStageBytes + 8 * (3 * kStages + 5) + 16;
-    static_assert(kAOff + kStages * 64 <= 512 && kSmem <= 232448, "TMEM columns, shared memory");
+    static constexpr int kAOff = 2 * BN;                  // first TMEM column of A: [slot][hi 32 | lo 32]
+    static constexpr size_t kBarOff = (size_t)kRaw * kRawBytes + (size_t)kSlots * kSlotBytes;
+    static constexpr size_t kSmem = 1024 + kBarOff + 8 * (2 * kRaw + 2 * kSlots + 5) + 16;
+    static_assert(kAOff + kSlots * 64 <= 512 && kSmem <= 232448, "TMEM columns, shared memory");
 };
 
 // D[tmem] (+)= A[tmem] * B[smem]^T, tf32 inputs.
+template <bool PAIR>
 __device__ __forceinline__ void mma_tf32_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
                                             uint32_t accumulate) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}" ::"r"(
-            d_tmem),
-        "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
+    if constexpr (PAIR)
+        asm volatile(
+            "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::2.kind::tf32 [%0], [%1], %2, %3, p;\n}" ::"r"(
+                d_tmem),
+            "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
+            : "memory");
+    else
+        asm volatile(
+            "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}" ::"r"(
+                d_tmem),
+            "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
+            : "memory");
+}
+// Arrives on `bar` of every CTA of the tile once the MMAs issued so far are done.
+template <bool PAIR>
+__device__ __forceinline__ void commit_all(uint32_t bar) {
+    if constexpr (PAIR)
+        asm volatile(
+            "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+            "h"((uint16_t)3)
+            : "memory");
+    else
+        mma_commit(bar);
+}
+__device__ __forceinline__ void commit_pair_local(uint32_t bar) {
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void tmem_alloc2(uint32_t dst, uint32_t ncols) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst), "r"(ncols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_dealloc2(uint32_t taddr, uint32_t ncols) {
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+}
+// Arrives on CTA 0's `bar` of the tile. The operands that it announces are ordered by tcgen05.wait::st and
+// fence.proxy.async; a release at cluster scope would wait for all of the warp's writes (1100
+// clocks).
+template <bool PAIR>
+__device__ __forceinline__ void arrive_leader(uint32_t bar) {
+    if constexpr (PAIR)
+        asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(map_rank(bar, 0u)) : "memory");
+    else
+        mbar_arrive(bar);
 }
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
     asm volatile(
@@ -429,29 +489,38 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-// Tile t: rows m0 (of A) and n0 (of B), batch entry z, feature slice y.
+// Tile t: first rows m0 (of A, this CTA's) and n0 (of B), batch entry z, feature slice y.
 struct TileAt {
     int64_t m0, n0;
     int z, y;
 };
-template <int BN>
-__device__ __forceinline__ TileAt tile_at(const GParams& p, int64_t t) {
+template <int BN, bool PAIR>
+__device__ __forceinline__ TileAt tile_at(const GParams& p, int64_t t, uint32_t rank) {
     TileAt a;
     const int64_t per_z = p.tiles_z * p.splits;
     a.z = (int)(t / per_z);
     t -= (int64_t)a.z * per_z;
     a.y = (int)(t / p.tiles_z);
     const int64_t tile = t - (int64_t)a.y * p.tiles_z;
-    if (p.lower) {
-        int64_t i = (int64_t)((sqrtf(8.f * (float)tile + 1.f) - 1.f) * 0.5f);  // fp64 is a slow pipe here
+    if (p.lower && PAIR) {
+        // row tiles 2q and 2q + 1 of B have q + 1 tiles of A each
+        int64_t q = (int64_t)(sqrtf((float)tile + 0.25f) - 0.5f);
+        while (q * (q + 1) > tile) --q;
+        while ((q + 1) * (q + 2) <= tile) ++q;
+        const int64_t r = tile - q * (q + 1), odd = r >= q + 1 ? 1 : 0;
+        a.n0 = (2 * q + odd) * BN;
+        a.m0 = (r - odd * (q + 1)) * 2 * kBM;
+    } else if (p.lower) {
+        int64_t i = (int64_t)((sqrtf(8.f * (float)tile + 1.f) - 1.f) * 0.5f);
         while (i * (i + 1) / 2 > tile) --i;
         while ((i + 1) * (i + 2) / 2 <= tile) ++i;
         a.n0 = i * BN;
         a.m0 = (tile - i * (i + 1) / 2) * kBM;
     } else {
-        a.m0 = (tile / p.tiles_n) * kBM;
+        a.m0 = (tile / p.tiles_n) * (PAIR ? 2 * kBM : kBM);
         a.n0 = (tile % p.tiles_n) * BN;
     }
+    a.m0 += rank * kBM;
     return a;
 }
 // 32-feature chunks of slice y
@@ -461,114 +530,179 @@ __device__ __forceinline__ int64_t chunks_of(const GParams& p, int y) {
     return (Kz + kKC - 1) / kKC;
 }
 
-template <int BN>
+template <int BN, bool PAIR, bool FIT>
 __global__ void __launch_bounds__(kThreadsT, 1)
 gemm3t_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GParams p) {
-    using C = TCfg<BN>;
+    using C = TCfg<BN, PAIR>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint64_t* bars = (uint64_t*)(smem + (size_t)C::kStages * C::kStageBytes);
-    uint64_t* raw_full = bars;               // [kStages] TMA bytes landed (count 1 + tx)
-    uint64_t* ready = raw_full + C::kStages; // [kStages] A in TMEM, B's lo written (8 warps)
-    uint64_t* empty = ready + C::kStages;    // [kStages] MMAs done reading (count 1)
-    uint64_t* acc_full = empty + C::kStages; // [2] a group is accumulated (count 1)
-    uint64_t* acc_empty = acc_full + 2;      // [2] the accumulator is drained (8 warps)
+    uint8_t* slots = smem + (size_t)C::kRaw * C::kRawBytes;
+    uint64_t* raw_full = (uint64_t*)(smem + C::kBarOff);  // [kRaw] TMA bytes landed (count 1 + tx)
+    uint64_t* raw_empty = raw_full + C::kRaw;             // [kRaw] chunk read (8 warps)
+    uint64_t* ready = raw_empty + C::kRaw;                // [kSlots] operands written (8 warps a CTA; CTA 0's)
+    uint64_t* empty = ready + C::kSlots;                  // [kSlots] MMAs done reading (count 1)
+    uint64_t* acc_full = empty + C::kSlots;               // [2] a group is accumulated (count 1)
+    uint64_t* acc_empty = acc_full + 2;                   // [2] the accumulator is drained (8 warps a CTA; CTA 0's)
     uint64_t* mma_done = acc_empty + 2;
     uint32_t* tmem_slot = (uint32_t*)(mma_done + 1);
     volatile int* abort = (volatile int*)(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    const uint32_t rank = PAIR ? cluster_rank() : 0u;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < C::kStages; ++s) {
-            mbar_init(smem_u32(&raw_full[s]), 1);
-            mbar_init(smem_u32(&ready[s]), 8);
+        for (int r = 0; r < C::kRaw; ++r) {
+            mbar_init(smem_u32(&raw_full[r]), 1);
+            mbar_init(smem_u32(&raw_empty[r]), 8);
+        }
+        for (int s = 0; s < C::kSlots; ++s) {
+            mbar_init(smem_u32(&ready[s]), 8 * C::kCtas);
             mbar_init(smem_u32(&empty[s]), 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(&acc_full[b]), 1);
-            mbar_init(smem_u32(&acc_empty[b]), 8);
+            mbar_init(smem_u32(&acc_empty[b]), 8 * C::kCtas);
         }
         mbar_init(smem_u32(mma_done), 1);
         *abort = 0;
         fence_mbar_init();
     }
     if (warp == 16) {
-        tmem_alloc(smem_u32(tmem_slot), 512);
-        tmem_relinquish();
+        if constexpr (PAIR) {
+            tmem_alloc2(smem_u32(tmem_slot), 512);
+        } else {
+            tmem_alloc(smem_u32(tmem_slot), 512);
+            tmem_relinquish();
+        }
     }
     tc_fence_before();
     __syncthreads();
+    if constexpr (PAIR) cluster_sync();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     const int64_t total = p.tiles_z * p.splits * p.nz;
+    const int64_t t0 = PAIR ? blockIdx.x >> 1 : blockIdx.x, tstep = PAIR ? gridDim.x >> 1 : gridDim.x;
 
     if (warp < 8) {
-        // ---------------- split warps: 0-3 A's rows into TMEM, 4-7 B's lo into shared memory
+        // ---------------- split warps: 0-3 A's rows into TMEM, 4-7 B's hi and lo into shared memory
         uint32_t it = 0;
         bool ok = true;
-        for (int64_t t = blockIdx.x; ok && t < total; t += gridDim.x) {
-            const int64_t nkc = chunks_of(p, tile_at<BN>(p, t).y);
+        for (int64_t t = t0; ok && t < total; t += tstep) {
+            const int64_t nkc = chunks_of(p, tile_at<BN, PAIR>(p, t, rank).y);
             for (int64_t kc = 0; kc < nkc; ++kc, ++it) {
-                const uint32_t s = it % C::kStages, ph = (it / C::kStages) & 1u;
-                bool got = true;
-                if (lane == 0) got = wait_bounded(smem_u32(&raw_full[s]), ph, abort, p.err);
-                got = __shfl_sync(0xffffffffu, got, 0);
-                if (!got) {
+                const uint32_t r = it % C::kRaw, rph = (it / C::kRaw) & 1u;
+                const uint32_t s = it % C::kSlots, ph = (it / C::kSlots) & 1u;
+                if (!warp_wait(smem_u32(&raw_full[r]), rph, abort, p.err)) {
                     ok = false;
                     break;
                 }
-                uint8_t* st = smem + (size_t)s * C::kStageBytes;
+                const uint8_t* raw = smem + (size_t)r * C::kRawBytes;
+                auto release = [&]() {  // the raw chunk is in registers; wait for the slot
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&raw_empty[r]));
+                    return warp_wait(smem_u32(&empty[s]), ph ^ 1u, abort, p.err);
+                };
                 if (warp < 4) {
-                    // the stage's TMEM slot is free: its MMAs were done before TMA refilled the stage
-                    tc_fence_after();
-                    const int row = warp * 32 + lane;
-                    const uint8_t* src = st + (uint32_t)row * kRowBytes;
-                    const uint32_t dst = tmem + ((uint32_t)(warp * 32) << 16) + C::kAOff + s * 64u;
+                    uint32_t x[32];
+                    if constexpr (FIT) {
+                        const uint8_t* box = raw + (uint32_t)warp * 4096u + (lane & 3) * 4;
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        uint32_t hi[16], lo[16];
+                        for (int e = 0; e < 32; ++e)
+                            x[e] = *reinterpret_cast<const uint32_t*>(box + e * kRowBytes + (((lane >> 2) ^ (e & 7)) << 4));
+                    } else {
+                        const int row = warp * 32 + lane;
+                        const uint8_t* src = raw + (uint32_t)row * kRowBytes;
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            const float4 v =
-                                *reinterpret_cast<const float4*>(src + (((4 * h + c) ^ (row & 7)) << 4));
-                            const float x[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                float hf, lf;
-                                split_tf32(x[i], hf, lf);
-                                hi[4 * c + i] = __float_as_uint(x[i]);
-                                lo[4 * c + i] = __float_as_uint(lf);
-                            }
+                        for (int c = 0; c < 8; ++c) {
+                            const uint4 v = *reinterpret_cast<const uint4*>(src + ((c ^ (row & 7)) << 4));
+                            x[4 * c] = v.x, x[4 * c + 1] = v.y, x[4 * c + 2] = v.z, x[4 * c + 3] = v.w;
                         }
-                        tmem_st16(dst + 16 * h, hi);
-                        tmem_st16(dst + 32 + 16 * h, lo);
                     }
+                    if (!release()) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    const uint32_t dst = tmem + ((uint32_t)(warp * 32) << 16) + C::kAOff + s * 64u;
+                    tmem_st16(dst, x);
+                    tmem_st16(dst + 16, x + 16);
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) {
+                        float h, l;
+                        split_tf32(__uint_as_float(x[e]), h, l);
+                        x[e] = __float_as_uint(l);
+                    }
+                    tmem_st16(dst + 32, x);
+                    tmem_st16(dst + 48, x + 16);
                     tmem_wait_st();
                     tc_fence_before();
                 } else {
-                    split_tile<C::kBBytes>(st + C::kABytes, st + C::kABytes + C::kBBytes, threadIdx.x - 128);
+                    constexpr int kPer = C::kBRows / 16;  // 16-byte groups a thread
+                    const int pt = threadIdx.x - 128, w = warp - 4;
+                    const uint8_t* src = raw + C::kABytes;
+                    float4 v[kPer];
+                    if constexpr (FIT) {
+                        // warp w: features kBRows / 4 * w ..., lane: example
+                        const uint8_t* row = src + (uint32_t)(w * kPer / 8) * 4096u + (uint32_t)lane * kRowBytes;
+#pragma unroll
+                        for (int j = 0; j < kPer; ++j)
+                            v[j] = *reinterpret_cast<const float4*>(row + (((j + w * kPer % 8) ^ (lane & 7)) << 4));
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < kPer; ++j)
+                            v[j] = *reinterpret_cast<const float4*>(src + (uint32_t)(pt + 128 * j) * 16u);
+                    }
+                    if (!release()) {
+                        ok = false;
+                        break;
+                    }
+                    uint8_t* hi = slots + (size_t)s * C::kSlotBytes;
+                    uint8_t* lo = hi + C::kBBytes;
+#pragma unroll
+                    for (int j = 0; j < kPer; ++j) {
+                        const float in[4] = {v[j].x, v[j].y, v[j].z, v[j].w};
+                        float h, l[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) split_tf32(in[i], h, l[i]);
+                        if constexpr (FIT) {
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                const int fr = 4 * (kPer * w + j) + i;  // feature row of the operand
+                                const uint32_t off =
+                                    (uint32_t)fr * kRowBytes + (uint32_t)((((lane >> 2) ^ (fr & 7)) << 4) + (lane & 3) * 4);
+                                *reinterpret_cast<float*>(hi + off) = in[i];
+                                *reinterpret_cast<float*>(lo + off) = l[i];
+                            }
+                        } else {
+                            const uint32_t off = (uint32_t)(pt + 128 * j) * 16u;
+                            *reinterpret_cast<float4*>(hi + off) = v[j];
+                            *reinterpret_cast<float4*>(lo + off) = make_float4(l[0], l[1], l[2], l[3]);
+                        }
+                    }
                     fence_proxy_async();
                 }
                 __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&ready[s]));
+                if (lane == 0) arrive_leader<PAIR>(smem_u32(&ready[s]));
             }
         }
+        if (PAIR && ok && threadIdx.x == 0)
+            // every arrival of the pair's MMAs on this CTA's barriers lands before it exits
+            for (uint32_t k = it > (uint32_t)C::kSlots ? it - C::kSlots : 0u; k < it; ++k)
+                if (!wait_bounded(smem_u32(&empty[k % C::kSlots]), (k / C::kSlots) & 1u, abort, p.err)) break;
     } else if (warp < 16) {
         // ---------------- epilogue: groups -> registers -> S
         const int q4 = warp & 3, half = (warp - 8) >> 2, row = q4 * 32 + lane;
         const uint32_t tbase = tmem + ((uint32_t)(q4 * 32) << 16) + half * C::kCols;
         uint32_t cnt = 0;
         bool got = true;
-        for (int64_t t = blockIdx.x; got && t < total; t += gridDim.x) {
-            const TileAt at = tile_at<BN>(p, t);
+        for (int64_t t = t0; got && t < total; t += tstep) {
+            const TileAt at = tile_at<BN, PAIR>(p, t, rank);
             const uint32_t groups = (uint32_t)((chunks_of(p, at.y) + C::kGroup - 1) / C::kGroup);
             float acc[C::kCols];
 #pragma unroll
             for (int c = 0; c < C::kCols; ++c) acc[c] = 0.f;
             for (uint32_t g = 0; g < groups; ++g, ++cnt) {
                 const uint32_t b = cnt & 1u;
-                if (lane == 0) got = wait_bounded(smem_u32(&acc_full[b]), (cnt >> 1) & 1u, abort, p.err);
-                got = __shfl_sync(0xffffffffu, got, 0);
+                got = warp_wait(smem_u32(&acc_full[b]), (cnt >> 1) & 1u, abort, p.err);
                 if (!got) break;
                 tc_fence_after();
 #pragma unroll
@@ -580,10 +714,11 @@ gemm3t_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                 }
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&acc_empty[b]));
+                if (lane == 0) arrive_leader<PAIR>(smem_u32(&acc_empty[b]));
             }
             const int64_t m = at.m0 + row, nb = at.n0 + half * C::kCols;
-            if (!got || m >= p.n_t) continue;
+            // (the upper half of a pair's tile on the diagonal lies above it)
+            if (!got || m >= p.n_t || (PAIR && p.lower && at.m0 > at.n0)) continue;
             float* Sz = p.S + (int64_t)at.y * p.slab + (int64_t)at.z * p.s_z + m;
             const int lim = (int)(p.n_q - nb < C::kCols ? p.n_q - nb : C::kCols);
             if (p.beta == 0.f) {
@@ -605,420 +740,108 @@ gemm3t_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         }
     } else if (warp == 17 && lane == 0) {
         // ---------------- TMA producer
-        uint32_t it = 0, last_par[C::kStages];
-        bool issued[C::kStages], ok = true;
-        for (int s = 0; s < C::kStages; ++s) issued[s] = false;
-        for (int64_t t = blockIdx.x; ok && t < total; t += gridDim.x) {
-            const TileAt at = tile_at<BN>(p, t);
+        uint32_t it = 0, last_par[C::kRaw];
+        bool issued[C::kRaw], ok = true;
+        for (int r = 0; r < C::kRaw; ++r) issued[r] = false;
+        for (int64_t t = t0; ok && t < total; t += tstep) {
+            const TileAt at = tile_at<BN, PAIR>(p, t, rank);
             const int64_t nkc = chunks_of(p, at.y);
             const int64_t kbase = (int64_t)at.y * p.kslice;
+            const int m0 = (int)at.m0, n0 = (int)at.n0 + (int)rank * C::kBRows;
             for (int64_t kc = 0; kc < nkc; ++kc, ++it) {
-                const uint32_t s = it % C::kStages, ph = (it / C::kStages) & 1u;
-                if (!wait_bounded(smem_u32(&empty[s]), ph ^ 1u, abort, p.err)) {
+                const uint32_t r = it % C::kRaw, ph = (it / C::kRaw) & 1u;
+                if (!wait_bounded(smem_u32(&raw_empty[r]), ph ^ 1u, abort, p.err)) {
                     ok = false;
                     break;
                 }
-                const uint32_t st = smem_u32(smem + (size_t)s * C::kStageBytes), bar = smem_u32(&raw_full[s]);
+                const uint32_t st = smem_u32(smem + (size_t)r * C::kRawBytes), bar = smem_u32(&raw_full[r]);
                 const int k = (int)(kbase + kc * kKC);
-                mbar_arrive_tx(bar, C::kABytes + C::kBBytes);
-                if (p.batched) {
-                    tma_load_3d(st, &tmA, k, (int)at.m0, at.z, bar);
-                    tma_load_3d(st + C::kABytes, &tmB, k, (int)at.n0, at.z, bar);
+                mbar_arrive_tx(bar, C::kRawBytes);
+                if constexpr (FIT) {
+                    const int x = (int)(at.z * p.n_t);
+#pragma unroll
+                    for (int b = 0; b < kBM / 32; ++b) tma_load_2d(st + 4096u * b, &tmA, x + m0 + 32 * b, k, bar);
+#pragma unroll
+                    for (int b = 0; b < C::kBRows / 32; ++b)
+                        tma_load_2d(st + C::kABytes + 4096u * b, &tmA, x + n0 + 32 * b, k, bar);
+                } else if (p.batched) {
+                    tma_load_3d(st, &tmA, k, m0, at.z, bar);
+                    tma_load_3d(st + C::kABytes, &tmB, k, n0, at.z, bar);
                 } else {
-                    tma_load_2d(st, &tmA, k, (int)at.m0, bar);
-                    tma_load_2d(st + C::kABytes, &tmB, k, (int)at.n0, bar);
+                    tma_load_2d(st, &tmA, k, m0, bar);
+                    tma_load_2d(st + C::kABytes, &tmB, k, n0, bar);
                 }
-                issued[s] = true;
-                last_par[s] = ph;
+                issued[r] = true;
+                last_par[r] = ph;
             }
         }
-        for (int s = 0; s < C::kStages; ++s)
-            if (issued[s]) {
-                const uint64_t t0 = global_ns();
-                while (!mbar_try_wait(smem_u32(&raw_full[s]), last_par[s]))
-                    if (global_ns() - t0 > kTimeoutNs) {
+        // copies still in flight when the consumers stopped early land before the CTA exits
+        for (int r = 0; r < C::kRaw; ++r)
+            if (issued[r]) {
+                const uint64_t ns = global_ns();
+                while (!mbar_try_wait(smem_u32(&raw_full[r]), last_par[r]))
+                    if (global_ns() - ns > kTimeoutNs) {
                         atomicOr(p.err, kErrTimeout);
                         break;
                     }
             }
-    } else if (warp == 16 && lane == 0) {
-        // ---------------- MMA issuer
-        constexpr uint32_t idesc = idesc_tf32(kBM, BN);
+    } else if (warp == 16 && rank == 0) {
+        // ---------------- MMA issuer: the warp waits, one lane issues
+        constexpr uint32_t idesc = idesc_tf32(kBM * C::kCtas, BN);
         uint32_t it = 0, cnt = 0;
         bool ok = true;
-        for (int64_t t = blockIdx.x; ok && t < total; t += gridDim.x) {
-            const int64_t nkc = chunks_of(p, tile_at<BN>(p, t).y);
-            for (int64_t kc = 0; kc < nkc; ++kc, ++it) {
-                const uint32_t s = it % C::kStages, ph = (it / C::kStages) & 1u, b = cnt & 1u;
+        for (int64_t t = t0; ok && t < total; t += tstep) {
+            const int nkc = (int)chunks_of(p, tile_at<BN, PAIR>(p, t, rank).y);
+            for (int kc = 0; kc < nkc; ++kc, ++it) {
+                const uint32_t s = it % C::kSlots, ph = (it / C::kSlots) & 1u, b = cnt & 1u;
                 const bool start = kc % C::kGroup == 0, last = kc % C::kGroup == C::kGroup - 1 || kc == nkc - 1;
-                if ((start && !wait_bounded(smem_u32(&acc_empty[b]), ((cnt >> 1) & 1u) ^ 1u, abort, p.err)) ||
-                    !wait_bounded(smem_u32(&ready[s]), ph, abort, p.err)) {
+                if ((start && !warp_wait(smem_u32(&acc_empty[b]), ((cnt >> 1) & 1u) ^ 1u, abort, p.err)) ||
+                    !warp_wait(smem_u32(&ready[s]), ph, abort, p.err)) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
-                const uint32_t st = smem_u32(smem + (size_t)s * C::kStageBytes);
+                const uint32_t st = smem_u32(slots + (size_t)s * C::kSlotBytes);
                 const uint32_t ahi = tmem + C::kAOff + s * 64u, alo = ahi + 32u, d = tmem + b * BN;
-                const uint64_t bhi = sw128_desc(st + C::kABytes), blo = sw128_desc(st + C::kABytes + C::kBBytes);
+                const uint64_t bhi = sw128_desc(st), blo = sw128_desc(st + C::kBBytes);
+                if (elect_one()) {
 #pragma unroll
-                for (int k = 0; k < kKC / 8; ++k) {  // K = 8 tf32: 8 TMEM columns, 32 bytes of shared memory
-                    mma_tf32_ta(d, ahi + 8 * k, bhi + 2 * k, idesc, start && k == 0 ? 0u : 1u);
-                    mma_tf32_ta(d, ahi + 8 * k, blo + 2 * k, idesc, 1u);
-                    mma_tf32_ta(d, alo + 8 * k, bhi + 2 * k, idesc, 1u);
-                }
-                mma_commit(smem_u32(&empty[s]));
-                if (last) {
-                    mma_commit(smem_u32(&acc_full[b]));
-                    ++cnt;
-                }
-            }
-        }
-        mma_commit(smem_u32(mma_done));
-        const uint64_t t0 = global_ns();
-        while (!mbar_try_wait(smem_u32(mma_done), 0))
-            if (global_ns() - t0 > kTimeoutNs) {
-                atomicOr(p.err, kErrTimeout);
-                break;
-            }
-    }
-
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 16) {
-        tc_fence_after();
-        tmem_dealloc(tmem, 512);
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Fisher fit on the tensor cores: M_l += Phi_l^T Phi_l for the lower 128 x 128
-// tiles of every layer l (layer l's features at column l*D of each row of Phi).
-// The MMA operands are features x examples, K-major (32 examples per chunk), but
-// Phi holds examples x features. Lane 0 of warp 17 copies each chunk raw with TMA
-// (32 examples x 32 features per box, 128-byte swizzle, 4 boxes per operand) into
-// a ring of raw stages. As in gemm3t_kernel the A operand goes to TMEM: warps 0-3
-// read the boxes with a lane per feature (32 lanes on one 128-byte row:
-// conflict-free), which is the TMEM lane, and write the 32 examples' hi and lo.
-// Warps 4-7 read B transposed (lane = example, 16 bytes of features per load:
-// conflict-free thanks to the swizzle), split every value to hi/lo and write both
-// into the K-major swizzled operand layout (conflict-free: the 32 lanes hit 32
-// distinct banks). A tile on the diagonal has A = B and loads one operand.
-// Shared memory bounds it: 1152 of a chunk's clocks at 128 bytes each, 1792 with
-// both operands there (seven layers of D = 4096, 8192 examples: 6.74 ms, 6.24 ms here).
-// A's features are the tile's columns of M, so that a warp's 32 lanes are 32
-// neighbouring entries of a row of M.
-template <int ROWS>
-__device__ __forceinline__ void store_split_t(const float4 (&vals)[ROWS / 16], uint8_t* hi, uint8_t* lo, int pt) {
-    constexpr int kPer = ROWS / 16;
-    const int lane = pt & 31, w = pt >> 5;
-#pragma unroll
-    for (int j = 0; j < kPer; ++j) {
-        const float in[4] = {vals[j].x, vals[j].y, vals[j].z, vals[j].w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int fr = (ROWS / 4) * w + 4 * j + i;  // feature row of the tile
-            const uint32_t off = (uint32_t)fr * kRowBytes + (uint32_t)((((lane >> 2) ^ (fr & 7)) << 4) + (lane & 3) * 4);
-            float h, l;
-            split_tf32(in[i], h, l);
-            *reinterpret_cast<float*>(hi + off) = h;
-            *reinterpret_cast<float*>(lo + off) = l;
-        }
-    }
-}
-// Warp w's 32 features of one raw operand (box w: row = example, 128 bytes of
-// features, 16-byte groups swizzled by the row's low three bits).
-__device__ __forceinline__ void load_raw_t(const uint8_t* raw, float4 (&vals)[8], int pt) {
-    const int lane = pt & 31, w = pt >> 5;
-    const uint8_t* row = raw + (uint32_t)w * 4096u + (uint32_t)lane * kRowBytes;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) vals[j] = *reinterpret_cast<const float4*>(row + ((j ^ (lane & 7)) << 4));
-}
-
-struct FCfg {
-    static constexpr int kStages = 3;                       // B hi/lo stages and TMEM slots of A
-    static constexpr int kRawStages = 4;                    // raw TMA chunks
-    static constexpr uint32_t kABytes = kBM * kRowBytes;    // 16 KiB: one operand, hi or lo or raw
-    static constexpr uint32_t kStageBytes = 2 * kABytes;    // hi and lo of B
-    static constexpr uint32_t kRawBytes = 2 * kABytes;      // raw chunk of both operands
-    // The tensor pipe's fp32 accumulation rounds toward zero, so a long same-sign sum
-    // (a diagonal entry of M) drifts low by up to an ulp per accumulate. Groups of kGroup
-    // chunks (24 accumulates) alternate between two accumulators and the epilogue warps
-    // drain them into round-to-nearest fp32 registers while the MMAs move on.
-    static constexpr int kGroup = 2;
-    static constexpr int kAOff = 2 * 128;                   // first TMEM column of A
-    static constexpr size_t kBarOff = (size_t)kStages * kStageBytes + (size_t)kRawStages * kRawBytes;
-    static constexpr size_t kSmem = 1024 + kBarOff + 8 * (2 * kStages + 2 * kRawStages + 5) + 16;
-    static_assert(kSmem <= 232448 && kAOff + 64 * kStages <= 512, "fit3t shared memory, TMEM columns");
-};
-
-struct FParams {
-    char* state;       // layer states, `bytes` apart; M at +64
-    size_t bytes;
-    int64_t D, n;
-    int tiles;         // lower tiles per layer
-    int total;         // tiles of all layers
-    unsigned int* err;
-};
-
-struct FTile {
-    int layer;
-    int64_t r0, c0;  // M's rows and columns
-    bool diag;
-};
-__device__ __forceinline__ FTile fit_tile(const FParams& p, int u) {
-    FTile f;
-    f.layer = u / p.tiles;
-    const int t = u - f.layer * p.tiles;
-    int by = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);  // lower-tile index -> (by, bx), bx <= by
-    while ((by + 1) * (by + 2) / 2 <= t) ++by;
-    while (by * (by + 1) / 2 > t) --by;
-    const int bx = t - by * (by + 1) / 2;
-    f.r0 = (int64_t)by * kBM;
-    f.c0 = (int64_t)bx * kBM;
-    f.diag = bx == by;
-    return f;
-}
-
-__global__ void __launch_bounds__(kThreadsT, 1) fit3t_kernel(const __grid_constant__ CUtensorMap tm, const FParams p) {
-    constexpr int BN = 128;
-    using C = FCfg;
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t* raw0 = smem + (size_t)C::kStages * C::kStageBytes;
-    uint64_t* bars = (uint64_t*)(smem + C::kBarOff);
-    uint64_t* ready = bars;                         // operands split (8 warps)
-    uint64_t* empty = bars + C::kStages;            // count 1 (MMA commit)
-    uint64_t* raw_full = empty + C::kStages;        // count 1 + TMA bytes
-    uint64_t* raw_empty = raw_full + C::kRawStages; // raw chunk read (8 warps)
-    uint64_t* acc_full = raw_empty + C::kRawStages; // [2] a group is accumulated (MMA commit)
-    uint64_t* acc_empty = acc_full + 2;             // [2] drained (8 warps)
-    uint64_t* mma_done = acc_empty + 2;
-    uint32_t* tmem_slot = (uint32_t*)(mma_done + 1);
-    volatile int* abort = (volatile int*)(tmem_slot + 1);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < C::kStages; ++s) {
-            mbar_init(smem_u32(&ready[s]), 8);
-            mbar_init(smem_u32(&empty[s]), 1);
-        }
-        for (int r = 0; r < C::kRawStages; ++r) {
-            mbar_init(smem_u32(&raw_full[r]), 1);
-            mbar_init(smem_u32(&raw_empty[r]), 8);
-        }
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(smem_u32(&acc_full[b]), 1);
-            mbar_init(smem_u32(&acc_empty[b]), 8);
-        }
-        mbar_init(smem_u32(mma_done), 1);
-        *abort = 0;
-        fence_mbar_init();
-    }
-    if (warp == 16) {
-        tmem_alloc(smem_u32(tmem_slot), 512);
-        tmem_relinquish();
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
-    const int64_t nkc = (p.n + kKC - 1) / kKC;
-
-    if (warp < 8) {
-        // ---------------- split warps: raw chunk -> A in TMEM (0-3), B hi/lo in shared memory (4-7)
-        uint32_t it = 0;
-        bool ok = true;
-        for (int u = blockIdx.x; ok && u < p.total; u += gridDim.x) {
-            const bool diag = fit_tile(p, u).diag;
-            for (int64_t kc = 0; kc < nkc; ++kc, ++it) {
-                const uint32_t r = it % C::kRawStages, rph = (it / C::kRawStages) & 1u;
-                const uint32_t s = it % C::kStages, ph = (it / C::kStages) & 1u;
-                bool got = true;
-                if (lane == 0) got = wait_bounded(smem_u32(&raw_full[r]), rph, abort, p.err);
-                got = __shfl_sync(0xffffffffu, got, 0);
-                if (!got) {
-                    ok = false;
-                    break;
-                }
-                const uint8_t* raw = raw0 + (size_t)r * C::kRawBytes;
-                if (warp < 4) {
-                    const uint8_t* box = raw + (uint32_t)warp * 4096u + (lane & 3) * 4;
-                    uint32_t x[32];
-#pragma unroll
-                    for (int e = 0; e < 32; ++e)
-                        x[e] = *reinterpret_cast<const uint32_t*>(box + e * kRowBytes + (((lane >> 2) ^ (e & 7)) << 4));
-                    __syncwarp();
-                    if (lane == 0) {
-                        mbar_arrive(smem_u32(&raw_empty[r]));
-                        got = wait_bounded(smem_u32(&empty[s]), ph ^ 1u, abort, p.err);
+                    for (int k = 0; k < kKC / 8; ++k) {  // K = 8 tf32: 8 TMEM columns, 32 bytes of shared memory
+                        mma_tf32_ta<PAIR>(d, ahi + 8 * k, bhi + 2 * k, idesc, start && k == 0 ? 0u : 1u);
+                        mma_tf32_ta<PAIR>(d, ahi + 8 * k, blo + 2 * k, idesc, 1u);
+                        mma_tf32_ta<PAIR>(d, alo + 8 * k, bhi + 2 * k, idesc, 1u);
                     }
-                    got = __shfl_sync(0xffffffffu, got, 0);
-                    if (!got) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint32_t dst = tmem + ((uint32_t)(warp * 32) << 16) + C::kAOff + s * 64u;
-                    tmem_st16(dst, x);
-                    tmem_st16(dst + 16, x + 16);
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) {
-                        float h, l;
-                        split_tf32(__uint_as_float(x[e]), h, l);
-                        x[e] = __float_as_uint(l);
-                    }
-                    tmem_st16(dst + 32, x);
-                    tmem_st16(dst + 48, x + 16);
-                    tmem_wait_st();
-                    tc_fence_before();
-                } else {
-                    const int pt = threadIdx.x - 128;
-                    float4 v[8];
-                    load_raw_t(raw + (diag ? 0u : C::kABytes), v, pt);
-                    __syncwarp();
-                    if (lane == 0) {
-                        mbar_arrive(smem_u32(&raw_empty[r]));
-                        got = wait_bounded(smem_u32(&empty[s]), ph ^ 1u, abort, p.err);
-                    }
-                    got = __shfl_sync(0xffffffffu, got, 0);
-                    if (!got) {
-                        ok = false;
-                        break;
-                    }
-                    uint8_t* st = smem + (size_t)s * C::kStageBytes;
-                    store_split_t<BN>(v, st, st + C::kABytes, pt);
-                    fence_proxy_async();
+                    commit_all<PAIR>(smem_u32(&empty[s]));
+                    if (last) commit_all<PAIR>(smem_u32(&acc_full[b]));
                 }
                 __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&ready[s]));
+                cnt += last;
             }
         }
-    } else if (warp < 16) {
-        // ---------------- epilogue: groups -> registers -> M (lane: column of M, register: row)
-        const int q4 = warp & 3, half = (warp - 8) >> 2, row = q4 * 32 + lane;
-        const uint32_t tbase = tmem + ((uint32_t)(q4 * 32) << 16) + half * 64;
-        const uint32_t groups = (uint32_t)((nkc + C::kGroup - 1) / C::kGroup);
-        uint32_t cnt = 0;
-        bool got = true;
-        for (int u = blockIdx.x; got && u < p.total; u += gridDim.x) {
-            const FTile f = fit_tile(p, u);
-            float acc[64];
-#pragma unroll
-            for (int c = 0; c < 64; ++c) acc[c] = 0.f;
-            for (uint32_t g = 0; g < groups; ++g, ++cnt) {
-                const uint32_t b = cnt & 1u;
-                if (lane == 0) got = wait_bounded(smem_u32(&acc_full[b]), (cnt >> 1) & 1u, abort, p.err);
-                got = __shfl_sync(0xffffffffu, got, 0);
-                if (!got) break;
-                tc_fence_after();
-#pragma unroll
-                for (int c0 = 0; c0 < 64; c0 += 16) {
-                    float v[16];
-                    tmem_ld16(tbase + b * BN + c0, v);
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) acc[c0 + i] += v[i];
-                }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&acc_empty[b]));
-            }
-            const int64_t c = f.c0 + row, r0 = f.r0 + half * 64;
-            if (!got || c >= p.D) continue;
-            float* M = (float*)(p.state + (size_t)f.layer * p.bytes + 64) + c;
-            const int lim = (int)(p.D - r0 < 64 ? p.D - r0 : 64);
-#pragma unroll
-            for (int c0 = 0; c0 < 64; c0 += 8) {
-                float old[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) old[i] = c0 + i < lim ? M[(r0 + c0 + i) * p.D] : 0.f;
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    if (c0 + i < lim) M[(r0 + c0 + i) * p.D] = old[i] + acc[c0 + i];
-            }
-        }
-    } else if (warp == 17) {
-        if (lane == 0) {
-            // ---------------- TMA producer: raw chunks of 32 examples, A: features c0.., B: r0..
-            uint32_t it = 0, last_par[C::kRawStages];
-            bool issued[C::kRawStages], ok = true;
-            for (int r = 0; r < C::kRawStages; ++r) issued[r] = false;
-            for (int u = blockIdx.x; ok && u < p.total; u += gridDim.x) {
-                const FTile f = fit_tile(p, u);
-                const int xa = (int)(f.layer * p.D + f.c0), xb = (int)(f.layer * p.D + f.r0);
-                const uint32_t bytes = f.diag ? C::kABytes : C::kRawBytes;
-                for (int64_t kc = 0; kc < nkc; ++kc, ++it) {
-                    const uint32_t r = it % C::kRawStages, rph = (it / C::kRawStages) & 1u;
-                    if (!wait_bounded(smem_u32(&raw_empty[r]), rph ^ 1u, abort, p.err)) {
-                        ok = false;
-                        break;
-                    }
-                    const uint32_t dst = smem_u32(raw0 + (size_t)r * C::kRawBytes), bar = smem_u32(&raw_full[r]);
-                    const int y = (int)(kc * kKC);
-                    mbar_arrive_tx(bar, bytes);
-#pragma unroll
-                    for (int b = 0; b < 4; ++b) tma_load_2d(dst + (uint32_t)b * 4096u, &tm, xa + 32 * b, y, bar);
-                    if (!f.diag)
-#pragma unroll
-                        for (int b = 0; b < 4; ++b)
-                            tma_load_2d(dst + C::kABytes + (uint32_t)b * 4096u, &tm, xb + 32 * b, y, bar);
-                    issued[r] = true;
-                    last_par[r] = rph;
-                }
-            }
-            // copies still in flight when the consumers stopped early land before the CTA exits
-            for (int r = 0; r < C::kRawStages; ++r)
-                if (issued[r]) {
-                    const uint64_t t0 = global_ns();
-                    while (!mbar_try_wait(smem_u32(&raw_full[r]), last_par[r]))
-                        if (global_ns() - t0 > kTimeoutNs) {
-                            atomicOr(p.err, kErrTimeout);
-                            break;
-                        }
-                }
-        }
-    } else if (lane == 0) {
-        // ---------------- MMA issuer
-        constexpr uint32_t idesc = idesc_tf32(kBM, BN);
-        uint32_t it = 0, cnt = 0;
-        bool ok = true;
-        for (int u = blockIdx.x; ok && u < p.total; u += gridDim.x)
-            for (int64_t kc = 0; kc < nkc; ++kc, ++it) {
-                const uint32_t s = it % C::kStages, ph = (it / C::kStages) & 1u, b = cnt & 1u;
-                const bool start = kc % C::kGroup == 0, last = kc % C::kGroup == C::kGroup - 1 || kc == nkc - 1;
-                if ((start && !wait_bounded(smem_u32(&acc_empty[b]), ((cnt >> 1) & 1u) ^ 1u, abort, p.err)) ||
-                    !wait_bounded(smem_u32(&ready[s]), ph, abort, p.err)) {
-                    ok = false;
+        if (elect_one()) {
+            if constexpr (PAIR)
+                commit_pair_local(smem_u32(mma_done));
+            else
+                mma_commit(smem_u32(mma_done));
+            const uint64_t ns = global_ns();
+            while (!mbar_try_wait(smem_u32(mma_done), 0))
+                if (global_ns() - ns > kTimeoutNs) {
+                    atomicOr(p.err, kErrTimeout);
                     break;
                 }
-                tc_fence_after();
-                const uint32_t st = smem_u32(smem + (size_t)s * C::kStageBytes);
-                const uint32_t ahi = tmem + C::kAOff + s * 64u, alo = ahi + 32u, d = tmem + b * BN;
-                const uint64_t bhi = sw128_desc(st), blo = sw128_desc(st + C::kABytes);
-#pragma unroll
-                for (int k = 0; k < kKC / 8; ++k) {
-                    mma_tf32_ta(d, ahi + 8 * k, bhi + 2 * k, idesc, start && k == 0 ? 0u : 1u);
-                    mma_tf32_ta(d, ahi + 8 * k, blo + 2 * k, idesc, 1u);
-                    mma_tf32_ta(d, alo + 8 * k, bhi + 2 * k, idesc, 1u);
-                }
-                mma_commit(smem_u32(&empty[s]));
-                if (last) {
-                    mma_commit(smem_u32(&acc_full[b]));
-                    ++cnt;
-                }
-            }
-        mma_commit(smem_u32(mma_done));
-        const uint64_t t0 = global_ns();
-        while (!mbar_try_wait(smem_u32(mma_done), 0))
-            if (global_ns() - t0 > kTimeoutNs) {
-                atomicOr(p.err, kErrTimeout);
-                break;
-            }
+        }
+        __syncwarp();
     }
 
     tc_fence_before();
     __syncthreads();
+    if constexpr (PAIR) cluster_sync();
     if (warp == 16) {
         tc_fence_after();
-        tmem_dealloc(tmem, 512);
+        if constexpr (PAIR)
+            tmem_dealloc2(tmem, 512);
+        else
+            tmem_dealloc(tmem, 512);
     }
 }
 
@@ -1069,6 +892,35 @@ bool make_map_f32_3d(CUtensorMap* tm, const float* X, int64_t rows, int64_t K, i
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// 256 x 128 tiles that hold the 128 x 128 tiles of a lower triangle of nt x nt
+int64_t pair_lower_tiles(int64_t nt) {
+    const int64_t q = nt / 2;
+    return nt & 1 ? (q + 1) * (q + 1) : q * (q + 1);
+}
+
+template <int BN, bool FIT>
+cudaError_t launch_pairs(const CUtensorMap& tmA, const CUtensorMap& tmB, const GParams& p, int sms, cudaStream_t s) {
+    using T = TCfg<BN, true>;
+    cudaError_t e = smem_attr_once<gemm3t_kernel<BN, true, FIT>>((int)T::kSmem);
+    if (e != cudaSuccess) return e;
+    const int64_t total = p.tiles_z * p.splits * p.nz, half = sms > 1 ? sms / 2 : 1;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)(2 * (total < half ? total : half)));
+    cfg.blockDim = dim3(kThreadsT);
+    cfg.dynamicSmemBytes = T::kSmem;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    note_launches(1);
+    e = cudaLaunchKernelEx(&cfg, gemm3t_kernel<BN, true, FIT>, tmA, tmB, p);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 template <int BN>
 cudaError_t launch_bn(GParams p, cudaStream_t s, int64_t nz = 1, size_t a_z_bytes = 0, size_t b_z_bytes = 0) {
     using C = GCfg<BN>;
@@ -1099,14 +951,26 @@ cudaError_t launch_bn(GParams p, cudaStream_t s, int64_t nz = 1, size_t a_z_byte
     p.cs = cs;
     p.tiles_n = (int)tiles_n;
     if (cs == 1) {
-        using T = TCfg<BN>;
-        p.tiles_z = tiles;
         p.nz = (int)nz;
-        const int64_t total = tiles * p.splits * nz;
-        cudaError_t e = smem_attr_once<gemm3t_kernel<BN>>((int)T::kSmem);
+        // A pair's chunk takes about three quarters of a single CTA's (see above), so its whole rounds of
+        // tiles decide: few or odd 128-row tiles can leave half of the pairs' rows empty.
+        const int64_t pairs = p.lower ? pair_lower_tiles(tiles_n) : (tiles_m + 1) / 2 * tiles_n;
+        const int64_t per = (int64_t)p.splits * nz, half = sms > 1 ? sms / 2 : 1;
+        if (3 * ((pairs * per + half - 1) / half) <= 4 * ((tiles * per + sms - 1) / sms)) {
+            p.tiles_z = pairs;
+            // B's box: the half of a tile's rows that one CTA of the pair loads
+            if (nz > 1 ? !make_map_f32_3d(&tmB, p.B, p.n_q, p.K, p.ldb, nz, b_z_bytes, BN / 2)
+                       : !make_map_f32(&tmB, p.B, p.n_q, p.K, p.ldb, BN / 2))
+                return cudaErrorInvalidValue;
+            return launch_pairs<BN, false>(tmA, tmB, p, sms, s);
+        }
+        using T = TCfg<BN, false>;
+        p.tiles_z = tiles;
+        const int64_t total = tiles * per;
+        cudaError_t e = smem_attr_once<gemm3t_kernel<BN, false, false>>((int)T::kSmem);
         if (e != cudaSuccess) return e;
         note_launches(1);
-        gemm3t_kernel<BN><<<(unsigned)(total < sms ? total : sms), kThreadsT, T::kSmem, s>>>(tmA, tmB, p);
+        gemm3t_kernel<BN, false, false><<<(unsigned)(total < sms ? total : sms), kThreadsT, T::kSmem, s>>>(tmA, tmB, p);
         return cudaGetLastError();
     }
     // few tiles: a cluster of cs CTAs splits K
@@ -1281,18 +1145,19 @@ bool fit_tc_supported(int n_layers, int64_t D, const float* phi, int64_t n, int6
 
 cudaError_t launch_fit_tc(int n_layers, int64_t D, void* state, size_t state_bytes, const float* phi, int64_t n,
                           int64_t ld, unsigned int* err, cudaStream_t s) {
-    using C = FCfg;
-    const int64_t nt = (D + kBM - 1) / kBM;
     // features of all layers, examples as rows; zero fill past the last layer's features and the last example
     CUtensorMap tm;
     if (!make_map_f32(&tm, phi, n, (int64_t)n_layers * D, ld, kKC)) return cudaErrorInvalidValue;
-    FParams p{};
-    p.state = (char*)state;
-    p.bytes = state_bytes;
-    p.D = D;
-    p.n = n;
-    p.tiles = (int)(nt * (nt + 1) / 2);
-    p.total = p.tiles * n_layers;
+    GParams p{};
+    p.S = (float*)((char*)state + 64);
+    p.s_z = (int64_t)(state_bytes / 4);
+    p.n_t = p.n_q = p.ld_S = D;
+    p.K = n;
+    p.alpha = p.beta = 1.f;
+    p.lower = 1;
+    p.splits = 1;
+    p.nz = n_layers;
+    p.tiles_z = pair_lower_tiles((D + kBM - 1) / kBM);
     p.err = err;
     static std::atomic<int> sms_cache{0};
     int sms = sms_cache.load(std::memory_order_relaxed);
@@ -1302,11 +1167,7 @@ cudaError_t launch_fit_tc(int n_layers, int64_t D, void* state, size_t state_byt
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 1;
         sms_cache.store(sms, std::memory_order_relaxed);
     }
-    cudaError_t e = smem_attr_once<fit3t_kernel>((int)C::kSmem);
-    if (e != cudaSuccess) return e;
-    note_launches(1);
-    fit3t_kernel<<<(unsigned)(p.total < sms ? p.total : sms), kThreadsT, C::kSmem, s>>>(tm, p);
-    return cudaGetLastError();
+    return launch_pairs<128, true>(tm, tm, p, sms, s);
 }
 
 }  // namespace tda

@@ -52,6 +52,22 @@ __device__ __forceinline__ bool wait_bounded(uint32_t bar, uint32_t parity, vola
         }
     }
 }
+// wait_bounded by a whole (converged) warp: all lanes poll, so that a phase already complete costs one
+// try_wait and a vote. (Lane 0 polling and a shuffle of its answer took about 250 clocks.)
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* abort, unsigned int* err) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    bool got = true;
+    if ((threadIdx.x & 31) == 0) got = wait_bounded(bar, parity, abort, err);
+    return __shfl_sync(0xffffffffu, got, 0);
+}
+// One lane of a converged warp, always the same one. The compiler knows that a single lane is active
+// behind it and keeps the operands of tcgen05 instructions in uniform registers; behind
+// `lane == 0` it rebuilds them for each instruction (80 clocks an MMA).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(r));
+    return r != 0;
+}
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* tm, int c0, int c1, int c2,
                                             uint32_t bar) {
     asm volatile(
