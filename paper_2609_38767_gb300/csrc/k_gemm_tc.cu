@@ -128,7 +128,7 @@ score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     uint32_t* tmem_slot = (uint32_t*)(mma_done + 1);
     volatile int* abort = (volatile int*)(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::kStages; ++s) {
             mbar_init(smem_u32(&full[s]), 4);
@@ -183,10 +183,7 @@ score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         for (int64_t kc = kc0; kc < kc1; ++kc, ++it) {
             const int s = it % C::kStages;
             const uint32_t ph = (it / C::kStages) & 1u;
-            bool got = true;
-            if (lane == 0) got = wait_bounded(smem_u32(&raw_full[s]), ph, abort, p.err);
-            got = __shfl_sync(0xffffffffu, got, 0);
-            __syncwarp();
+            bool got = warp_wait(smem_u32(&raw_full[s]), ph, abort, p.err);
             if (!got) break;
             uint8_t* st = smem + (size_t)s * C::kStageBytes;
             split_tile<C::kABytes>(st, st + C::kABytes, pt);
@@ -231,8 +228,8 @@ score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     }
             }
     }
-    if (warp == kMmaWarp && lane == 0) {
-        // ---------------- MMA issuer
+    if (warp == kMmaWarp) {
+        // ---------------- MMA issuer: the warp waits, one lane issues
         const uint32_t idesc = idesc_tf32(kBM, BN);
         uint32_t it = 0;
         for (int64_t kc = kc0; kc < kc1; ++kc, ++it) {
@@ -240,29 +237,35 @@ score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             const uint32_t ph = (it / C::kStages) & 1u;
             const uint32_t g = it / C::kGroup, a = g % C::kAcc;  // group g goes to accumulator a
             const bool start = it % C::kGroup == 0;
-            if (start && !wait_bounded(smem_u32(&acc_empty[a]), ((g / C::kAcc) & 1u) ^ 1u, abort, p.err)) break;
-            if (!wait_bounded(smem_u32(&full[s]), ph, abort, p.err)) break;
+            if (start && !warp_wait(smem_u32(&acc_empty[a]), ((g / C::kAcc) & 1u) ^ 1u, abort, p.err)) break;
+            if (!warp_wait(smem_u32(&full[s]), ph, abort, p.err)) break;
             tc_fence_after();
             const uint32_t st = smem_u32(smem + (size_t)s * C::kStageBytes);
             const uint64_t ahi = sw128_desc(st), alo = sw128_desc(st + C::kABytes);
             const uint64_t bhi = sw128_desc(st + 2 * C::kABytes), blo = sw128_desc(st + 2 * C::kABytes + C::kBBytes);
             const uint32_t d = tmem + a * BN;
+            if (elect_one()) {
 #pragma unroll
-            for (int k = 0; k < kKC / 8; ++k) {  // K = 8 tf32 = 32 bytes per instruction
-                mma_tf32(d, ahi + 2 * k, bhi + 2 * k, idesc, start && k == 0 ? 0u : 1u);
-                mma_tf32(d, ahi + 2 * k, blo + 2 * k, idesc, 1u);
-                mma_tf32(d, alo + 2 * k, bhi + 2 * k, idesc, 1u);
+                for (int k = 0; k < kKC / 8; ++k) {  // K = 8 tf32 = 32 bytes per instruction
+                    mma_tf32(d, ahi + 2 * k, bhi + 2 * k, idesc, start && k == 0 ? 0u : 1u);
+                    mma_tf32(d, ahi + 2 * k, blo + 2 * k, idesc, 1u);
+                    mma_tf32(d, alo + 2 * k, bhi + 2 * k, idesc, 1u);
+                }
+                mma_commit(smem_u32(&empty[s]));
+                if (it % C::kGroup == C::kGroup - 1 || kc == kc1 - 1) mma_commit(smem_u32(&acc_full[a]));
             }
-            mma_commit(smem_u32(&empty[s]));
-            if (it % C::kGroup == C::kGroup - 1 || kc == kc1 - 1) mma_commit(smem_u32(&acc_full[a]));
+            __syncwarp();
         }
-        mma_commit(smem_u32(mma_done));
-        const uint64_t t0 = global_ns();
-        while (!mbar_try_wait(smem_u32(mma_done), 0))
-            if (global_ns() - t0 > kTimeoutNs) {
-                atomicOr(p.err, kErrTimeout);
-                break;
-            }
+        if (elect_one()) {
+            mma_commit(smem_u32(mma_done));
+            const uint64_t t0 = global_ns();
+            while (!mbar_try_wait(smem_u32(mma_done), 0))
+                if (global_ns() - t0 > kTimeoutNs) {
+                    atomicOr(p.err, kErrTimeout);
+                    break;
+                }
+        }
+        __syncwarp();
     }
     __syncwarp();
     if (warp >= 4 && warp < 8) {
@@ -278,8 +281,7 @@ score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         bool got = true;
         for (uint32_t g = 0; g < groups; ++g) {
             const uint32_t a = g % C::kAcc;
-            if (lane == 0) got = wait_bounded(smem_u32(&acc_full[a]), (g / C::kAcc) & 1u, abort, p.err);
-            got = __shfl_sync(0xffffffffu, got, 0);
+            got = warp_wait(smem_u32(&acc_full[a]), (g / C::kAcc) & 1u, abort, p.err);
             if (!got) break;
             tc_fence_after();
 #pragma unroll

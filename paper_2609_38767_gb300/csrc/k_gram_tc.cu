@@ -159,7 +159,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmAq, const __grid_constant__
     volatile int* abort = (volatile int*)(tmem_slot + 1);
     float* red = (float*)(tmem_slot + 4);   // packed: [2 column halves][128 rows][ldr examples] partial sums
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.stages; ++s) {
             mbar_init(smem_u32(&full[s]), 1);
@@ -235,8 +235,8 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmAq, const __grid_constant__
                         break;
                     }
             }
-    } else if (warp == 1 && lane == 0) {
-        // ---------------- MMA issuer
+    } else if (warp == 1) {
+        // ---------------- MMA issuer: the warp waits, one lane issues
         uint32_t s = 0, ph = 0, cnt = 0;
         bool ok = true;
         constexpr uint32_t idesc = idesc_bf16(kTM, kTN);
@@ -246,7 +246,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmAq, const __grid_constant__
                 const uint32_t boff = SELF && ti == tj ? 0u : kABytes;
                 for (int blk = 0; ok && blk < nb; ++blk, ++cnt) {
                     const uint32_t b = cnt & 1u;
-                    if (!wait_bounded(smem_u32(&tempty[b]), ((cnt >> 1) & 1u) ^ 1u, abort, p.err)) {
+                    if (!warp_wait(smem_u32(&tempty[b]), ((cnt >> 1) & 1u) ^ 1u, abort, p.err)) {
                         ok = false;
                         break;
                     }
@@ -256,32 +256,39 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmAq, const __grid_constant__
                     const int left = side_b ? p.nk_out - (blk - nbx) * kb : p.nk_in - blk * kb;
                     const int n = left < kb ? left : kb;
                     for (int c = 0; c < n; ++c) {
-                        if (!wait_bounded(smem_u32(&full[s]), ph, abort, p.err)) {
+                        if (!warp_wait(smem_u32(&full[s]), ph, abort, p.err)) {
                             ok = false;
                             break;
                         }
                         tc_fence_after();
                         const uint32_t st = smem_u32(smem + (size_t)s * C::kStageBytes);
                         const uint64_t ad = sw128_desc(st), bd = sw128_desc(st + boff);
+                        if (elect_one()) {
 #pragma unroll
-                        for (int k = 0; k < kChunkK / 16; ++k)
-                            mma_bf16(tmem + b * 256u, ad + 2 * k, bd + 2 * k, idesc, (c > 0 || k > 0) ? 1u : 0u);
-                        mma_commit(smem_u32(&empty[s]));
+                            for (int k = 0; k < kChunkK / 16; ++k)
+                                mma_bf16(tmem + b * 256u, ad + 2 * k, bd + 2 * k, idesc, (c > 0 || k > 0) ? 1u : 0u);
+                            mma_commit(smem_u32(&empty[s]));
+                        }
+                        __syncwarp();
                         if (++s == (uint32_t)p.stages) s = 0, ph ^= 1u;
                     }
                     if (!ok) break;
-                    mma_commit(smem_u32(&tfull[b]));
+                    if (elect_one()) mma_commit(smem_u32(&tfull[b]));
+                    __syncwarp();
                 }
                 if (++tj == p.tiles_t) tj = SELF ? ++ti : (++ti, 0);
             }
         }
-        mma_commit(smem_u32(mma_done));
-        const uint64_t t0 = global_ns();
-        while (!mbar_try_wait(smem_u32(mma_done), 0))
-            if (global_ns() - t0 > kTimeoutNs) {
-                atomicOr(p.err, kErrTimeout);
-                break;
-            }
+        if (elect_one()) {
+            mma_commit(smem_u32(mma_done));
+            const uint64_t t0 = global_ns();
+            while (!mbar_try_wait(smem_u32(mma_done), 0))
+                if (global_ns() - t0 > kTimeoutNs) {
+                    atomicOr(p.err, kErrTimeout);
+                    break;
+                }
+        }
+        __syncwarp();
     } else if (warp >= 2) {
         // ---------------- epilogue: warp ew covers TMEM lane quadrant warp % 4, column half h
         const int ew = warp - 2, q4 = warp & 3, h = ew >> 2, row = q4 * 32 + lane;
@@ -305,8 +312,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmAq, const __grid_constant__
                 for (int c = 0; c < kCols; ++c) x[c] = 0.f;
                 for (int blk = 0; ok && blk < nb; ++blk, ++cnt) {
                     const uint32_t b = cnt & 1u;
-                    if (lane == 0) ok = wait_bounded(smem_u32(&tfull[b]), (cnt >> 1) & 1u, abort, p.err);
-                    ok = __shfl_sync(0xffffffffu, ok, 0);
+                    ok = warp_wait(smem_u32(&tfull[b]), (cnt >> 1) & 1u, abort, p.err);
                     if (!ok) break;  // the other roles see the abort flag; the barrier below ends the unit
                     tc_fence_after();
                     const uint32_t tb = tbase + b * 256u;

@@ -85,7 +85,7 @@ materialize_tc_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_cons
     uint64_t* mma_done = tempty + 2;
     uint32_t* tmem_slot = (uint32_t*)(mma_done + 1);
     volatile int* abort = (volatile int*)(tmem_slot + 1);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(smem_u32(&full[s]), 1);
@@ -149,34 +149,38 @@ materialize_tc_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_cons
                 }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ---------------- MMA issuer
-            uint32_t ring = 0, tile = 0;
-            bool ok = true;
-            for (int64_t u = blockIdx.x; ok && u < p.n_units; u += gridDim.x, ++tile) {
-                const uint32_t b = tile & 1u, use = tile >> 1;
-                if (!wait_bounded(smem_u32(&tempty[b]), (use & 1u) ^ 1u, abort, p.err)) break;
+        // ---------------- MMA issuer: the warp waits, one lane issues
+        uint32_t ring = 0, tile = 0;
+        bool ok = true;
+        for (int64_t u = blockIdx.x; ok && u < p.n_units; u += gridDim.x, ++tile) {
+            const uint32_t b = tile & 1u, use = tile >> 1;
+            if (!warp_wait(smem_u32(&tempty[b]), (use & 1u) ^ 1u, abort, p.err)) break;
+            tc_fence_after();
+            for (int kc = 0; kc < nk; ++kc, ++ring) {
+                const int s = ring % kStages;
+                const uint32_t ph = (ring / kStages) & 1u;
+                if (!warp_wait(smem_u32(&full[s]), ph, abort, p.err)) {
+                    ok = false;
+                    break;
+                }
                 tc_fence_after();
-                for (int kc = 0; kc < nk; ++kc, ++ring) {
-                    const int s = ring % kStages;
-                    const uint32_t ph = (ring / kStages) & 1u;
-                    if (!wait_bounded(smem_u32(&full[s]), ph, abort, p.err)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint32_t st = smem_u32(smem + (size_t)s * kStageBytes);
-                    const uint64_t ad = sw128_mn_desc(st, kBox, 1024), bd = sw128_mn_desc(st + kABytes, kBox, 1024);
-                    // 16 tokens per MMA = two 8-token groups = 2 KiB further into every box
+                const uint32_t st = smem_u32(smem + (size_t)s * kStageBytes);
+                const uint64_t ad = sw128_mn_desc(st, kBox, 1024), bd = sw128_mn_desc(st + kABytes, kBox, 1024);
+                // 16 tokens per MMA = two 8-token groups = 2 KiB further into every box
+                if (elect_one()) {
 #pragma unroll
                     for (int k = 0; k < kTK / 16; ++k)
                         mma_bf16(tmem + b * kTN, ad + (uint64_t)(k * 2048 >> 4), bd + (uint64_t)(k * 2048 >> 4),
                                  kIdesc, (kc > 0 || k > 0) ? 1u : 0u);
                     mma_commit(smem_u32(&empty[s]));
                 }
-                if (!ok) break;
-                mma_commit(smem_u32(&tfull[b]));
+                __syncwarp();
             }
+            if (!ok) break;
+            if (elect_one()) mma_commit(smem_u32(&tfull[b]));
+            __syncwarp();
+        }
+        if (elect_one()) {
             mma_commit(smem_u32(mma_done));
             const uint64_t t0 = global_ns();
             while (!mbar_try_wait(smem_u32(mma_done), 0))
@@ -185,6 +189,7 @@ materialize_tc_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_cons
                     break;
                 }
         }
+        __syncwarp();
     } else {
         // ---------------- epilogue: TMEM -> shared (swizzled 32 x 32 blocks) -> TMA store to G
         const int q = warp & 3;
@@ -193,9 +198,7 @@ materialize_tc_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_cons
         bool prev_stored = false;  // lane 0: whether the previous block (the other buffer) went out
         for (int64_t u = blockIdx.x; u < p.n_units; u += gridDim.x, ++tile) {
             const uint32_t b = tile & 1u, use = tile >> 1;
-            bool got = true;
-            if (lane == 0) got = wait_bounded(smem_u32(&tfull[b]), use & 1u, abort, p.err);
-            got = __shfl_sync(0xffffffffu, got, 0);
+            bool got = warp_wait(smem_u32(&tfull[b]), use & 1u, abort, p.err);
             if (epi_any(!got)) break;
             tc_fence_after();
             const int64_t e = u / (p.n_rb * p.n_cb), rc = u % (p.n_rb * p.n_cb);

@@ -1749,7 +1749,7 @@ __global__ void __launch_bounds__(256) scale_lower_kernel(St<float> st) {
 // the backward solve's tensor-core products; the diagonal blocks hold W^T there). Each thread has
 // four 16-byte loads in flight and the block index comes from an fp32 estimate corrected in
 // integers: with 32 x 32 blocks, scalar loads and an fp64 square root per block this took 417 us
-// for seven layers of D = 4096, 73056 us here.
+// for seven layers of D = 4096, 73 us here.
 __global__ void __launch_bounds__(256) upper_from_lower_kernel(St<float> st, int n_layers) {
     __shared__ float t[64][65];
     const int64_t D = st.D, nb = D / 64, pairs = nb * (nb - 1) / 2;

@@ -172,7 +172,7 @@ project_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     uint32_t* tmem_slot = (uint32_t*)(red_full + 1);
     volatile int* abort = (volatile int*)(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::kStages; ++s) {
             mbar_init(smem_u32(&full[s]), 1);
@@ -248,19 +248,19 @@ project_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                         break;
                     }
             }
-    } else if (warp == 1 && lane == 0) {
-        // ---------------- MMA issuer
+    } else if (warp == 1) {
+        // ---------------- MMA issuer: the warp waits, one lane issues
         uint32_t s = 0, ph = 0, cnt = 0, tile = 0;
         bool ok = true;
         constexpr uint32_t idesc = idesc_bf16(kTileM, K);
         for (; ok && it.x < p.n_slots; it.next(p, ncl, crank), ++tile) {
             const uint32_t b = tile % C::kBufs, use = tile / C::kBufs;
-            if (!wait_bounded(smem_u32(&tempty[b]), (use & 1u) ^ 1u, abort, p.err)) break;
+            if (!warp_wait(smem_u32(&tempty[b]), (use & 1u) ^ 1u, abort, p.err)) break;
             for (int kc = 0; kc < nk_tot; ++kc, ++cnt) {
                 const uint32_t a = cnt & 1u;
-                if (!wait_bounded(smem_u32(&sready[s]), ph, abort, p.err) ||
-                    !(F32 ? wait_bounded(smem_u32(&afull[a]), (cnt >> 1) & 1u, abort, p.err)
-                          : wait_bounded(smem_u32(&full[s]), ph, abort, p.err))) {
+                if (!warp_wait(smem_u32(&sready[s]), ph, abort, p.err) ||
+                    !(F32 ? warp_wait(smem_u32(&afull[a]), (cnt >> 1) & 1u, abort, p.err)
+                          : warp_wait(smem_u32(&full[s]), ph, abort, p.err))) {
                     ok = false;
                     break;
                 }
@@ -270,32 +270,39 @@ project_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 const uint32_t st = smem_u32(smem + (size_t)s * C::kStageBytes);
                 const uint64_t bd = sw128_desc(st + C::kTileBytes);
                 const uint32_t dh = tmem + b * C::kBufCols + (side_b ? C::kSideCols : 0), dl = dh + K;
+                if (elect_one()) {
 #pragma unroll
-                for (int k = 0; k < kChunkK / 16; ++k) {  // K = 16: 32 bytes of bf16, 8 columns of pieces
-                    const uint32_t acc = start && k == 0 ? 0u : 1u;
-                    if constexpr (F32) {
-                        const uint32_t at = tmem + C::kAOff + a * kACols;
-                        mma_bf16_ta(dh, at + 8 * k, bd + 2 * k, idesc, acc);
-                        mma_bf16_ta(dl, at + kPieceCols + 8 * k, bd + 2 * k, idesc, acc);
-                        mma_bf16_ta(dl, at + 2 * kPieceCols + 8 * k, bd + 2 * k, idesc, 1u);
-                    } else {
-                        mma_bf16(dh, sw128_desc(st) + 2 * k, bd + 2 * k, idesc, acc);
+                    for (int k = 0; k < kChunkK / 16; ++k) {  // K = 16: 32 bytes of bf16, 8 columns of pieces
+                        const uint32_t acc = start && k == 0 ? 0u : 1u;
+                        if constexpr (F32) {
+                            const uint32_t at = tmem + C::kAOff + a * kACols;
+                            mma_bf16_ta(dh, at + 8 * k, bd + 2 * k, idesc, acc);
+                            mma_bf16_ta(dl, at + kPieceCols + 8 * k, bd + 2 * k, idesc, acc);
+                            mma_bf16_ta(dl, at + 2 * kPieceCols + 8 * k, bd + 2 * k, idesc, 1u);
+                        } else {
+                            mma_bf16(dh, sw128_desc(st) + 2 * k, bd + 2 * k, idesc, acc);
+                        }
                     }
+                    if constexpr (F32) mma_commit(smem_u32(&aempty[a]));
+                    mma_commit(smem_u32(&sempty[s]));
                 }
-                if constexpr (F32) mma_commit(smem_u32(&aempty[a]));
-                mma_commit(smem_u32(&sempty[s]));
+                __syncwarp();
                 if (++s == (uint32_t)C::kStages) s = 0, ph ^= 1u;
             }
             if (!ok) break;
-            mma_commit(smem_u32(&tfull[b]));
+            if (elect_one()) mma_commit(smem_u32(&tfull[b]));
+            __syncwarp();
         }
-        mma_commit(smem_u32(mma_done));
-        const uint64_t t0 = global_ns();
-        while (!mbar_try_wait(smem_u32(mma_done), 0))
-            if (global_ns() - t0 > kTimeoutNs) {
-                atomicOr(p.err, kErrTimeout);
-                break;
-            }
+        if (elect_one()) {
+            mma_commit(smem_u32(mma_done));
+            const uint64_t t0 = global_ns();
+            while (!mbar_try_wait(smem_u32(mma_done), 0))
+                if (global_ns() - t0 > kTimeoutNs) {
+                    atomicOr(p.err, kErrTimeout);
+                    break;
+                }
+        }
+        __syncwarp();
     } else if (warp == 2 || warp == 3) {
         // ---------------- sign generators: the 64 threads share a tile's K rows, kParts threads per row
         constexpr int kParts = 64 / K, kChunks = 8 / kParts;
@@ -312,9 +319,7 @@ project_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 #pragma unroll
                 for (int c = 0; c < kChunks; ++c)
                     q[c] = lds128(lut_s + ((((uint32_t)(w >> (8 * (part * kChunks + c)))) & 0xFFu) << 4));
-                bool got = true;
-                if (lane == 0) got = wait_bounded(smem_u32(&sempty[s]), ph ^ 1u, abort, p.err);
-                got = __shfl_sync(0xffffffffu, got, 0);
+                bool got = warp_wait(smem_u32(&sempty[s]), ph ^ 1u, abort, p.err);
                 if (!got) {
                     ok = false;
                     break;
@@ -337,9 +342,7 @@ project_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         for (; ok && it.x < p.n_slots; it.next(p, ncl, crank))
             for (int kc = 0; kc < nk_tot; ++kc, ++cnt) {
                 const uint32_t a = cnt & 1u;
-                bool got = true;
-                if (lane == 0) got = wait_bounded(smem_u32(&full[s]), ph, abort, p.err);
-                got = __shfl_sync(0xffffffffu, got, 0);
+                bool got = warp_wait(smem_u32(&full[s]), ph, abort, p.err);
                 if (!got) {
                     ok = false;
                     break;
@@ -365,12 +368,8 @@ project_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     }
                 }
                 __syncwarp();
-                if (lane == 0) {
-                    mbar_arrive(smem_u32(&rempty[s]));
-                    got = wait_bounded(smem_u32(&aempty[a]), ((cnt >> 1) & 1u) ^ 1u, abort, p.err);
-                }
-                got = __shfl_sync(0xffffffffu, got, 0);
-                if (!got) {
+                if (lane == 0) mbar_arrive(smem_u32(&rempty[s]));
+                if (!warp_wait(smem_u32(&aempty[a]), ((cnt >> 1) & 1u) ^ 1u, abort, p.err)) {
                     ok = false;
                     break;
                 }
@@ -469,9 +468,7 @@ project_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         while (ok && it.x < p.n_slots) {
             const int64_t cur = it.x;
             const uint32_t b = tile % C::kBufs, use = tile / C::kBufs;
-            bool got = true;
-            if (lane == 0) got = wait_bounded(smem_u32(&tfull[b]), use & 1u, abort, p.err);
-            got = __shfl_sync(0xffffffffu, got, 0);
+            bool got = warp_wait(smem_u32(&tfull[b]), use & 1u, abort, p.err);
             if (epi_any(!got)) break;
             tc_fence_after();
             const int rows = p.pack > 1 ? p.pack * (int)p.T : p.R;

@@ -408,7 +408,7 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     uint32_t* tmem_slot = (uint32_t*)(red_full + 1);
     volatile int* abort = (volatile int*)(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::kStages; ++s) {
             mbar_init(smem_u32(&full[s]), 1);
@@ -486,14 +486,14 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                         break;
                     }
             }
-    } else if (warp == 1 && lane == 0) {
-        // ---------------- MMA issuer
+    } else if (warp == 1) {
+        // ---------------- MMA issuer: the warp waits, one lane issues
         uint32_t ring = 0, grp = 0;
         bool ok = true;
         const uint32_t idesc = idesc_bf16(kTileM, K);
         for (int ng; ok && (ng = it.take<G>(p, ncl, crank, gx, gt)) > 0; ++grp) {
             const uint32_t b = grp & 1u, use = grp >> 1;
-            if (!wait_bounded(smem_u32(&tempty[b]), (use & 1u) ^ 1u, abort, p.err)) {
+            if (!warp_wait(smem_u32(&tempty[b]), (use & 1u) ^ 1u, abort, p.err)) {
                 ok = false;
                 break;
             }
@@ -501,8 +501,8 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             for (int kc = 0; kc < nk_tot; ++kc, ++ring) {
                 const int s = ring % C::kStages;
                 const uint32_t ph = (ring / C::kStages) & 1u;
-                if (!wait_bounded(smem_u32(&full[s]), ph, abort, p.err) ||
-                    (!SL && !wait_bounded(smem_u32(&sready[s]), ph, abort, p.err))) {
+                if (!warp_wait(smem_u32(&full[s]), ph, abort, p.err) ||
+                    (!SL && !warp_wait(smem_u32(&sready[s]), ph, abort, p.err))) {
                     ok = false;
                     break;
                 }
@@ -511,26 +511,33 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                 const int kk = side_b ? kc - p.nk_in : kc;
                 uint8_t* stage = sA + (size_t)s * C::kStageBytes;
                 const uint64_t bd = sw128_desc(smem_u32(stage + (size_t)G * kTileBytes));
-                for (int u = 0; u < ng; ++u) {
-                    const uint32_t d_tmem = tmem + b * C::kBufCols + u * C::kAccCols + (side_b ? K : 0);
-                    const uint64_t ad = sw128_desc(smem_u32(stage + (size_t)u * kTileBytes));
+                if (elect_one()) {
+                    for (int u = 0; u < ng; ++u) {
+                        const uint32_t d_tmem = tmem + b * C::kBufCols + u * C::kAccCols + (side_b ? K : 0);
+                        const uint64_t ad = sw128_desc(smem_u32(stage + (size_t)u * kTileBytes));
 #pragma unroll
-                    for (int k = 0; k < kChunkK / 16; ++k)
-                        mma_bf16(d_tmem, ad + 2 * k, bd + 2 * k, idesc, (kk > 0 || k > 0) ? 1u : 0u);
+                        for (int k = 0; k < kChunkK / 16; ++k)
+                            mma_bf16(d_tmem, ad + 2 * k, bd + 2 * k, idesc, (kk > 0 || k > 0) ? 1u : 0u);
+                    }
+                    mma_commit(smem_u32(&empty[s]));
                 }
-                mma_commit(smem_u32(&empty[s]));
+                __syncwarp();
             }
             if (!ok) break;
-            mma_commit(smem_u32(&tfull[b]));
+            if (elect_one()) mma_commit(smem_u32(&tfull[b]));
+            __syncwarp();
         }
-        // all MMAs this thread issued have completed once mma_done fires
-        mma_commit(smem_u32(mma_done));
-        const uint64_t t0 = global_ns();
-        while (!mbar_try_wait(smem_u32(mma_done), 0))
-            if (global_ns() - t0 > kTimeoutNs) {
-                atomicOr(p.err, kErrTimeout);
-                break;
-            }
+        // all MMAs issued have completed once mma_done fires
+        if (elect_one()) {
+            mma_commit(smem_u32(mma_done));
+            const uint64_t t0 = global_ns();
+            while (!mbar_try_wait(smem_u32(mma_done), 0))
+                if (global_ns() - t0 > kTimeoutNs) {
+                    atomicOr(p.err, kErrTimeout);
+                    break;
+                }
+        }
+        __syncwarp();
     } else if (!SL && (warp == 2 || warp == 3)) {
         // ---------------- sign generators (two warps, one half-row each)
         uint32_t ring = 0;
@@ -552,10 +559,7 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 #pragma unroll
                     for (int j = 0; j < 2; ++j) expand_signs(q[j], sign_word(key, (uint32_t)(col0 + 32 * j), rb), lut);
                 }
-                bool got = true;
-                if (lane == 0) got = wait_bounded(smem_u32(&empty[s]), ph ^ 1u, abort, p.err);
-                got = __shfl_sync(0xffffffffu, got, 0);
-                __syncwarp();
+                bool got = warp_wait(smem_u32(&empty[s]), ph ^ 1u, abort, p.err);
                 if (!got) {
                     ok = false;
                     break;
@@ -596,9 +600,7 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             do {
                 const uint32_t b = grp & 1u, use = grp >> 1;
                 if (u == 0) {
-                    bool got = true;
-                    if (lane == 0) got = wait_bounded(smem_u32(&tfull[b]), use & 1u, abort, p.err);
-                    got = __shfl_sync(0xffffffffu, got, 0);
+                    bool got = warp_wait(smem_u32(&tfull[b]), use & 1u, abort, p.err);
                     if (epi_any(!got)) {
                         ok = false;
                         break;
@@ -682,9 +684,7 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 
         for (int ng; !stop && (ng = it.take<G>(p, ncl, crank, gx, gt)) > 0; ++grp) {
             const uint32_t b = grp & 1u, use = grp >> 1;
-            bool got = true;
-            if (lane == 0) got = wait_bounded(smem_u32(&tfull[b]), use & 1u, abort, p.err);
-            got = __shfl_sync(0xffffffffu, got, 0);
+            bool got = warp_wait(smem_u32(&tfull[b]), use & 1u, abort, p.err);
             if (epi_any(!got)) {
                 stop = true;
                 break;

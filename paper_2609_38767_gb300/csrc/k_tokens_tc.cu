@@ -142,7 +142,7 @@ token_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     uint64_t* mma_done = bars + 14;
     uint32_t* tmem_slot = (uint32_t*)(bars + 17);
     volatile int* abort = (volatile int*)(tmem_slot + 1);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int i = 0; i < 2; ++i) {
             mbar_init(smem_u32(&a_raw[i]), 1);
@@ -172,9 +172,7 @@ token_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         uint32_t it = 0;
         for (int u = blockIdx.x; u < p.n_tt; u += gridDim.x, ++it) {
             const uint32_t ab = it % kABufs, ph = (it / kABufs) & 1u;
-            bool got = true;
-            if (lane == 0) got = wait_bounded(smem_u32(&a_raw[ab]), ph, abort, p.err);
-            got = __shfl_sync(0xffffffffu, got, 0);
+            bool got = warp_wait(smem_u32(&a_raw[ab]), ph, abort, p.err);
             if (!got) break;
             uint8_t* hi = abuf + ab * kABuf;
             uint8_t* lo = hi + KC * kATile;
@@ -194,28 +192,28 @@ token_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             if (lane == 0) mbar_arrive(smem_u32(&a_full[ab]));
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // ---------------- MMA issuer
-            constexpr uint32_t idesc = idesc_tf32(kTM, kTN);
-            uint32_t it = 0, rb = 0, tt = 0;
-            bool ok = true;
-            for (int u = blockIdx.x; ok && u < p.n_tt; u += gridDim.x, ++it) {
-                const uint32_t ab = it % kABufs;
-                if (!wait_bounded(smem_u32(&a_full[ab]), (it / kABufs) & 1u, abort, p.err)) break;
+        // ---------------- MMA issuer: the warp waits, one lane issues
+        constexpr uint32_t idesc = idesc_tf32(kTM, kTN);
+        uint32_t it = 0, rb = 0, tt = 0;
+        bool ok = true;
+        for (int u = blockIdx.x; ok && u < p.n_tt; u += gridDim.x, ++it) {
+            const uint32_t ab = it % kABufs;
+            if (!warp_wait(smem_u32(&a_full[ab]), (it / kABufs) & 1u, abort, p.err)) break;
+            tc_fence_after();
+            const uint32_t ahs = smem_u32(abuf + ab * kABuf);
+            for (int j = 0; j < p.n_nt; ++j, ++rb, ++tt) {
+                const uint32_t s = rb & 1u, b = tt & 1u;
+                if (!warp_wait(smem_u32(&tempty[b]), ((tt >> 1) & 1u) ^ 1u, abort, p.err) ||
+                    !warp_wait(smem_u32(&b_full[s]), (rb >> 1) & 1u, abort, p.err)) {
+                    ok = false;
+                    break;
+                }
                 tc_fence_after();
-                const uint32_t ahs = smem_u32(abuf + ab * kABuf);
-                for (int j = 0; j < p.n_nt; ++j, ++rb, ++tt) {
-                    const uint32_t s = rb & 1u, b = tt & 1u;
-                    if (!wait_bounded(smem_u32(&tempty[b]), ((tt >> 1) & 1u) ^ 1u, abort, p.err) ||
-                        !wait_bounded(smem_u32(&b_full[s]), (rb >> 1) & 1u, abort, p.err)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint32_t bhs = smem_u32(bbuf + s * kBBuf);
-                    const uint32_t d = tmem + b * C::kBufCols;
-                    // lo * hi and hi * lo of every k, then hi * hi (K = 8 tf32 = 32 bytes per instruction);
-                    // KC = 2: the first chunk's hi * hi in an accumulator of its own
+                const uint32_t bhs = smem_u32(bbuf + s * kBBuf);
+                const uint32_t d = tmem + b * C::kBufCols;
+                // lo * hi and hi * lo of every k, then hi * hi (K = 8 tf32 = 32 bytes per instruction);
+                // KC = 2: the first chunk's hi * hi in an accumulator of its own
+                if (elect_one()) {
 #pragma unroll
                     for (int pr = 0; pr < 3; ++pr)
 #pragma unroll
@@ -232,12 +230,17 @@ token_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     mma_commit(smem_u32(&b_empty[s]));
                     mma_commit(smem_u32(&tfull[b]));
                 }
-                if (!ok) break;
-                mma_commit(smem_u32(&a_empty[ab]));
+                __syncwarp();
             }
+            if (!ok) break;
+            if (elect_one()) mma_commit(smem_u32(&a_empty[ab]));
+            __syncwarp();
+        }
+        if (elect_one()) {
             mma_commit(smem_u32(mma_done));
             drain_wait(smem_u32(mma_done), 0, p.err);
         }
+        __syncwarp();
     } else if (warp == 2) {
         if (lane == 0) {
             // ---------------- TMA producer
@@ -305,9 +308,7 @@ token_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             prefetch(0);
             for (int j = 0; j < p.n_nt; ++j, ++tt) {
                 const uint32_t b = tt & 1u;
-                bool got = true;
-                if (lane == 0) got = wait_bounded(smem_u32(&tfull[b]), (tt >> 1) & 1u, abort, p.err);
-                got = __shfl_sync(0xffffffffu, got, 0);
+                bool got = warp_wait(smem_u32(&tfull[b]), (tt >> 1) & 1u, abort, p.err);
                 if (epi_any(!got)) {
                     stop = true;
                     break;
