@@ -1306,7 +1306,7 @@ constexpr int64_t kBlockedMinD = 2048;  // smaller layers keep the one-launch cl
 // above the diagonal inside each 64 x 64 diagonal block (solve_kernel reads it), the 32 x 32
 // inverses to Dinv (APPLY's other path). D = 4096, seven layers: 85 us a 128-column block as a
 // column-by-column left-looking factorisation, plus 49 us and 33 us for the second half's solve
-// and update as launches of their own; 114 us the 256 columns here.
+// and update as launches of their own; 97 us the 256 columns here.
 constexpr int kDiagThreads = 512;
 constexpr int kLdS = kBB + 4;  // 16-byte rows, four banks apart
 struct DiagSmem {
@@ -1333,28 +1333,35 @@ __device__ void factor128(float (*S)[kLdS], DiagSmem& sm, float* inv, int64_t co
                 const float4 v = *reinterpret_cast<const float4*>(&S[r][c0 + c]);
                 a[c] = v.x, a[c + 1] = v.y, a[c + 2] = v.z, a[c + 3] = v.w;
             }
-            if (r >= c0 && r < c0 + 16) sm.col[0][r - c0] = a[0];
-            bar_rows();
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                float cj[16];
+            const bool own = r >= c0 && r < c0 + 16;
+            float cj[16];
+            auto column = [&](int j) {  // the panel's diagonal rows of column j, to every row
+                if (own) sm.col[j & 1][r - c0] = a[j];
+                bar_rows();
 #pragma unroll
                 for (int c = 0; c < 16; c += 4) {
                     const float4 v = *reinterpret_cast<const float4*>(&sm.col[j & 1][c]);
                     cj[c] = v.x, cj[c + 1] = v.y, cj[c + 2] = v.z, cj[c + 3] = v.w;
                 }
+            };
+            column(0);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
                 const float p = cj[j], iv = p > 0.f ? rsqrtf(p) : NAN;
                 const float lr = a[j] * iv;  // L_rj (rows above the pivot: unused)
-                a[j] = lr;
+                float lc[16];                // L_cj
 #pragma unroll
-                for (int c = j + 1; c < 16; ++c) a[c] -= lr * (cj[c] * iv);
+                for (int c = j + 1; c < 16; ++c) lc[c] = cj[c] * iv;
+                a[j] = lr;
+                if (j < 15) {  // the next pivot's column first: its way to the other rows is the chain
+                    a[j + 1 < 16 ? j + 1 : 15] -= lr * lc[j < 15 ? j + 1 : 15];
+                    column(j < 15 ? j + 1 : 15);
+                }
+#pragma unroll
+                for (int c = j + 2; c < 16; ++c) a[c] -= lr * lc[c];
                 if (r == c0 + j) {
                     inv[c0 + j] = iv;
                     if (!(p > 0.f) && h[kPcFailedPivot] == 0.0) h[kPcFailedPivot] = (double)(col0 + c0 + j + 1);
-                }
-                if (j < 15) {
-                    if (r >= c0 && r < c0 + 16) sm.col[(j + 1) & 1][r - c0] = a[j < 15 ? j + 1 : 15];
-                    bar_rows();
                 }
             }
             if (r >= c0) {
@@ -1418,52 +1425,66 @@ __device__ void invert64(float (*S)[kLdS], DiagSmem& sm, const float* inv) {
     __syncthreads();
     // W10 = -W11 (L10 W00) for the two 64-blocks: thread (block, row i, four columns)
     float(*T)[kNB][kNB + 1] = reinterpret_cast<float(*)[kNB][kNB + 1]>(&sm.P[0][0]);
-    const int blk = tid >> 8, i = (tid >> 3) & 31, k0 = (tid & 7) * 4, lo = 64 * blk, hi = lo + kNB;
+    // (columns kq, kq + 8, ...: neighbouring lanes on neighbouring rows of W00, no bank conflicts)
+    const int blk = tid >> 8, i = (tid >> 3) & 31, kq = tid & 7, lo = 64 * blk, hi = lo + kNB;
     float t[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 8
-    for (int m = 0; m < kNB; ++m) {  // (L10 W00)[i][k] = sum_{m >= k} L10[i][m] W00[m][k]
-        const float l = S[hi + i][lo + m];
+#pragma unroll
+    for (int m = 0; m < kNB; m += 4) {  // (L10 W00)[i][k] = sum_{m >= k} L10[i][m] W00[m][k]
+        const float4 l4 = *reinterpret_cast<const float4*>(&S[hi + i][lo + m]);
+        const float l[4] = {l4.x, l4.y, l4.z, l4.w};
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-            const int k = k0 + v;
-            const float w = m > k ? S[lo + k][lo + m] : (m == k ? inv[lo + k] : 0.f);
-            t[v] = fmaf(l, w, t[v]);
+            const int k = kq + 8 * v;
+            const float4 w4 = *reinterpret_cast<const float4*>(&S[lo + k][lo + m]);
+            const float w[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                t[v] = fmaf(l[u], m + u > k ? w[u] : (m + u == k ? inv[lo + k] : 0.f), t[v]);
         }
     }
 #pragma unroll
-    for (int v = 0; v < 4; ++v) T[blk][i][k0 + v] = t[v];
+    for (int v = 0; v < 4; ++v) T[blk][i][kq + 8 * v] = t[v];
     __syncthreads();
     float o[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 8
     for (int m = 0; m < kNB; ++m) {  // W11[i][m], m <= i
         const float w = m < i ? S[hi + m][hi + i] : (m == i ? inv[hi + i] : 0.f);
 #pragma unroll
-        for (int v = 0; v < 4; ++v) o[v] = fmaf(w, T[blk][m][k0 + v], o[v]);
+        for (int v = 0; v < 4; ++v) o[v] = fmaf(w, T[blk][m][kq + 8 * v], o[v]);
     }
     __syncthreads();
 #pragma unroll
-    for (int v = 0; v < 4; ++v) S[lo + k0 + v][hi + i] = -o[v];
+    for (int v = 0; v < 4; ++v) S[lo + kq + 8 * v][hi + i] = -o[v];
     __syncthreads();
 }
 
-// Rows of S21 solved against S11: X L11^T = A, 64 columns at a time with W. 4 x 4 entries a thread.
+// Rows of S21 solved against S11: X L11^T = A, 64 columns at a time with W. A thread has four rows
+// and columns ci, ci + 16, ci + 32, ci + 48 (16 lanes on 16 neighbouring rows or columns of S11).
 __device__ void solve_half(DiagSmem& sm) {
-    const int tid = threadIdx.x, r0 = (tid >> 4) * 4, i0 = (tid & 15) * 4;
+    const int tid = threadIdx.x, r0 = (tid >> 4) * 4, ci = tid & 15;
     for (int b = 0; b < 2; ++b) {
         const int c0 = 64 * b;
         float acc[4][4];
+        auto store = [&]() {  // a row's 16 threads are half a warp: they alone read and write it
+            __syncwarp();
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int v = 0; v < 4; ++v) sm.S21[r0 + u][c0 + ci + 16 * v] = acc[u][v];
+            __syncwarp();
+        };
         if (b == 1) {  // columns 64..127 less the solved columns' share
 #pragma unroll
             for (int u = 0; u < 4; ++u)
 #pragma unroll
-                for (int v = 0; v < 4; ++v) acc[u][v] = sm.S21[r0 + u][c0 + i0 + v];
+                for (int v = 0; v < 4; ++v) acc[u][v] = sm.S21[r0 + u][c0 + ci + 16 * v];
 #pragma unroll 2
             for (int k = 0; k < 64; k += 4) {
                 float4 x[4], y[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     x[u] = *reinterpret_cast<const float4*>(&sm.S21[r0 + u][k]);
-                    y[u] = *reinterpret_cast<const float4*>(&sm.S11[c0 + i0 + u][k]);
+                    y[u] = *reinterpret_cast<const float4*>(&sm.S11[c0 + ci + 16 * u][k]);
                 }
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
@@ -1471,37 +1492,40 @@ __device__ void solve_half(DiagSmem& sm) {
                     for (int v = 0; v < 4; ++v)
                         acc[u][v] -= x[u].x * y[v].x + x[u].y * y[v].y + x[u].z * y[v].z + x[u].w * y[v].w;
             }
-            __syncthreads();
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                *reinterpret_cast<float4*>(&sm.S21[r0 + u][c0 + i0]) =
-                    make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]);
-            __syncthreads();
+            store();
         }
+        float iv[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) iv[v] = sm.inv[0][c0 + ci + 16 * v];
 #pragma unroll
         for (int u = 0; u < 4; ++u)
 #pragma unroll
             for (int v = 0; v < 4; ++v) acc[u][v] = 0.f;
         // out[r][i] = sum_{k <= i} x[r][k] W[i][k], W[i][k] = S11[c0 + k][c0 + i] for k < i
-        for (int k = 0; k < i0 + 4; ++k) {
-            float w[4];
 #pragma unroll
-            for (int v = 0; v < 4; ++v)
-                w[v] = k < i0 + v ? sm.S11[c0 + k][c0 + i0 + v] : (k == i0 + v ? sm.inv[0][c0 + k] : 0.f);
+        for (int k = 0; k < 64; k += 4) {
+            float x[4][4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const float x = sm.S21[r0 + u][c0 + k];
+                const float4 q = *reinterpret_cast<const float4*>(&sm.S21[r0 + u][c0 + k]);
+                x[u][0] = q.x, x[u][1] = q.y, x[u][2] = q.z, x[u][3] = q.w;
+            }
 #pragma unroll
-                for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(x, w[v], acc[u][v]);
+            for (int v = 0; v < 4; ++v) {
+                if (k >= 16 * v + 16) continue;  // W is lower triangular
+                const int i = ci + 16 * v;
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    const float s = sm.S11[c0 + k + t][c0 + i];
+                    const float w = k + t < i ? s : (k + t == i ? iv[v] : 0.f);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) acc[u][v] = fmaf(x[u][t], w, acc[u][v]);
+                }
             }
         }
-        __syncthreads();
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            *reinterpret_cast<float4*>(&sm.S21[r0 + u][c0 + i0]) =
-                make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]);
-        __syncthreads();
+        store();
     }
+    __syncthreads();
 }
 
 __global__ void __launch_bounds__(kDiagThreads) diag_panel_kernel(St<float> st, int64_t lo) {
@@ -1533,23 +1557,23 @@ __global__ void __launch_bounds__(kDiagThreads) diag_panel_kernel(St<float> st, 
     invert64(sm.S11, sm, sm.inv[0]);
     if (two) {
         solve_half(sm);
-        // S22 -= L21 L21^T on and below the diagonal: 8 x 4 tiles
+        // S22 -= L21 L21^T on and below the diagonal: tiles of 8 rows by 4 columns, the
+        // columns 2 (ti + 1) apart so that neighbouring lanes read neighbouring rows of S21 (no bank conflicts)
         for (int u = tid; u < 16 * 17; u += kDiagThreads) {
-            // row pairs of 4-wide tiles: tile row ti has 2 (ti + 1) tiles
+            // tile row ti has 2 (ti + 1) tiles
             int ti = (int)((sqrtf(4.f * (float)u + 1.f) - 1.f) * 0.5f);
             while (ti * (ti + 1) > u) --ti;
             while ((ti + 1) * (ti + 2) <= u) ++ti;
-            const int i0 = 8 * ti, j0 = 4 * (u - ti * (ti + 1));
+            const int i0 = 8 * ti, j0 = u - ti * (ti + 1), js = 2 * (ti + 1);  // columns j0 + js v
             float acc[8][4];
 #pragma unroll
-            for (int a = 0; a < 8; ++a) {
-                const float4 v = *reinterpret_cast<const float4*>(&sm.S22[i0 + a][j0]);
-                acc[a][0] = v.x, acc[a][1] = v.y, acc[a][2] = v.z, acc[a][3] = v.w;
-            }
+            for (int a = 0; a < 8; ++a)
+#pragma unroll
+                for (int v = 0; v < 4; ++v) acc[a][v] = sm.S22[i0 + a][j0 + js * v];
             for (int k = 0; k < kBB; k += 4) {
                 float4 y[4];
 #pragma unroll
-                for (int v = 0; v < 4; ++v) y[v] = *reinterpret_cast<const float4*>(&sm.S21[j0 + v][k]);
+                for (int v = 0; v < 4; ++v) y[v] = *reinterpret_cast<const float4*>(&sm.S21[j0 + js * v][k]);
 #pragma unroll
                 for (int a = 0; a < 8; ++a) {
                     const float4 x = *reinterpret_cast<const float4*>(&sm.S21[i0 + a][k]);
@@ -1560,7 +1584,8 @@ __global__ void __launch_bounds__(kDiagThreads) diag_panel_kernel(St<float> st, 
             }
 #pragma unroll
             for (int a = 0; a < 8; ++a)
-                *reinterpret_cast<float4*>(&sm.S22[i0 + a][j0]) = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
+#pragma unroll
+                for (int v = 0; v < 4; ++v) sm.S22[i0 + a][j0 + js * v] = acc[a][v];
         }
         __syncthreads();
         factor128(sm.S22, sm, sm.inv[1], lo + kBB, h);
