@@ -318,7 +318,7 @@ token_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 float acc[G];
 #pragma unroll
                 for (int gq = 0; gq < G; ++gq) {
-                    float s = 0.f, s1 = 0.f;
+                    float sum[4] = {0.f, 0.f, 0.f, 0.f};  // four chains: less rounding
 #pragma unroll
                     for (int c = 0; c < KG; c += 16) {
                         float v[16];
@@ -330,12 +330,9 @@ token_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                             for (int i = 0; i < 16; ++i) v[i] += w[i];
                         }
 #pragma unroll
-                        for (int i = 0; i < 16; i += 2) {
-                            s = fmaf(g[c + i], v[i], s);
-                            s1 = fmaf(g[c + i + 1], v[i + 1], s1);
-                        }
+                        for (int i = 0; i < 16; ++i) sum[i & 3] = fmaf(g[c + i], v[i], sum[i & 3]);
                     }
-                    s += s1;
+                    const float s = (sum[0] + sum[1]) + (sum[2] + sum[3]);
                     acc[gq] = rmw ? p.beta * old[gq] + p.scale * s : p.scale * s;
                 }
                 tc_fence_before();
