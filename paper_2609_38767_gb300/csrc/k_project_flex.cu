@@ -31,7 +31,7 @@
 // pair of generator warps, each taking every other stage, measured 6 % slower).
 //
 // Measured, fp32: 64 examples of 512 tokens, 2048 -> 2048, k = 32 (537 MB): 7.6 ms
-// on the CUDA cores, 136 us here. bf16: see plan_bf16_flex().
+// on the CUDA cores, 102 us here. bf16: see plan_bf16_flex().
 //
 // Warp roles (fp32 512, bf16 256 threads, one persistent CTA per SM): warp 0 TMA
 // producer; warp 1 TMEM allocator and MMA issuer; warps 2-3 sign generators;
@@ -617,13 +617,27 @@ int max_clusters(int cs) {
     return n;
 }
 
+// Clocks of a 64-feature chunk, measured over 1 to 700 examples of 20 to 1024 tokens. Here: 4.2 a bf16
+// row of the tile (what one SM draws from L2 and HBM), 9 an fp32 row, at least the signs and the
+// barriers of a stage, or the splitting of fp32 rows.
+// k_project_tc.cu: per 128-row tile, without and with the workspace's equal runs (bal).
+template <int K, bool F32>
+double chunk_clocks(int R) {
+    const double data = R * (F32 ? 9.0 : 4.2), least = F32 ? 800.0 : (K <= 16 ? 430.0 : (K <= 32 ? 460.0 : 670.0));
+    return data > least ? data : least;
+}
+double stream_chunk_clocks(int K, bool bal) { return K >= 64 ? 950.0 : (bal ? 600.0 : 560.0); }
+double row_clocks(int K) { return K >= 64 ? 110.0 : (K >= 32 ? 50.0 : 35.0); }  // contraction of a token row
+double hbm_clocks(const tda_layer_desc& L, int64_t N, int el, int sms) {        // 22 bytes a clock and SM
+    return (double)N * L.T * (L.d_in + L.d_out) * el / (22.0 * sms);
+}
+
 // bf16 with k_in = k_out in {16, 32, 64}: whether this kernel's plan beats the streaming kernel of
 // k_project_tc.cu. That one takes 128-row tiles, whole examples per CTA, clusters of 2 or 4 below one
-// example per SM, or with the workspace (bal) equal runs of tiles; its chunk takes 960 clocks (as
-// above), at k = 64 1100, and 1350 without the workspace's smaller staging (the sign warps). 64
-// examples of 1024 tokens, 4096 -> 4096, k = 64 with the workspace: 302 us there, 224 us here; 16
-// of them: 97 us there, 120 us here. With two tiles a stage (four tiles per SM and more) and whole examples or equal runs for every SM it runs at HBM
-// speed and is kept.
+// example per SM, or with the workspace (bal) equal runs of tiles. With two tiles a stage (four
+// tiles per SM and more) and whole examples or equal runs for every SM it runs at HBM speed and is
+// kept. 4096 -> 4096, k = 64: 64 examples of 1024 tokens with the workspace 241 us there and 209 us
+// here, 16 of them 84 us there and 114 us here, without the workspace 130 us there.
 bool plan_bf16_flex(const tda_layer_desc& L, int64_t N, int sms, double cost, int K, bool bal) {
     const int pack = L.T <= 64 ? (int)(kTileM / L.T) : 1;
     const int64_t slots = (N + pack - 1) / pack, nt = pack > 1 ? 1 : (L.T + kTileM - 1) / kTileM;
@@ -634,13 +648,12 @@ bool plan_bf16_flex(const tda_layer_desc& L, int64_t N, int sms, double cost, in
     if (pack == 1 && N < sms) cs = 2 * N >= sms ? 2 : 4;
     while (cs > nt) cs >>= 1;
     const double chunks = (double)((L.d_in + kChunkK - 1) / kChunkK + (L.d_out + kChunkK - 1) / kChunkK);
-    const double t = K >= 64 ? (bal ? 1100.0 : 1350.0) : 960.0;
     const int64_t room = sms / cs, rounds = (slots + room - 1) / room;
-    const double tile = chunks * t + kTileM * (K >= 64 ? 45.0 : 20.0);
-    if (bal) return cost < 0.95 * ((double)((slots * nt + sms - 1) / sms) * tile + 3000.0);
-    const double mine = (double)rounds * ((nt + cs - 1) / cs) * tile +
-                        rounds * (cs > 1 ? 3000.0 : 500.0);
-    return cost < 0.95 * mine;
+    const double tile = chunks * stream_chunk_clocks(K, bal) + kTileM * row_clocks(K), hbm = hbm_clocks(L, N, 2, sms);
+    double stream = bal ? (double)((slots * nt + sms - 1) / sms) * tile + 3000.0
+                        : rounds * ((double)((nt + cs - 1) / cs) * tile + (cs > 1 ? 3000.0 : 500.0));
+    if (stream < hbm) stream = hbm;
+    return cost < 0.97 * stream;
 }
 
 struct Plan {
@@ -649,25 +662,23 @@ struct Plan {
     double cost;  // clocks
 };
 
-// Tile rows and cluster size with the least time of the busiest CTA: its tiles times the time of a
-// 64-feature chunk (one SM draws about 17 bytes a clock from HBM however few others do: 7.5 clocks a
-// bf16 row, 15 an fp32 row; at least 400 for the signs and the barriers), but at least what HBM
-// takes in all (22 bytes a clock and SM); ties go to fewer, larger tiles and smaller clusters. A
-// tile's contraction and an example's reduction count too. T past a multiple of the tile is cut into equal tiles (T = 130: two of 65 rows).
+// Tile rows and cluster size with the least time of the busiest CTA (its tiles, their contraction, the
+// reductions over the cluster), but at least what HBM takes in all; ties go to fewer, larger tiles and
+// smaller clusters. T past a multiple of the tile is cut into equal tiles (T = 130: two of 65 rows).
 template <int K, bool F32>
 Plan plan(const tda_layer_desc& L, int64_t N, int sms) {
     Plan best{};
     const double chunks = (double)((L.d_in + kChunkK - 1) / kChunkK + (L.d_out + kChunkK - 1) / kChunkK);
-    const double floor_clk = (double)N * L.T * (L.d_in + L.d_out) * (F32 ? 4.0 : 2.0) / (22.0 * sms);
+    const double floor_clk = hbm_clocks(L, N, F32 ? 4 : 2, sms);
     auto consider = [&](int R, int pack, int nt) {
-        const double t = R * (F32 ? 15.0 : 7.5) > 400.0 ? R * (F32 ? 15.0 : 7.5) : 400.0;
+        const double t = chunk_clocks<K, F32>(R);
         const int64_t slots = (N + pack - 1) / pack;
         for (int cs = 1; cs <= 8 && cs <= nt; cs *= 2) {
             const int64_t room = sms / cs, fit = max_clusters<K, F32>(cs) < room ? max_clusters<K, F32>(cs) : room;
             if (fit < 1) continue;
             const int64_t clusters = slots < fit ? slots : fit, rounds = (slots + clusters - 1) / clusters;
             const double tiles = (double)rounds * ((nt + cs - 1) / cs);
-            double cost = tiles * (chunks * t + R * (K >= 64 ? 45.0 : 20.0)) + rounds * (cs > 1 ? 3000.0 : 500.0);
+            double cost = tiles * (chunks * t + R * row_clocks(K)) + rounds * (cs > 1 ? 3000.0 : 500.0);
             if (cost < floor_clk) cost = floor_clk;
             if (best.R == 0 || cost < best.cost * 0.98) best = Plan{R, cs, pack, nt, slots, clusters, cost};
         }
