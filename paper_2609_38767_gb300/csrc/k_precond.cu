@@ -1306,13 +1306,12 @@ constexpr int64_t kBlockedMinD = 2048;  // smaller layers keep the one-launch cl
 // above the diagonal inside each 64 x 64 diagonal block (solve_kernel reads it), the 32 x 32
 // inverses to Dinv (APPLY's other path). D = 4096, seven layers: 85 us a 128-column block as a
 // column-by-column left-looking factorisation, plus 49 us and 33 us for the second half's solve
-// and update as launches of their own; 97 us the 256 columns here.
+// and update as launches of their own; 73 us the 256 columns here.
 constexpr int kDiagThreads = 512;
 constexpr int kLdS = kBB + 4;  // 16-byte rows, four banks apart
 struct DiagSmem {
-    float S11[kBB][kLdS];
+    float S[2][kBB][kLdS];  // the halves' diagonal blocks
     float S21[kBB][kLdS];
-    float S22[kBB][kLdS];
     float P[16][kLdS];      // a 16-column panel, transposed; invert64's scratch
     float inv[2][kBB];      // 1 / L_jj of both halves
     float col[2][16];       // the pivot column's entries in the panel's diagonal rows
@@ -1322,8 +1321,10 @@ static_assert(sizeof(float) * 2 * 32 * 33 <= sizeof(float) * 16 * kLdS, "invert6
 
 __device__ __forceinline__ void bar_rows() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 
-__device__ void factor128(float (*S)[kLdS], DiagSmem& sm, float* inv, int64_t col0, double* h) {
+__device__ __forceinline__ void factor128(DiagSmem& sm, int half, int64_t col0, double* h) {
     const int tid = threadIdx.x;
+    float(*S)[kLdS] = sm.S[half];
+    float* inv = sm.inv[half];
     for (int c0 = 0; c0 < kBB; c0 += 16) {
         if (tid < kBB) {
             const int r = tid;
@@ -1405,7 +1406,9 @@ __device__ void factor128(float (*S)[kLdS], DiagSmem& sm, float* inv, int64_t co
 }
 
 // W^T of both 64 x 64 diagonal blocks into their strict upper triangles (W's diagonal is inv).
-__device__ void invert64(float (*S)[kLdS], DiagSmem& sm, const float* inv) {
+__device__ __forceinline__ void invert64(DiagSmem& sm, int half) {
+    float(*S)[kLdS] = sm.S[half];
+    const float* inv = sm.inv[half];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (warp < 4) {  // 32 x 32 block `warp`: lane c solves L X[:, c] = e_c, column order
         const int b0 = warp * kNB, c = lane;
@@ -1458,9 +1461,9 @@ __device__ void invert64(float (*S)[kLdS], DiagSmem& sm, const float* inv) {
     __syncthreads();
 }
 
-// Rows of S21 solved against S11: X L11^T = A, 64 columns at a time with W. A thread has four rows
+// Rows of S21 solved against the first block, S11: X L11^T = A, 64 columns at a time with W. A thread has four rows
 // and columns ci, ci + 16, ci + 32, ci + 48 (16 lanes on 16 neighbouring rows or columns of S11).
-__device__ void solve_half(DiagSmem& sm) {
+__device__ __forceinline__ void solve_half(DiagSmem& sm) {
     const int tid = threadIdx.x, r0 = (tid >> 4) * 4, ci = tid & 15;
     for (int b = 0; b < 2; ++b) {
         const int c0 = 64 * b;
@@ -1484,7 +1487,7 @@ __device__ void solve_half(DiagSmem& sm) {
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     x[u] = *reinterpret_cast<const float4*>(&sm.S21[r0 + u][k]);
-                    y[u] = *reinterpret_cast<const float4*>(&sm.S11[c0 + ci + 16 * u][k]);
+                    y[u] = *reinterpret_cast<const float4*>(&sm.S[0][c0 + ci + 16 * u][k]);
                 }
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
@@ -1501,7 +1504,7 @@ __device__ void solve_half(DiagSmem& sm) {
         for (int u = 0; u < 4; ++u)
 #pragma unroll
             for (int v = 0; v < 4; ++v) acc[u][v] = 0.f;
-        // out[r][i] = sum_{k <= i} x[r][k] W[i][k], W[i][k] = S11[c0 + k][c0 + i] for k < i
+        // out[r][i] = sum_{k <= i} x[r][k] W[i][k], W[i][k] = S[0][c0 + k][c0 + i] for k < i
 #pragma unroll
         for (int k = 0; k < 64; k += 4) {
             float x[4][4];
@@ -1516,7 +1519,7 @@ __device__ void solve_half(DiagSmem& sm) {
                 const int i = ci + 16 * v;
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
-                    const float s = sm.S11[c0 + k + t][c0 + i];
+                    const float s = sm.S[0][c0 + k + t][c0 + i];
                     const float w = k + t < i ? s : (k + t == i ? iv[v] : 0.f);
 #pragma unroll
                     for (int u = 0; u < 4; ++u) acc[u][v] = fmaf(x[u][t], w, acc[u][v]);
@@ -1537,25 +1540,30 @@ __global__ void __launch_bounds__(kDiagThreads) diag_panel_kernel(St<float> st, 
     double* h = st.header(l);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool two = lo + kBB < D;
-    // a warp per row, 16 bytes a lane
+    // a warp per row, 16 bytes a lane, nothing above the diagonal (one SM draws 17 bytes a clock)
 #pragma unroll 4
     for (int r = warp; r < kBB; r += kDiagThreads / 32) {
         const int c = 4 * lane;
-        float4 v = *reinterpret_cast<const float4*>(M + (lo + r) * D + lo + c);
-        float* d = &sm.S11[r][c];
-        d[0] = c <= r ? v.x : 0.f, d[1] = c + 1 <= r ? v.y : 0.f, d[2] = c + 2 <= r ? v.z : 0.f, d[3] = c + 3 <= r ? v.w : 0.f;
+        auto diagonal = [&](int half) {
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (c <= r) v = *reinterpret_cast<const float4*>(M + (lo + half * kBB + r) * D + lo + half * kBB + c);
+            *reinterpret_cast<float4*>(&sm.S[half][r][c]) =
+                make_float4(v.x, c + 1 <= r ? v.y : 0.f, c + 2 <= r ? v.z : 0.f, c + 3 <= r ? v.w : 0.f);
+        };
+        diagonal(0);
         if (two) {
             *reinterpret_cast<float4*>(&sm.S21[r][c]) =
                 *reinterpret_cast<const float4*>(M + (lo + kBB + r) * D + lo + c);
-            v = *reinterpret_cast<const float4*>(M + (lo + kBB + r) * D + lo + kBB + c);
-            d = &sm.S22[r][c];
-            d[0] = c <= r ? v.x : 0.f, d[1] = c + 1 <= r ? v.y : 0.f, d[2] = c + 2 <= r ? v.z : 0.f, d[3] = c + 3 <= r ? v.w : 0.f;
+            diagonal(1);
         }
     }
     __syncthreads();
-    factor128(sm.S11, sm, sm.inv[0], lo, h);
-    invert64(sm.S11, sm, sm.inv[0]);
-    if (two) {
+    // a loop and not two copies: every launch starts with a cold instruction cache
+#pragma unroll 1
+    for (int half = 0; half < (two ? 2 : 1); ++half) {
+        factor128(sm, half, lo + half * kBB, h);
+        invert64(sm, half);
+        if (half == 1 || !two) break;
         solve_half(sm);
         // S22 -= L21 L21^T on and below the diagonal: tiles of 8 rows by 4 columns, the
         // columns 2 (ti + 1) apart so that neighbouring lanes read neighbouring rows of S21 (no bank conflicts)
@@ -1569,7 +1577,8 @@ __global__ void __launch_bounds__(kDiagThreads) diag_panel_kernel(St<float> st, 
 #pragma unroll
             for (int a = 0; a < 8; ++a)
 #pragma unroll
-                for (int v = 0; v < 4; ++v) acc[a][v] = sm.S22[i0 + a][j0 + js * v];
+                for (int v = 0; v < 4; ++v) acc[a][v] = sm.S[1][i0 + a][j0 + js * v];
+#pragma unroll 2
             for (int k = 0; k < kBB; k += 4) {
                 float4 y[4];
 #pragma unroll
@@ -1585,18 +1594,16 @@ __global__ void __launch_bounds__(kDiagThreads) diag_panel_kernel(St<float> st, 
 #pragma unroll
             for (int a = 0; a < 8; ++a)
 #pragma unroll
-                for (int v = 0; v < 4; ++v) sm.S22[i0 + a][j0 + js * v] = acc[a][v];
+                for (int v = 0; v < 4; ++v) sm.S[1][i0 + a][j0 + js * v] = acc[a][v];
         }
         __syncthreads();
-        factor128(sm.S22, sm, sm.inv[1], lo + kBB, h);
-        invert64(sm.S22, sm, sm.inv[1]);
     }
     // L on and below the diagonal, W^T above it inside the 64 x 64 diagonal blocks (the rest of a
     // half's upper triangle is the other 64-block's, written by upper_from_lower_kernel)
     for (int r = warp; r < kBB; r += kDiagThreads / 32) {
         const int c = 4 * lane;
         for (int half = 0; half < (two ? 2 : 1); ++half) {
-            const float* src = half ? &sm.S22[r][c] : &sm.S11[r][c];
+            const float* src = &sm.S[half][r][c];
             float* dst = M + (lo + half * kBB + r) * D + lo + half * kBB + c;
             if (c / 64 <= r / 64) *reinterpret_cast<float4*>(dst) = *reinterpret_cast<const float4*>(src);
         }
@@ -1606,7 +1613,7 @@ __global__ void __launch_bounds__(kDiagThreads) diag_panel_kernel(St<float> st, 
     float* Dg = st.Dinv(l) + (lo / kNB) * (kNB * kNB);
     for (int e = tid; e < (two ? 8 : 4) * kNB * kNB; e += kDiagThreads) {
         const int b = e >> 10, r = (e >> 5) & 31, c = e & 31, half = b >> 2, o = (b & 3) * kNB;
-        const float(*S)[kLdS] = half ? sm.S22 : sm.S11;
+        const float(*S)[kLdS] = sm.S[half];
         Dg[e] = c < r ? S[o + c][o + r] : (c == r ? sm.inv[half][o + r] : 0.f);
     }
 }
