@@ -63,6 +63,10 @@ struct GParams {
     int batched;           // grid z = batch entry: A and B maps are 3-D (z the third coordinate)
     int64_t s_z;           // S element offset between batch entries
     int64_t tiles_z;       // persistent kernel: tiles per batch entry
+    int64_t tiles_1;       // of which with the first B (all, without a second product)
+    int tiles_n2;          // second product, the same A: its tiles along B, B2 rows, output
+    int64_t n_q2, ld_S2, s_z2;
+    float* S2;
     int nz;                // persistent kernel: batch entries
     unsigned int* err;
 };
@@ -495,6 +499,7 @@ __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.
 struct TileAt {
     int64_t m0, n0;
     int z, y;
+    bool second;
 };
 template <int BN, bool PAIR>
 __device__ __forceinline__ TileAt tile_at(const GParams& p, int64_t t, uint32_t rank) {
@@ -504,7 +509,11 @@ __device__ __forceinline__ TileAt tile_at(const GParams& p, int64_t t, uint32_t 
     t -= (int64_t)a.z * per_z;
     a.y = (int)(t / p.tiles_z);
     const int64_t tile = t - (int64_t)a.y * p.tiles_z;
-    if (p.lower && PAIR) {
+    a.second = PAIR && tile >= p.tiles_1;
+    if (a.second) {
+        a.m0 = (tile - p.tiles_1) / p.tiles_n2 * (2 * kBM);
+        a.n0 = (tile - p.tiles_1) % p.tiles_n2 * BN;
+    } else if (p.lower && PAIR) {
         // row tiles 2q and 2q + 1 of B have q + 1 tiles of A each
         int64_t q = (int64_t)(sqrtf((float)tile + 0.25f) - 0.5f);
         while (q * (q + 1) > tile) --q;
@@ -534,7 +543,8 @@ __device__ __forceinline__ int64_t chunks_of(const GParams& p, int y) {
 
 template <int BN, bool PAIR, bool FIT>
 __global__ void __launch_bounds__(kThreadsT, 1)
-gemm3t_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GParams p) {
+gemm3t_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+              const __grid_constant__ CUtensorMap tmB2, const GParams p) {
     using C = TCfg<BN, PAIR>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -701,9 +711,10 @@ gemm3t_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             const uint32_t groups = (uint32_t)((chunks_of(p, at.y) + C::kGroup - 1) / C::kGroup);
             const int64_t m = at.m0 + row, nb = at.n0 + half * C::kCols;
             // (the upper half of a pair's tile on the diagonal lies above it)
-            const bool write = !(PAIR && p.lower && at.m0 > at.n0);
-            float* Sz = p.S + (int64_t)at.y * p.slab + (int64_t)at.z * p.s_z + m;
-            const int lim = (int)(p.n_q - nb < C::kCols ? p.n_q - nb : C::kCols);
+            const bool write = !(PAIR && p.lower && !at.second && at.m0 > at.n0);
+            float* Sz = (at.second ? p.S2 + (int64_t)at.z * p.s_z2 : p.S + (int64_t)at.y * p.slab + (int64_t)at.z * p.s_z) + m;
+            const int64_t ld_S = at.second ? p.ld_S2 : p.ld_S, n_q = at.second ? p.n_q2 : p.n_q;
+            const int lim = (int)(n_q - nb < C::kCols ? n_q - nb : C::kCols);
             // the previous values start on their way to L2: short products (256 features) end before
             // HBM has answered (rank-256 updates of 7 x 4096: 85 -> 77 us on average). A warp's 32 values of a
             // column are one or two lines.
@@ -711,7 +722,7 @@ gemm3t_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
 #pragma unroll
                 for (int c = lane; c < C::kCols; c += 32)
                     if (c < lim && at.m0 + q4 * 32 < p.n_t)
-                        asm volatile("prefetch.global.L2 [%0];" ::"l"(Sz - lane + (nb + c) * p.ld_S));
+                        asm volatile("prefetch.global.L2 [%0];" ::"l"(Sz - lane + (nb + c) * ld_S));
             float acc[C::kCols];
 #pragma unroll
             for (int c = 0; c < C::kCols; ++c) acc[c] = 0.f;
@@ -735,17 +746,17 @@ gemm3t_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             if (p.beta == 0.f) {
 #pragma unroll
                 for (int c = 0; c < C::kCols; ++c)
-                    if (c < lim) Sz[(nb + c) * p.ld_S] = p.alpha * acc[c];
+                    if (c < lim) Sz[(nb + c) * ld_S] = p.alpha * acc[c];
             } else {
                 // 8 previous values are on their way together
 #pragma unroll
                 for (int c0 = 0; c0 < C::kCols; c0 += 8) {
                     float old[8];
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) old[i] = c0 + i < lim ? __ldcg(Sz + (nb + c0 + i) * p.ld_S) : 0.f;
+                    for (int i = 0; i < 8; ++i) old[i] = c0 + i < lim ? __ldcg(Sz + (nb + c0 + i) * ld_S) : 0.f;
 #pragma unroll
                     for (int i = 0; i < 8; ++i)
-                        if (c0 + i < lim) Sz[(nb + c0 + i) * p.ld_S] = p.beta * old[i] + p.alpha * acc[c0 + i];
+                        if (c0 + i < lim) Sz[(nb + c0 + i) * ld_S] = p.beta * old[i] + p.alpha * acc[c0 + i];
                 }
             }
         }
@@ -777,10 +788,10 @@ gemm3t_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                         tma_load_2d(st + C::kABytes + 4096u * b, &tmA, x + n0 + 32 * b, k, bar);
                 } else if (p.batched) {
                     tma_load_3d(st, &tmA, k, m0, at.z, bar);
-                    tma_load_3d(st + C::kABytes, &tmB, k, n0, at.z, bar);
+                    tma_load_3d(st + C::kABytes, at.second ? &tmB2 : &tmB, k, n0, at.z, bar);
                 } else {
                     tma_load_2d(st, &tmA, k, m0, bar);
-                    tma_load_2d(st + C::kABytes, &tmB, k, n0, bar);
+                    tma_load_2d(st + C::kABytes, at.second ? &tmB2 : &tmB, k, n0, bar);
                 }
                 issued[r] = true;
                 last_par[r] = ph;
@@ -910,7 +921,8 @@ int64_t pair_lower_tiles(int64_t nt) {
 }
 
 template <int BN, bool FIT>
-cudaError_t launch_pairs(const CUtensorMap& tmA, const CUtensorMap& tmB, const GParams& p, int sms, cudaStream_t s) {
+cudaError_t launch_pairs(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmB2, const GParams& p,
+                         int sms, cudaStream_t s) {
     using T = TCfg<BN, true>;
     cudaError_t e = smem_attr_once<gemm3t_kernel<BN, true, FIT>>((int)T::kSmem);
     if (e != cudaSuccess) return e;
@@ -928,12 +940,13 @@ cudaError_t launch_pairs(const CUtensorMap& tmA, const CUtensorMap& tmB, const G
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     note_launches(1);
-    e = cudaLaunchKernelEx(&cfg, gemm3t_kernel<BN, true, FIT>, tmA, tmB, p);
+    e = cudaLaunchKernelEx(&cfg, gemm3t_kernel<BN, true, FIT>, tmA, tmB, tmB2, p);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <int BN>
-cudaError_t launch_bn(GParams p, cudaStream_t s, int64_t nz = 1, size_t a_z_bytes = 0, size_t b_z_bytes = 0) {
+cudaError_t launch_bn(GParams p, cudaStream_t s, int64_t nz = 1, size_t a_z_bytes = 0, size_t b_z_bytes = 0,
+                      const GemmSecond* second = nullptr) {
     using C = GCfg<BN>;
     CUtensorMap tmA, tmB;
     if (nz > 1) {
@@ -956,7 +969,7 @@ cudaError_t launch_bn(GParams p, cudaStream_t s, int64_t nz = 1, size_t a_z_byte
     const int64_t nkc = ((p.kslice ? p.kslice : p.K) + kKC - 1) / kKC;
     int cs = 1;
     // split K over a cluster only while the tiles of all batch entries leave SMs idle
-    while (cs < 4 && tiles * p.splits * nz * cs * 2 <= sms && nkc >= 8 * cs * 2) cs *= 2;
+    while (!second && cs < 4 && tiles * p.splits * nz * cs * 2 <= sms && nkc >= 8 * cs * 2) cs *= 2;
     // the leader's stage buffers must hold the members' partial tiles
     while (cs > 1 && (size_t)(cs - 1) * kBM * BN * 4 > (size_t)C::kStages * C::kStageBytes) cs >>= 1;
     p.cs = cs;
@@ -965,15 +978,30 @@ cudaError_t launch_bn(GParams p, cudaStream_t s, int64_t nz = 1, size_t a_z_byte
         p.nz = (int)nz;
         // A pair's chunk takes about three quarters of a single CTA's (see above), so its whole rounds of
         // tiles decide: few or odd 128-row tiles can leave half of the pairs' rows empty.
-        const int64_t pairs = p.lower ? pair_lower_tiles(tiles_n) : (tiles_m + 1) / 2 * tiles_n;
+        int64_t pairs = p.lower ? pair_lower_tiles(tiles_n) : (tiles_m + 1) / 2 * tiles_n;
+        CUtensorMap tmB2 = tmB;
+        if (second) {  // always in pairs
+            p.tiles_1 = pairs;
+            p.tiles_n2 = (int)((second->n_b + BN - 1) / BN);
+            pairs += (tiles_m + 1) / 2 * p.tiles_n2;
+            p.n_q2 = second->n_b;
+            p.S2 = second->C;
+            p.ld_S2 = second->ldc;
+            p.s_z2 = second->c_z;
+            if (nz > 1 ? !make_map_f32_3d(&tmB2, second->B, second->n_b, p.K, second->ldb, nz, second->b_z_bytes, BN / 2)
+                       : !make_map_f32(&tmB2, second->B, second->n_b, p.K, second->ldb, BN / 2))
+                return cudaErrorInvalidValue;
+        } else {
+            p.tiles_1 = pairs;
+        }
         const int64_t per = (int64_t)p.splits * nz, half = sms > 1 ? sms / 2 : 1;
-        if (3 * ((pairs * per + half - 1) / half) <= 4 * ((tiles * per + sms - 1) / sms)) {
+        if (second || 3 * ((pairs * per + half - 1) / half) <= 4 * ((tiles * per + sms - 1) / sms)) {
             p.tiles_z = pairs;
             // B's box: the half of a tile's rows that one CTA of the pair loads
             if (nz > 1 ? !make_map_f32_3d(&tmB, p.B, p.n_q, p.K, p.ldb, nz, b_z_bytes, BN / 2)
                        : !make_map_f32(&tmB, p.B, p.n_q, p.K, p.ldb, BN / 2))
                 return cudaErrorInvalidValue;
-            return launch_pairs<BN, false>(tmA, tmB, p, sms, s);
+            return launch_pairs<BN, false>(tmA, tmB, tmB2, p, sms, s);
         }
         using T = TCfg<BN, false>;
         p.tiles_z = tiles;
@@ -981,9 +1009,10 @@ cudaError_t launch_bn(GParams p, cudaStream_t s, int64_t nz = 1, size_t a_z_byte
         cudaError_t e = smem_attr_once<gemm3t_kernel<BN, false, false>>((int)T::kSmem);
         if (e != cudaSuccess) return e;
         note_launches(1);
-        gemm3t_kernel<BN, false, false><<<(unsigned)(total < sms ? total : sms), kThreadsT, T::kSmem, s>>>(tmA, tmB, p);
+        gemm3t_kernel<BN, false, false><<<(unsigned)(total < sms ? total : sms), kThreadsT, T::kSmem, s>>>(tmA, tmB, tmB, p);
         return cudaGetLastError();
     }
+    if (second) return cudaErrorInvalidValue;
     // few tiles: a cluster of cs CTAs splits K
     cudaError_t e = smem_attr_once<score3x_kernel<BN>>((int)C::kSmem);
     if (e != cudaSuccess) return e;
@@ -1084,26 +1113,16 @@ cudaError_t launch_score_tc_slices(const float* Qhat, int64_t n_q, int64_t ld_q,
     return launch_bn<128>(p, s);
 }
 
-cudaError_t launch_gemm_nt_tc_batched(const float* A, int64_t n_a, int64_t lda, size_t a_z_bytes, const float* B,
-                                      int64_t n_b, int64_t ldb, size_t b_z_bytes, int64_t K, float* C, int64_t ldc,
-                                      int64_t c_z, int64_t nz, float alpha, float beta, bool lower,
-                                      unsigned int* err, cudaStream_t s);
-
 // C[n][m] = beta * C[n][m] + alpha * sum_k A[m][k] B[n][k] (C row stride ldc): the
 // score GEMM with a sign, used by the blocked Cholesky and triangular solves. With
 // lower = true, A and B must be the same n x n operand rows (a symmetric rank-K
 // update) and only the 128 x 128 tiles on or below the diagonal (m0 <= n0) are
-// formed; entries above the diagonal inside a diagonal tile are written too.
-cudaError_t launch_gemm_nt_tc(const float* A, int64_t n_a, int64_t lda, const float* B, int64_t n_b, int64_t ldb,
-                              int64_t K, float* C, int64_t ldc, float alpha, float beta, bool lower,
-                              unsigned int* err, cudaStream_t s) {
-    return launch_gemm_nt_tc_batched(A, n_a, lda, 0, B, n_b, ldb, 0, K, C, ldc, 0, 1, alpha, beta, lower, err, s);
-}
-
+// formed; entries above the diagonal inside a diagonal tile are written too. `second` (batch
+// entries as in the first): C2 = beta * C2 + alpha * A B2^T with the same A, in the same launch.
 cudaError_t launch_gemm_nt_tc_batched(const float* A, int64_t n_a, int64_t lda, size_t a_z_bytes, const float* B,
                                       int64_t n_b, int64_t ldb, size_t b_z_bytes, int64_t K, float* C, int64_t ldc,
                                       int64_t c_z, int64_t nz, float alpha, float beta, bool lower,
-                                      unsigned int* err, cudaStream_t s) {
+                                      unsigned int* err, cudaStream_t s, const GemmSecond* second) {
     if (nz < 1 || nz > 65535) return cudaErrorInvalidValue;
     if (nz > 1 && ((a_z_bytes & 15) || (b_z_bytes & 15) || !a_z_bytes || !b_z_bytes)) return cudaErrorInvalidValue;
     GParams p{};
@@ -1125,8 +1144,8 @@ cudaError_t launch_gemm_nt_tc_batched(const float* A, int64_t n_a, int64_t lda, 
     p.s_z = c_z;
     p.err = err;
     if (lower && (n_a != n_b || n_b <= 64)) return cudaErrorInvalidValue;
-    if (n_b <= 64) return launch_bn<64>(p, s, nz, a_z_bytes, b_z_bytes);
-    return launch_bn<128>(p, s, nz, a_z_bytes, b_z_bytes);
+    if (n_b <= 64) return launch_bn<64>(p, s, nz, a_z_bytes, b_z_bytes, second);
+    return launch_bn<128>(p, s, nz, a_z_bytes, b_z_bytes, second);
 }
 
 bool gemm_tc_available() {
@@ -1168,7 +1187,7 @@ cudaError_t launch_fit_tc(int n_layers, int64_t D, void* state, size_t state_byt
     p.lower = 1;
     p.splits = 1;
     p.nz = n_layers;
-    p.tiles_z = pair_lower_tiles((D + kBM - 1) / kBM);
+    p.tiles_z = p.tiles_1 = pair_lower_tiles((D + kBM - 1) / kBM);
     p.err = err;
     static std::atomic<int> sms_cache{0};
     int sms = sms_cache.load(std::memory_order_relaxed);
@@ -1178,7 +1197,7 @@ cudaError_t launch_fit_tc(int n_layers, int64_t D, void* state, size_t state_byt
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 1;
         sms_cache.store(sms, std::memory_order_relaxed);
     }
-    return launch_pairs<128, true>(tm, tm, p, sms, s);
+    return launch_pairs<128, true>(tm, tm, tm, p, sms, s);
 }
 
 }  // namespace tda

@@ -22,12 +22,12 @@
 //           block step is a small matrix product instead of a serial chain.
 // Every launch covers all layers of the call (grid z or y = layer).
 //
-// Blocked path (fp32 state, D a multiple of 128 and at least 2048): the same
+// Blocked path (fp32 state, D a multiple of 128 and at least 256): the same
 // right-looking Cholesky in 256-column panels. Per panel: the 256 x 256 diagonal
 // block is factored in shared memory by one CTA (diag_panel_kernel), the rows
 // below it are solved against it (solve_kernel, x L_BB^T = a), and the trailing
 // lower triangle takes the rank-256 update M -= P P^T on the tensor cores (3xTF32,
-// launch_gemm_nt_tc). After the last panel, L^T is copied into M's upper triangle.
+// launch_gemm_nt_tc_batched). After the last panel, L^T is copied into M's upper triangle.
 // APPLY then solves the query rows panel by panel: a 256-wide triangular solve, and
 // the rest of every row updated by a tensor-core product with L's panel (forward)
 // or with L^T's panel from the upper triangle (backward).
@@ -1291,7 +1291,13 @@ cudaError_t apply_impl(int n_layers, int64_t D, const void* state, const float* 
 
 // ---------------------------------------------------------------- blocked path (fp32)
 constexpr int kBB = 128;                // panel width
-constexpr int64_t kBlockedMinD = 2048;  // smaller layers keep the one-launch cluster path
+// FACTOR and FACTOR_APPLY of layers of whole 128-column blocks, against the one-launch cluster kernel,
+// seven layers and 64 queries: D = 256 129 us here and 190 us there (one layer: 125 and 170 us),
+// D = 512 316 and 448 us, D = 1024 690 and 1110 us. At D = 128 the difference is the
+// launches' (77 and 110 us) and the cluster kernel's smaller inverses are as accurate, so it stays.
+constexpr int64_t kBlockedMinD = 256;
+// APPLY by itself: below, states may come from the cluster kernel, which leaves no L^T
+constexpr int64_t kBlockedApplyD = 2048;
 
 // ---- diagonal panels. A panel is 256 columns (128 at the end of an odd D / 128): the rows and
 // columns [lo, lo + 256) of a layer, factored by one CTA with everything in shared memory, since
@@ -1540,6 +1546,7 @@ __global__ void __launch_bounds__(kDiagThreads) diag_panel_kernel(St<float> st, 
     double* h = st.header(l);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool two = lo + kBB < D;
+    if (tid == 0) h[kPcW64] = 64.0;  // solve_kernel: the 64 x 64 inverses are there
     // a warp per row, 16 bytes a lane, nothing above the diagonal (one SM draws 17 bytes a clock)
 #pragma unroll 4
     for (int r = warp; r < kBB; r += kDiagThreads / 32) {
@@ -1620,8 +1627,8 @@ __global__ void __launch_bounds__(kDiagThreads) diag_panel_kernel(St<float> st, 
 
 // Row vectors solved against the panel's diagonal block B = [lo, lo + nb) of layer l (grid y),
 // nb = 256 or 128: FWD x <- L_BB^{-1} x, else x <- L_BB^{-T} x, for rows of nb values at column lo of
-// X (row stride ldx, layer l's rows at byte offset l * layer_bytes from base). Used for the rows of
-// M below a panel (FWD) and for the query rows of APPLY (both directions).
+// two sets of rows (the first blocks_a CTAs of a layer have rows_a). Used for the rows of M below a
+// panel (FWD) and for the query rows of APPLY (both directions).
 // R rows a CTA, their nb values in shared memory; 64 columns at a time: the solved columns' share
 // is taken off with L, then the 64 x 64 inverse applied, both from one slab S[k][i] of
 // coefficients (k: solved or own column, i: column of the block). A thread has RT x 4 entries, so
@@ -1632,22 +1639,31 @@ template <int R>
 struct SolveCfg {
     static constexpr int RT = R / 16;                       // 16 row groups x 16 column groups
     static constexpr int kLdX = 2 * kBB + 4;
-    static constexpr size_t kSmem = sizeof(float) * ((size_t)R * kLdX + (size_t)2 * kBB * 64 + 64);
+    static constexpr size_t kSmem = sizeof(float) * ((size_t)R * kLdX + (size_t)2 * kBB * 64 + kNB * (kNB + 1));
+};
+struct SolveRows {
+    char* base;          // layer l's rows at byte l * layer_bytes
+    size_t layer_bytes;
+    int64_t ldx, n_rows;
 };
 template <int R, bool FWD>
-__global__ void __launch_bounds__(256) solve_kernel(St<float> st, int64_t lo, int nb, char* base, size_t layer_bytes,
-                                                    int64_t ldx, int64_t n_rows) {
+__global__ void __launch_bounds__(256) solve_kernel(St<float> st, int64_t lo, int nb, SolveRows rows_a, SolveRows rows_b,
+                                                    int blocks_a) {
     using C = SolveCfg<R>;
     constexpr int RT = C::RT;
     extern __shared__ __align__(16) float ssm[];
     float(*xs)[C::kLdX] = reinterpret_cast<float(*)[C::kLdX]>(ssm);
     float(*S)[64] = reinterpret_cast<float(*)[64]>(ssm + R * C::kLdX);  // [k][i ^ 4 (k & 7)]
+    float(*T)[kNB + 1] = reinterpret_cast<float(*)[kNB + 1]>(ssm + R * C::kLdX + 2 * kBB * 64);
     const int l = blockIdx.y;
     const int64_t D = st.D;
     const float* M = st.M(l) + lo * D + lo;
+    const bool w64 = st.header(l)[kPcW64] == 64.0;
     const int tid = threadIdx.x, rg = tid >> 4, i0 = (tid & 15) * 4;
-    const int64_t row0 = (int64_t)blockIdx.x * R;
-    float* X = (float*)(base + (size_t)l * layer_bytes) + lo;
+    const bool second = (int)blockIdx.x >= blocks_a;
+    const SolveRows w = second ? rows_b : rows_a;
+    const int64_t row0 = (int64_t)(second ? blockIdx.x - blocks_a : blockIdx.x) * R, n_rows = w.n_rows, ldx = w.ldx;
+    float* X = (float*)(w.base + (size_t)l * w.layer_bytes) + lo;
     // n 16-byte loads, eight of a thread's in flight together: ld(e) loads item e, st(e, value) stores it
     auto copy = [&](int n, auto&& ld, auto&& st) {
         for (int e0 = tid; e0 < n; e0 += 8 * 256) {
@@ -1690,18 +1706,43 @@ __global__ void __launch_bounds__(256) solve_kernel(St<float> st, int64_t lo, in
                      const int k = e / 16;
                      *reinterpret_cast<float4*>(&S[k][(e % 16 * 4) ^ ((k & 7) << 2)]) = v;
                  });
-        // the block as stored: L left of the diagonal, W^T right of it. FWD: S[k][i] = W[i][k] =
-        // stored[k][i] for k < i; else S[k][i] = W[k][i] = stored[i][k] for k > i
-        copy(64 * 16, [&](int e) { return *reinterpret_cast<const float4*>(M + (int64_t)(c0 + e / 16) * D + c0 + e % 16 * 4); },
-             [&](int e, const float4& v4) {
-                 const int a = e / 16, c = e % 16 * 4;
-                 const float v[4] = {v4.x, v4.y, v4.z, v4.w};
+        if (w64) {
+            // the block as stored: L left of the diagonal, W^T right of it. FWD: S[k][i] = W[i][k] =
+            // stored[k][i] for k < i; else S[k][i] = W[k][i] = stored[i][k] for k > i
+            copy(64 * 16, [&](int e) { return *reinterpret_cast<const float4*>(M + (int64_t)(c0 + e / 16) * D + c0 + e % 16 * 4); },
+                 [&](int e, const float4& v4) {
+                     const int a = e / 16, c = e % 16 * 4;
+                     const float v[4] = {v4.x, v4.y, v4.z, v4.w};
 #pragma unroll
-                 for (int t = 0; t < 4; ++t) {
-                     const int i = FWD ? c + t : a, k = FWD ? a : c + t, kr = nk + k;
-                     S[kr][i ^ ((kr & 7) << 2)] = (FWD ? k < i : k > i) ? v[t] : (k == i ? 1.f / v[t] : 0.f);
-                 }
-             });
+                     for (int t = 0; t < 4; ++t) {
+                         const int i = FWD ? c + t : a, k = FWD ? a : c + t, kr = nk + k;
+                         S[kr][i ^ ((kr & 7) << 2)] = (FWD ? k < i : k > i) ? v[t] : (k == i ? 1.f / v[t] : 0.f);
+                     }
+                 });
+        } else {
+            // a state factored before these inverses were kept: from the 32 x 32 ones,
+            // W = [W00 0; -W11 (L10 W00) W11]
+            const float *D0 = st.Dinv(l) + (lo + c0) / kNB * (kNB * kNB), *D1 = D0 + kNB * kNB;
+            for (int e = tid; e < kNB * kNB; e += 256) {
+                const int i = e / kNB, k = e % kNB;
+                float t = 0.f;
+                for (int m = k; m < kNB; ++m) t = fmaf(M[(int64_t)(c0 + kNB + i) * D + c0 + m], D0[m * kNB + k], t);
+                T[i][k] = t;
+            }
+            __syncthreads();
+            for (int e = tid; e < 64 * 64; e += 256) {
+                const int r = e / 64, c = e % 64;
+                float w = 0.f;
+                if (c <= r && r < kNB)
+                    w = D0[r * kNB + c];
+                else if (c <= r && c >= kNB)
+                    w = D1[(r - kNB) * kNB + c - kNB];
+                else if (c <= r)
+                    for (int m = 0; m <= r - kNB; ++m) w = fmaf(-D1[(r - kNB) * kNB + m], T[m][c], w);
+                const int i = FWD ? r : c, kr = nk + (FWD ? c : r);
+                S[kr][i ^ ((kr & 7) << 2)] = w;
+            }
+        }
         __syncthreads();
         float acc[RT][4];  // the solved columns' share less x, so that both products add
 #pragma unroll
@@ -1828,29 +1869,34 @@ bool blocked_pc(int64_t D, tda_dtype sdt) {
 }
 
 template <int R, bool FWD>
-cudaError_t launch_solve_r(St<float> st, int n_layers, int64_t lo, int nb, char* base, size_t layer_bytes, int64_t ldx,
-                           int64_t n_rows, cudaStream_t s) {
+cudaError_t launch_solve_r(St<float> st, int n_layers, int64_t lo, int nb, const SolveRows& a, const SolveRows& b,
+                           cudaStream_t s) {
     cudaError_t e = smem_attr_once<solve_kernel<R, FWD>>((int)SolveCfg<R>::kSmem);
     if (e != cudaSuccess) return e;
+    const int64_t na = (a.n_rows + R - 1) / R, nb_b = (b.n_rows + R - 1) / R;
+    if (na + nb_b == 0) return cudaSuccess;
     note_launches(1);
-    solve_kernel<R, FWD><<<dim3((unsigned)((n_rows + R - 1) / R), n_layers), 256, SolveCfg<R>::kSmem, s>>>(
-        st, lo, nb, base, layer_bytes, ldx, n_rows);
+    solve_kernel<R, FWD><<<dim3((unsigned)(na + nb_b), n_layers), 256, SolveCfg<R>::kSmem, s>>>(st, lo, nb, a, b, (int)na);
     return cudaGetLastError();
 }
 
 // 128 rows a CTA once those fill the chip, else 16 (a quarter of the products per slab value read)
 template <bool FWD>
-cudaError_t launch_solve(St<float> st, int n_layers, int64_t lo, int nb, char* base, size_t layer_bytes, int64_t ldx,
-                         int64_t n_rows, cudaStream_t s) {
-    return (n_rows + 127) / 128 * n_layers >= 114
-               ? launch_solve_r<128, FWD>(st, n_layers, lo, nb, base, layer_bytes, ldx, n_rows, s)
-               : ((n_rows + 31) / 32 * n_layers >= 114
-                      ? launch_solve_r<32, FWD>(st, n_layers, lo, nb, base, layer_bytes, ldx, n_rows, s)
-                      : launch_solve_r<16, FWD>(st, n_layers, lo, nb, base, layer_bytes, ldx, n_rows, s));
+cudaError_t launch_solve(St<float> st, int n_layers, int64_t lo, int nb, const SolveRows& a, const SolveRows& b,
+                         cudaStream_t s) {
+    auto ctas = [&](int r) { return ((a.n_rows + r - 1) / r + (b.n_rows + r - 1) / r) * n_layers; };
+    return ctas(128) >= 114 ? launch_solve_r<128, FWD>(st, n_layers, lo, nb, a, b, s)
+                            : (ctas(32) >= 114 ? launch_solve_r<32, FWD>(st, n_layers, lo, nb, a, b, s)
+                                               : launch_solve_r<16, FWD>(st, n_layers, lo, nb, a, b, s));
 }
 
-cudaError_t factor_blocked(int n_layers, int64_t D, void* state, int64_t n_total, double la, double lr,
-                           cudaStream_t s) {
+// Factorisation in panels of 256 columns: the diagonal block, the rows below it, then the trailing
+// lower triangle of all layers in one launch, M -= P P^T, P = L[hi:D, lo:hi]. With queries (qhat,
+// n_q > 0) their rows ride along: x L^T = q is one more set of rows below each panel, so that the
+// forward substitution needs no launches of its own (seven layers of D = 4096, 256 queries: 1.0 ms
+// as 32 launches).
+cudaError_t factor_blocked(int n_layers, int64_t D, void* state, int64_t n_total, double la, double lr, float* qhat,
+                           int64_t n_q, int64_t ld_qhat, cudaStream_t s) {
     cudaError_t e = smem_attr_once<diag_panel_kernel>((int)sizeof(DiagSmem));
     if (e != cudaSuccess) return e;
     unsigned int* err = device_error_word();
@@ -1860,19 +1906,21 @@ cudaError_t factor_blocked(int n_layers, int64_t D, void* state, int64_t n_total
     prepare_kernel<float><<<n_layers, 256, 0, s>>>(st, n_total, la, lr);
     const unsigned rows_per = (unsigned)((D < 1024 ? D : 1024) * (n_layers < 8 ? 8 / n_layers : 1));
     scale_lower_kernel<<<dim3(rows_per < (unsigned)D ? rows_per : (unsigned)D, n_layers), 256, 0, s>>>(st);
-    // panels of 256 columns: the diagonal block, the rows below it, then the trailing lower
-    // triangle of all layers in one launch: M -= P P^T, P = L[hi:D, lo:hi]
     float* M0 = (float*)((char*)state + 64);  // layer l's M is st.bytes further on
     const int64_t cz = (int64_t)(st.bytes / 4);
+    const size_t lb = (size_t)D * 4;
     for (int64_t lo = 0; lo < D; lo += 2 * kBB) {
         note_launches(1);
         diag_panel_kernel<<<n_layers, kDiagThreads, sizeof(DiagSmem), s>>>(st, lo);
-        const int64_t hi = lo + 2 * kBB, rest = D - hi;
-        if (rest <= 0) break;
-        e = launch_solve<true>(st, n_layers, lo, 2 * kBB, (char*)M0 + (size_t)hi * D * 4, st.bytes, D, rest, s);
+        const int64_t hi = lo + 2 * kBB < D ? lo + 2 * kBB : D, rest = D - hi;
+        e = launch_solve<true>(st, n_layers, lo, (int)(hi - lo), SolveRows{(char*)M0 + (size_t)hi * D * 4, st.bytes, D, rest},
+                               SolveRows{(char*)qhat, lb, ld_qhat, n_q}, s);
         if (e != cudaSuccess) return e;
-        e = launch_gemm_nt_tc_batched(M0 + hi * D + lo, rest, D, st.bytes, M0 + hi * D + lo, rest, D, st.bytes,
-                                      2 * kBB, M0 + hi * D + hi, D, cz, n_layers, -1.f, 1.f, true, err, s);
+        if (rest <= 0) break;
+        const float* P = M0 + hi * D + lo;
+        const GemmSecond q2{qhat + lo, n_q, ld_qhat, lb, qhat + hi, ld_qhat, D};
+        e = launch_gemm_nt_tc_batched(P, rest, D, st.bytes, P, rest, D, st.bytes, 2 * kBB, M0 + hi * D + hi, D, cz,
+                                      n_layers, -1.f, 1.f, true, err, s, n_q > 0 ? &q2 : nullptr);
         if (e != cudaSuccess) return e;
     }
     const int64_t nb = D / 64;
@@ -1883,27 +1931,32 @@ cudaError_t factor_blocked(int n_layers, int64_t D, void* state, int64_t n_total
     return cudaGetLastError();
 }
 
+// (D >= kBlockedMinD suffices where the state is factored in the same call)
 bool apply_blocked_ok(int64_t D, tda_dtype sdt, const void* qhat, int64_t ld_qhat, int64_t n_q) {
     return blocked_pc(D, sdt) && ((uintptr_t)qhat & 15) == 0 && (ld_qhat & 3) == 0 && n_q < (1LL << 24);
 }
 
-cudaError_t apply_blocked(int n_layers, int64_t D, const void* state, const float* q, int64_t n_q, int64_t ld_q,
-                          float* qhat, int64_t ld_qhat, cudaStream_t s) {
+cudaError_t copy_queries(int n_layers, int64_t D, const float* q, int64_t n_q, int64_t ld_q, float* qhat,
+                         int64_t ld_qhat, cudaStream_t s) {
+    if (q == qhat && ld_q == ld_qhat) return cudaSuccess;
+    return cudaMemcpy2DAsync(qhat, (size_t)ld_qhat * 4, q, (size_t)ld_q * 4, (size_t)n_layers * D * 4, (size_t)n_q,
+                             cudaMemcpyDeviceToDevice, s);
+}
+
+// Both substitutions of the rows of qhat in place, or (forward = false) the backward one alone.
+cudaError_t apply_blocked(int n_layers, int64_t D, const void* state, int64_t n_q, float* qhat, int64_t ld_qhat,
+                          bool forward, cudaStream_t s) {
     cudaError_t e = cudaSuccess;
     unsigned int* err = device_error_word();
     if (!err) return cudaErrorUnknown;
     St<float> st = state_of<float>(const_cast<void*>(state), D);
-    if (q != qhat || ld_q != ld_qhat) {
-        e = cudaMemcpy2DAsync(qhat, (size_t)ld_qhat * 4, q, (size_t)ld_q * 4, (size_t)n_layers * D * 4, (size_t)n_q,
-                              cudaMemcpyDeviceToDevice, s);
-        if (e != cudaSuccess) return e;
-    }
     const size_t lb = (size_t)D * 4;  // layer l's columns start l * D floats into each row
     const float* M0 = (const float*)((const char*)state + 64);  // layer l's M is st.bytes further on
     constexpr int64_t kPanel = 2 * kBB;
-    for (int64_t lo = 0; lo < D; lo += kPanel) {
+    const SolveRows rows{(char*)qhat, lb, ld_qhat, n_q}, none{};
+    for (int64_t lo = 0; forward && lo < D; lo += kPanel) {
         const int64_t hi = lo + kPanel < D ? lo + kPanel : D;
-        e = launch_solve<true>(st, n_layers, lo, (int)(hi - lo), (char*)qhat, lb, ld_qhat, n_q, s);
+        e = launch_solve<true>(st, n_layers, lo, (int)(hi - lo), rows, none, s);
         if (e != cudaSuccess) return e;
         if (hi == D) break;
         e = launch_gemm_nt_tc_batched(M0 + hi * D + lo, D - hi, D, st.bytes, qhat + lo, n_q, ld_qhat, lb, kPanel,
@@ -1912,7 +1965,7 @@ cudaError_t apply_blocked(int n_layers, int64_t D, const void* state, const floa
     }
     for (int64_t lo = (D - 1) / kPanel * kPanel; lo >= 0; lo -= kPanel) {
         const int64_t hi = lo + kPanel < D ? lo + kPanel : D;
-        e = launch_solve<false>(st, n_layers, lo, (int)(hi - lo), (char*)qhat, lb, ld_qhat, n_q, s);
+        e = launch_solve<false>(st, n_layers, lo, (int)(hi - lo), rows, none, s);
         if (e != cudaSuccess) return e;
         if (lo == 0) break;
         // rows [0, lo) of U = L^T, columns [lo, hi): U[i][j] = L[j][i]
@@ -1956,7 +2009,8 @@ cudaError_t launch_pc_fit(int n_layers, int64_t D, tda_dtype sdt, void* state, c
 
 cudaError_t launch_pc_factor(int n_layers, int64_t D, tda_dtype sdt, void* state, int64_t n_total,
                              double lambda_abs, double lambda_rel, cudaStream_t s) {
-    if (blocked_pc(D, sdt)) return factor_blocked(n_layers, D, state, n_total, lambda_abs, lambda_rel, s);
+    if (blocked_pc(D, sdt))
+        return factor_blocked(n_layers, D, state, n_total, lambda_abs, lambda_rel, nullptr, 0, 0, s);
     if (sdt == TDA_F64) return factor_impl<double>(n_layers, D, state, n_total, lambda_abs, lambda_rel, s);
     return factor_impl<float>(n_layers, D, state, n_total, lambda_abs, lambda_rel, s);
 }
@@ -1964,17 +2018,25 @@ cudaError_t launch_pc_factor(int n_layers, int64_t D, tda_dtype sdt, void* state
 cudaError_t launch_pc_factor_apply(int n_layers, int64_t D, tda_dtype sdt, void* state, int64_t n_total,
                                    double lambda_abs, double lambda_rel, const float* q, int64_t n_q, int64_t ld_q,
                                    void* qhat, int64_t ld_qhat, cudaStream_t s) {
+    cudaError_t e;
+    if (n_q >= 1 && apply_blocked_ok(D, sdt, qhat, ld_qhat, n_q)) {
+        if ((e = copy_queries(n_layers, D, q, n_q, ld_q, (float*)qhat, ld_qhat, s)) != cudaSuccess) return e;
+        e = factor_blocked(n_layers, D, state, n_total, lambda_abs, lambda_rel, (float*)qhat, n_q, ld_qhat, s);
+        if (e != cudaSuccess) return e;
+        return apply_blocked(n_layers, D, state, n_q, (float*)qhat, ld_qhat, false, s);
+    }
     // fp32 state, whole 32-column blocks, up to 256 queries: factorisation and both
-    // substitutions in one cluster launch per call (below the blocked path's sizes);
+    // substitutions in one cluster launch per call;
     // otherwise FACTOR, then APPLY
-    if (sdt == TDA_F32 && !blocked_pc(D, sdt) && D % kNB == 0 && D >= 2 * kNB && n_q >= 1 && n_q <= 256) {
+    if (sdt == TDA_F32 && !(D >= kBlockedApplyD && blocked_pc(D, sdt)) && D % kNB == 0 && D >= 2 * kNB && n_q >= 1 &&
+        n_q <= 256) {
         const QArgs qa{q, (float*)qhat, n_q, ld_q, ld_qhat};
-        cudaError_t e = factor_cluster<16, true>(n_layers, D, state, n_total, lambda_abs, lambda_rel, qa, s);
+        e = factor_cluster<16, true>(n_layers, D, state, n_total, lambda_abs, lambda_rel, qa, s);
         if (e == cudaErrorNotSupported)
             e = factor_cluster<8, true>(n_layers, D, state, n_total, lambda_abs, lambda_rel, qa, s);
         if (e != cudaErrorNotSupported) return e;
     }
-    cudaError_t e = launch_pc_factor(n_layers, D, sdt, state, n_total, lambda_abs, lambda_rel, s);
+    e = launch_pc_factor(n_layers, D, sdt, state, n_total, lambda_abs, lambda_rel, s);
     if (e != cudaSuccess) return e;
     return launch_pc_apply(n_layers, D, sdt, state, q, n_q, ld_q, qhat, ld_qhat, s);
 }
@@ -1983,8 +2045,10 @@ cudaError_t launch_pc_apply(int n_layers, int64_t D, tda_dtype sdt, const void* 
                             int64_t n_q, int64_t ld_q, void* qhat, int64_t ld_qhat, cudaStream_t s) {
     if (n_q == 0) return cudaSuccess;
     // a blocked factorisation left L^T in M's upper triangle: tensor-core substitutions
-    if (apply_blocked_ok(D, sdt, qhat, ld_qhat, n_q))
-        return apply_blocked(n_layers, D, state, q, n_q, ld_q, (float*)qhat, ld_qhat, s);
+    if (D >= kBlockedApplyD && apply_blocked_ok(D, sdt, qhat, ld_qhat, n_q)) {
+        const cudaError_t e = copy_queries(n_layers, D, q, n_q, ld_q, (float*)qhat, ld_qhat, s);
+        return e != cudaSuccess ? e : apply_blocked(n_layers, D, state, n_q, (float*)qhat, ld_qhat, true, s);
+    }
     const size_t el = sdt == TDA_F64 ? 8 : 4;
     const size_t budget = 160 * 1024;
     if (sdt == TDA_F64) {

@@ -210,16 +210,20 @@ cudaError_t launch_score_tc(const float* Qhat, int64_t n_q, int64_t ld_q, const 
 int score_tc_tiles(int64_t n_q, int64_t n_t);
 bool gemm_tc_available();  // tcgen05 and the tensor-map encoder are usable on this device
 // C[n][m] = beta C[n][m] + alpha sum_k A[m][k] B[n][k] on tcgen05 (3xTF32); lower: square
-// symmetric update, tiles on or below the diagonal only. Same operand rules as the score.
-cudaError_t launch_gemm_nt_tc(const float* A, int64_t n_a, int64_t lda, const float* B, int64_t n_b, int64_t ldb,
-                              int64_t K, float* C, int64_t ldc, float alpha, float beta, bool lower,
-                              unsigned int* err, cudaStream_t s);
-// The same for nz independent problems in one launch (grid z): problem z's A, B start
-// a_z_bytes, b_z_bytes (multiples of 16) after the previous one's, its C c_z floats after.
+// symmetric update, tiles on or below the diagonal only. Same operand rules as the score. nz
+// independent problems in one launch: problem z's A, B start a_z_bytes, b_z_bytes (multiples of 16)
+// after the previous one's, its C c_z floats after. `second`: another B and C for the same A.
+struct GemmSecond {
+    const float* B;
+    int64_t n_b, ldb;
+    size_t b_z_bytes;
+    float* C;
+    int64_t ldc, c_z;
+};
 cudaError_t launch_gemm_nt_tc_batched(const float* A, int64_t n_a, int64_t lda, size_t a_z_bytes, const float* B,
                                       int64_t n_b, int64_t ldb, size_t b_z_bytes, int64_t K, float* C, int64_t ldc,
                                       int64_t c_z, int64_t nz, float alpha, float beta, bool lower,
-                                      unsigned int* err, cudaStream_t s);
+                                      unsigned int* err, cudaStream_t s, const GemmSecond* second = nullptr);
 cudaError_t launch_score_tc_slices(const float* Qhat, int64_t n_q, int64_t ld_q, const float* Phi, int64_t n_t,
                                    int64_t ld_phi, int64_t D, int splits, float* part, unsigned int* err,
                                    cudaStream_t s);
@@ -237,7 +241,7 @@ cudaError_t launch_topk(const float* S, int64_t n_q, int64_t n_t, int64_t ld_S, 
                         int32_t* idx, float* val, cudaStream_t s);
 
 // State header layout of the preconditioner (doubles).
-enum { kPcLambda = 0, kPcMeanEig = 1, kPcFailedPivot = 2, kPcNTotal = 3, kPcHeaderDoubles = 8 };
+enum { kPcLambda = 0, kPcMeanEig = 1, kPcFailedPivot = 2, kPcNTotal = 3, kPcW64 = 4, kPcHeaderDoubles = 8 };
 
 // Per-kernel launch set-up that does not change between launches, done once per device
 // (a stream job launches hundreds of kernels a step, and the host's time per launch adds up):

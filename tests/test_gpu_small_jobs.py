@@ -153,3 +153,57 @@ def test_blocked_failed_pivot(dev, bad):
         tda.tda_precondition_info(1, D, tda.TDA_F32, state)
     assert e.value.status == tda.TDA_ERR_NOT_SPD and f"pivot {bad + 1}" in str(e.value)
     assert torch.isnan(out).all()
+
+
+# as test_blocked_panels (condition number, rows a feature); D below 2048: FACTOR_APPLY runs the panels, APPLY by
+# itself the row-by-row substitution on the state that they leave
+@pytest.mark.parametrize("D,nl,nq,ld", [(256, 3, 5, 0), (384, 1, 33, 4), (1024, 2, 1, 0), (1152, 1, 130, 4), (1536, 3, 300, 0), (2176, 1, 40, 8)])
+def test_blocked_factor_apply(dev, D, nl, nq, ld):
+    rng = np.random.default_rng(D + 1)
+    n, w = 4 * D, nl * D
+    ph = torch.from_numpy(rng.standard_normal((n, w)).astype(np.float32)).to(dev)
+    q = torch.from_numpy(rng.standard_normal((nq, w + ld)).astype(np.float32)).to(dev)
+    state = torch.empty(nl * tda.tda_precondition_state_bytes(D, tda.TDA_F32), dtype=torch.uint8, device=dev)
+    out, alone, inplace = torch.full((nq, w + ld), 3.0, device=dev), torch.empty((nq, w), device=dev), q.clone()
+    args = (nl, D, tda.TDA_F32, state)
+    for o in (out, inplace):
+        tda.tda_precondition(tda.TDA_PC_RESET, *args)
+        tda.tda_precondition(tda.TDA_PC_FIT_ACCUM, *args, phi=ph, n=n, ld_phi=w)
+        tda.tda_precondition(tda.TDA_PC_FACTOR_APPLY, *args, n_total=n, lambda_rel_mean_eig=0.1,
+                             q=o if o is inplace else q, n_q=nq, ld_q=w + ld, qhat=o, ld_qhat=w + ld)
+    tda.tda_precondition(tda.TDA_PC_APPLY, *args, q=q, n_q=nq, ld_q=w + ld, qhat=alone, ld_qhat=w)
+    tda.tda_device_status()
+    tda.tda_precondition_info(nl, D, tda.TDA_F32, state)
+    for l in range(nl):
+        x = ph[:, l * D:(l + 1) * D].double()
+        F = x.T @ x / n
+        F.diagonal().add_(0.1 * F.diagonal().mean())
+        ref = torch.linalg.solve(F, q[:, l * D:(l + 1) * D].double().T).T
+        for o in (out, inplace, alone):
+            got = o[:, l * D:(l + 1) * D].double()
+            assert float((got - ref).norm() / ref.norm()) <= 2e-5
+    assert (out[:, w:] == 3.0).all() and torch.equal(inplace[:, :w], out[:, :w])
+
+
+def test_blocked_state_without_64_column_inverses(dev):
+    # a factored state from before the 64 x 64 inverses were kept: no mark in the header, nothing of use right of
+    # the diagonal inside the 64-column blocks
+    D, nq = 2048, 20
+    rng = np.random.default_rng(9)
+    ph = torch.from_numpy(rng.standard_normal((4 * D, D)).astype(np.float32)).to(dev)
+    q = torch.from_numpy(rng.standard_normal((nq, D)).astype(np.float32)).to(dev)
+    state = torch.empty(tda.tda_precondition_state_bytes(D, tda.TDA_F32), dtype=torch.uint8, device=dev)
+    args = (1, D, tda.TDA_F32, state)
+    tda.tda_precondition(tda.TDA_PC_RESET, *args)
+    tda.tda_precondition(tda.TDA_PC_FIT_ACCUM, *args, phi=ph, n=4 * D, ld_phi=D)
+    tda.tda_precondition(tda.TDA_PC_FACTOR, *args, n_total=4 * D, lambda_rel_mean_eig=0.1)
+    new, old = torch.empty((nq, D), device=dev), torch.empty((nq, D), device=dev)
+    tda.tda_precondition(tda.TDA_PC_APPLY, *args, q=q, n_q=nq, ld_q=D, qhat=new, ld_qhat=D)
+    state[32:40] = 0
+    m = state[64:64 + 4 * D * D].view(torch.float32).view(D // 64, 64, D // 64, 64)
+    up = torch.triu(torch.ones(64, 64, dtype=torch.bool, device=dev), 1)
+    for b in range(D // 64):
+        m[b, :, b, :][up] = float("nan")
+    tda.tda_precondition(tda.TDA_PC_APPLY, *args, q=q, n_q=nq, ld_q=D, qhat=old, ld_qhat=D)
+    tda.tda_device_status()
+    assert float((new - old).norm() / new.norm()) <= 2e-5
