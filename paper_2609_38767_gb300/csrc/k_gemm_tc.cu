@@ -67,6 +67,7 @@ struct GParams {
     int tiles_n2;          // second product, the same A: its tiles along B, B2 rows, output
     int64_t n_q2, ld_S2, s_z2;
     float* S2;
+    int red;               // add to S through TMA (beta = 1; S, its rows and entries 16-byte aligned)
     int nz;                // persistent kernel: batch entries
     unsigned int* err;
 };
@@ -410,6 +411,11 @@ score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 // quadrant, half of the columns each) add every finished group into round-to-nearest registers
 // beside the next group's MMAs, then write the tile beside the next tile's.
 //
+// RED: S += alpha * product with TMA reductions from shared memory (one rounding, as in registers).
+// For products of few features, whose epilogue's loads of the old values took longer than the
+// MMAs: the rank-256 updates of 7 x 4096 rows take 49 us on average, 101 us before. L2 flushes subnormal sums, so the fit
+// and the scores keep the loads.
+//
 // Measured: scores of 256 x 8192, 7168 features: 205 us with both operands in shared memory and one
 // pass over the accumulators (1.3e-5 off), 188 us with A in TMEM (9e-7 off), 114 us in pairs.
 // Fit of seven layers of D = 4096, 8192 examples: 6.74 ms, 6.24 ms, 3.61 ms.
@@ -418,20 +424,22 @@ score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 // the pair: in CTA 0), 17 TMA. Every wait is bounded.
 constexpr int kThreadsT = 18 * 32;
 
-template <int BN, bool PAIR>
+template <int BN, bool PAIR, bool RED = false>
 struct TCfg {
     static constexpr int kCtas = PAIR ? 2 : 1;
     static constexpr int kBRows = BN / kCtas;             // rows of B in this CTA
     static constexpr uint32_t kABytes = kBM * kRowBytes;  // 16 KiB
     static constexpr uint32_t kBBytes = kBRows * kRowBytes;
     static constexpr uint32_t kRawBytes = kABytes + kBBytes;
-    static constexpr int kRaw = PAIR ? 6 : 4;             // raw chunks
+    static constexpr int kRaw = PAIR && !RED ? 6 : 4;     // raw chunks
     static constexpr int kSlots = PAIR ? 4 : 3;           // A in TMEM, B's hi and lo in shared memory
     static constexpr uint32_t kSlotBytes = 2 * kBBytes;
     static constexpr int kGroup = 2;
     static constexpr int kCols = BN / 2;                  // columns per epilogue thread
     static constexpr int kAOff = 2 * BN;                  // first TMEM column of A: [slot][hi 32 | lo 32]
-    static constexpr size_t kBarOff = (size_t)kRaw * kRawBytes + (size_t)kSlots * kSlotBytes;
+    static constexpr size_t kOutOff = (size_t)kRaw * kRawBytes + (size_t)kSlots * kSlotBytes;
+    static constexpr uint32_t kOutBytes = kCols * 128;    // RED: kCols rows of 32 output columns, per epilogue warp
+    static constexpr size_t kBarOff = kOutOff + (RED ? 8 * kOutBytes : 0);
     static constexpr size_t kSmem = 1024 + kBarOff + 8 * (2 * kRaw + 2 * kSlots + 5) + 16;
     static_assert(kAOff + kSlots * 64 <= 512 && kSmem <= 232448, "TMEM columns, shared memory");
 };
@@ -541,11 +549,12 @@ __device__ __forceinline__ int64_t chunks_of(const GParams& p, int y) {
     return (Kz + kKC - 1) / kKC;
 }
 
-template <int BN, bool PAIR, bool FIT>
+template <int BN, bool PAIR, bool FIT, bool RED>
 __global__ void __launch_bounds__(kThreadsT, 1)
 gemm3t_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-              const __grid_constant__ CUtensorMap tmB2, const GParams p) {
-    using C = TCfg<BN, PAIR>;
+              const __grid_constant__ CUtensorMap tmB2, const __grid_constant__ CUtensorMap tmS,
+              const __grid_constant__ CUtensorMap tmS2, const GParams p) {
+    using C = TCfg<BN, PAIR, RED>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t* slots = smem + (size_t)C::kRaw * C::kRawBytes;
@@ -716,9 +725,8 @@ gemm3t_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             const int64_t ld_S = at.second ? p.ld_S2 : p.ld_S, n_q = at.second ? p.n_q2 : p.n_q;
             const int lim = (int)(n_q - nb < C::kCols ? n_q - nb : C::kCols);
             // the previous values start on their way to L2: short products (256 features) end before
-            // HBM has answered (rank-256 updates of 7 x 4096: 85 -> 77 us on average). A warp's 32 values of a
-            // column are one or two lines.
-            if (p.beta != 0.f && write)
+            // HBM has answered. A warp's 32 values of a column are one or two lines.
+            if (!RED && p.beta != 0.f && write)
 #pragma unroll
                 for (int c = lane; c < C::kCols; c += 32)
                     if (c < lim && at.m0 + q4 * 32 < p.n_t)
@@ -742,6 +750,25 @@ gemm3t_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                 __syncwarp();
                 if (lane == 0) arrive_leader<PAIR>(smem_u32(&acc_empty[b]));
             }
+            if constexpr (RED) {
+                if (!got || !write || at.m0 + q4 * 32 >= p.n_t || lim <= 0) continue;
+                uint8_t* out = smem + C::kOutOff + (size_t)(warp - 8) * C::kOutBytes;
+                if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // the last tile has left
+                __syncwarp();
+#pragma unroll
+                for (int c = 0; c < C::kCols; ++c) *reinterpret_cast<float*>(out + c * 128 + lane * 4) = p.alpha * acc[c];
+                fence_proxy_async();
+                __syncwarp();
+                if (lane == 0) {
+                    asm volatile(
+                        "cp.reduce.async.bulk.tensor.3d.global.shared::cta.add.tile.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(
+                            (uint64_t)(at.second ? &tmS2 : &tmS)),
+                        "r"((int)at.m0 + q4 * 32), "r"((int)nb), "r"(at.z), "r"(smem_u32(out))
+                        : "memory");
+                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                }
+                continue;
+            }
             if (!got || m >= p.n_t || !write) continue;
             if (p.beta == 0.f) {
 #pragma unroll
@@ -760,6 +787,7 @@ gemm3t_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
                 }
             }
         }
+        if (RED && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     } else if (warp == 17 && lane == 0) {
         // ---------------- TMA producer
         uint32_t it = 0, last_par[C::kRaw];
@@ -920,11 +948,11 @@ int64_t pair_lower_tiles(int64_t nt) {
     return nt & 1 ? (q + 1) * (q + 1) : q * (q + 1);
 }
 
-template <int BN, bool FIT>
-cudaError_t launch_pairs(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmB2, const GParams& p,
-                         int sms, cudaStream_t s) {
-    using T = TCfg<BN, true>;
-    cudaError_t e = smem_attr_once<gemm3t_kernel<BN, true, FIT>>((int)T::kSmem);
+template <int BN, bool FIT, bool RED>
+cudaError_t launch_pairs(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmB2, const CUtensorMap& tmS,
+                         const CUtensorMap& tmS2, const GParams& p, int sms, cudaStream_t s) {
+    using T = TCfg<BN, true, RED>;
+    cudaError_t e = smem_attr_once<gemm3t_kernel<BN, true, FIT, RED>>((int)T::kSmem);
     if (e != cudaSuccess) return e;
     const int64_t total = p.tiles_z * p.splits * p.nz, half = sms > 1 ? sms / 2 : 1;
     cudaLaunchConfig_t cfg = {};
@@ -940,8 +968,23 @@ cudaError_t launch_pairs(const CUtensorMap& tmA, const CUtensorMap& tmB, const C
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     note_launches(1);
-    e = cudaLaunchKernelEx(&cfg, gemm3t_kernel<BN, true, FIT>, tmA, tmB, tmB2, p);
+    e = cudaLaunchKernelEx(&cfg, gemm3t_kernel<BN, true, FIT, RED>, tmA, tmB, tmB2, tmS, tmS2, p);
     return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+// 3-D map over nz outputs fp32 S[rows][ld] (columns 0..cols-1), entry z s_z floats from the last; box
+// 32 columns x box_rows rows, no swizzle.
+bool make_map_out(CUtensorMap* tm, float* S, int64_t rows, int64_t cols, int64_t ld, int64_t nz, int64_t s_z,
+                  int box_rows) {
+    EncodeTiledFn enc = encode_fn();
+    if (!enc) return false;
+    cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)nz};
+    cuuint64_t strides[2] = {(cuuint64_t)(ld * 4), (cuuint64_t)((nz > 1 ? s_z : ld) * 4)};
+    cuuint32_t box[3] = {32, (cuuint32_t)box_rows, 1};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return enc(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, S, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 template <int BN>
@@ -1001,15 +1044,24 @@ cudaError_t launch_bn(GParams p, cudaStream_t s, int64_t nz = 1, size_t a_z_byte
             if (nz > 1 ? !make_map_f32_3d(&tmB, p.B, p.n_q, p.K, p.ldb, nz, b_z_bytes, BN / 2)
                        : !make_map_f32(&tmB, p.B, p.n_q, p.K, p.ldb, BN / 2))
                 return cudaErrorInvalidValue;
-            return launch_pairs<BN, false>(tmA, tmB, tmB2, p, sms, s);
+            if (p.red) {
+                // output boxes: 32 columns x the rows of half a tile
+                CUtensorMap tmS, tmS2;
+                if (!make_map_out(&tmS, p.S, p.n_q, p.n_t, p.ld_S, nz, p.s_z, BN / 2)) return cudaErrorInvalidValue;
+                tmS2 = tmS;
+                if (second && !make_map_out(&tmS2, p.S2, p.n_q2, p.n_t, p.ld_S2, nz, p.s_z2, BN / 2))
+                    return cudaErrorInvalidValue;
+                return launch_pairs<BN, false, true>(tmA, tmB, tmB2, tmS, tmS2, p, sms, s);
+            }
+            return launch_pairs<BN, false, false>(tmA, tmB, tmB2, tmA, tmA, p, sms, s);
         }
         using T = TCfg<BN, false>;
         p.tiles_z = tiles;
         const int64_t total = tiles * per;
-        cudaError_t e = smem_attr_once<gemm3t_kernel<BN, false, false>>((int)T::kSmem);
+        cudaError_t e = smem_attr_once<gemm3t_kernel<BN, false, false, false>>((int)T::kSmem);
         if (e != cudaSuccess) return e;
         note_launches(1);
-        gemm3t_kernel<BN, false, false><<<(unsigned)(total < sms ? total : sms), kThreadsT, T::kSmem, s>>>(tmA, tmB, tmB, p);
+        gemm3t_kernel<BN, false, false, false><<<(unsigned)(total < sms ? total : sms), kThreadsT, T::kSmem, s>>>(tmA, tmB, tmB, tmA, tmA, p);
         return cudaGetLastError();
     }
     if (second) return cudaErrorInvalidValue;
@@ -1144,6 +1196,8 @@ cudaError_t launch_gemm_nt_tc_batched(const float* A, int64_t n_a, int64_t lda, 
     p.s_z = c_z;
     p.err = err;
     if (lower && (n_a != n_b || n_b <= 64)) return cudaErrorInvalidValue;
+    auto aligned = [](const float* S, int64_t ld, int64_t z) { return !(((uintptr_t)S | (size_t)(ld * 4) | (size_t)(z * 4)) & 15); };
+    p.red = beta == 1.f && aligned(C, ldc, c_z) && (!second || aligned(second->C, second->ldc, second->c_z));
     if (n_b <= 64) return launch_bn<64>(p, s, nz, a_z_bytes, b_z_bytes, second);
     return launch_bn<128>(p, s, nz, a_z_bytes, b_z_bytes, second);
 }
@@ -1197,7 +1251,7 @@ cudaError_t launch_fit_tc(int n_layers, int64_t D, void* state, size_t state_byt
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 1;
         sms_cache.store(sms, std::memory_order_relaxed);
     }
-    return launch_pairs<128, true>(tm, tm, tm, p, sms, s);
+    return launch_pairs<128, true, false>(tm, tm, tm, tm, tm, p, sms, s);
 }
 
 }  // namespace tda
