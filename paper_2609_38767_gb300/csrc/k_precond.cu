@@ -1880,14 +1880,25 @@ cudaError_t launch_solve_r(St<float> st, int n_layers, int64_t lo, int nb, const
     return cudaGetLastError();
 }
 
-// 128 rows a CTA once those fill the chip, else 16 (a quarter of the products per slab value read)
+// Rows a CTA: the fewest microseconds over the rounds of 152 CTAs (measured, 256 columns: 26 us for the
+// slabs and the chain, 0.26 us a row).
 template <bool FWD>
 cudaError_t launch_solve(St<float> st, int n_layers, int64_t lo, int nb, const SolveRows& a, const SolveRows& b,
                          cudaStream_t s) {
-    auto ctas = [&](int r) { return ((a.n_rows + r - 1) / r + (b.n_rows + r - 1) / r) * n_layers; };
-    return ctas(128) >= 114 ? launch_solve_r<128, FWD>(st, n_layers, lo, nb, a, b, s)
-                            : (ctas(32) >= 114 ? launch_solve_r<32, FWD>(st, n_layers, lo, nb, a, b, s)
-                                               : launch_solve_r<16, FWD>(st, n_layers, lo, nb, a, b, s));
+    int best = 0;
+    double least = 0.0;
+    for (int r : {128, 96, 64, 32, 16}) {
+        const int64_t ctas = ((a.n_rows + r - 1) / r + (b.n_rows + r - 1) / r) * n_layers;
+        const double us = (double)((ctas + 151) / 152) * (26.0 + 0.26 * r);
+        if (!best || us < least) best = r, least = us;
+    }
+    switch (best) {
+        case 128: return launch_solve_r<128, FWD>(st, n_layers, lo, nb, a, b, s);
+        case 96: return launch_solve_r<96, FWD>(st, n_layers, lo, nb, a, b, s);
+        case 64: return launch_solve_r<64, FWD>(st, n_layers, lo, nb, a, b, s);
+        case 32: return launch_solve_r<32, FWD>(st, n_layers, lo, nb, a, b, s);
+        default: return launch_solve_r<16, FWD>(st, n_layers, lo, nb, a, b, s);
+    }
 }
 
 // Factorisation in panels of 256 columns: the diagonal block, the rows below it, then the trailing
