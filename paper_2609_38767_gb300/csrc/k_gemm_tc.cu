@@ -461,38 +461,6 @@ __device__ __forceinline__ void mma_tf32_ta(uint32_t d_tmem, uint32_t a_tmem, ui
             "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
             : "memory");
 }
-// Arrives on `bar` of every CTA of the tile once the MMAs issued so far are done.
-template <bool PAIR>
-__device__ __forceinline__ void commit_all(uint32_t bar) {
-    if constexpr (PAIR)
-        asm volatile(
-            "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
-            "h"((uint16_t)3)
-            : "memory");
-    else
-        mma_commit(bar);
-}
-__device__ __forceinline__ void commit_pair_local(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void tmem_alloc2(uint32_t dst, uint32_t ncols) {
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst), "r"(ncols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc2(uint32_t taddr, uint32_t ncols) {
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
-}
-// Arrives on CTA 0's `bar` of the tile. The operands that it announces are ordered by tcgen05.wait::st and
-// fence.proxy.async; a release at cluster scope would wait for all of the warp's writes (1100
-// clocks).
-template <bool PAIR>
-__device__ __forceinline__ void arrive_leader(uint32_t bar) {
-    if constexpr (PAIR)
-        asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(map_rank(bar, 0u)) : "memory");
-    else
-        mbar_arrive(bar);
-}
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(

@@ -28,25 +28,26 @@
 // be kept. The buffers alternate, so the epilogue of one block overlaps the
 // MMAs of the next.
 //
-// What bounds it: each M = 128, N = 256, K = 16 MMA reads 12 KB of operands
-// from shared memory and the TMA writes as much, ~190 B/clock per SM against
+// What bounds it: in one CTA, each M = 128, N = 256, K = 16 MMA reads 12 KB of
+// operands from shared memory and the TMA writes as much, ~190 B/clock per SM against
 // ~128 B/clock of shared-memory bandwidth, so the tile tops out near two
-// thirds of the MMA rate. The epilogue (256 threads, 128 columns each) reads
-// 128 KB of TMEM per block, half the time of a two-chunk block's MMAs.
+// thirds of the MMA rate. Pairs of CTAs (PAIR, cta_group::2) read 8 KB. The epilogue
+// (256 threads, 128 columns each) reads 128 KB of TMEM per block, more than
+// half the time of a two-chunk block's MMAs; sixteen warps for it were 12 % slower.
 //
 // Measured (similarity alone): 2048 -> 2048, T = 50, 16 x 512 pairs 34.9 ms on the
 // CUDA cores (T not a power of two), now 0.22 ms = 0.76 PFLOP/s useful (100 of 128
-// and 250 of 256 tile rows); 8192 -> 8192 at T = 8 / 32 / 128 / 512: 1.14 / 1.25 /
+// and 250 of 256 tile rows), then 0.142 ms in pairs and blocks of 256; 8192 -> 8192 at T = 8 / 32 / 128 / 512: 1.14 / 1.25 /
 // 1.27 / 0.99 PFLOP/s with one accumulation per tile and no overlap between tiles,
-// now 1.56 / 1.46 / 1.53 / 1.39.
+// now 1.80 / 1.73 / 1.77 / 1.49.
 //
 // Norms (SELF): one 128-row tile of packed examples against itself needs one
 // 16 KB copy per chunk (A and B operand are the same tile) and is bound by
 // HBM (512 examples of 50 tokens, 2048 -> 2048: 3.9 ms on the CUDA cores, now
-// 78 us); T > 128 loops over the tile pairs i <= j, off-diagonal ones doubled.
+// 58 us); T > 128 loops over the tile pairs i <= j, off-diagonal ones doubled.
 //
 // Warp roles (320 threads, one persistent CTA per SM): warp 0 TMA producer,
-// warp 1 TMEM allocator and MMA issuer (lane 0), warps 2-9 epilogue (two warps
+// warp 1 TMEM allocator and MMA issuer (of a pair: in CTA 0), warps 2-9 epilogue (two warps
 // per TMEM lane quadrant, each half of the columns). Waits are bounded (about
 // 1 s) and set kErrTimeout on expiry, as in the projection kernel.
 #include <cuda.h>
@@ -67,13 +68,14 @@ constexpr uint32_t kABytes = kTM * kChunkK * 2;          // 16 KiB
 constexpr uint32_t kTmemCols = 512;                      // two accumulator buffers of at most 256 columns
 constexpr int kMaxStages = 8;
 constexpr size_t kSmemMax = 232448;                      // 227 KiB of dynamic shared memory per CTA
-constexpr size_t kTailBytes = 16 * 8 + 8 * (2 * kMaxStages + 5) + 16;  // warp sums, barriers, TMEM slot, abort flag
+constexpr size_t kTailBytes = 16 * 8 + 8 * (3 * kMaxStages + 5) + 16;  // warp sums, barriers, TMEM slot, abort flag
 
-template <bool SELF>
+template <bool SELF, bool PAIR = false>
 struct Cfg {
     static constexpr int kTN = SELF ? 128 : 256;         // train token rows per tile (MMA N)
     static constexpr int kCols = kTN / 2;                // columns per epilogue thread
-    static constexpr uint32_t kStageBytes = kABytes + kTN * kChunkK * 2;
+    static constexpr int kBRows = PAIR ? kTN / 2 : kTN;  // of which in this CTA
+    static constexpr uint32_t kStageBytes = kABytes + kBRows * kChunkK * 2;
 };
 
 struct GParams {
@@ -84,7 +86,7 @@ struct GParams {
     int pq, pt;             // examples per query tile and per train tile (T <= 128), else 0
     int ldr;                // floats per row of the per-example partial sums (packed)
     int64_t n_units;        // tile pairs (packed) or example pairs (T > 128); SELF: tiles or examples
-    int64_t n_qtiles;       // packed query tiles
+    int64_t n_qtiles;       // packed query tiles, or pairs of them
     int tiles_q, tiles_t;   // token tiles per query / train example (T > 128)
     float alpha, beta;
     float* S;
@@ -92,6 +94,20 @@ struct GParams {
 };
 
 #include "tc_ptx.cuh"
+
+// mma_bf16 of one CTA or a pair
+template <bool PAIR>
+__device__ __forceinline__ void mma_bf16_g(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                           uint32_t accumulate) {
+    if constexpr (PAIR)
+        asm volatile(
+            "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(
+                d_tmem),
+            "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+            : "memory");
+    else
+        mma_bf16(d_tmem, adesc, bdesc, idesc, accumulate);
+}
 
 __device__ __forceinline__ void emit(const GParams& p, int64_t q, int64_t i, float v) {
     float* dst = p.S + q * p.ld_S + i;
@@ -139,12 +155,12 @@ __device__ __forceinline__ void y_block_short(const float (&x)[COLS], uint32_t t
     }
 }
 
-template <bool SELF>
+template <bool SELF, bool PAIR>
 __global__ void __launch_bounds__(kThreads, 1)
 gram_tc_kernel(const __grid_constant__ CUtensorMap tmAq, const __grid_constant__ CUtensorMap tmAt,
                const __grid_constant__ CUtensorMap tmBq, const __grid_constant__ CUtensorMap tmBt,
                const GParams p) {
-    using C = Cfg<SELF>;
+    using C = Cfg<SELF, PAIR>;
     constexpr int kTN = C::kTN, kCols = C::kCols;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -155,7 +171,8 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmAq, const __grid_constant__
     uint64_t* tfull = bars + 2 * kMaxStages;  // [2] block accumulated
     uint64_t* tempty = tfull + 2;           // [2] block drained (one arrive per epilogue warp)
     uint64_t* mma_done = tempty + 2;
-    uint32_t* tmem_slot = (uint32_t*)(mma_done + 1);
+    uint64_t* pfull = mma_done + 1;         // [stages] PAIR: landed in CTA 1
+    uint32_t* tmem_slot = (uint32_t*)(pfull + kMaxStages);
     volatile int* abort = (volatile int*)(tmem_slot + 1);
     float* red = (float*)(tmem_slot + 4);   // packed: [2 column halves][128 rows][ldr examples] partial sums
 
@@ -164,23 +181,33 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmAq, const __grid_constant__
         for (int s = 0; s < p.stages; ++s) {
             mbar_init(smem_u32(&full[s]), 1);
             mbar_init(smem_u32(&empty[s]), 1);
+            mbar_init(smem_u32(&pfull[s]), 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(&tfull[b]), 1);
-            mbar_init(smem_u32(&tempty[b]), kEpiWarps);
+            mbar_init(smem_u32(&tempty[b]), PAIR ? 2 * kEpiWarps : kEpiWarps);
         }
         mbar_init(smem_u32(mma_done), 1);
         *abort = 0;
         fence_mbar_init();
     }
     if (warp == 1) {
-        tmem_alloc(smem_u32(tmem_slot), kTmemCols);
-        tmem_relinquish();
+        if constexpr (PAIR) {
+            tmem_alloc2(smem_u32(tmem_slot), kTmemCols);
+        } else {
+            tmem_alloc(smem_u32(tmem_slot), kTmemCols);
+            tmem_relinquish();
+        }
     }
     tc_fence_before();
     __syncthreads();
+    if constexpr (PAIR) cluster_sync();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    const uint32_t rank = PAIR ? cluster_rank() : 0u;
+    const int64_t u0 = PAIR ? blockIdx.x >> 1 : blockIdx.x, ustep = PAIR ? gridDim.x >> 1 : gridDim.x;
+    // packed: this CTA's query tile of unit u
+    auto qtile = [&](int64_t u) { return SELF ? u : (PAIR ? 2 * (u % p.n_qtiles) + rank : u % p.n_qtiles); };
     const bool packed = p.pq > 0;
     const int nk_tot = p.nk_in + p.nk_out;
     const int nbx = (p.nk_in + p.kbx - 1) / p.kbx, nb = nbx + (p.nk_out + p.kby - 1) / p.kby;
@@ -192,13 +219,13 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmAq, const __grid_constant__
         uint32_t s = 0, ph = 0, last_par[kMaxStages];
         bool issued[kMaxStages], ok = true;
         for (int i = 0; i < kMaxStages; ++i) issued[i] = false;
-        for (int64_t u = blockIdx.x; ok && u < p.n_units; u += gridDim.x) {
+        for (int64_t u = u0; ok && u < p.n_units; u += ustep) {
             int ti = 0, tj = 0;
             for (int tp = 0; ok && tp < tpp; ++tp) {
                 int rq, eq, rt, et;
                 if (packed) {  // rows of the [n*T][d] views
-                    rq = (int)((SELF ? u : u % p.n_qtiles) * p.pq * p.T);
-                    rt = SELF ? rq : (int)((u / p.n_qtiles) * p.pt * p.T);
+                    rq = (int)(qtile(u) * p.pq * p.T);
+                    rt = SELF ? rq : (int)((u / p.n_qtiles) * p.pt * p.T) + (int)rank * C::kBRows;
                     eq = et = 0;
                 } else {       // token tiles of one query and one train example
                     eq = (int)(SELF ? u : u % p.n_q);
@@ -234,13 +261,28 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmAq, const __grid_constant__
                         atomicOr(p.err, kErrTimeout);
                         break;
                     }
+                // every arrival of the pair's MMAs on this CTA's barriers lands before it exits
+                if (PAIR && ok && !wait_bounded(smem_u32(&empty[i]), last_par[i], abort, p.err)) ok = false;
+            }
+    } else if (warp == 1 && rank == 1) {
+        // ---------------- CTA 1 of a pair: tells CTA 0, which issues the MMAs, that a stage has landed
+        uint32_t s = 0, ph = 0;
+        bool ok = true;
+        for (int64_t u = u0; ok && u < p.n_units; u += ustep)
+            for (int kc = 0; kc < nk_tot; ++kc) {
+                if (!warp_wait(smem_u32(&full[s]), ph, abort, p.err)) {
+                    ok = false;
+                    break;
+                }
+                if (lane == 0) arrive_leader<PAIR>(smem_u32(&pfull[s]));
+                if (++s == (uint32_t)p.stages) s = 0, ph ^= 1u;
             }
     } else if (warp == 1) {
         // ---------------- MMA issuer: the warp waits, one lane issues
         uint32_t s = 0, ph = 0, cnt = 0;
         bool ok = true;
-        constexpr uint32_t idesc = idesc_bf16(kTM, kTN);
-        for (int64_t u = blockIdx.x; ok && u < p.n_units; u += gridDim.x) {
+        constexpr uint32_t idesc = idesc_bf16(PAIR ? 2 * kTM : kTM, kTN);
+        for (int64_t u = u0; ok && u < p.n_units; u += ustep) {
             int ti = 0, tj = 0;
             for (int tp = 0; ok && tp < tpp; ++tp) {
                 const uint32_t boff = SELF && ti == tj ? 0u : kABytes;
@@ -256,7 +298,8 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmAq, const __grid_constant__
                     const int left = side_b ? p.nk_out - (blk - nbx) * kb : p.nk_in - blk * kb;
                     const int n = left < kb ? left : kb;
                     for (int c = 0; c < n; ++c) {
-                        if (!warp_wait(smem_u32(&full[s]), ph, abort, p.err)) {
+                        if (!warp_wait(smem_u32(&full[s]), ph, abort, p.err) ||
+                            (PAIR && !warp_wait(smem_u32(&pfull[s]), ph, abort, p.err))) {
                             ok = false;
                             break;
                         }
@@ -266,21 +309,24 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmAq, const __grid_constant__
                         if (elect_one()) {
 #pragma unroll
                             for (int k = 0; k < kChunkK / 16; ++k)
-                                mma_bf16(tmem + b * 256u, ad + 2 * k, bd + 2 * k, idesc, (c > 0 || k > 0) ? 1u : 0u);
-                            mma_commit(smem_u32(&empty[s]));
+                                mma_bf16_g<PAIR>(tmem + b * 256u, ad + 2 * k, bd + 2 * k, idesc, (c > 0 || k > 0) ? 1u : 0u);
+                            commit_all<PAIR>(smem_u32(&empty[s]));
                         }
                         __syncwarp();
                         if (++s == (uint32_t)p.stages) s = 0, ph ^= 1u;
                     }
                     if (!ok) break;
-                    if (elect_one()) mma_commit(smem_u32(&tfull[b]));
+                    if (elect_one()) commit_all<PAIR>(smem_u32(&tfull[b]));
                     __syncwarp();
                 }
                 if (++tj == p.tiles_t) tj = SELF ? ++ti : (++ti, 0);
             }
         }
         if (elect_one()) {
-            mma_commit(smem_u32(mma_done));
+            if constexpr (PAIR)
+                commit_pair_local(smem_u32(mma_done));
+            else
+                mma_commit(smem_u32(mma_done));
             const uint64_t t0 = global_ns();
             while (!mbar_try_wait(smem_u32(mma_done), 0))
                 if (global_ns() - t0 > kTimeoutNs) {
@@ -303,7 +349,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmAq, const __grid_constant__
         const int own = packed && SELF ? row / T * T : 0;
         uint32_t cnt = 0;
         bool ok = true, stop = false;
-        for (int64_t u = blockIdx.x; !stop && u < p.n_units; u += gridDim.x) {
+        for (int64_t u = u0; !stop && u < p.n_units; u += ustep) {
             float tot = 0.f;  // T > 128 and SELF: this thread's share of the sum
             int ti = 0, tj = 0;
             for (int tp = 0; tp < tpp; ++tp) {
@@ -395,7 +441,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmAq, const __grid_constant__
                     }
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&tempty[b]));
+                    if (lane == 0) arrive_leader<PAIR>(smem_u32(&tempty[b]));
                 }
                 if (!ok) break;
                 tot = SELF && ti != tj ? fmaf(2.f, tile, tot) : tot + tile;  // (i, j) stands for (j, i) too
@@ -436,7 +482,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmAq, const __grid_constant__
                             for (int t = lanes > 1 ? lane : 0; t < T; t += lanes) v += r[(size_t)t * p.ldr];
                         }
                         if (lanes > 1) v = warp_sum(v);
-                        const int64_t qq = (SELF ? u : u % p.n_qtiles) * p.pq + qi;
+                        const int64_t qq = qtile(u) * p.pq + qi;
                         const int64_t ii = SELF ? 0 : (u / p.n_qtiles) * p.pt + g;
                         if (lanes == 1 || lane == 0) {
                             if (SELF) {
@@ -454,9 +500,13 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmAq, const __grid_constant__
 
     tc_fence_before();
     __syncthreads();
+    if constexpr (PAIR) cluster_sync();
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem, kTmemCols);
+        if constexpr (PAIR)
+            tmem_dealloc2(tmem, kTmemCols);
+        else
+            tmem_dealloc(tmem, kTmemCols);
     }
 }
 
@@ -519,16 +569,59 @@ int sm_count() {
     return n;
 }
 
+template <bool SELF, bool PAIR>
+cudaError_t launch_kernel(const tda_layer_desc& L, const void* Aq, const void* Bq, int64_t n_q, const void* At,
+                          const void* Bt, int64_t n_t, GParams p, cudaStream_t s) {
+    using C = Cfg<SELF, PAIR>;
+    const bool packed = L.T <= kTM;
+    CUtensorMap mAq, mAt, mBq, mBt;
+    if (!make_side(&mAq, &mBq, L, Aq, Bq, n_q, packed, kTM) || !make_side(&mAt, &mBt, L, At, Bt, n_t, packed, C::kBRows))
+        return cudaErrorInvalidValue;
+    if (PAIR) p.n_qtiles = (p.n_qtiles + 1) / 2;
+    if (SELF)
+        p.n_units = packed ? p.n_qtiles : n_q;
+    else
+        p.n_units = packed ? p.n_qtiles * ((n_t + p.pt - 1) / p.pt) : n_q * n_t;
+    // partial sums of a packed tile: rows of an odd stride (no bank conflicts)
+    const int64_t T = L.T;
+    p.ldr = !packed || SELF ? 1 : (int)(T < 16 ? C::kCols / T : (C::kCols - 1) / T + 2) | 1;
+    const size_t red = packed ? 2 * (size_t)kTM * p.ldr * sizeof(float) : 0;
+    const int64_t stages = ((int64_t)kSmemMax - 1024 - (int64_t)kTailBytes - (int64_t)red) / C::kStageBytes;
+    if (stages < 2) return cudaErrorInvalidValue;
+    p.stages = stages < kMaxStages ? (int)stages : kMaxStages;
+    const size_t smem = 1024 + (size_t)p.stages * C::kStageBytes + kTailBytes + red;
+    cudaError_t e = smem_attr_once<gram_tc_kernel<SELF, PAIR>>((int)kSmemMax);
+    if (e != cudaSuccess) return e;
+    const int64_t room = PAIR ? (sm_count() > 1 ? sm_count() / 2 : 1) : sm_count();
+    const int64_t grid = (p.n_units < room ? p.n_units : room) * (PAIR ? 2 : 1);
+    note_launches(1);
+    if constexpr (PAIR) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 2;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3((unsigned)grid);
+        cfg.blockDim = dim3(kThreads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = s;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        e = cudaLaunchKernelEx(&cfg, gram_tc_kernel<SELF, PAIR>, mAq, mAt, mBq, mBt, p);
+        if (e != cudaSuccess) return e;
+    } else {
+        gram_tc_kernel<SELF, PAIR><<<(unsigned)grid, kThreads, smem, s>>>(mAq, mAt, mBq, mBt, p);
+    }
+    return cudaGetLastError();
+}
+
 template <bool SELF>
 cudaError_t launch(const tda_layer_desc& L, const void* Aq, const void* Bq, int64_t n_q, const void* At,
                    const void* Bt, int64_t n_t, GParams p, cudaStream_t s) {
     using C = Cfg<SELF>;
-    const int64_t T = L.T;
+    const int64_t T = L.T, sms = sm_count();
     const bool packed = T <= kTM;
-    CUtensorMap mAq, mAt, mBq, mBt;
-    if (!make_side(&mAq, &mBq, L, Aq, Bq, n_q, packed, kTM) ||
-        !make_side(&mAt, &mBt, L, At, Bt, n_t, packed, C::kTN))
-        return cudaErrorInvalidValue;
     p.n_q = n_q;
     p.n_t = n_t;
     p.T = T;
@@ -536,8 +629,8 @@ cudaError_t launch(const tda_layer_desc& L, const void* Aq, const void* Bq, int6
     p.nk_out = (int)((L.d_out + kChunkK - 1) / kChunkK);
     // Block lengths that keep the accuracy of an fp32 FMA chain over d features (1.8e-7 at d = 256,
     // 5.7e-7 at 2048, 8.9e-7 at 4096): 64, 128 or 256 features, whose truncation is 1.1e-7, 2.2e-7 or
-    // 4.5e-7. Short sequences (T < 16) pay the most per Y block and take it twice as long.
-    auto block = [](int nk) { return nk <= 8 ? 1 : (nk < 64 ? 2 : 4); };
+    // 4.5e-7 (2048 -> 2048, T = 50: 4.4e-7 with 256, 183 -> 143 us from 128). Short sequences (T < 16) pay the most per Y block and take it twice as long.
+    auto block = [](int nk) { return nk <= 8 ? 1 : (nk < 32 ? 2 : 4); };
     p.kbx = block(p.nk_in);
     p.kby = block(p.nk_out) * (packed && T < 16 ? 2 : 1);
     p.pq = packed ? (int)(kTM / T) : 0;
@@ -545,23 +638,17 @@ cudaError_t launch(const tda_layer_desc& L, const void* Aq, const void* Bq, int6
     p.tiles_q = packed ? 1 : (int)((T + kTM - 1) / kTM);
     p.tiles_t = packed ? 1 : (int)((T + C::kTN - 1) / C::kTN);
     p.n_qtiles = packed ? (n_q + p.pq - 1) / p.pq : 0;
-    if (SELF)
-        p.n_units = packed ? p.n_qtiles : n_q;
-    else
-        p.n_units = packed ? p.n_qtiles * ((n_t + p.pt - 1) / p.pt) : n_q * n_t;
-    // partial sums of a packed tile: rows of an odd stride (no bank conflicts)
-    p.ldr = !packed || SELF ? 1 : (int)(T < 16 ? C::kCols / T : (C::kCols - 1) / T + 2) | 1;
-    const size_t red = packed ? 2 * (size_t)kTM * p.ldr * sizeof(float) : 0;
-    const int64_t stages = ((int64_t)kSmemMax - 1024 - (int64_t)kTailBytes - (int64_t)red) / C::kStageBytes;
-    if (stages < 2) return cudaErrorInvalidValue;
-    p.stages = stages < kMaxStages ? (int)stages : kMaxStages;
-    const size_t smem = 1024 + (size_t)p.stages * C::kStageBytes + kTailBytes + red;
-    cudaError_t e = smem_attr_once<gram_tc_kernel<SELF>>((int)kSmemMax);
-    if (e != cudaSuccess) return e;
-    const int64_t grid = p.n_units < sm_count() ? p.n_units : sm_count();
-    note_launches(1);
-    gram_tc_kernel<SELF><<<(unsigned)grid, kThreads, smem, s>>>(mAq, mAt, mBq, mBt, p);
-    return cudaGetLastError();
+    if constexpr (!SELF) {
+        // Pairs of CTAs take two query tiles against one train tile: each has half of the train rows to
+        // copy and to read (512 clocks of shared memory a chunk instead of 768). 8192 -> 8192, T = 32, 64 x
+        // 512 examples: 682 us in single CTAs, 634 us in pairs. Not where an odd tile count makes more
+        // rounds, nor for few features, where a pair's start costs more (256 -> 256: 19 and 21 us).
+        const int64_t tt = packed ? (n_t + p.pt - 1) / p.pt : 0;
+        const int64_t ones = (p.n_qtiles * tt + sms - 1) / sms, half = sms > 1 ? sms / 2 : 1;
+        const int64_t pairs = ((p.n_qtiles + 1) / 2 * tt + half - 1) / half;
+        if (packed && p.n_qtiles >= 2 && pairs <= ones && p.nk_in + p.nk_out >= 48) return launch_kernel<false, true>(L, Aq, Bq, n_q, At, Bt, n_t, p, s);
+    }
+    return launch_kernel<SELF, false>(L, Aq, Bq, n_q, At, Bt, n_t, p, s);
 }
 
 }  // namespace

@@ -166,6 +166,40 @@ __device__ __forceinline__ bool wait_bounded_cluster(uint32_t bar, uint32_t pari
     }
 }
 
+// ---- pairs of CTAs that share a tile (cta_group::2; PAIR false: one CTA a tile)
+// Arrives on `bar` of every CTA of the tile once the MMAs issued so far are done.
+template <bool PAIR>
+__device__ __forceinline__ void commit_all(uint32_t bar) {
+    if constexpr (PAIR)
+        asm volatile(
+            "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+            "h"((uint16_t)3)
+            : "memory");
+    else
+        mma_commit(bar);
+}
+__device__ __forceinline__ void commit_pair_local(uint32_t bar) {
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void tmem_alloc2(uint32_t dst, uint32_t ncols) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst), "r"(ncols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_dealloc2(uint32_t taddr, uint32_t ncols) {
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+}
+// Arrives on CTA 0's `bar` of the tile. The operands that it announces are ordered by tcgen05.wait::st and
+// fence.proxy.async; a release at cluster scope would wait for all of the warp's writes (1100
+// clocks).
+template <bool PAIR>
+__device__ __forceinline__ void arrive_leader(uint32_t bar) {
+    if constexpr (PAIR)
+        asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(map_rank(bar, 0u)) : "memory");
+    else
+        mbar_arrive(bar);
+}
+
 // OR of `v` over the 128 epilogue threads, through named barrier 1.
 __device__ __forceinline__ bool epi_any(bool v) {
     uint32_t r;

@@ -45,7 +45,10 @@ def scale(Aq, Bq, At, Bt):
 @pytest.mark.parametrize("nq,nt,T,di,do", [
     (5, 300, 1, 64, 40), (7, 140, 2, 136, 64), (9, 100, 3, 72, 64), (30, 61, 5, 200, 136), (5, 12, 21, 520, 1032),
     (70, 131, 50, 64, 72), (5, 9, 63, 64, 64), (6, 9, 65, 128, 136), (20, 31, 100, 64, 64), (3, 5, 127, 64, 200),
-    (3, 5, 129, 72, 64), (2, 3, 200, 264, 128), (2, 3, 257, 64, 72), (13, 14, 300, 64, 64)])
+    (3, 5, 129, 72, 64), (2, 3, 200, 264, 128), (2, 3, 257, 64, 72), (13, 14, 300, 64, 64),
+    # pairs of CTAs: odd and even query tiles, one example a tile, ragged last train tile
+    (5, 9, 50, 1544, 1608), (3, 7, 128, 2048, 1032), (140, 70, 1, 1600, 1536), (17, 33, 13, 3072, 64),
+    (4, 11, 64, 64, 3080)])
 def test_gram_any_token_count(dev, orc, nq, nt, T, di, do):
     Aq, Bq = factors(nq, T, di, do, 51)
     At, Bt = factors(nt, T, di, do, 52)
