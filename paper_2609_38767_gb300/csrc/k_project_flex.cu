@@ -27,14 +27,15 @@
 // partial blocks are reduce-scattered over distributed shared memory: every CTA
 // sums and writes 1/cs of Phi.
 //
-// Signs: a byte of a sign word becomes eight bf16 signs by one table read (a second
-// pair of generator warps, each taking every other stage, measured 6 % slower).
+// Signs: a byte of a sign word becomes eight bf16 signs by one table read. bf16 factors at k = 64 have
+// two pairs of generator warps that take every other stage (96 x 130 tokens, 1000 -> 4096: 70 us
+// with one pair, 60 us with two); elsewhere a second pair costs 1 to 3 %.
 //
 // Measured, fp32: 64 examples of 512 tokens, 2048 -> 2048, k = 32 (537 MB): 7.6 ms
 // on the CUDA cores, 102 us here. bf16: see plan_bf16_flex().
 //
-// Warp roles (fp32 512, bf16 256 threads, one persistent CTA per SM): warp 0 TMA
-// producer; warp 1 TMEM allocator and MMA issuer; warps 2-3 sign generators;
+// Warp roles (fp32 512, bf16 256 or 320 threads, one persistent CTA per SM): warp 0 TMA
+// producer; warp 1 TMEM allocator and MMA issuer; warps 2-3 (8-9) sign generators;
 // warps 4-7 epilogue; fp32: warps 8-15 split. Every wait is bounded (about 1 s); on
 // expiry the kernel records kErrTimeout, drains its copies, frees its TMEM and
 // returns.
@@ -60,7 +61,8 @@ constexpr size_t kLutBytes = 256 * 16;
 
 template <int K, bool F32>
 struct Cfg {
-    static constexpr int kThreads = F32 ? 512 : 256;
+    static constexpr int kSignPairs = !F32 && K >= 64 ? 2 : 1;  // warps 2-3, 8-9
+    static constexpr int kThreads = F32 ? 512 : 256 + 64 * (kSignPairs - 1);
     static constexpr uint32_t kTileBytes = (F32 ? 2 : 1) * kBoxBytes;
     static constexpr uint32_t kSignBytes = K * 128;
     static constexpr uint32_t kStageBytes = kTileBytes + kSignBytes;
@@ -303,15 +305,20 @@ project_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 }
         }
         __syncwarp();
-    } else if (warp == 2 || warp == 3) {
-        // ---------------- sign generators: the 64 threads share a tile's K rows, kParts threads per row
+    } else if (warp == 2 || warp == 3 || (C::kSignPairs == 2 && warp >= 8)) {
+        // ---------------- sign generators: a pair of warps takes a stage, its 64 threads share a tile's K
+        // rows, kParts threads per row; two pairs take turns
         constexpr int kParts = 64 / K, kChunks = 8 / kParts;
         const int g = (warp & 1) * 32 + lane, col = g / kParts, part = g % kParts;
         const uint32_t lut_s = smem_u32(lut);
-        uint32_t s = 0, ph = 0;
+        uint32_t s = 0, ph = 0, turn = warp >= 8 ? 1u : 0u;
         bool ok = true;
         for (; ok && it.x < p.n_slots; it.next(p, ncl, crank))
-            for (int kc = 0; kc < nk_tot; ++kc) {
+            for (int kc = 0; kc < nk_tot; ++kc, turn ^= 1u) {
+                if (C::kSignPairs == 2 && turn) {  // the other pair's
+                    if (++s == (uint32_t)C::kStages) s = 0, ph ^= 1u;
+                    continue;
+                }
                 const bool side_b = kc >= p.nk_in;
                 const uint64_t w = sign_word(side_b ? p.key_out : p.key_in, (uint32_t)col,
                                              (uint64_t)(side_b ? kc - p.nk_in : kc));
@@ -623,7 +630,7 @@ int max_clusters(int cs) {
 // k_project_tc.cu: per 128-row tile, without and with the workspace's equal runs (bal).
 template <int K, bool F32>
 double chunk_clocks(int R) {
-    const double data = R * (F32 ? 9.0 : 4.2), least = F32 ? 800.0 : (K <= 16 ? 430.0 : (K <= 32 ? 460.0 : 670.0));
+    const double data = R * (F32 ? 9.0 : 4.2), least = F32 ? 800.0 : (K <= 16 ? 430.0 : (K <= 32 ? 460.0 : 590.0));
     return data > least ? data : least;
 }
 double stream_chunk_clocks(int K, bool bal) { return K >= 64 ? 950.0 : (bal ? 600.0 : 560.0); }
