@@ -1634,7 +1634,7 @@ __global__ void __launch_bounds__(kDiagThreads) diag_panel_kernel(St<float> st, 
 // coefficients (k: solved or own column, i: column of the block). A thread has RT x 4 entries, so
 // a slab value read from shared memory serves RT products. R = 128 for many rows, 16 where few
 // rows would leave SMs idle. Seven layers, 256 columns: 3840 rows each 131 us as two 128-column
-// solves (a warp per row) and a product between them, 118 us here; 256 rows each 29 us.
+// solves (a warp per row) and a product between them, 99 us here; 256 rows each 26 us.
 template <int R>
 struct SolveCfg {
     static constexpr int RT = R / 16;                       // 16 row groups x 16 column groups
@@ -1684,41 +1684,69 @@ __global__ void __launch_bounds__(256) solve_kernel(St<float> st, int64_t lo, in
                                       : make_float4(0.f, 0.f, 0.f, 0.f);
          },
          [&](int e, const float4& v) { *reinterpret_cast<float4*>(&xs[e / q4][e % q4 * 4]) = v; });
+    // Block b's coefficients: the solved columns' (4 nblk x 64 items of 16 bytes at most) and W's, one to
+    // four of the thread's items each. They are loaded into registers beside the previous block's
+    // products and stored behind them.
     const int nblk = nb / 64;
+    float4 pl[12], pw[4];
+    auto block = [&](int s, int& c0, int& k0, int& nk) {  // its columns and the solved ones
+        const int b = FWD ? s : nblk - 1 - s;
+        c0 = 64 * b;
+        k0 = FWD ? 0 : c0 + 64;
+        nk = FWD ? c0 : nb - c0 - 64;
+    };
+    auto load = [&](int s) {
+        int c0, k0, nk;
+        block(s, c0, k0, nk);
+#pragma unroll
+        for (int u = 0; u < 12; ++u) {
+            const int e = tid + 256 * u;
+            if (16 * u < nk)  // FWD: L[c0 + e % 64][e / 64 * 4 ..]; else L[k0 + e / 16][c0 + e % 16 * 4 ..]
+                pl[u] = *reinterpret_cast<const float4*>(FWD ? M + (int64_t)(c0 + e % 64) * D + e / 64 * 4
+                                                             : M + (int64_t)(k0 + e / 16) * D + c0 + e % 16 * 4);
+        }
+        if (w64)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int e = tid + 256 * u;
+                pw[u] = *reinterpret_cast<const float4*>(M + (int64_t)(c0 + e / 16) * D + c0 + e % 16 * 4);
+            }
+    };
+    load(0);
     for (int s = 0; s < nblk; ++s) {
-        const int b = FWD ? s : nblk - 1 - s, c0 = 64 * b;   // this block's columns
-        const int k0 = FWD ? 0 : c0 + 64, nk = FWD ? c0 : nb - c0 - 64;  // the solved columns
+        int c0, k0, nk;
+        block(s, c0, k0, nk);
         __syncthreads();  // the previous block's slab is read
         // slab rows 0 .. nk-1: L between the block's columns and the solved ones; rows nk .. nk+63: W
-        if (FWD)  // S[k][i] = L[c0 + i][k], a warp's lanes along i: every store hits 32 banks
-            copy(16 * nk, [&](int e) { return *reinterpret_cast<const float4*>(M + (int64_t)(c0 + e % 64) * D + e / 64 * 4); },
-                 [&](int e, const float4& v) {
-                     const int i = e % 64, k = e / 64 * 4;
-                     S[k][i ^ ((k & 7) << 2)] = v.x;
-                     S[k + 1][i ^ (((k + 1) & 7) << 2)] = v.y;
-                     S[k + 2][i ^ (((k + 2) & 7) << 2)] = v.z;
-                     S[k + 3][i ^ (((k + 3) & 7) << 2)] = v.w;
-                 });
-        else      // S[k][i] = L[k0 + k][c0 + i]
-            copy(16 * nk,
-                 [&](int e) { return *reinterpret_cast<const float4*>(M + (int64_t)(k0 + e / 16) * D + c0 + e % 16 * 4); },
-                 [&](int e, const float4& v) {
-                     const int k = e / 16;
-                     *reinterpret_cast<float4*>(&S[k][(e % 16 * 4) ^ ((k & 7) << 2)]) = v;
-                 });
+#pragma unroll
+        for (int u = 0; u < 12; ++u) {
+            const int e = tid + 256 * u;
+            if (16 * u >= nk) continue;
+            const float4 v = pl[u];
+            if (FWD) {  // S[k][i] = L[c0 + i][k], a warp's lanes along i: every store hits 32 banks
+                const int i = e % 64, k = e / 64 * 4;
+                S[k][i ^ ((k & 7) << 2)] = v.x;
+                S[k + 1][i ^ (((k + 1) & 7) << 2)] = v.y;
+                S[k + 2][i ^ (((k + 2) & 7) << 2)] = v.z;
+                S[k + 3][i ^ (((k + 3) & 7) << 2)] = v.w;
+            } else {    // S[k][i] = L[k0 + k][c0 + i]
+                const int k = e / 16;
+                *reinterpret_cast<float4*>(&S[k][(e % 16 * 4) ^ ((k & 7) << 2)]) = v;
+            }
+        }
         if (w64) {
             // the block as stored: L left of the diagonal, W^T right of it. FWD: S[k][i] = W[i][k] =
             // stored[k][i] for k < i; else S[k][i] = W[k][i] = stored[i][k] for k > i
-            copy(64 * 16, [&](int e) { return *reinterpret_cast<const float4*>(M + (int64_t)(c0 + e / 16) * D + c0 + e % 16 * 4); },
-                 [&](int e, const float4& v4) {
-                     const int a = e / 16, c = e % 16 * 4;
-                     const float v[4] = {v4.x, v4.y, v4.z, v4.w};
 #pragma unroll
-                     for (int t = 0; t < 4; ++t) {
-                         const int i = FWD ? c + t : a, k = FWD ? a : c + t, kr = nk + k;
-                         S[kr][i ^ ((kr & 7) << 2)] = (FWD ? k < i : k > i) ? v[t] : (k == i ? 1.f / v[t] : 0.f);
-                     }
-                 });
+            for (int u = 0; u < 4; ++u) {
+                const int e = tid + 256 * u, a = e / 16, c = e % 16 * 4;
+                const float v[4] = {pw[u].x, pw[u].y, pw[u].z, pw[u].w};
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    const int i = FWD ? c + t : a, k = FWD ? a : c + t, kr = nk + k;
+                    S[kr][i ^ ((kr & 7) << 2)] = (FWD ? k < i : k > i) ? v[t] : (k == i ? 1.f / v[t] : 0.f);
+                }
+            }
         } else {
             // a state factored before these inverses were kept: from the 32 x 32 ones,
             // W = [W00 0; -W11 (L10 W00) W11]
@@ -1744,6 +1772,7 @@ __global__ void __launch_bounds__(256) solve_kernel(St<float> st, int64_t lo, in
             }
         }
         __syncthreads();
+        if (s + 1 < nblk) load(s + 1);
         float acc[RT][4];  // the solved columns' share less x, so that both products add
 #pragma unroll
         for (int u = 0; u < RT; ++u) {
@@ -1799,21 +1828,33 @@ __global__ void __launch_bounds__(256) solve_kernel(St<float> st, int64_t lo, in
     }
 }
 
-// Lower triangle of M <- M / n_total + lambda I for the blocked path: one row per
-// loop step of a CTA, the row's columns across the threads (coalesced, no per-element
-// index division). grid (row groups, layer).
+// Lower triangle of M <- M / n_total + lambda I for the blocked path: a warp per row, 16 bytes a lane
+// (which scales up to three entries right of the diagonal too: they are overwritten later).
+// grid (row groups, layer).
 __global__ void __launch_bounds__(256) scale_lower_kernel(St<float> st) {
-    const int l = blockIdx.y;
+    const int l = blockIdx.y, lane = threadIdx.x & 31;
     const int64_t D = st.D;
     const double* h = st.header(l);
     const float inv_n = (float)(1.0 / h[kPcNTotal]), lam = (float)h[kPcLambda];
     float* M = st.M(l);
-    for (int64_t a = blockIdx.x; a < D; a += gridDim.x) {
+    for (int64_t a = blockIdx.x * 8 + (threadIdx.x >> 5); a < D; a += gridDim.x * 8) {
         float* row = M + a * D;
-        for (int64_t b = threadIdx.x; b <= a; b += 256) {
-            float v = row[b] * inv_n;
-            if (b == a) v += lam;
-            row[b] = v;
+        for (int64_t b0 = 4 * lane; b0 <= a; b0 += 4 * 128) {
+            float4 v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (b0 + 128 * u <= a) v[u] = *reinterpret_cast<const float4*>(row + b0 + 128 * u);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int64_t b = b0 + 128 * u;
+                if (b > a) break;
+                float4 w = make_float4(v[u].x * inv_n, v[u].y * inv_n, v[u].z * inv_n, v[u].w * inv_n);
+                if (b == a) w.x += lam;
+                if (b + 1 == a) w.y += lam;
+                if (b + 2 == a) w.z += lam;
+                if (b + 3 == a) w.w += lam;
+                *reinterpret_cast<float4*>(row + b) = w;
+            }
         }
     }
 }
@@ -1915,8 +1956,8 @@ cudaError_t factor_blocked(int n_layers, int64_t D, void* state, int64_t n_total
     St<float> st = state_of<float>(state, D);
     note_launches(2);
     prepare_kernel<float><<<n_layers, 256, 0, s>>>(st, n_total, la, lr);
-    const unsigned rows_per = (unsigned)((D < 1024 ? D : 1024) * (n_layers < 8 ? 8 / n_layers : 1));
-    scale_lower_kernel<<<dim3(rows_per < (unsigned)D ? rows_per : (unsigned)D, n_layers), 256, 0, s>>>(st);
+    const int64_t per = (D + 7) / 8, most = 152 * 8 / n_layers > 1 ? 152 * 8 / n_layers : 1;
+    scale_lower_kernel<<<dim3((unsigned)(per < most ? per : most), n_layers), 256, 0, s>>>(st);
     float* M0 = (float*)((char*)state + 64);  // layer l's M is st.bytes further on
     const int64_t cz = (int64_t)(st.bytes / 4);
     const size_t lb = (size_t)D * 4;
