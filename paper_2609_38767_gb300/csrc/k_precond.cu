@@ -1634,10 +1634,11 @@ __global__ void __launch_bounds__(kDiagThreads) diag_panel_kernel(St<float> st, 
 // coefficients (k: solved or own column, i: column of the block). A thread has RT x 4 entries, so
 // a slab value read from shared memory serves RT products. R = 128 for many rows, 16 where few
 // rows would leave SMs idle. Seven layers, 256 columns: 3840 rows each 131 us as two 128-column
-// solves (a warp per row) and a product between them, 99 us here; 256 rows each 26 us.
+// solves (a warp per row) and a product between them, 91 us here; 256 rows each 26 us.
 template <int R>
 struct SolveCfg {
-    static constexpr int RT = R / 16;                       // 16 row groups x 16 column groups
+    static constexpr int NT = R >= 96 ? 512 : 256;          // threads (R = 96: 99 us with 256, 91 with 512)
+    static constexpr int RT = R / (NT / 16);                // NT / 16 row groups x 16 column groups
     static constexpr int kLdX = 2 * kBB + 4;
     static constexpr size_t kSmem = sizeof(float) * ((size_t)R * kLdX + (size_t)2 * kBB * 64 + kNB * (kNB + 1));
 };
@@ -1647,10 +1648,10 @@ struct SolveRows {
     int64_t ldx, n_rows;
 };
 template <int R, bool FWD>
-__global__ void __launch_bounds__(256) solve_kernel(St<float> st, int64_t lo, int nb, SolveRows rows_a, SolveRows rows_b,
+__global__ void __launch_bounds__(SolveCfg<R>::NT) solve_kernel(St<float> st, int64_t lo, int nb, SolveRows rows_a, SolveRows rows_b,
                                                     int blocks_a) {
     using C = SolveCfg<R>;
-    constexpr int RT = C::RT;
+    constexpr int RT = C::RT, NT = C::NT, kPl = 12 * 256 / NT, kPw = 4 * 256 / NT;
     extern __shared__ __align__(16) float ssm[];
     float(*xs)[C::kLdX] = reinterpret_cast<float(*)[C::kLdX]>(ssm);
     float(*S)[64] = reinterpret_cast<float(*)[64]>(ssm + R * C::kLdX);  // [k][i ^ 4 (k & 7)]
@@ -1666,14 +1667,14 @@ __global__ void __launch_bounds__(256) solve_kernel(St<float> st, int64_t lo, in
     float* X = (float*)(w.base + (size_t)l * w.layer_bytes) + lo;
     // n 16-byte loads, eight of a thread's in flight together: ld(e) loads item e, st(e, value) stores it
     auto copy = [&](int n, auto&& ld, auto&& st) {
-        for (int e0 = tid; e0 < n; e0 += 8 * 256) {
+        for (int e0 = tid; e0 < n; e0 += 8 * NT) {
             float4 v[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u)
-                if (e0 + 256 * u < n) v[u] = ld(e0 + 256 * u);
+                if (e0 + NT * u < n) v[u] = ld(e0 + NT * u);
 #pragma unroll
             for (int u = 0; u < 8; ++u)
-                if (e0 + 256 * u < n) st(e0 + 256 * u, v[u]);
+                if (e0 + NT * u < n) st(e0 + NT * u, v[u]);
         }
     };
     const int q4 = nb / 4;
@@ -1688,7 +1689,7 @@ __global__ void __launch_bounds__(256) solve_kernel(St<float> st, int64_t lo, in
     // four of the thread's items each. They are loaded into registers beside the previous block's
     // products and stored behind them.
     const int nblk = nb / 64;
-    float4 pl[12], pw[4];
+    float4 pl[kPl], pw[kPw];
     auto block = [&](int s, int& c0, int& k0, int& nk) {  // its columns and the solved ones
         const int b = FWD ? s : nblk - 1 - s;
         c0 = 64 * b;
@@ -1699,16 +1700,16 @@ __global__ void __launch_bounds__(256) solve_kernel(St<float> st, int64_t lo, in
         int c0, k0, nk;
         block(s, c0, k0, nk);
 #pragma unroll
-        for (int u = 0; u < 12; ++u) {
-            const int e = tid + 256 * u;
-            if (16 * u < nk)  // FWD: L[c0 + e % 64][e / 64 * 4 ..]; else L[k0 + e / 16][c0 + e % 16 * 4 ..]
+        for (int u = 0; u < kPl; ++u) {
+            const int e = tid + NT * u;
+            if (NT / 16 * u < nk)  // FWD: L[c0 + e % 64][e / 64 * 4 ..]; else L[k0 + e / 16][c0 + e % 16 * 4 ..]
                 pl[u] = *reinterpret_cast<const float4*>(FWD ? M + (int64_t)(c0 + e % 64) * D + e / 64 * 4
                                                              : M + (int64_t)(k0 + e / 16) * D + c0 + e % 16 * 4);
         }
         if (w64)
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int e = tid + 256 * u;
+            for (int u = 0; u < kPw; ++u) {
+                const int e = tid + NT * u;
                 pw[u] = *reinterpret_cast<const float4*>(M + (int64_t)(c0 + e / 16) * D + c0 + e % 16 * 4);
             }
     };
@@ -1719,9 +1720,9 @@ __global__ void __launch_bounds__(256) solve_kernel(St<float> st, int64_t lo, in
         __syncthreads();  // the previous block's slab is read
         // slab rows 0 .. nk-1: L between the block's columns and the solved ones; rows nk .. nk+63: W
 #pragma unroll
-        for (int u = 0; u < 12; ++u) {
-            const int e = tid + 256 * u;
-            if (16 * u >= nk) continue;
+        for (int u = 0; u < kPl; ++u) {
+            const int e = tid + NT * u;
+            if (NT / 16 * u >= nk) continue;
             const float4 v = pl[u];
             if (FWD) {  // S[k][i] = L[c0 + i][k], a warp's lanes along i: every store hits 32 banks
                 const int i = e % 64, k = e / 64 * 4;
@@ -1738,8 +1739,8 @@ __global__ void __launch_bounds__(256) solve_kernel(St<float> st, int64_t lo, in
             // the block as stored: L left of the diagonal, W^T right of it. FWD: S[k][i] = W[i][k] =
             // stored[k][i] for k < i; else S[k][i] = W[k][i] = stored[i][k] for k > i
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int e = tid + 256 * u, a = e / 16, c = e % 16 * 4;
+            for (int u = 0; u < kPw; ++u) {
+                const int e = tid + NT * u, a = e / 16, c = e % 16 * 4;
                 const float v[4] = {pw[u].x, pw[u].y, pw[u].z, pw[u].w};
 #pragma unroll
                 for (int t = 0; t < 4; ++t) {
@@ -1751,14 +1752,14 @@ __global__ void __launch_bounds__(256) solve_kernel(St<float> st, int64_t lo, in
             // a state factored before these inverses were kept: from the 32 x 32 ones,
             // W = [W00 0; -W11 (L10 W00) W11]
             const float *D0 = st.Dinv(l) + (lo + c0) / kNB * (kNB * kNB), *D1 = D0 + kNB * kNB;
-            for (int e = tid; e < kNB * kNB; e += 256) {
+            for (int e = tid; e < kNB * kNB; e += NT) {
                 const int i = e / kNB, k = e % kNB;
                 float t = 0.f;
                 for (int m = k; m < kNB; ++m) t = fmaf(M[(int64_t)(c0 + kNB + i) * D + c0 + m], D0[m * kNB + k], t);
                 T[i][k] = t;
             }
             __syncthreads();
-            for (int e = tid; e < 64 * 64; e += 256) {
+            for (int e = tid; e < 64 * 64; e += NT) {
                 const int r = e / 64, c = e % 64;
                 float w = 0.f;
                 if (c <= r && r < kNB)
@@ -1821,7 +1822,7 @@ __global__ void __launch_bounds__(256) solve_kernel(St<float> st, int64_t lo, in
         store(1.f);
     }
     __syncthreads();
-    for (int e = tid; e < R * q4; e += 256) {
+    for (int e = tid; e < R * q4; e += NT) {
         const int r = e / q4, c = e % q4 * 4;
         if (row0 + r < n_rows)
             *reinterpret_cast<float4*>(X + (row0 + r) * ldx + c) = *reinterpret_cast<const float4*>(&xs[r][c]);
@@ -1917,7 +1918,7 @@ cudaError_t launch_solve_r(St<float> st, int n_layers, int64_t lo, int nb, const
     const int64_t na = (a.n_rows + R - 1) / R, nb_b = (b.n_rows + R - 1) / R;
     if (na + nb_b == 0) return cudaSuccess;
     note_launches(1);
-    solve_kernel<R, FWD><<<dim3((unsigned)(na + nb_b), n_layers), 256, SolveCfg<R>::kSmem, s>>>(st, lo, nb, a, b, (int)na);
+    solve_kernel<R, FWD><<<dim3((unsigned)(na + nb_b), n_layers), SolveCfg<R>::NT, SolveCfg<R>::kSmem, s>>>(st, lo, nb, a, b, (int)na);
     return cudaGetLastError();
 }
 
