@@ -301,17 +301,19 @@ tda_status tda_cosine(float* S, int64_t n_q, int64_t n_t, int64_t ld_S, const fl
  *                     state). Layers whose FACTOR failed get NaN rows.
  *                     Needs D <= 40960 (F32) or 20480 (F64).
  *   TDA_PC_FACTOR_APPLY  FACTOR, then APPLY, in one call (same arguments and
- *                     results as the two; a failed layer's rows are NaN). For an
- *                     F32 state with D a multiple of 32 below 2048 and n_q <= 256
- *                     both run in one launch: the query rows are solved alongside
- *                     the factorisation (forward substitution as extra rows of
- *                     each step) and then backward. qhat may not alias q.
- * Large layers (F32 state, D a multiple of 128, D >= 2048): FACTOR is a blocked
- * Cholesky in 256-column panels whose trailing updates run on the tensor cores
- * (3xTF32, fp32-accurate); it also leaves L^T in M's upper triangle, and APPLY
- * (qhat 16-byte aligned, ld_qhat a multiple of 4) then solves the query rows in
- * 128-column blocks with tensor-core updates. In this mode qhat may alias q
- * (same pointer and row stride: solved in place).
+ *                     results as the two; a failed layer's rows are NaN): the
+ *                     query rows are solved alongside the factorisation (forward
+ *                     substitution as extra rows of each step) and then backward.
+ *                     qhat may not alias q, except as below.
+ * F32 state, D a multiple of 64, D >= 256: FACTOR is a blocked Cholesky in
+ * 256-column panels whose trailing updates run on the tensor cores (3xTF32,
+ * fp32-accurate); it also leaves L^T in M's upper triangle (inside the 64 x 64
+ * diagonal blocks, the transposed inverse of the block). FACTOR_APPLY, and APPLY
+ * for D >= 2048, D a multiple of 128 (both with qhat 16-byte aligned, ld_qhat a
+ * multiple of 4), solve the query rows in 256-column blocks with tensor-core updates. In this mode
+ * qhat may alias q (same pointer and row stride: solved in place). Other F32
+ * layers with D a multiple of 32 run FACTOR_APPLY for n_q <= 256 in one launch.
+ * A state factored by an earlier version of the library can be passed to APPLY.
  * Arguments not used by an op are ignored (may be 0/NULL).
  * ------------------------------------------------------------------------- */
 #define TDA_PC_RESET 0
@@ -453,11 +455,10 @@ tda_status tda_mask_gather(const tda_layer_desc* L, tda_dtype dtype, const void*
  *         With TDA_F64 the sum is accumulated in fp64 (CUDA cores). With
  *         TDA_F32 on sm_103 (aligned rows, D >= 64) the sum runs on the tensor
  *         cores as three TF32 products per element pair (hi*hi + hi*lo + lo*hi
- *         of the split x = hi + lo), accurate to about fp32 rounding at the
- *         feature counts of a block (1e-5 relative at D = 7168). The tensor
- *         pipe's fp32 accumulators add with truncation, so the error grows with
- *         the features per call: rows of ~10^6 features are better scored in
- *         blocks of features accumulated with beta = 1.
+ *         of the split x = hi + lo), accurate to about fp32 rounding (1e-6
+ *         relative at D = 7168): the tensor pipe's fp32 accumulators add with
+ *         truncation, and every 64 features they are added to registers with
+ *         round-to-nearest.
  *   Phi   device fp32, n_t rows of D, row stride ld_phi.
  *   S     device fp32, row stride ld_S >= n_t. beta 0 overwrites (S may hold
  *         garbage); beta 1 accumulates layers.

@@ -1163,10 +1163,10 @@ cudaError_t launch_gemm_nt_tc_batched(const float* A, int64_t n_a, int64_t lda, 
     p.splits = 1;
     p.s_z = c_z;
     p.err = err;
-    if (lower && (n_a != n_b || n_b <= 64)) return cudaErrorInvalidValue;
+    if (lower && n_a != n_b) return cudaErrorInvalidValue;
     auto aligned = [](const float* S, int64_t ld, int64_t z) { return !(((uintptr_t)S | (size_t)(ld * 4) | (size_t)(z * 4)) & 15); };
     p.red = beta == 1.f && aligned(C, ldc, c_z) && (!second || aligned(second->C, second->ldc, second->c_z));
-    if (n_b <= 64) return launch_bn<64>(p, s, nz, a_z_bytes, b_z_bytes, second);
+    if (n_b <= 64 && !lower) return launch_bn<64>(p, s, nz, a_z_bytes, b_z_bytes, second);
     return launch_bn<128>(p, s, nz, a_z_bytes, b_z_bytes, second);
 }
 

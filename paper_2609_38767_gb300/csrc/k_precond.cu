@@ -22,7 +22,7 @@
 //           block step is a small matrix product instead of a serial chain.
 // Every launch covers all layers of the call (grid z or y = layer).
 //
-// Blocked path (fp32 state, D a multiple of 128 and at least 256): the same
+// Blocked path (fp32 state, D a multiple of 64 and at least 256): the same
 // right-looking Cholesky in 256-column panels. Per panel: the 256 x 256 diagonal
 // block is factored in shared memory by one CTA (diag_panel_kernel), the rows
 // below it are solved against it (solve_kernel, x L_BB^T = a), and the trailing
@@ -1291,15 +1291,16 @@ cudaError_t apply_impl(int n_layers, int64_t D, const void* state, const float* 
 
 // ---------------------------------------------------------------- blocked path (fp32)
 constexpr int kBB = 128;                // panel width
-// FACTOR and FACTOR_APPLY of layers of whole 128-column blocks, against the one-launch cluster kernel,
+// FACTOR and FACTOR_APPLY of layers of whole 64-column blocks, against the one-launch cluster kernel,
 // seven layers and 64 queries: D = 256 129 us here and 190 us there (one layer: 125 and 170 us),
 // D = 512 316 and 448 us, D = 1024 690 and 1110 us. At D = 128 the difference is the
 // launches' (77 and 110 us) and the cluster kernel's smaller inverses are as accurate, so it stays.
 constexpr int64_t kBlockedMinD = 256;
-// APPLY by itself: below, states may come from the cluster kernel, which leaves no L^T
-constexpr int64_t kBlockedApplyD = 2048;
+// APPLY by itself: states of other sizes may come from the cluster kernel, which leaves no L^T (earlier
+// versions factored them so)
+bool blocked_states(int64_t D) { return D >= 2048 && D % kBB == 0; }
 
-// ---- diagonal panels. A panel is 256 columns (128 at the end of an odd D / 128): the rows and
+// ---- diagonal panels. A panel is 256 columns (64, 128 or 192 at the end of other D): the rows and
 // columns [lo, lo + 256) of a layer, factored by one CTA with everything in shared memory, since
 // the pivots are a serial chain and the next panel waits for them. Per 128-column half:
 //   factor128   16 columns at a time: four warps, a thread per row with the 16 values in registers,
@@ -1545,7 +1546,8 @@ __global__ void __launch_bounds__(kDiagThreads) diag_panel_kernel(St<float> st, 
     float* M = st.M(l);
     double* h = st.header(l);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const bool two = lo + kBB < D;
+    const int n = D - lo < 2 * kBB ? (int)(D - lo) : 2 * kBB;  // the panel's rows, a multiple of 64
+    const bool two = n > kBB;
     if (tid == 0) h[kPcW64] = 64.0;  // solve_kernel: the 64 x 64 inverses are there
     // a warp per row, 16 bytes a lane, nothing above the diagonal (one SM draws 17 bytes a clock)
 #pragma unroll 4
@@ -1553,14 +1555,20 @@ __global__ void __launch_bounds__(kDiagThreads) diag_panel_kernel(St<float> st, 
         const int c = 4 * lane;
         auto diagonal = [&](int half) {
             float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (c <= r) v = *reinterpret_cast<const float4*>(M + (lo + half * kBB + r) * D + lo + half * kBB + c);
-            *reinterpret_cast<float4*>(&sm.S[half][r][c]) =
-                make_float4(v.x, c + 1 <= r ? v.y : 0.f, c + 2 <= r ? v.z : 0.f, c + 3 <= r ? v.w : 0.f);
+            const int row = half * kBB + r;
+            if (c <= r && row < n) v = *reinterpret_cast<const float4*>(M + (lo + row) * D + lo + half * kBB + c);
+            v = make_float4(v.x, c + 1 <= r ? v.y : 0.f, c + 2 <= r ? v.z : 0.f, c + 3 <= r ? v.w : 0.f);
+            if (row >= n) {  // past the last block: identity
+                v.x = c == r ? 1.f : 0.f, v.y = c + 1 == r ? 1.f : 0.f;
+                v.z = c + 2 == r ? 1.f : 0.f, v.w = c + 3 == r ? 1.f : 0.f;
+            }
+            *reinterpret_cast<float4*>(&sm.S[half][r][c]) = v;
         };
         diagonal(0);
         if (two) {
             *reinterpret_cast<float4*>(&sm.S21[r][c]) =
-                *reinterpret_cast<const float4*>(M + (lo + kBB + r) * D + lo + c);
+                kBB + r < n ? *reinterpret_cast<const float4*>(M + (lo + kBB + r) * D + lo + c)
+                            : make_float4(0.f, 0.f, 0.f, 0.f);
             diagonal(1);
         }
     }
@@ -1612,13 +1620,14 @@ __global__ void __launch_bounds__(kDiagThreads) diag_panel_kernel(St<float> st, 
         for (int half = 0; half < (two ? 2 : 1); ++half) {
             const float* src = &sm.S[half][r][c];
             float* dst = M + (lo + half * kBB + r) * D + lo + half * kBB + c;
-            if (c / 64 <= r / 64) *reinterpret_cast<float4*>(dst) = *reinterpret_cast<const float4*>(src);
+            if (c / 64 <= r / 64 && half * kBB + r < n)
+                *reinterpret_cast<float4*>(dst) = *reinterpret_cast<const float4*>(src);
         }
-        if (two)
+        if (kBB + r < n)
             *reinterpret_cast<float4*>(M + (lo + kBB + r) * D + lo + c) = *reinterpret_cast<const float4*>(&sm.S21[r][c]);
     }
     float* Dg = st.Dinv(l) + (lo / kNB) * (kNB * kNB);
-    for (int e = tid; e < (two ? 8 : 4) * kNB * kNB; e += kDiagThreads) {
+    for (int e = tid; e < n / kNB * kNB * kNB; e += kDiagThreads) {
         const int b = e >> 10, r = (e >> 5) & 31, c = e & 31, half = b >> 2, o = (b & 3) * kNB;
         const float(*S)[kLdS] = sm.S[half];
         Dg[e] = c < r ? S[o + c][o + r] : (c == r ? sm.inv[half][o + r] : 0.f);
@@ -1626,7 +1635,7 @@ __global__ void __launch_bounds__(kDiagThreads) diag_panel_kernel(St<float> st, 
 }
 
 // Row vectors solved against the panel's diagonal block B = [lo, lo + nb) of layer l (grid y),
-// nb = 256 or 128: FWD x <- L_BB^{-1} x, else x <- L_BB^{-T} x, for rows of nb values at column lo of
+// nb = 64 to 256: FWD x <- L_BB^{-1} x, else x <- L_BB^{-T} x, for rows of nb values at column lo of
 // two sets of rows (the first blocks_a CTAs of a layer have rows_a). Used for the rows of M below a
 // panel (FWD) and for the query rows of APPLY (both directions).
 // R rows a CTA, their nb values in shared memory; 64 columns at a time: the solved columns' share
@@ -1907,7 +1916,7 @@ __global__ void nan_failed_kernel(St<float> st, float* qhat, int64_t ld, int64_t
 }
 
 bool blocked_pc(int64_t D, tda_dtype sdt) {
-    return sdt == TDA_F32 && D % kBB == 0 && D >= kBlockedMinD && D < (1LL << 31) / kBB && gemm_tc_available();
+    return sdt == TDA_F32 && D % 64 == 0 && D >= kBlockedMinD && D < (1LL << 31) / kBB && gemm_tc_available();
 }
 
 template <int R, bool FWD>
@@ -2081,7 +2090,7 @@ cudaError_t launch_pc_factor_apply(int n_layers, int64_t D, tda_dtype sdt, void*
     // fp32 state, whole 32-column blocks, up to 256 queries: factorisation and both
     // substitutions in one cluster launch per call;
     // otherwise FACTOR, then APPLY
-    if (sdt == TDA_F32 && !(D >= kBlockedApplyD && blocked_pc(D, sdt)) && D % kNB == 0 && D >= 2 * kNB && n_q >= 1 &&
+    if (sdt == TDA_F32 && !(blocked_states(D) && blocked_pc(D, sdt)) && D % kNB == 0 && D >= 2 * kNB && n_q >= 1 &&
         n_q <= 256) {
         const QArgs qa{q, (float*)qhat, n_q, ld_q, ld_qhat};
         e = factor_cluster<16, true>(n_layers, D, state, n_total, lambda_abs, lambda_rel, qa, s);
@@ -2098,7 +2107,7 @@ cudaError_t launch_pc_apply(int n_layers, int64_t D, tda_dtype sdt, const void* 
                             int64_t n_q, int64_t ld_q, void* qhat, int64_t ld_qhat, cudaStream_t s) {
     if (n_q == 0) return cudaSuccess;
     // a blocked factorisation left L^T in M's upper triangle: tensor-core substitutions
-    if (D >= kBlockedApplyD && apply_blocked_ok(D, sdt, qhat, ld_qhat, n_q)) {
+    if (blocked_states(D) && apply_blocked_ok(D, sdt, qhat, ld_qhat, n_q)) {
         const cudaError_t e = copy_queries(n_layers, D, q, n_q, ld_q, (float*)qhat, ld_qhat, s);
         return e != cudaSuccess ? e : apply_blocked(n_layers, D, state, n_q, (float*)qhat, ld_qhat, true, s);
     }

@@ -157,7 +157,8 @@ def test_blocked_failed_pivot(dev, bad):
 
 # as test_blocked_panels (condition number, rows a feature); D below 2048: FACTOR_APPLY runs the panels, APPLY by
 # itself the row-by-row substitution on the state that they leave
-@pytest.mark.parametrize("D,nl,nq,ld", [(256, 3, 5, 0), (384, 1, 33, 4), (1024, 2, 1, 0), (1152, 1, 130, 4), (1536, 3, 300, 0), (2176, 1, 40, 8)])
+@pytest.mark.parametrize("D,nl,nq,ld", [(256, 3, 5, 0), (320, 2, 40, 0), (384, 1, 33, 4), (448, 1, 9, 0), (576, 3, 65, 4),
+                                         (1600, 1, 70, 0), (2112, 1, 20, 0), (1024, 2, 1, 0), (1152, 1, 130, 4), (1536, 3, 300, 0), (2176, 1, 40, 8)])
 def test_blocked_factor_apply(dev, D, nl, nq, ld):
     rng = np.random.default_rng(D + 1)
     n, w = 4 * D, nl * D
