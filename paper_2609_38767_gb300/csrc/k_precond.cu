@@ -363,11 +363,11 @@ __global__ void __launch_bounds__(256) update_kernel(St<TS> st, int64_t k0) {
 // Panel step at k0, grid (row chunk, layer), 128 threads: a CTA eliminates the diagonal block
 // together with its 8 panel rows, A_ic -= (A_ij w_j) A_cj with w_j = 1 / A_jj, and scales column j
 // by 1/sqrt(A_jj) at the end, all columns at once. The serial chain is one pivot after the other,
-// so warp 0 does nothing else: it brings A_jj of the next column up to date and inverts it (an fp32
+// so warp 0 does nothing else: it brings A_jj of the next column up to date and inverts it (a 20-bit
 // guess and one cubic step) while warps 1-3 update the rest with the current column; one barrier a
 // column. Chunk 0 leaves L_kk in the block's slot of Dinv; f64_inverse_kernel replaces it by its
 // inverse after the last step. D = 256: 150 us a step in panel_kernel (one CTA: two warps of
-// serial chains), 29 us with every warp inverting every pivot before its updates.
+// serial chains), 35 us with every warp inverting every pivot before its updates, 27 us here.
 constexpr int kF64Rows = 8;
 
 // 1/p and 1/sqrt(p) for p > 0 to fp64 rounding: p = m 4^h with m in [1, 4); the fp32 guess for m
@@ -388,6 +388,15 @@ __device__ __forceinline__ double rcp_f64(double p) {
     const bool wide = h > 510 || h < -510;
     const double x = fma(r, fma(e, e, e), r) * pow2(wide ? -h : -2 * h);
     return wide ? x * pow2(-h) : x;
+}
+// 1/p on the pivots' serial chain: the hardware's 20-bit guess of a double's reciprocal needs no
+// conversions and no scaling inside 2^-1000 .. 2^1000, and the same iteration takes it past 2^-59.
+__device__ __forceinline__ double rcp_chain(double p) {
+    if (!(p > 9.4e-302 && p < 1.07e301)) return rcp_f64(p);
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(p));
+    const double e = fma(-p, r, 1.0);
+    return fma(r, fma(e, e, e), r);
 }
 __device__ __forceinline__ double rsqrt_f64(double p) {
     int h;
@@ -421,7 +430,7 @@ __global__ void __launch_bounds__(128) panel_f64_kernel(St<double> st, int64_t k
     if (warp == 0) {
         const double p = A[0][0];
         if (!(p > 0.0)) bad = 0;
-        const double w = p > 0.0 ? rcp_f64(p) : NAN;
+        const double w = p > 0.0 ? rcp_chain(p) : NAN;
         if (lane == 0) wj[0] = w;
     }
     __syncthreads();
@@ -430,7 +439,7 @@ __global__ void __launch_bounds__(128) panel_f64_kernel(St<double> st, int64_t k
         if (warp == 0) {
             const double a = A[j + 1][j], p = A[j + 1][j + 1] - a * w * a;
             if (!(p > 0.0) && bad < 0) bad = j + 1;
-            const double wn = p > 0.0 ? rcp_f64(p) : NAN;
+            const double wn = p > 0.0 ? rcp_chain(p) : NAN;
             if (lane == 0) {
                 A[j + 1][j + 1] = p;
                 wj[(j + 1) & 1] = wn;
