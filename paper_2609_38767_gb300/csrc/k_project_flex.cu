@@ -405,7 +405,17 @@ project_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 #pragma unroll
                 for (int j = 0; j < C::CB; ++j) acc[i][j] = 0.f;
         };
-        auto contract = [&](int t0, int t1) {  // staged rows [t0, t1)
+        auto contract = [&](int t0, int t1) {  // acc += rows t0 .. t1 - 1 of the staged At, Bt
+            // into sums of their own where there are registers: a chain of at most kSR rows, not of the
+            // CTA's share of the example, rounds less (560 tokens: 3.1e-7 off in one chain)
+            constexpr bool kOwn = !F32 || K < 64;
+            float sum[C::RB][C::CB];
+            auto& to = *(kOwn ? &sum : &acc);
+            if constexpr (kOwn)
+#pragma unroll
+                for (int i = 0; i < C::RB; ++i)
+#pragma unroll
+                    for (int j = 0; j < C::CB; ++j) sum[i][j] = 0.f;
 #pragma unroll 2
             for (int t = t0; t < t1; ++t) {
                 float y[C::RB], x[C::CB];
@@ -416,8 +426,13 @@ project_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 #pragma unroll
                 for (int i = 0; i < C::RB; ++i)
 #pragma unroll
-                    for (int j = 0; j < C::CB; ++j) acc[i][j] = fmaf(y[i], x[j], acc[i][j]);
+                    for (int j = 0; j < C::CB; ++j) to[i][j] = fmaf(y[i], x[j], to[i][j]);
             }
+            if constexpr (kOwn)
+#pragma unroll
+                for (int i = 0; i < C::RB; ++i)
+#pragma unroll
+                    for (int j = 0; j < C::CB; ++j) acc[i][j] += sum[i][j];
         };
         auto write = [&](int64_t n) {
             float* out = p.phi + n * p.ld_phi;
