@@ -1924,8 +1924,10 @@ __global__ void nan_failed_kernel(St<float> st, float* qhat, int64_t ld, int64_t
         qhat[(e / D) * ld + (int64_t)l * D + e % D] = NAN;
 }
 
-bool blocked_pc(int64_t D, tda_dtype sdt) {
-    return sdt == TDA_F32 && D % 64 == 0 && D >= kBlockedMinD && D < (1LL << 31) / kBB && gemm_tc_available();
+// (layers are a grid's y coordinate)
+bool blocked_pc(int n_layers, int64_t D, tda_dtype sdt) {
+    return sdt == TDA_F32 && n_layers <= 65535 && D % 64 == 0 && D >= kBlockedMinD && D < (1LL << 31) / kBB &&
+           gemm_tc_available();
 }
 
 template <int R, bool FWD>
@@ -2003,8 +2005,11 @@ cudaError_t factor_blocked(int n_layers, int64_t D, void* state, int64_t n_total
 }
 
 // (D >= kBlockedMinD suffices where the state is factored in the same call)
-bool apply_blocked_ok(int64_t D, tda_dtype sdt, const void* qhat, int64_t ld_qhat, int64_t n_q) {
-    return blocked_pc(D, sdt) && ((uintptr_t)qhat & 15) == 0 && (ld_qhat & 3) == 0 && n_q < (1LL << 24);
+bool apply_blocked_ok(int n_layers, int64_t D, tda_dtype sdt, int64_t ld_q, const void* qhat, int64_t ld_qhat,
+                      int64_t n_q) {
+    // 2-D copies: row strides below 2^31 bytes
+    return blocked_pc(n_layers, D, sdt) && ((uintptr_t)qhat & 15) == 0 && (ld_qhat & 3) == 0 && n_q < (1LL << 24) &&
+           ld_q < (1LL << 29) && ld_qhat < (1LL << 29);
 }
 
 cudaError_t copy_queries(int n_layers, int64_t D, const float* q, int64_t n_q, int64_t ld_q, float* qhat,
@@ -2080,7 +2085,7 @@ cudaError_t launch_pc_fit(int n_layers, int64_t D, tda_dtype sdt, void* state, c
 
 cudaError_t launch_pc_factor(int n_layers, int64_t D, tda_dtype sdt, void* state, int64_t n_total,
                              double lambda_abs, double lambda_rel, cudaStream_t s) {
-    if (blocked_pc(D, sdt))
+    if (blocked_pc(n_layers, D, sdt))
         return factor_blocked(n_layers, D, state, n_total, lambda_abs, lambda_rel, nullptr, 0, 0, s);
     if (sdt == TDA_F64) return factor_impl<double>(n_layers, D, state, n_total, lambda_abs, lambda_rel, s);
     return factor_impl<float>(n_layers, D, state, n_total, lambda_abs, lambda_rel, s);
@@ -2090,7 +2095,7 @@ cudaError_t launch_pc_factor_apply(int n_layers, int64_t D, tda_dtype sdt, void*
                                    double lambda_abs, double lambda_rel, const float* q, int64_t n_q, int64_t ld_q,
                                    void* qhat, int64_t ld_qhat, cudaStream_t s) {
     cudaError_t e;
-    if (n_q >= 1 && apply_blocked_ok(D, sdt, qhat, ld_qhat, n_q)) {
+    if (n_q >= 1 && apply_blocked_ok(n_layers, D, sdt, ld_q, qhat, ld_qhat, n_q)) {
         if ((e = copy_queries(n_layers, D, q, n_q, ld_q, (float*)qhat, ld_qhat, s)) != cudaSuccess) return e;
         e = factor_blocked(n_layers, D, state, n_total, lambda_abs, lambda_rel, (float*)qhat, n_q, ld_qhat, s);
         if (e != cudaSuccess) return e;
@@ -2099,8 +2104,8 @@ cudaError_t launch_pc_factor_apply(int n_layers, int64_t D, tda_dtype sdt, void*
     // fp32 state, whole 32-column blocks, up to 256 queries: factorisation and both
     // substitutions in one cluster launch per call;
     // otherwise FACTOR, then APPLY
-    if (sdt == TDA_F32 && !(blocked_states(D) && blocked_pc(D, sdt)) && D % kNB == 0 && D >= 2 * kNB && n_q >= 1 &&
-        n_q <= 256) {
+    if (sdt == TDA_F32 && !(blocked_states(D) && blocked_pc(n_layers, D, sdt)) && D % kNB == 0 && D >= 2 * kNB &&
+        n_q >= 1 && n_q <= 256) {
         const QArgs qa{q, (float*)qhat, n_q, ld_q, ld_qhat};
         e = factor_cluster<16, true>(n_layers, D, state, n_total, lambda_abs, lambda_rel, qa, s);
         if (e == cudaErrorNotSupported)
@@ -2116,7 +2121,7 @@ cudaError_t launch_pc_apply(int n_layers, int64_t D, tda_dtype sdt, const void* 
                             int64_t n_q, int64_t ld_q, void* qhat, int64_t ld_qhat, cudaStream_t s) {
     if (n_q == 0) return cudaSuccess;
     // a blocked factorisation left L^T in M's upper triangle: tensor-core substitutions
-    if (blocked_states(D) && apply_blocked_ok(D, sdt, qhat, ld_qhat, n_q)) {
+    if (blocked_states(D) && apply_blocked_ok(n_layers, D, sdt, ld_q, qhat, ld_qhat, n_q)) {
         const cudaError_t e = copy_queries(n_layers, D, q, n_q, ld_q, (float*)qhat, ld_qhat, s);
         return e != cudaSuccess ? e : apply_blocked(n_layers, D, state, n_q, (float*)qhat, ld_qhat, true, s);
     }

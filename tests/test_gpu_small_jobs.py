@@ -208,3 +208,23 @@ def test_blocked_state_without_64_column_inverses(dev):
     tda.tda_precondition(tda.TDA_PC_APPLY, *args, q=q, n_q=nq, ld_q=D, qhat=old, ld_qhat=D)
     tda.tda_device_status()
     assert float((new - old).norm() / new.norm()) <= 2e-5
+
+
+def test_factor_apply_row_strides_past_the_copies(dev):
+    # one row whose stride no 2-D copy takes: solved by the cluster kernel, as every row of this width once was
+    D = 256
+    rng = np.random.default_rng(4)
+    ph = torch.from_numpy(rng.standard_normal((4 * D, D)).astype(np.float32)).to(dev)
+    q = torch.from_numpy(rng.standard_normal((1, D)).astype(np.float32)).to(dev)
+    outs = []
+    for ld in (D, 1 << 29):
+        state = torch.empty(tda.tda_precondition_state_bytes(D, tda.TDA_F32), dtype=torch.uint8, device=dev)
+        args = (1, D, tda.TDA_F32, state)
+        out = torch.empty((1, D), device=dev)
+        tda.tda_precondition(tda.TDA_PC_RESET, *args)
+        tda.tda_precondition(tda.TDA_PC_FIT_ACCUM, *args, phi=ph, n=4 * D, ld_phi=D)
+        tda.tda_precondition(tda.TDA_PC_FACTOR_APPLY, *args, n_total=4 * D, lambda_rel_mean_eig=0.1, q=q, n_q=1, ld_q=ld,
+                             qhat=out, ld_qhat=ld)
+        outs.append(out)
+    tda.tda_device_status()
+    assert float((outs[0] - outs[1]).norm() / outs[0].norm()) <= 4e-5
