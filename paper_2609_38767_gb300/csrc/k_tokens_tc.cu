@@ -81,10 +81,13 @@ __device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t adesc, uint64
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-// x to TF32's 10 mantissa bits, nearest (a value that would round past the largest is truncated).
+// x to TF32's 10 mantissa bits, nearest. From the value that would round past the largest on, the bits
+// below are cut off; a NaN keeps its quiet bit (0x7FFFFFFF, the NaN of CUDA arithmetic and of the tensor pipe,
+// would carry into the sign and become zero). An infinity's lo is a NaN, so its products are NaN.
 __device__ __forceinline__ float round_tf32(float x) {
-    const uint32_t u = __float_as_uint(x), r = u + 0x1000u;
-    return __uint_as_float(((r & 0x7F800000u) == 0x7F800000u ? u : r) & 0xFFFFE000u);
+    const uint32_t u = __float_as_uint(x), mag = u & 0x7FFFFFFFu;
+    const uint32_t r = mag >= 0x7F7FF000u ? u : u + 0x1000u;
+    return __uint_as_float((r & 0xFFFFE000u) | (mag > 0x7F800000u ? 0x00400000u : 0u));
 }
 __device__ __forceinline__ void split_tf32(float x, float& hi, float& lo) {
     hi = round_tf32(x);
