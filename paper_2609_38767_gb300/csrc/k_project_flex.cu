@@ -2,15 +2,21 @@
 // tiles and clusters cut to the batch, for any k_in, k_out up to 64: fp32 factors of
 // any batch, and bf16 factors where whole examples per SM would leave SMs idle.
 //
-// fp32 factors, exact to fp32 rounding: every value is cut into three bf16 pieces,
-// x = h + m + l (8 significant bits each, by truncation: h + m + l = x exactly), and
-// the signs S are +-1, so the products h S, m S, l S are exact and only sums round.
-// At = A S_in keeps two fp32 accumulators, sum h S and sum (m + l) S: within one,
-// the terms are so coarse against its ulp that the tensor pipe's truncating
-// additions lose almost nothing (2048 features: 1.2e-6 off with an fp32 chain on the
-// CUDA cores, 2e-7 here). The epilogue adds the two with round-to-nearest and
-// contracts Phi += Bt^T At over the tokens in fp32, as the other kernels do. bf16
-// factors are the MMA's A operand as TMA wrote them, one accumulator a side.
+// fp32 factors: every value is cut into three bf16 pieces, x = h + m + l (8 significant bits each, by
+// truncation: h + m + l = x exactly), and the signs S are +-1, so the products h S, m S, l S are exact and
+// only sums round: sum h S in one fp32 accumulator, sum (m + l) S in another. bf16 factors are the MMA's A
+// operand as TMA wrote them, one accumulator.
+//
+// Accuracy: the tensor pipe adds 16 features at a time into its accumulators with truncation. Among values
+// of similar size it loses almost nothing (the terms are coarse against the sum's ulp), but every loss
+// points to zero, so that wide layers with a few large features drift (cubed normals, 49152 features: 5.3e-5
+// off in one sum; rounded fp32 chain 4.0e-6, bf16 1.9e-6). So an accumulator takes four chunks (256
+// features; bf16, whose rounded chain is almost exact, two), and the epilogue adds it to the token's row of
+// At or Bt with round-to-nearest (3.8e-7; bf16 3.9e-7). The accumulators form groups in two TMEM buffers:
+// one group is added beside the next one's MMAs, and bf16 has four accumulators a group, so that barriers and
+// commits are as rare as with fp32. At the end of a tile the epilogue contracts the rows, Phi += Bt^T At, in
+// fp32, as the other kernels do. One sum a side and one accumulator a group against this: fp32 2048 -> 2048,
+// k = 64, 64 x 512 tokens 133.8 and 129.7 us; bf16 4096 -> 4096, k = 64 x 48, 64 x 300 tokens 94.9 and 96.9 us.
 //
 // The pieces go to TMEM, not to shared memory: the MMA takes its A operand from
 // TMEM (a lane per token, two bf16 features per column), the split warps read
@@ -53,7 +59,7 @@ constexpr int kChunkK = 64;   // features per stage: one bf16 box or two 32-feat
 constexpr uint32_t kBoxBytes = kTileM * 128;  // room of one box (a 128-byte row per token)
 constexpr size_t kSmemMax = 232448;
 constexpr int kMaxStages = 8;
-constexpr int kSR = 64;       // token rows staged at a time
+constexpr int kSR = 64;       // token rows added in one chain
 constexpr int kPieceCols = kChunkK / 2;       // TMEM columns of one piece of a chunk
 constexpr int kACols = 3 * kPieceCols;
 constexpr int kABufs = 2;
@@ -66,12 +72,12 @@ struct Cfg {
     static constexpr uint32_t kTileBytes = (F32 ? 2 : 1) * kBoxBytes;
     static constexpr uint32_t kSignBytes = K * 128;
     static constexpr uint32_t kStageBytes = kTileBytes + kSignBytes;
-    static constexpr int kSideCols = (F32 ? 2 : 1) * K;    // one side's accumulators (fp32: h, m+l)
-    static constexpr int kBufCols = 2 * kSideCols;         // At, Bt
-    static constexpr int kBufs = F32 && K > 32 ? 1 : 2;
-    static constexpr int kAOff = kBufs * kBufCols;         // first column of the A pieces (fp32)
+    static constexpr int kGroup = F32 ? 4 : 8;             // chunks accumulated in TMEM before they are drained
+    static constexpr int kAccs = F32 ? 2 : 4;              // their accumulators: h and m + l, or two chunks each
+    static constexpr int kBufCols = kAccs * K;
+    static constexpr int kAOff = 2 * kBufCols;             // first column of the A pieces (fp32)
     static constexpr int kStageLd = K + 4;
-    static constexpr size_t kStaging = 2ull * kSR * kStageLd * 4;
+    static constexpr size_t kStaging = 2ull * kTileM * kStageLd * 4;
     static constexpr size_t kTail = kLutBytes + 8 * (4 * kMaxStages + 2 * kABufs + 4 + 3) + 16;
     static constexpr int kFit = (int)((kSmemMax - 1024 - kStaging - kTail) / kStageBytes);
     static constexpr int kStages = kFit > kMaxStages ? kMaxStages : kFit;
@@ -113,15 +119,27 @@ __device__ __forceinline__ void mma_bf16_ta(uint32_t d_tmem, uint32_t a_tmem, ui
         "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(
-            taddr),
-        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
-        "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
-        : "memory");
+
+// 32 lanes x N consecutive fp32 columns of TMEM into registers, one wait.
+template <int N>
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&v)[N]) {
+    static_assert(N == 16 || N == 32 || N == 64, "columns");
+    uint32_t r[N];
+#pragma unroll
+    for (int c = 0; c < N; c += 16)
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+            : "=r"(r[c]), "=r"(r[c + 1]), "=r"(r[c + 2]), "=r"(r[c + 3]), "=r"(r[c + 4]), "=r"(r[c + 5]), "=r"(r[c + 6]),
+              "=r"(r[c + 7]), "=r"(r[c + 8]), "=r"(r[c + 9]), "=r"(r[c + 10]), "=r"(r[c + 11]), "=r"(r[c + 12]),
+              "=r"(r[c + 13]), "=r"(r[c + 14]), "=r"(r[c + 15])
+            : "r"(taddr + c));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int c = 0; c < N; ++c) {
+        asm volatile("" : "+r"(r[c]));  // not read before the wait
+        v[c] = __uint_as_float(r[c]);
+    }
 }
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // The upper halves of two fp32 bit patterns: the truncated bf16 pair (lo in the low half).
 __device__ __forceinline__ uint32_t pack_hi(uint32_t lo, uint32_t hi) { return __byte_perm(lo, hi, 0x7632); }
@@ -156,8 +174,8 @@ project_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     using C = Cfg<K, F32>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    float* stX = (float*)(smem + (size_t)C::kStages * C::kStageBytes);  // [kSR][K+4] At rows
-    float* stY = stX + kSR * C::kStageLd;                               // [kSR][K+4] Bt rows
+    float* stX = (float*)(smem + (size_t)C::kStages * C::kStageBytes);  // [kTileM][K+4] At rows
+    float* stY = stX + kTileM * C::kStageLd;                            // [kTileM][K+4] Bt rows
     uint8_t* lut = smem + (size_t)C::kStages * C::kStageBytes + C::kStaging;
     uint64_t* bars = (uint64_t*)(lut + kLutBytes);
     uint64_t* full = bars;                     // [stages] boxes landed (count 1 + tx)
@@ -166,8 +184,8 @@ project_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     uint64_t* sempty = bars + 3 * kMaxStages;  // [stages] MMAs done with the signs, bf16: and the boxes (1)
     uint64_t* afull = bars + 4 * kMaxStages;   // [2] pieces in TMEM (8)
     uint64_t* aempty = afull + kABufs;         // [2] MMAs done with the pieces (1)
-    uint64_t* tfull = aempty + kABufs;         // [2] accumulators ready (1)
-    uint64_t* tempty = tfull + 2;              // [2] accumulators drained (4)
+    uint64_t* tfull = aempty + kABufs;         // [2] a group is accumulated (1)
+    uint64_t* tempty = tfull + 2;              // [2] the accumulators are drained (4)
     uint64_t* mma_done = tempty + 2;
     uint64_t* red_go = mma_done + 1;           // the other members' staging rows are free (cs - 1)
     uint64_t* red_full = red_go + 1;           // the other members' slices have landed here (cs - 1)
@@ -252,49 +270,56 @@ project_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             }
     } else if (warp == 1) {
         // ---------------- MMA issuer: the warp waits, one lane issues
-        uint32_t s = 0, ph = 0, cnt = 0, tile = 0;
+        uint32_t s = 0, ph = 0, cnt = 0, grp = 0;
         bool ok = true;
         constexpr uint32_t idesc = idesc_bf16(kTileM, K);
-        for (; ok && it.x < p.n_slots; it.next(p, ncl, crank), ++tile) {
-            const uint32_t b = tile % C::kBufs, use = tile / C::kBufs;
-            if (!warp_wait(smem_u32(&tempty[b]), (use & 1u) ^ 1u, abort, p.err)) break;
-            for (int kc = 0; kc < nk_tot; ++kc, ++cnt) {
-                const uint32_t a = cnt & 1u;
-                if (!warp_wait(smem_u32(&sready[s]), ph, abort, p.err) ||
-                    !(F32 ? warp_wait(smem_u32(&afull[a]), (cnt >> 1) & 1u, abort, p.err)
-                          : warp_wait(smem_u32(&full[s]), ph, abort, p.err))) {
+        for (; ok && it.x < p.n_slots; it.next(p, ncl, crank))
+            for (int k0 = 0; ok && k0 < nk_tot; ++grp) {  // groups end with a side
+                const uint32_t b = grp & 1u;
+                const int side_end = k0 < p.nk_in ? p.nk_in : nk_tot;
+                const int n = side_end - k0 < C::kGroup ? side_end - k0 : C::kGroup;
+                if (!warp_wait(smem_u32(&tempty[b]), ((grp >> 1) & 1u) ^ 1u, abort, p.err)) {
                     ok = false;
                     break;
                 }
-                tc_fence_after();
-                const bool side_b = kc >= p.nk_in;
-                const bool start = kc == 0 || kc == p.nk_in;
-                const uint32_t st = smem_u32(smem + (size_t)s * C::kStageBytes);
-                const uint64_t bd = sw128_desc(st + C::kTileBytes);
-                const uint32_t dh = tmem + b * C::kBufCols + (side_b ? C::kSideCols : 0), dl = dh + K;
-                if (elect_one()) {
-#pragma unroll
-                    for (int k = 0; k < kChunkK / 16; ++k) {  // K = 16: 32 bytes of bf16, 8 columns of pieces
-                        const uint32_t acc = start && k == 0 ? 0u : 1u;
-                        if constexpr (F32) {
-                            const uint32_t at = tmem + C::kAOff + a * kACols;
-                            mma_bf16_ta(dh, at + 8 * k, bd + 2 * k, idesc, acc);
-                            mma_bf16_ta(dl, at + kPieceCols + 8 * k, bd + 2 * k, idesc, acc);
-                            mma_bf16_ta(dl, at + 2 * kPieceCols + 8 * k, bd + 2 * k, idesc, 1u);
-                        } else {
-                            mma_bf16(dh, sw128_desc(st) + 2 * k, bd + 2 * k, idesc, acc);
-                        }
+                for (int c = 0; c < n; ++c, ++cnt) {
+                    const uint32_t a = cnt & 1u;
+                    if (!warp_wait(smem_u32(&sready[s]), ph, abort, p.err) ||
+                        !(F32 ? warp_wait(smem_u32(&afull[a]), (cnt >> 1) & 1u, abort, p.err)
+                              : warp_wait(smem_u32(&full[s]), ph, abort, p.err))) {
+                        ok = false;
+                        break;
                     }
-                    if constexpr (F32) mma_commit(smem_u32(&aempty[a]));
-                    mma_commit(smem_u32(&sempty[s]));
+                    tc_fence_after();
+                    const uint32_t st = smem_u32(smem + (size_t)s * C::kStageBytes);
+                    const uint64_t bd = sw128_desc(st + C::kTileBytes);
+                    // bf16: two chunks an accumulator
+                    const uint32_t dh = tmem + b * C::kBufCols + (F32 ? 0 : c / 2 * K), dl = dh + K;
+                    const bool clear = F32 ? c == 0 : c % 2 == 0;
+                    if (elect_one()) {
+#pragma unroll
+                        for (int k = 0; k < kChunkK / 16; ++k) {  // K = 16: 32 bytes of bf16, 8 columns of pieces
+                            const uint32_t acc = clear && k == 0 ? 0u : 1u;
+                            if constexpr (F32) {
+                                const uint32_t at = tmem + C::kAOff + a * kACols;
+                                mma_bf16_ta(dh, at + 8 * k, bd + 2 * k, idesc, acc);
+                                mma_bf16_ta(dl, at + kPieceCols + 8 * k, bd + 2 * k, idesc, acc);
+                                mma_bf16_ta(dl, at + 2 * kPieceCols + 8 * k, bd + 2 * k, idesc, 1u);
+                            } else {
+                                mma_bf16(dh, sw128_desc(st) + 2 * k, bd + 2 * k, idesc, acc);
+                            }
+                        }
+                        if constexpr (F32) mma_commit(smem_u32(&aempty[a]));
+                        mma_commit(smem_u32(&sempty[s]));
+                    }
+                    __syncwarp();
+                    if (++s == (uint32_t)C::kStages) s = 0, ph ^= 1u;
                 }
+                if (!ok) break;
+                if (elect_one()) mma_commit(smem_u32(&tfull[b]));
                 __syncwarp();
-                if (++s == (uint32_t)C::kStages) s = 0, ph ^= 1u;
+                k0 += n;
             }
-            if (!ok) break;
-            if (elect_one()) mma_commit(smem_u32(&tfull[b]));
-            __syncwarp();
-        }
         if (elect_one()) {
             mma_commit(smem_u32(mma_done));
             const uint64_t t0 = global_ns();
@@ -394,9 +419,9 @@ project_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 if (++s == (uint32_t)C::kStages) s = 0, ph ^= 1u;
             }
     } else if (warp >= 4) {
-        // ---------------- epilogue: TMEM -> shared -> Phi += Bt^T At, kSR token rows at a time
+        // ---------------- epilogue: groups of chunks -> sums in shared memory -> Phi += Bt^T At
         const int q4 = warp & 3, et = threadIdx.x - 128, rg = et >> 3, cg = et & 7;
-        uint32_t tile = 0, red_use = 0;
+        uint32_t grp = 0, red_use = 0;
         bool ok = true;
         float acc[C::RB][C::CB];
         auto clear = [&]() {
@@ -405,7 +430,7 @@ project_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
 #pragma unroll
                 for (int j = 0; j < C::CB; ++j) acc[i][j] = 0.f;
         };
-        auto contract = [&](int t0, int t1) {  // acc += rows t0 .. t1 - 1 of the staged At, Bt
+        auto contract = [&](int t0, int t1) {  // acc += rows t0 .. t1 - 1 (at most kSR) of At, Bt
             // into sums of their own where there are registers: a chain of at most kSR rows, not of the
             // CTA's share of the example, rounds less (560 tokens: 3.1e-7 off in one chain)
             constexpr bool kOwn = !F32 || K < 64;
@@ -489,59 +514,67 @@ project_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         clear();
         while (ok && it.x < p.n_slots) {
             const int64_t cur = it.x;
-            const uint32_t b = tile % C::kBufs, use = tile / C::kBufs;
-            bool got = warp_wait(smem_u32(&tfull[b]), use & 1u, abort, p.err);
-            if (epi_any(!got)) break;
-            tc_fence_after();
             const int rows = p.pack > 1 ? p.pack * (int)p.T : p.R;
-            int j = 0;  // packed: example of the tile whose rows come next
-            for (int r0 = 0; r0 < rows; r0 += kSR) {
-                const int srow = q4 * 32 + lane - r0;
-                if (srow >= 0 && srow < kSR) {
-                    const uint32_t tb = tmem + ((uint32_t)(q4 * 32) << 16) + b * C::kBufCols;
+            // every accumulator is added with round-to-nearest to this thread's row of At or Bt, in shared
+            // memory or (bf16, which has the registers) in registers
+            for (int side = 0; ok && side < 2; ++side) {
+                const int nk = side ? p.nk_out : p.nk_in;
+                const bool active = q4 * 32 < rows;
+                float* dst = (side ? stY : stX) + (q4 * 32 + lane) * C::kStageLd;
+                float sum[K];  // bf16
 #pragma unroll
-                    for (int side = 0; side < 2; ++side)
+                for (int i = 0; i < K; ++i) sum[i] = 0.f;
+                for (int k0 = 0; k0 < nk; k0 += C::kGroup, ++grp) {
+                    const uint32_t b = grp & 1u;
+                    ok = warp_wait(smem_u32(&tfull[b]), (grp >> 1) & 1u, abort, p.err);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t tb = tmem + ((uint32_t)(q4 * 32) << 16) + b * C::kBufCols;
+                    if (F32 && active) {
 #pragma unroll
                         for (int c0 = 0; c0 < K; c0 += 16) {
-                            float v[16];
-                            tmem_ld16(tb + side * C::kSideCols + c0, v);
-                            if constexpr (F32) {
-                                float lo[16];
-                                tmem_ld16(tb + side * C::kSideCols + K + c0, lo);
+                            float v[16], lo[16];
+                            tmem_ld16(tb + c0, v);
+                            tmem_ld16(tb + K + c0, lo);
 #pragma unroll
-                                for (int i = 0; i < 16; ++i) v[i] += lo[i];
+                            for (int i = 0; i < 16; i += 4) {
+                                float4* d4 = reinterpret_cast<float4*>(dst + c0 + i);
+                                const float4 o = k0 > 0 ? *d4 : make_float4(0.f, 0.f, 0.f, 0.f);
+                                *d4 = make_float4(o.x + (v[i] + lo[i]), o.y + (v[i + 1] + lo[i + 1]),
+                                                  o.z + (v[i + 2] + lo[i + 2]), o.w + (v[i + 3] + lo[i + 3]));
                             }
-                            float* dst = (side ? stY : stX) + srow * C::kStageLd + c0;
-#pragma unroll
-                            for (int i = 0; i < 16; i += 4)
-                                *reinterpret_cast<float4*>(dst + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
                         }
-                }
-                epi_sync();
-                const int end = rows - r0 < kSR ? rows - r0 : kSR;
-                if (p.pack == 1) {
-                    contract(0, end);
-                } else {
-                    // packed: example j's rows j*T .. may span two staged parts
-                    for (int t = 0; t < end;) {
-                        const int stop = (j + 1) * (int)p.T - r0 < end ? (j + 1) * (int)p.T - r0 : end;
-                        contract(t, stop);
-                        t = stop;
-                        if (stop + r0 == (j + 1) * (int)p.T) {
-                            const int64_t e = cur * p.pack + j;
-                            if (e < p.N) write(e);
-                            clear();
-                            ++j;
+                    } else if (active) {
+                        for (int a = 0; a < C::kAccs && k0 + 2 * a < nk; ++a) {
+                            float v[K];
+                            tmem_ld<K>(tb + a * K, v);
+#pragma unroll
+                            for (int i = 0; i < K; ++i) sum[i] += v[i];
                         }
                     }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&tempty[b]));
                 }
-                epi_sync();
+                if (!F32 && active)
+#pragma unroll
+                    for (int i = 0; i < K; i += 4)
+                        *reinterpret_cast<float4*>(dst + i) = make_float4(sum[i], sum[i + 1], sum[i + 2], sum[i + 3]);
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&tempty[b]));
+            if (epi_any(!ok)) break;  // the rows are whole
+            if (p.pack == 1) {
+                for (int t = 0; t < rows; t += kSR) contract(t, t + kSR < rows ? t + kSR : rows);
+            } else {
+                for (int j = 0; j < p.pack; ++j) {  // example j of the tile: T <= kSR rows
+                    const int64_t e = cur * p.pack + j;
+                    if (e >= p.N) break;
+                    contract(j * (int)p.T, (j + 1) * (int)p.T);
+                    write(e);
+                    clear();
+                }
+            }
+            epi_sync();  // the rows are read
             it.next(p, ncl, crank);
-            ++tile;
             if (p.pack == 1 && it.x != cur) {
                 ok = flush(cur);
                 clear();

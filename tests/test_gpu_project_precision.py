@@ -1,0 +1,45 @@
+"""Accuracy of the tensor-core projection of wide layers whose features differ widely in size (cubed normal values),
+where a long truncating sum of the tensor pipe drifts towards zero.
+
+Tolerance: a sum of at most 256 features takes 16 additions that truncate, each by at most one ulp (2^-23) of the
+running sum; every later addition rounds to nearest, 64 to 128 of them per entry here (a random walk of half ulps:
+at most 5e-7). Both sides of the projection: 2 * 16 * 2^-23 + 2 * 5e-7 = 4.8e-6 of an example's features."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2609_38767_gb300 as tda
+from paper_2609_38767_gb300 import build as tbuild
+
+pytestmark = pytest.mark.gpu
+TOL = 4.8e-6
+
+
+@pytest.fixture(scope="module")
+def dev():
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    tbuild.build()
+    tda.load()
+    return torch.device("cuda:0")
+
+
+def check(dev, orc, dtype, N, T, di, do, ki, ko):
+    rng = np.random.default_rng(di + ko)
+    td, code = (torch.bfloat16, tda.TDA_BF16) if dtype == "bf16" else (torch.float32, tda.TDA_F32)
+    A, B = (torch.from_numpy((rng.standard_normal((N, T, d)) ** 3).astype(np.float32)).to(td) for d in (di, do))
+    L = tda.LayerDesc(di, do, T, ki, ko, seed=7, layer=2)
+    phi = torch.empty((N, ki * ko), device=dev)
+    Ad, Bd = A.to(dev), B.to(dev)
+    assert tda.tda_project_engine(L, code, Ad, Bd) == 1
+    tda.tda_project(L, code, Ad, Bd, N, phi, ki * ko, tda.TDA_ROUTE_FACTORED)
+    tda.tda_device_status()
+    ref = orc.project(A.double().numpy(), B.double().numpy(), ki, ko, 7, 2).reshape(N, -1)
+    got = phi.cpu().numpy().astype(np.float64)
+    assert max(np.linalg.norm(got[n] - ref[n]) / np.linalg.norm(ref[n]) for n in range(N)) <= TOL
+
+
+@pytest.mark.parametrize("dtype,N,T,di,do,ki,ko", [
+    ("f32", 2, 40, 16384, 64, 32, 32), ("f32", 3, 33, 64, 16388, 64, 64), ("f32", 1, 150, 16384, 300, 16, 12),
+    ("bf16", 2, 40, 16384, 64, 32, 48), ("bf16", 1, 130, 72, 16392, 8, 24)])
+def test_wide_layers_of_uneven_features(dev, orc, dtype, N, T, di, do, ki, ko):
+    check(dev, orc, dtype, N, T, di, do, ki, ko)
