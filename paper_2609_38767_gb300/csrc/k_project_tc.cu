@@ -70,6 +70,7 @@ constexpr int kChunkK = 64;            // K elements per stage (128 bytes of bf1
 constexpr uint32_t kTileBytes = kTileM * kChunkK * 2;  // 16 KiB per factor tile
 constexpr size_t kSmemMax = 232448;    // 227 KiB of dynamic shared memory per CTA
 constexpr int kMaxStages = 12;
+constexpr int kDrain = 2;              // ODD: chunks that an accumulator takes before it is added to the sums
 
 // SR: token rows the epilogue stages in shared memory at a time (32, 64 or 128).
 // Fewer rows leave room for more stages in the ring, i.e. more factor bytes in
@@ -491,7 +492,37 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         uint32_t ring = 0, grp = 0;
         bool ok = true;
         const uint32_t idesc = idesc_bf16(kTileM, K);
-        for (int ng; ok && (ng = it.take<G>(p, ncl, crank, gx, gt)) > 0; ++grp) {
+        if constexpr (ODD)  // groups of kDrain chunks, in turn into two accumulators behind the sums
+            while (ok && it.take<G>(p, ncl, crank, gx, gt) > 0)
+                for (int k0 = 0; ok && k0 < nk_tot; ++grp) {  // groups end with a side
+                    const uint32_t b = grp & 1u;
+                    const int end = k0 < p.nk_in ? p.nk_in : nk_tot, n = end - k0 < kDrain ? end - k0 : kDrain;
+                    ok = warp_wait(smem_u32(&tempty[b]), ((grp >> 1) & 1u) ^ 1u, abort, p.err);
+                    for (int c = 0; ok && c < n; ++c, ++ring) {
+                        const int s = ring % C::kStages;
+                        const uint32_t ph = (ring / C::kStages) & 1u;
+                        if (!warp_wait(smem_u32(&full[s]), ph, abort, p.err) ||
+                            !warp_wait(smem_u32(&sready[s]), ph, abort, p.err)) {
+                            ok = false;
+                            break;
+                        }
+                        tc_fence_after();
+                        uint8_t* stage = sA + (size_t)s * C::kStageBytes;
+                        const uint64_t ad = sw128_desc(smem_u32(stage)), bd = sw128_desc(smem_u32(stage + kTileBytes));
+                        if (elect_one()) {
+#pragma unroll
+                            for (int k = 0; k < kChunkK / 16; ++k)
+                                mma_bf16(tmem + 2 * K + b * K, ad + 2 * k, bd + 2 * k, idesc, (c > 0 || k > 0) ? 1u : 0u);
+                            mma_commit(smem_u32(&empty[s]));
+                        }
+                        __syncwarp();
+                    }
+                    if (!ok) break;
+                    if (elect_one()) mma_commit(smem_u32(&tfull[b]));
+                    __syncwarp();
+                    k0 += n;
+                }
+        for (int ng; !ODD && ok && (ng = it.take<G>(p, ncl, crank, gx, gt)) > 0; ++grp) {
             const uint32_t b = grp & 1u, use = grp >> 1;
             if (!warp_wait(smem_u32(&tempty[b]), (use & 1u) ^ 1u, abort, p.err)) {
                 ok = false;
@@ -599,7 +630,41 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                 for (int c = 0; c < C::CB; ++c) acc[a][c] = 0.f;
             do {
                 const uint32_t b = grp & 1u, use = grp >> 1;
-                if (u == 0) {
+                const uint32_t tbase =
+                    tmem + ((uint32_t)(q * 32) << 16) + (ODD ? 0u : b * C::kBufCols + (uint32_t)u * C::kAccCols);
+                if constexpr (ODD) {
+                    // every group is added with round-to-nearest to the sums of its side, TMEM columns
+                    // [0, K) and [K, 2K): one truncating sum of all features drifts (cubed normal values,
+                    // 49152 features: 5.3e-5 off, the CUDA cores' rounded chain 1.8e-6, this 4.2e-7).
+                    // 64 x 500 tokens, 4096 -> 4096, k = 100 x 72: 197 us in one sum, 205 us so
+                    bool got = true;
+                    for (int k0 = 0; k0 < nk_tot; ++grp) {
+                        const int first = k0 < p.nk_in ? 0 : p.nk_in, end = k0 < p.nk_in ? p.nk_in : nk_tot;
+                        const uint32_t gb = grp & 1u, sums = tbase + (first ? K : 0);
+                        got = warp_wait(smem_u32(&tfull[gb]), (grp >> 1) & 1u, abort, p.err);
+                        if (!got) break;
+                        tc_fence_after();
+#pragma unroll 2
+                        for (int c0 = 0; c0 < K; c0 += 16) {
+                            float v[16], o[16];
+                            uint32_t r[16];
+                            tmem_ld16(tbase + 2 * K + gb * K + c0, v);
+                            if (k0 > first) tmem_ld16(sums + c0, o);
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) r[i] = __float_as_uint(k0 > first ? o[i] + v[i] : v[i]);
+                            tmem_st16(sums + c0, r);
+                        }
+                        tmem_wait_st();
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(smem_u32(&tempty[gb]));
+                        k0 += end - k0 < kDrain ? end - k0 : kDrain;
+                    }
+                    if (epi_any(!got)) {
+                        ok = false;
+                        break;
+                    }
+                } else if (u == 0) {
                     bool got = warp_wait(smem_u32(&tfull[b]), use & 1u, abort, p.err);
                     if (epi_any(!got)) {
                         ok = false;
@@ -607,8 +672,6 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                     }
                     tc_fence_after();
                 }
-                const uint32_t tbase =
-                    tmem + ((uint32_t)(q * 32) << 16) + b * C::kBufCols + (uint32_t)u * C::kAccCols;
                 for (int h = 0; h < kParts; ++h) {
                     if (q / kWarpsPer == h) {
                         const int srow = (q % kWarpsPer) * 32 + lane;
@@ -621,7 +684,7 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                             for (int i = 0; i < 16; i += 4)
                                 *reinterpret_cast<float4*>(dst + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
                         }
-                        if (u == ng - 1) {
+                        if (!ODD && u == ng - 1) {
                             tc_fence_before();
                             __syncwarp();
                             if (lane == 0) mbar_arrive(smem_u32(&tempty[b]));
@@ -643,7 +706,7 @@ project_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                     epi_sync();
                 }
                 if (++u == ng) {
-                    ++grp;
+                    if (!ODD) ++grp;
                     ng = it.take<G>(p, ncl, crank, gx, gt);
                     u = 0;
                 }

@@ -43,3 +43,10 @@ def check(dev, orc, dtype, N, T, di, do, ki, ko):
     ("bf16", 2, 40, 16384, 64, 32, 48), ("bf16", 1, 130, 72, 16392, 8, 24)])
 def test_wide_layers_of_uneven_features(dev, orc, dtype, N, T, di, do, ki, ko):
     check(dev, orc, dtype, N, T, di, do, ki, ko)
+
+
+@pytest.mark.parametrize("N,T,di,do,ki,ko", [(2, 40, 16384, 64, 100, 72), (3, 200, 64, 16392, 72, 128),
+                                             (160, 130, 1000, 72, 65, 3), (1, 520, 72, 64, 128, 96)])
+def test_wide_layers_of_uneven_features_k_above_64(dev, orc, N, T, di, do, ki, ko):
+    # groups that end with a side, several tiles an example, clusters and whole examples a CTA
+    check(dev, orc, "bf16", N, T, di, do, ki, ko)
