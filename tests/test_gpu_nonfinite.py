@@ -48,3 +48,27 @@ def test_token_scores_keep_nan(dev, ki, ko):
     lost[:, 1, 7] = lost[2] = True
     assert np.isnan(outs[1][lost]).all()
     np.testing.assert_array_equal(outs[1][~lost], outs[0][~lost])
+
+
+@pytest.mark.parametrize("T,k", [(3, 32), (40, 64), (130, 24)])
+def test_fp32_pieces_extremes(dev, orc, T, k):
+    # k above 16: the kernel that cuts fp32 factors into three bf16 pieces, packed and whole tiles. Tiny values, values
+    # of the largest exponent, an infinity and both NaN patterns stay in their example
+    N, d = 5, 64
+    A, B = (synth.factors(seed, 64, N, T, d, sc, 0, 0, "f32", 0.02) for seed, sc in ((synth.SEED_A, 1.0), (synth.SEED_B, 0.1)))
+    A[0] *= np.float32(1e-30)
+    B[0] *= np.float32(1e-3)
+    A[1] *= np.float32(1e36)
+    B[1] *= np.float32(1e-30)
+    A[2, 1, 5] = np.inf
+    B[3, 0, 7] = np.nan
+    A[4, 2, 9] = np.array(0x7FFFFFFF, np.uint32).view(np.float32)
+    L = tda.LayerDesc(d, d, T, k, k, seed=7, layer=2)
+    phi = torch.empty((N, k * k), device=dev)
+    tda.tda_project(L, tda.TDA_F32, torch.from_numpy(A).to(dev), torch.from_numpy(B).to(dev), N, phi, k * k,
+                    tda.TDA_ROUTE_FACTORED)
+    tda.tda_device_status()
+    got = phi.cpu().numpy().astype(np.float64)
+    ref = orc.project(A[:2].astype(np.float64), B[:2].astype(np.float64), k, k, 7, 2).reshape(2, -1)
+    assert max(np.linalg.norm(got[n] - ref[n]) / np.linalg.norm(ref[n]) for n in range(2)) <= 1e-5
+    assert not np.isfinite(got[2]).any() and np.isnan(got[3:]).all()

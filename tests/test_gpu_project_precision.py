@@ -50,3 +50,20 @@ def test_wide_layers_of_uneven_features(dev, orc, dtype, N, T, di, do, ki, ko):
 def test_wide_layers_of_uneven_features_k_above_64(dev, orc, N, T, di, do, ki, ko):
     # groups that end with a side, several tiles an example, clusters and whole examples a CTA
     check(dev, orc, "bf16", N, T, di, do, ki, ko)
+
+
+@pytest.mark.parametrize("N,T,di,do,ki,ko", [(4000, 5, 64, 72, 8, 5), (64, 32, 576, 256, 16, 16), (8, 32, 576, 256, 16, 16),
+                                             (1, 1, 516, 4, 1, 1), (300, 64, 64, 64, 12, 16)])
+def test_fp32_packed_tiles_of_few_columns(dev, orc, N, T, di, do, ki, ko):
+    # fp32 factors at k up to 16 past the limits of the CUDA-core kernel for short jobs (16384 tokens, 512 features)
+    rng = np.random.default_rng(N)
+    A, B = (rng.standard_normal((N, T, d)).astype(np.float32) for d in (di, do))
+    L = tda.LayerDesc(di, do, T, ki, ko, seed=7, layer=2)
+    phi = torch.full((N, ki * ko + 1), 7.0, device=dev)
+    tda.tda_project(L, tda.TDA_F32, torch.from_numpy(A).to(dev), torch.from_numpy(B).to(dev), N, phi, ki * ko + 1,
+                    tda.TDA_ROUTE_FACTORED)
+    tda.tda_device_status()
+    ref = orc.project(A.astype(np.float64), B.astype(np.float64), ki, ko, 7, 2).reshape(N, -1)
+    got = phi.cpu().numpy().astype(np.float64)
+    assert (got[:, ki * ko] == 7.0).all()
+    assert max(np.linalg.norm(got[n, :ki * ko] - ref[n]) / np.linalg.norm(ref[n]) for n in range(N)) <= TOL
