@@ -370,39 +370,21 @@ __global__ void __launch_bounds__(256) update_kernel(St<TS> st, int64_t k0) {
 // serial chains), 35 us with every warp inverting every pivot before its updates, 27 us here.
 constexpr int kF64Rows = 8;
 
-// 1/p and 1/sqrt(p) for p > 0 to fp64 rounding: p = m 4^h with m in [1, 4); the fp32 guess for m
-// is within 2^-21, and one step of Householder's third-order iteration takes it past 2^-60.
-__device__ __forceinline__ double pow2(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
-__device__ __forceinline__ double split_pow4(double p, int& h) {
-    int sub = 0;
-    if (p < 2.3e-308) p *= 18014398509481984.0, sub = 27;  // subnormal: times 2^54
-    const long long b = __double_as_longlong(p);
-    const int e = (int)(b >> 52) - 1023, odd = e & 1;
-    h = ((e - odd) >> 1) - sub;
-    return __longlong_as_double((b & 0xFFFFFFFFFFFFFll) | ((long long)(1023 + odd) << 52));
-}
-__device__ __forceinline__ double rcp_f64(double p) {
-    int h;
-    const double m = split_pow4(p, h), r = (double)__frcp_rn((float)m);
-    const double e = fma(-m, r, 1.0);
-    const bool wide = h > 510 || h < -510;
-    const double x = fma(r, fma(e, e, e), r) * pow2(wide ? -h : -2 * h);
-    return wide ? x * pow2(-h) : x;
-}
-// 1/p on the pivots' serial chain: the hardware's 20-bit guess of a double's reciprocal needs no
-// conversions and no scaling inside 2^-1000 .. 2^1000, and the same iteration takes it past 2^-59.
+// 1/p on the pivots' serial chain, for p between kRcpMin and kRcpMax: the hardware's 20-bit guess of a
+// double's reciprocal, and one step of Householder's third-order iteration takes it past 2^-59 before rounding.
+constexpr double kRcpMin = 9.4e-302, kRcpMax = 1.07e301;
 __device__ __forceinline__ double rcp_chain(double p) {
-    if (!(p > 9.4e-302 && p < 1.07e301)) return rcp_f64(p);
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(p));
     const double e = fma(-p, r, 1.0);
     return fma(r, fma(e, e, e), r);
 }
-__device__ __forceinline__ double rsqrt_f64(double p) {
-    int h;
-    const double m = split_pow4(p, h), r = (double)rsqrtf((float)m);
-    const double e = fma(-m * r, r, 1.0);
-    return fma(r * e, fma(0.375, e, 0.5), r) * pow2(-h);
+// What the updates by a pivot p multiply with: w = 1/p, or near the ends of the exponent range, where 1/p
+// may overflow or lose bits, w = 1/sqrt(p) to be multiplied with twice (twice: true).
+__device__ __forceinline__ double pivot_factor(double p, bool& twice) {
+    twice = !(p > kRcpMin && p < kRcpMax);
+    if (!twice) return rcp_chain(p);
+    return p > 0.0 ? rsqrt(p) : NAN;
 }
 
 __global__ void __launch_bounds__(128) panel_f64_kernel(St<double> st, int64_t k0) {
@@ -425,42 +407,51 @@ __global__ void __launch_bounds__(128) panel_f64_kernel(St<double> st, int64_t k
         A[i][j] = v;
     }
     __syncthreads();
-    __shared__ double wj[2];  // 1 / A_jj of the current and the next column
+    __shared__ double wj[2];  // pivot_factor of the current and the next column
+    __shared__ int wtwice[2];
     int bad = -1;             // warp 0: first non-positive pivot
+    bool twice = false;
     if (warp == 0) {
         const double p = A[0][0];
         if (!(p > 0.0)) bad = 0;
-        const double w = p > 0.0 ? rcp_chain(p) : NAN;
-        if (lane == 0) wj[0] = w;
+        const double w = pivot_factor(p, twice);
+        if (lane == 0) wj[0] = w, wtwice[0] = twice;
     }
     __syncthreads();
     for (int j = 0; j < kNB - 1; ++j) {
         const double w = wj[j & 1];
         if (warp == 0) {
-            const double a = A[j + 1][j], p = A[j + 1][j + 1] - a * w * a;
+            const double a = A[j + 1][j], aw = a * w, p = A[j + 1][j + 1] - (twice ? aw * aw : aw * a);
             if (!(p > 0.0) && bad < 0) bad = j + 1;
-            const double wn = p > 0.0 ? rcp_chain(p) : NAN;
+            const double wn = pivot_factor(p, twice);
             if (lane == 0) {
                 A[j + 1][j + 1] = p;
                 wj[(j + 1) & 1] = wn;
+                wtwice[(j + 1) & 1] = twice;
             }
         } else {
             const int u = warp - 1;
-            // the diagonal block's rows below j + 1: column c of row `lane`
-            if (lane > j + 1) {
-                const double t = A[lane][j] * w;
-                for (int c = j + 1 + u; c <= lane; c += 3) A[lane][c] -= t * A[c][j];
-            }
-            // the panel rows: 8 rows x the columns after j, 12 columns at a time
-            const int pr = kNB + (lane & 7);
-            const double tp = A[pr][j] * w;
-            for (int c = j + 1 + u * 4 + (lane >> 3); c < kNB; c += 12) A[pr][c] -= tp * A[c][j];
+            auto update = [&](auto&& col) {  // col(c): the column's entry c, times w where that is due twice
+                // the diagonal block's rows below j + 1: column c of row `lane`
+                if (lane > j + 1) {
+                    const double t = A[lane][j] * w;
+                    for (int c = j + 1 + u; c <= lane; c += 3) A[lane][c] -= t * col(c);
+                }
+                // the panel rows: 8 rows x the columns after j, 12 columns at a time
+                const int pr = kNB + (lane & 7);
+                const double tp = A[pr][j] * w;
+                for (int c = j + 1 + u * 4 + (lane >> 3); c < kNB; c += 12) A[pr][c] -= tp * col(c);
+            };
+            if (wtwice[j & 1])
+                update([&](int c) { return A[c][j] * w; });
+            else
+                update([&](int c) { return A[c][j]; });
         }
         __syncthreads();
     }
     if (warp == 0) {
         const double p = A[lane][lane];
-        inv[lane] = p > 0.0 ? rsqrt_f64(p) : NAN;
+        inv[lane] = p > 0.0 ? rsqrt(p) : NAN;
         if (blockIdx.x == 0 && lane == 0 && bad >= 0 && bad < nb) {
             double* h = st.header(l);
             if (h[kPcFailedPivot] == 0.0) h[kPcFailedPivot] = (double)(k0 + bad + 1);
