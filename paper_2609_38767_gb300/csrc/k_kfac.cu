@@ -226,17 +226,23 @@ __device__ void gemm_nn(double* out, const double* X, const double* Y, int n, in
     }
     cluster_barrier();  // the whole product is in every CTA
 }
-// V <- V (3I - V^T V) / 2: one Newton-Schulz step towards orthonormal columns (T1, T2: scratch)
-__device__ void orthonormalise(double* V, double* T1, double* T2, int n, int ld, int cs, int rank) {
+// V <- V (3I - V^T V) / 2: one Newton-Schulz step towards orthonormal columns (T1, T2: scratch). A
+// deviation of d becomes n d^2 at most, so the step is not the last one if d was above 1e-9: returns whether
+// it was (in every CTA alike: they hold the same V^T V).
+__device__ bool orthonormalise(double* V, double* T1, double* T2, int n, int ld, int cs, int rank) {
     gemm_nn(T1, V, V, n, ld, true, cs, rank);
+    int far = 0;
     for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
         const int i = e / n, j = e % n;
-        T1[i * ld + j] = ((i == j) ? 1.5 : 0.0) - 0.5 * T1[i * ld + j];
+        const double t = T1[i * ld + j], one = i == j ? 1.0 : 0.0;
+        far |= fabs(t - one) > 1e-9;
+        T1[i * ld + j] = 1.5 * one - 0.5 * t;
     }
-    __syncthreads();
+    far = __syncthreads_or(far);
     gemm_nn(T2, V, T1, n, ld, false, cs, rank);
     for (int e = threadIdx.x; e < n * n; e += blockDim.x) V[(e / n) * ld + e % n] = T2[(e / n) * ld + e % n];
     __syncthreads();
+    return far;
 }
 
 // Eigenbases of C = S / M for the a side (blockIdx.x 0) and the g side (1) of
@@ -247,7 +253,7 @@ __device__ void orthonormalise(double* V, double* T1, double* T2, int n, int ld,
 //   and with products shared by the cluster: a Newton-Schulz step
 //   V <- V (3I - V^T V) / 2, A = V^T C V afresh, and twice the first-order
 //   rotation of all pairs at once, V <- V (I + E) with E_ij = A_ij / (A_jj - A_ii),
-//   made orthonormal by another Newton-Schulz step (errors of 1e-7 become 1e-14,
+//   made orthonormal by Newton-Schulz steps, one mostly (errors of 1e-7 become 1e-14,
 //   then rounding; pairs with a gap below 1000 |A_ij| are left out). fp64 sweeps
 //   finish what is left: none, mostly, where two used to take most of the time
 //   (three k = 32 layers: 576 us, 220 now). The header gets the fp64 sweep count.
@@ -316,7 +322,9 @@ jacobi_kernel(double* __restrict__ st0, int64_t stride, int64_t ka, int64_t kg, 
             gemm_nn(A, V, Tm, n, ld, false, cs, rank);
             for (int e = threadIdx.x; e < n * n; e += blockDim.x) V[(e / n) * ld + e % n] = A[(e / n) * ld + e % n];
             __syncthreads();
-            orthonormalise(V, Tm, A, n, ld, cs, rank);
+            // many pairs just past the gap's limit turn V by up to 0.06: then one last step is not enough
+            for (int r = 0; orthonormalise(V, Tm, A, n, ld, cs, rank) && it == 1 && r < 3; ++r) {
+            }
             form_a();
         }
         sweeps = jacobi_sweeps<double>(A, ld, V, ld, n, cs64, sn, P, Q, red, &done, 1e-28, 60);
