@@ -20,7 +20,7 @@
 //
 // Accuracy: the tensor pipe adds into its fp32 accumulators with truncation,
 // a loss of about a quarter ulp per addition that always points to zero (d =
-// 2048, 128 additions: 3.6e-6 low). So K goes in blocks of one to eight 64-feature
+// 2048, 128 additions: 3.6e-6 low). So K goes in blocks of one to four 64-feature
 // chunks, each into one of two 256-column TMEM buffers, and the epilogue adds
 // the blocks in registers with round-to-nearest: X's blocks are summed (128
 // registers a thread), and since the identity is bilinear every Y block is
@@ -627,12 +627,14 @@ cudaError_t launch(const tda_layer_desc& L, const void* Aq, const void* Bq, int6
     p.T = T;
     p.nk_in = (int)((L.d_in + kChunkK - 1) / kChunkK);
     p.nk_out = (int)((L.d_out + kChunkK - 1) / kChunkK);
-    // Block lengths that keep the accuracy of an fp32 FMA chain over d features (1.8e-7 at d = 256,
-    // 5.7e-7 at 2048, 8.9e-7 at 4096): 64, 128 or 256 features, whose truncation is 1.1e-7, 2.2e-7 or
-    // 4.5e-7 (2048 -> 2048, T = 50: 4.4e-7 with 256, 183 -> 143 us from 128). Short sequences (T < 16) pay the most per Y block and take it twice as long.
+    // Block lengths that keep the accuracy of an fp32 FMA chain over d features (1.6e-7 at d = 256, 5.2e-7 at
+    // 2048, 8.5e-7 at 4096): 64, 128 or 256 features (1.5e-7, 2.5e-7 at d = 1024, 4.5e-7; 2048 -> 2048, T = 50:
+    // 183 -> 143 us from 128 to 256). T < 16 pays the most per Y block, but Y blocks of twice the length are off
+    // by half as much again (T = 5, d = 2048: 6.6e-7; 64 x 8192 pairs, T = 8, d = 256: 56 us, and 66 us so;
+    // 64 x 2048 pairs, d = 2048: 58 us either way).
     auto block = [](int nk) { return nk <= 8 ? 1 : (nk < 32 ? 2 : 4); };
     p.kbx = block(p.nk_in);
-    p.kby = block(p.nk_out) * (packed && T < 16 ? 2 : 1);
+    p.kby = block(p.nk_out);
     p.pq = packed ? (int)(kTM / T) : 0;
     p.pt = !packed ? 0 : (int)(T < 16 ? C::kCols / T * 2 : C::kTN / T);
     p.tiles_q = packed ? 1 : (int)((T + kTM - 1) / kTM);
