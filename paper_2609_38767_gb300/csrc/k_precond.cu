@@ -367,7 +367,7 @@ __global__ void __launch_bounds__(256) update_kernel(St<TS> st, int64_t k0) {
 // guess and one cubic step) while warps 1-3 update the rest with the current column; one barrier a
 // column. Chunk 0 leaves L_kk in the block's slot of Dinv; f64_inverse_kernel replaces it by its
 // inverse after the last step. D = 256: 150 us a step in panel_kernel (one CTA: two warps of
-// serial chains), 35 us with every warp inverting every pivot before its updates, 27 us here.
+// serial chains), 26 us here.
 constexpr int kF64Rows = 8;
 
 // 1/p on the pivots' serial chain, for p between kRcpMin and kRcpMax: the hardware's 20-bit guess of a
@@ -1915,10 +1915,9 @@ __global__ void nan_failed_kernel(St<float> st, float* qhat, int64_t ld, int64_t
         qhat[(e / D) * ld + (int64_t)l * D + e % D] = NAN;
 }
 
-// (layers are a grid's y coordinate)
-bool blocked_pc(int n_layers, int64_t D, tda_dtype sdt) {
-    return sdt == TDA_F32 && n_layers <= 65535 && D % 64 == 0 && D >= kBlockedMinD && D < (1LL << 31) / kBB &&
-           gemm_tc_available();
+// (layers are a grid's y coordinate: the entry point takes 65535 at most)
+bool blocked_pc(int64_t D, tda_dtype sdt) {
+    return sdt == TDA_F32 && D % 64 == 0 && D >= kBlockedMinD && D < (1LL << 31) / kBB && gemm_tc_available();
 }
 
 template <int R, bool FWD>
@@ -1996,10 +1995,10 @@ cudaError_t factor_blocked(int n_layers, int64_t D, void* state, int64_t n_total
 }
 
 // (D >= kBlockedMinD suffices where the state is factored in the same call)
-bool apply_blocked_ok(int n_layers, int64_t D, tda_dtype sdt, int64_t ld_q, const void* qhat, int64_t ld_qhat,
+bool apply_blocked_ok(int64_t D, tda_dtype sdt, int64_t ld_q, const void* qhat, int64_t ld_qhat,
                       int64_t n_q) {
     // 2-D copies: row strides below 2^31 bytes
-    return blocked_pc(n_layers, D, sdt) && ((uintptr_t)qhat & 15) == 0 && (ld_qhat & 3) == 0 && n_q < (1LL << 24) &&
+    return blocked_pc(D, sdt) && ((uintptr_t)qhat & 15) == 0 && (ld_qhat & 3) == 0 && n_q < (1LL << 24) &&
            ld_q < (1LL << 29) && ld_qhat < (1LL << 29);
 }
 
@@ -2076,7 +2075,7 @@ cudaError_t launch_pc_fit(int n_layers, int64_t D, tda_dtype sdt, void* state, c
 
 cudaError_t launch_pc_factor(int n_layers, int64_t D, tda_dtype sdt, void* state, int64_t n_total,
                              double lambda_abs, double lambda_rel, cudaStream_t s) {
-    if (blocked_pc(n_layers, D, sdt))
+    if (blocked_pc(D, sdt))
         return factor_blocked(n_layers, D, state, n_total, lambda_abs, lambda_rel, nullptr, 0, 0, s);
     if (sdt == TDA_F64) return factor_impl<double>(n_layers, D, state, n_total, lambda_abs, lambda_rel, s);
     return factor_impl<float>(n_layers, D, state, n_total, lambda_abs, lambda_rel, s);
@@ -2086,7 +2085,7 @@ cudaError_t launch_pc_factor_apply(int n_layers, int64_t D, tda_dtype sdt, void*
                                    double lambda_abs, double lambda_rel, const float* q, int64_t n_q, int64_t ld_q,
                                    void* qhat, int64_t ld_qhat, cudaStream_t s) {
     cudaError_t e;
-    if (n_q >= 1 && apply_blocked_ok(n_layers, D, sdt, ld_q, qhat, ld_qhat, n_q)) {
+    if (n_q >= 1 && apply_blocked_ok(D, sdt, ld_q, qhat, ld_qhat, n_q)) {
         if ((e = copy_queries(n_layers, D, q, n_q, ld_q, (float*)qhat, ld_qhat, s)) != cudaSuccess) return e;
         e = factor_blocked(n_layers, D, state, n_total, lambda_abs, lambda_rel, (float*)qhat, n_q, ld_qhat, s);
         if (e != cudaSuccess) return e;
@@ -2095,7 +2094,7 @@ cudaError_t launch_pc_factor_apply(int n_layers, int64_t D, tda_dtype sdt, void*
     // fp32 state, whole 32-column blocks, up to 256 queries: factorisation and both
     // substitutions in one cluster launch per call;
     // otherwise FACTOR, then APPLY
-    if (sdt == TDA_F32 && !(blocked_states(D) && blocked_pc(n_layers, D, sdt)) && D % kNB == 0 && D >= 2 * kNB &&
+    if (sdt == TDA_F32 && !(blocked_states(D) && blocked_pc(D, sdt)) && D % kNB == 0 && D >= 2 * kNB &&
         n_q >= 1 && n_q <= 256) {
         const QArgs qa{q, (float*)qhat, n_q, ld_q, ld_qhat};
         e = factor_cluster<16, true>(n_layers, D, state, n_total, lambda_abs, lambda_rel, qa, s);
@@ -2112,7 +2111,7 @@ cudaError_t launch_pc_apply(int n_layers, int64_t D, tda_dtype sdt, const void* 
                             int64_t n_q, int64_t ld_q, void* qhat, int64_t ld_qhat, cudaStream_t s) {
     if (n_q == 0) return cudaSuccess;
     // a blocked factorisation left L^T in M's upper triangle: tensor-core substitutions
-    if (blocked_states(D) && apply_blocked_ok(n_layers, D, sdt, ld_q, qhat, ld_qhat, n_q)) {
+    if (blocked_states(D) && apply_blocked_ok(D, sdt, ld_q, qhat, ld_qhat, n_q)) {
         const cudaError_t e = copy_queries(n_layers, D, q, n_q, ld_q, (float*)qhat, ld_qhat, s);
         return e != cudaSuccess ? e : apply_blocked(n_layers, D, state, n_q, (float*)qhat, ld_qhat, true, s);
     }
