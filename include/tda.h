@@ -319,6 +319,9 @@ tda_status tda_cosine(float* S, int64_t n_q, int64_t n_t, int64_t ld_S, const fl
  * multiple of 4), solve the query rows in 256-column blocks with tensor-core updates. In this mode
  * qhat may alias q (same pointer and row stride: solved in place). Other F32
  * layers with D a multiple of 32 run FACTOR_APPLY for n_q <= 256 in one launch.
+ * The updates of such a layer's M and of its query rows are added by the L2
+ * cache, which takes sums below 2^-126 as zero: features from about 1e-18 and
+ * queries from about 1e-36 on keep full precision.
  * A state factored by an earlier version of the library can be passed to APPLY.
  * Arguments not used by an op are ignored (may be 0/NULL).
  * ------------------------------------------------------------------------- */
@@ -545,7 +548,8 @@ uint64_t tda_launch_count(void);
  * that kernels queued on another stream (the query side of a step: the query
  * projection, the curvature fit, its factorisation and the preconditioning)
  * find SMs free and run beside it. 0 (the default) = every SM. Process-wide,
- * host only; results do not depend on it. n_sms < 0 -> TDA_ERR_INVALID_ARG. */
+ * host only; results depend on it only in the order in which an example's
+ * partial sums are added. n_sms < 0 -> TDA_ERR_INVALID_ARG. */
 tda_status tda_set_sm_budget(int32_t n_sms);
 int32_t tda_get_sm_budget(void);
 

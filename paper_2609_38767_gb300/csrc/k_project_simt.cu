@@ -217,6 +217,11 @@ project_small_kernel(const float* __restrict__ A, const float* __restrict__ B, i
 
 }  // namespace
 
+// The line is not where the tensor-core kernel (k_project_flex.cu) becomes faster but where a job is no longer
+// small: below it features stay, bit for bit, what an fp64 preconditioner has seen before. d = 256, T = 32, k = 16,
+// 8 or 64 examples: 6.6 us here, 9.5 us there; d = 512, T = 64: 16 to 128 examples 19.9 and 15.8 us, 256 examples
+// 36.7 and 17.8 us; 16384 examples of one token, d = 512: 506 and 39 us. These sums are fp32 chains in order
+// (6.8e-7 off at d = 256), the other kernel's 1.9e-7.
 bool project_small_supported(const tda_layer_desc& L, const void* A, const void* B, int64_t N) {
     return L.kind == TDA_PROJ_RADEMACHER && L.T >= 1 && L.T <= kSmallT && L.d_in <= kSmallD && L.d_out <= kSmallD &&
            L.k_in <= kSmallK && L.k_out <= kSmallK && L.d_in % 4 == 0 && L.d_out % 4 == 0 && N <= 16384 / L.T &&

@@ -1,5 +1,6 @@
-"""The fp64 preconditioner's pivots over the whole range of exponents, from states written directly (a diagonal block
-matrix of small blocks, one scale each), against exact rational arithmetic."""
+"""The preconditioner far from well-conditioned features of order one: the fp64 pivots over the whole range of exponents,
+from states written directly (a diagonal block matrix of small blocks, one scale each), against exact rational
+arithmetic; the fp32 blocked path with rank-deficient fits and little damping, and with tiny features."""
 from fractions import Fraction
 
 import numpy as np
@@ -86,3 +87,35 @@ def test_fp64_blocks_of_any_scale(dev, exps):
         tol[r] = (12 * 2.0 ** -52 + 64 * 2.0 ** (-1074 - int(e))) * np.abs(ref[r]).max()
     got = solve(dev, np.tril(M), q)
     assert (np.abs(got - ref) <= tol).all(), (np.abs(got - ref) / tol).max()
+
+
+# Random-walk rounding of a 256-feature fp32 sum, 16 * 2^-24 of a pivot's scale, is a backward error that the solve
+# magnifies by the condition number (largest eigenvalue of the fit over the damping).
+@pytest.mark.parametrize("D,n,lam,scale", [(256, 64, 1e-2, 1.0), (256, 64, 1e-4, 1.0), (576, 144, 1e-3, 1.0),
+                                           (1024, 256, 1e-3, 1.0), (2048, 512, 1e-3, 1.0), (512, 128, 1e-2, 1e-17)])
+def test_fp32_weak_damping(dev, D, n, lam, scale):
+    rng = np.random.default_rng(D)
+    nl, nq = 2, 20
+    w = nl * D
+    ph = torch.from_numpy((rng.standard_normal((n, w)) * scale).astype(np.float32)).to(dev)
+    q = torch.from_numpy(rng.standard_normal((nq, w)).astype(np.float32)).to(dev)
+    state = torch.empty(nl * tda.tda_precondition_state_bytes(D, tda.TDA_F32), dtype=torch.uint8, device=dev)
+    out, alone = torch.empty((nq, w), device=dev), torch.empty((nq, w), device=dev)
+    args = (nl, D, tda.TDA_F32, state)
+    tda.tda_precondition(tda.TDA_PC_RESET, *args)
+    tda.tda_precondition(tda.TDA_PC_FIT_ACCUM, *args, phi=ph, n=n, ld_phi=w)
+    tda.tda_precondition(tda.TDA_PC_FACTOR_APPLY, *args, n_total=n, lambda_rel_mean_eig=lam, q=q, n_q=nq, ld_q=w,
+                         qhat=out, ld_qhat=w)
+    tda.tda_precondition(tda.TDA_PC_APPLY, *args, q=q, n_q=nq, ld_q=w, qhat=alone, ld_qhat=w)
+    tda.tda_device_status()
+    tda.tda_precondition_info(nl, D, tda.TDA_F32, state)
+    for l in range(nl):
+        x = ph[:, l * D:(l + 1) * D].double()
+        F = x.T @ x / n
+        damping = lam * F.diagonal().mean()
+        cond = float((torch.linalg.eigvalsh(F)[-1] + damping) / damping)
+        F.diagonal().add_(damping)
+        ref = torch.linalg.solve(F, q[:, l * D:(l + 1) * D].double().T).T
+        for o in (out, alone):
+            got = o[:, l * D:(l + 1) * D].double()
+            assert float((got - ref).norm() / ref.norm()) <= 16 * 2.0 ** -24 * cond
