@@ -139,7 +139,7 @@ project_simt_kernel(const T* __restrict__ A, const T* __restrict__ B, int64_t Tn
 // tokens, run in the general kernel's order, so the features are the same bit for bit (an fp64
 // preconditioner state behind them sees no change). 64 examples, 256 -> 256, T = 32, k = 16:
 // 63 us in the general kernel, which computes 64 columns whatever k is, 16 tokens at a time;
-// about 25 us here.
+// 8 us here.
 constexpr int kSmallT = 64, kSmallD = 512, kSmallK = 16;
 constexpr int kSmallLd = kDChunk + 4;  // padded row: 16-byte loads of different tokens miss each other's banks
 
@@ -221,7 +221,7 @@ project_small_kernel(const float* __restrict__ A, const float* __restrict__ B, i
 // small: below it features stay, bit for bit, what an fp64 preconditioner has seen before. d = 256, T = 32, k = 16,
 // 8 or 64 examples: 6.6 us here, 9.5 us there; d = 512, T = 64: 16 to 128 examples 19.9 and 15.8 us, 256 examples
 // 36.7 and 17.8 us; 16384 examples of one token, d = 512: 506 and 39 us. These sums are fp32 chains in order
-// (6.8e-7 off at d = 256), the other kernel's 1.9e-7.
+// (T = 64, d = 512: 6.8e-7 off), the other kernel is closer (1.8e-7).
 bool project_small_supported(const tda_layer_desc& L, const void* A, const void* B, int64_t N) {
     return L.kind == TDA_PROJ_RADEMACHER && L.T >= 1 && L.T <= kSmallT && L.d_in <= kSmallD && L.d_out <= kSmallD &&
            L.k_in <= kSmallK && L.k_out <= kSmallK && L.d_in % 4 == 0 && L.d_out % 4 == 0 && N <= 16384 / L.T &&
