@@ -231,12 +231,15 @@ __device__ void gemm_nn(double* out, const double* X, const double* Y, int n, in
 // it was (in every CTA alike: they hold the same V^T V).
 __device__ bool orthonormalise(double* V, double* T1, double* T2, int n, int ld, int cs, int rank) {
     gemm_nn(T1, V, V, n, ld, true, cs, rank);
-    int far = 0;
+    // (the diagonal by two warps, the rest by their high words, 1e-9's is 0x3E112E0B: fp64 comparisons of
+    // all entries took 6 us of a call)
+    int far = (int)threadIdx.x < n && fabs(T1[threadIdx.x * ld + threadIdx.x] - 1.0) > 1e-9;
+    __syncthreads();
     for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
         const int i = e / n, j = e % n;
-        const double t = T1[i * ld + j], one = i == j ? 1.0 : 0.0;
-        far |= fabs(t - one) > 1e-9;
-        T1[i * ld + j] = 1.5 * one - 0.5 * t;
+        const double t = T1[i * ld + j];
+        far |= i != j && (__double2hiint(t) & 0x7FFFFFFF) > 0x3E112E0B;
+        T1[i * ld + j] = ((i == j) ? 1.5 : 0.0) - 0.5 * t;
     }
     far = __syncthreads_or(far);
     gemm_nn(T2, V, T1, n, ld, false, cs, rank);
