@@ -154,9 +154,10 @@ tda_status tda_project(const tda_layer_desc* L, tda_dtype dtype, const void* A, 
 /* Which kernel tda_project (route FACTORED) would run for these arguments on
  * the current device: 1 = a tcgen05/TMA tensor-core kernel (bf16 with k_in and
  * k_out at most 128, fp32 with at most 64, sm_103; fp32 batches of at most
- * 16384 tokens with T <= 64, widths <= 512 and k <= 16 run on the CUDA cores
- * all the same), 0 = the CUDA-core kernel, negative = the arguments are
- * invalid. Host only; for tests and benchmark reports. */
+ * 16384 tokens with T <= 64, widths <= 512 and k <= 16, and bf16 batches of few
+ * tokens with a k above 64 other than 128 x 128, run on the CUDA cores all the
+ * same), 0 = the CUDA-core kernel, negative = the arguments are invalid. Host
+ * only; for tests and benchmark reports. */
 int32_t tda_project_engine(const tda_layer_desc* L, tda_dtype dtype, const void* A, const void* B);
 
 /* ---------------------------------------------------------------------------

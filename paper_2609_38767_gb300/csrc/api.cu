@@ -319,7 +319,9 @@ tda_status tda_project(const tda_layer_desc* L, tda_dtype dtype, const void* A, 
         // ten on the tensor cores), the rest on the tensor cores
         if (dtype == TDA_F32 && project_small_supported(*L, A, B, N))
             return cuda_check(launch_project_small(*L, A, B, N, phi, ld_phi, s), "project (small)");
-        const bool stream = dtype == TDA_BF16 && project_tc_plain_supported(*L, A, B);
+        const bool odd = (L->k_in > 64 || L->k_out > 64) && !(L->k_in == 128 && L->k_out == 128);
+        const bool stream =
+            dtype == TDA_BF16 && project_tc_plain_supported(*L, A, B) && !(odd && project_short_supported(*L, N));
         const bool flex = project_flex_supported(*L, dtype, A, B);
         if (stream || flex) {
             unsigned int* err = device_error_word();

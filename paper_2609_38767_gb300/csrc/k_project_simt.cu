@@ -9,6 +9,7 @@
 // cover (identity maps, k above their blocks); project_small_kernel takes short
 // fp32 jobs of narrow layers, with the general kernel's sums bit for bit.
 #include <cuda_bf16.h>
+#include <math.h>
 
 #include "tda_internal.cuh"
 
@@ -226,6 +227,20 @@ bool project_small_supported(const tda_layer_desc& L, const void* A, const void*
     return L.kind == TDA_PROJ_RADEMACHER && L.T >= 1 && L.T <= kSmallT && L.d_in <= kSmallD && L.d_out <= kSmallD &&
            L.k_in <= kSmallK && L.k_out <= kSmallK && L.d_in % 4 == 0 && L.d_out % 4 == 0 && N <= 16384 / L.T &&
            !((uintptr_t)A & 15) && !((uintptr_t)B & 15);
+}
+
+// bf16 factors, the larger k in 65 .. 127 or unequal: whether the general kernel beats the tensor-core one, which
+// computes tiles of 128 tokens x 128 + 128 columns whatever the job is (28.5 us a tile and 8.3 ns a feature of both
+// widths). The general kernel takes 16 tokens and 64 x 64 features a CTA at a time, 1.2 us and 40 ns a feature, about
+// 240 CTAs at once. T = 8, k = 100 x 96, measured here and there: 16 examples d = 64 8.7 and 30 us, d = 256 22 and
+// 33 us, d = 1024 76 and 46 us; 152 examples d = 64 20 and 32 us, d = 256 63 and 36 us; 3000 examples d = 64 329 and
+// 561 us; T = 64, 16 examples, d = 64 26 and 30 us. Within 15 % of the line either may be the faster one.
+bool project_short_supported(const tda_layer_desc& L, int64_t N) {
+    if (L.T > 128) return false;
+    const double d = (double)(L.d_in + L.d_out), sms = (double)project_tc_max_grid();
+    const double ctas = (double)N * (double)((L.k_in + 63) / 64) * (double)((L.k_out + 63) / 64);
+    const double general = fmax(1.0, ctas / (240.0 / 152.0 * sms)) * ((double)((L.T + 15) / 16) * (1.2 + 0.04 * d) + 2.0);
+    return general < ceil((double)N / sms) * (28.5 + 0.0083 * d);
 }
 
 cudaError_t launch_project_small(const tda_layer_desc& L, const void* A, const void* B, int64_t N, float* phi,

@@ -75,6 +75,9 @@ cudaError_t launch_project_simt(const tda_layer_desc& L, tda_dtype dt, const voi
 
 // Short fp32 jobs of narrow layers, the generic kernel's sums bit for bit.
 bool project_small_supported(const tda_layer_desc& L, const void* A, const void* B, int64_t N);
+// bf16 factors with k above 64 other than 128 x 128: few tokens of narrow layers, where the general
+// kernel is the faster one.
+bool project_short_supported(const tda_layer_desc& L, int64_t N);
 cudaError_t launch_project_small(const tda_layer_desc& L, const void* A, const void* B, int64_t N, float* phi,
                                  int64_t ld_phi, cudaStream_t s);
 

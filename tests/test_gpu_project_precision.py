@@ -67,3 +67,20 @@ def test_fp32_packed_tiles_of_few_columns(dev, orc, N, T, di, do, ki, ko):
     got = phi.cpu().numpy().astype(np.float64)
     assert (got[:, ki * ko] == 7.0).all()
     assert max(np.linalg.norm(got[n, :ki * ko] - ref[n]) / np.linalg.norm(ref[n]) for n in range(N)) <= TOL
+
+
+@pytest.mark.parametrize("N,T,di,do,ki,ko", [(1, 1, 64, 64, 100, 100), (2, 8, 128, 128, 100, 90), (200, 8, 128, 136, 128, 72),
+                                             (16, 17, 256, 256, 96, 100), (16, 16, 256, 256, 96, 100), (300, 64, 64, 72, 65, 1),
+                                             (3, 128, 8, 8, 127, 128), (5, 33, 520, 8, 70, 128)])
+def test_short_jobs_of_k_above_64(dev, orc, N, T, di, do, ki, ko):
+    # either side of the line between the general and the tensor-core kernel: one result, padding columns untouched
+    rng = np.random.default_rng(N + T)
+    A, B = (torch.from_numpy(rng.standard_normal((N, T, d)).astype(np.float32)).bfloat16() for d in (di, do))
+    L = tda.LayerDesc(di, do, T, ki, ko, seed=7, layer=2)
+    phi = torch.full((N, ki * ko + 1), 7.0, device=dev)
+    tda.tda_project(L, tda.TDA_BF16, A.to(dev), B.to(dev), N, phi, ki * ko + 1, tda.TDA_ROUTE_FACTORED)
+    tda.tda_device_status()
+    ref = orc.project(A.double().numpy(), B.double().numpy(), ki, ko, 7, 2).reshape(N, -1)
+    got = phi.cpu().numpy().astype(np.float64)
+    assert (got[:, ki * ko] == 7.0).all()
+    assert max(np.linalg.norm(got[n, :ki * ko] - ref[n]) / np.linalg.norm(ref[n]) for n in range(N)) <= TOL
