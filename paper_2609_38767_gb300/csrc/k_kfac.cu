@@ -260,7 +260,7 @@ __device__ bool orthonormalise(double* V, double* T1, double* T2, int n, int ld,
 //   then rounding; pairs with a gap below 1000 |A_ij| are left out). fp64 sweeps
 //   finish what is left: none, mostly, where two used to take most of the time
 //   (three k = 32 layers: 576 us, 220 now). The header gets the fp64 sweep count.
-//   n > 64: fp64 sweeps from the start, V in the state's U.
+//   n > 64, and up to 2: fp64 sweeps from the start, V (n > 64) in the state's U.
 template <bool MIXED>
 __global__ void __launch_bounds__(kKfThreads)
 jacobi_kernel(double* __restrict__ st0, int64_t stride, int64_t ka, int64_t kg, int cs) {
@@ -636,7 +636,9 @@ cudaError_t launch_kfac_eigen(int n_layers, double* state, int64_t ka, int64_t k
     const int64_t stride = (int64_t)kfac_state_bytes(ka, kg) / 8;
     cudaError_t e;
     note_launches(1);
-    if (nmax <= 64) {
+    // up to 2 columns: the fp64 sweeps alone, without the refinement's cluster barriers (k = 1 6 us and 23 with them,
+    // k = 2 9 and 27 us, k = 3 33 to 43 and 34 us)
+    if (nmax <= 64 && nmax > 2) {
         const size_t smem = (size_t)3 * sq * 8 + (size_t)mh * (8 + 8) + (size_t)2 * sq * 4 + (size_t)mh * (4 + 4 + 4 + 4);
         // the largest shared memory of n <= 64, set once per device
         constexpr int kMax = (int)((size_t)3 * 64 * 65 * 8 + 33 * 16 + (size_t)2 * 64 * 65 * 4 + 33 * 16);
@@ -658,7 +660,7 @@ cudaError_t launch_kfac_eigen(int n_layers, double* state, int64_t ka, int64_t k
         if ((e = cudaLaunchKernelEx(&cfg, jacobi_kernel<true>, state, stride, ka, kg, cs))) return e;
         return cudaGetLastError();
     }
-    const size_t smem = (size_t)sq * 8 + (size_t)mh * (8 + 8 + 4 + 4);
+    const size_t smem = (size_t)(nmax <= 64 ? 2 : 1) * sq * 8 + (size_t)mh * (8 + 8 + 4 + 4);  // V in shared memory up to 64
     if ((e = cudaFuncSetAttribute(jacobi_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
         return e;
     jacobi_kernel<false><<<dim3(2, (unsigned)n_layers), kKfThreads, smem, s>>>(state, stride, ka, kg, 1);

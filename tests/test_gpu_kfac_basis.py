@@ -23,7 +23,8 @@ def dev():
 
 @pytest.mark.parametrize("k,spectrum,seed", [(64, "geometric", 2), (64, "crowded", 1), (64, "crowded", 2),
                                              (48, "crowded", 2), (48, "low rank", 1), (32, "crowded", 2),
-                                             (33, "linear", 1), (7, "crowded", 1)])
+                                             (33, "linear", 1), (7, "crowded", 1), (4, "crowded", 1),
+                                             (3, "crowded", 1), (3, "low rank", 1), (2, "linear", 1), (1, "linear", 1)])
 def test_eigenbases_are_orthonormal(dev, k, spectrum, seed):
     rng = np.random.default_rng(seed)
     U = np.linalg.qr(rng.standard_normal((k, k)))[0]
