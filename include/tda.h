@@ -231,7 +231,8 @@ tda_status tda_similarity_exact(const tda_layer_desc* L, tda_dtype dtype,
 /* Which kernel the GRAM route of tda_similarity_exact runs: 1 = the tcgen05
  * kernel (bf16 factors, d_in and d_out multiples of 8, 16-byte aligned
  * factors, sm_103), whose two token Grams (A_q A_i^T, B_q B_i^T)
- * are tensor-core GEMMs with fp32 accumulation; 0 = the CUDA-core kernel.
+ * are tensor-core GEMMs with fp32 accumulation (up to some 300 pairs of short,
+ * narrow examples run on the CUDA cores all the same); 0 = the CUDA-core kernel.
  * Host only. */
 int32_t tda_similarity_gram_engine(const tda_layer_desc* L, tda_dtype dtype, const void* Aq, const void* Bq,
                                    const void* At, const void* Bt);

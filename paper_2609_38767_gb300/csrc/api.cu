@@ -379,7 +379,7 @@ tda_status tda_similarity_exact(const tda_layer_desc* L, tda_dtype dtype, const 
         return cuda_check(launch_score(S, TDA_F32, n_q, 0, S, n_t, 0, 0, S, ld_S, beta, s), "zero S");
     }
     if (route == TDA_ROUTE_GRAM) {
-        if (gram_tc_supported(*L, dtype, Aq, Bq, At, Bt)) {
+        if (gram_tc_supported(*L, dtype, Aq, Bq, At, Bt) && !gram_short(*L, n_q, n_t, false)) {
             unsigned int* err = device_error_word();
             if (!err) return fail(TDA_ERR_CUDA, "device error word unavailable");
             return cuda_check(launch_gram_tc(*L, Aq, Bq, n_q, At, Bt, n_t, S, ld_S, beta, 1.f, err, s),
@@ -507,7 +507,8 @@ tda_status tda_norms(tda_op op, const tda_layer_desc* L, tda_dtype dtype, const 
     cudaStream_t s = (cudaStream_t)stream;
     if (N == 0) return TDA_OK;
     if (L->T == 0) return cuda_check(cudaMemsetAsync(out, 0, sizeof(float) * (size_t)N, s), "zero norms");
-    if (op == TDA_OP_NORM_EXACT && route == TDA_ROUTE_GRAM && gram_tc_supported(*L, dtype, A, B, A, B)) {
+    if (op == TDA_OP_NORM_EXACT && route == TDA_ROUTE_GRAM && gram_tc_supported(*L, dtype, A, B, A, B) &&
+        !gram_short(*L, N, 0, true)) {
         unsigned int* err = device_error_word();
         if (!err) return fail(TDA_ERR_CUDA, "device error word unavailable");
         return cuda_check(launch_gram_self_tc(*L, A, B, N, out, err, s), "norms (gram, tensor cores)");

@@ -674,6 +674,20 @@ bool gram_tc_supported(const tda_layer_desc& L, tda_dtype dt, const void* Aq, co
     return true;
 }
 
+// Few pairs of short, narrow examples: a tile's epilogue sums all of its pq x pt outputs, of which such a job uses a
+// few, while the CUDA-core kernel has a CTA for every pair. Times of both in us, d both widths together. T = 3, 64 ->
+// 64, 1 x 8 pairs: 5 us on the CUDA cores and 15 us here; T = 1, one pair: 4.5 and 73 us; T = 5, 128 -> 128, 4 x 16: 8.8 and
+// 10.9 us, 256 -> 256: 14.5 and 13.8 us; norms, T = 3, 64 -> 64: 4.7 and 5.7 us, 128 -> 128: 7.6 and 7.1 us. Jobs of more
+// pairs than two an SM stay here, whose time does not grow with them.
+bool gram_short(const tda_layer_desc& L, int64_t n_q, int64_t n_t, bool norms) {
+    const int64_t most = 2 * (int64_t)sm_count();
+    if (L.T >= 16 || n_q > most || n_t > most || (norms ? n_q : n_q * n_t) > most) return false;
+    const double T = (double)L.T, d = (double)(L.d_in + L.d_out), chain = (0.018 + 0.0009 * T) * d;
+    if (norms) return 2.2 + chain < 4.0 + 0.09 * T + 0.0105 * d;
+    const int64_t outputs = (int64_t)(kTM / L.T) * (Cfg<false>::kCols / L.T * 2);
+    return 2.6 + chain < 5.6 + 0.0022 * (double)outputs + 0.0085 * d;
+}
+
 // S[q][i] = beta * S[q][i] + alpha * <DW_q, DW_i>_F for bf16 factors. A side with more examples
 // than one launch addresses goes in pieces, each its own block of S.
 cudaError_t launch_gram_tc(const tda_layer_desc& L, const void* Aq, const void* Bq, int64_t n_q, const void* At,

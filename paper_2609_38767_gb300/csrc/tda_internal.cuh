@@ -157,6 +157,8 @@ cudaError_t launch_similarity_materialized(const tda_layer_desc& L, tda_dtype dt
 // Route (c) and exact norms on tcgen05 for bf16 factors (k_gram_tc.cu).
 bool gram_tc_supported(const tda_layer_desc& L, tda_dtype dt, const void* Aq, const void* Bq, const void* At,
                        const void* Bt);
+// Jobs that the CUDA-core kernel does faster all the same (norms: n_q examples).
+bool gram_short(const tda_layer_desc& L, int64_t n_q, int64_t n_t, bool norms);
 cudaError_t launch_gram_tc(const tda_layer_desc& L, const void* Aq, const void* Bq, int64_t n_q, const void* At,
                            const void* Bt, int64_t n_t, float* S, int64_t ld_S, float beta, float alpha,
                            unsigned int* err, cudaStream_t s);
