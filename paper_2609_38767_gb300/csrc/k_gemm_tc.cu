@@ -40,11 +40,10 @@ struct GCfg {
     static constexpr uint32_t kBBytes = BN * kRowBytes;
     static constexpr uint32_t kStageBytes = 2 * kABytes + 2 * kBBytes;  // hi and lo of both operands
     // The tensor pipe's fp32 accumulation truncates (about a quarter ulp per addition,
-    // always toward zero), so groups of kGroup K chunks (24 additions) rotate over kAcc
-    // accumulators (all 512 TMEM columns) and the epilogue warps add every finished group
-    // into round-to-nearest fp32 registers while the MMAs fill the next ones.
+    // always toward zero), so every K chunk (12 additions) goes to the next of kAcc accumulators (all 512 TMEM
+    // columns) and the epilogue warps add it into round-to-nearest fp32 registers while the MMAs fill the next
+    // ones. 11 x 211 scores of 256 features: 6.7e-7 off, 9.2e-7 with two chunks each (8.6 and 8.3 us).
     static constexpr int kAcc = 512 / BN < 8 ? 512 / BN : 8;
-    static constexpr int kGroup = 2;
     static constexpr uint32_t kTmemCols = 512;
     static constexpr size_t kSmem =
         1024 + (size_t)kStages * kStageBytes + 8 * (3 * kStages + 2 * kAcc + 3) + 16;  // + barriers, TMEM slot, abort flag
@@ -69,6 +68,7 @@ struct GParams {
     float* S2;
     int red;               // add to S through TMA (beta = 1; S, its rows and entries 16-byte aligned)
     int nz;                // persistent kernel: batch entries
+    int gm;                // persistent kernel: chunks accumulated before they are drained, less one (0 or 1)
     unsigned int* err;
 };
 
@@ -125,7 +125,7 @@ score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     uint64_t* full = bars;                   // count 4 (producer warps)
     uint64_t* empty = bars + C::kStages;     // count 1 (MMA commit)
     uint64_t* raw_full = empty + C::kStages; // [kStages] TMA bytes landed (count 1 + tx)
-    uint64_t* acc_full = raw_full + C::kStages;  // [kAcc] a group is in the accumulator (MMA commit)
+    uint64_t* acc_full = raw_full + C::kStages;  // [kAcc] a chunk is in the accumulator (MMA commit)
     uint64_t* acc_empty = acc_full + C::kAcc;    // [kAcc] the accumulator is drained (count 4)
     uint64_t* red_go = acc_empty + C::kAcc;  // count 1 (leader's remote arrive)
     uint64_t* red_full = red_go + 1;         // count cs-1
@@ -240,9 +240,8 @@ score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         for (int64_t kc = kc0; kc < kc1; ++kc, ++it) {
             const int s = it % C::kStages;
             const uint32_t ph = (it / C::kStages) & 1u;
-            const uint32_t g = it / C::kGroup, a = g % C::kAcc;  // group g goes to accumulator a
-            const bool start = it % C::kGroup == 0;
-            if (start && !warp_wait(smem_u32(&acc_empty[a]), ((g / C::kAcc) & 1u) ^ 1u, abort, p.err)) break;
+            const uint32_t a = it % C::kAcc;  // this chunk's accumulator
+            if (!warp_wait(smem_u32(&acc_empty[a]), ((it / C::kAcc) & 1u) ^ 1u, abort, p.err)) break;
             if (!warp_wait(smem_u32(&full[s]), ph, abort, p.err)) break;
             tc_fence_after();
             const uint32_t st = smem_u32(smem + (size_t)s * C::kStageBytes);
@@ -252,12 +251,12 @@ score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             if (elect_one()) {
 #pragma unroll
                 for (int k = 0; k < kKC / 8; ++k) {  // K = 8 tf32 = 32 bytes per instruction
-                    mma_tf32(d, ahi + 2 * k, bhi + 2 * k, idesc, start && k == 0 ? 0u : 1u);
+                    mma_tf32(d, ahi + 2 * k, bhi + 2 * k, idesc, k == 0 ? 0u : 1u);
                     mma_tf32(d, ahi + 2 * k, blo + 2 * k, idesc, 1u);
                     mma_tf32(d, alo + 2 * k, bhi + 2 * k, idesc, 1u);
                 }
                 mma_commit(smem_u32(&empty[s]));
-                if (it % C::kGroup == C::kGroup - 1 || kc == kc1 - 1) mma_commit(smem_u32(&acc_full[a]));
+                mma_commit(smem_u32(&acc_full[a]));
             }
             __syncwarp();
         }
@@ -274,12 +273,11 @@ score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
     __syncwarp();
     if (warp >= 4 && warp < 8) {
-        // ---------------- epilogue: TMEM groups -> registers -> (cluster reduction) -> S
+        // ---------------- epilogue: TMEM chunks -> registers -> (cluster reduction) -> S
         const int q = warp & 3;
         const int row = q * 32 + lane;  // Phi row within the tile
         const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16);
-        const uint32_t nchunks = kc1 > kc0 ? (uint32_t)(kc1 - kc0) : 0u;
-        const uint32_t groups = (nchunks + C::kGroup - 1) / C::kGroup;
+        const uint32_t groups = kc1 > kc0 ? (uint32_t)(kc1 - kc0) : 0u;
         float acc[BN];
 #pragma unroll
         for (int c = 0; c < BN; ++c) acc[c] = 0.f;
@@ -406,8 +404,8 @@ score3x_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 // A's hi is the fp32 value as it is (a kind::tf32 MMA reads its upper 19 bits).
 //
 // Accuracy: the tensor pipe's fp32 accumulation rounds toward zero, so a long same-sign sum (a
-// diagonal entry of M) drifts low by up to an ulp per accumulate. Groups of kGroup chunks (24
-// accumulates) alternate between two accumulators, and eight epilogue warps (two per TMEM lane
+// diagonal entry of M) drifts low by up to an ulp per accumulate. Groups of two chunks (24 accumulates; scores
+// of up to 384 features: one) alternate between two accumulators, and eight epilogue warps (two per TMEM lane
 // quadrant, half of the columns each) add every finished group into round-to-nearest registers
 // beside the next group's MMAs, then write the tile beside the next tile's.
 //
@@ -434,7 +432,6 @@ struct TCfg {
     static constexpr int kRaw = PAIR && !RED ? 6 : 4;     // raw chunks
     static constexpr int kSlots = PAIR ? 4 : 3;           // A in TMEM, B's hi and lo in shared memory
     static constexpr uint32_t kSlotBytes = 2 * kBBytes;
-    static constexpr int kGroup = 2;
     static constexpr int kCols = BN / 2;                  // columns per epilogue thread
     static constexpr int kAOff = 2 * BN;                  // first TMEM column of A: [slot][hi 32 | lo 32]
     static constexpr size_t kOutOff = (size_t)kRaw * kRawBytes + (size_t)kSlots * kSlotBytes;
@@ -676,7 +673,7 @@ gemm3t_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
         bool got = true;
         for (int64_t t = t0; got && t < total; t += tstep) {
             const TileAt at = tile_at<BN, PAIR>(p, t, rank);
-            const uint32_t groups = (uint32_t)((chunks_of(p, at.y) + C::kGroup - 1) / C::kGroup);
+            const uint32_t groups = (uint32_t)((chunks_of(p, at.y) + p.gm) >> p.gm);
             const int64_t m = at.m0 + row, nb = at.n0 + half * C::kCols;
             // (the upper half of a pair's tile on the diagonal lies above it)
             const bool write = !(PAIR && p.lower && !at.second && at.m0 > at.n0);
@@ -803,7 +800,7 @@ gemm3t_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ C
             const int nkc = (int)chunks_of(p, tile_at<BN, PAIR>(p, t, rank).y);
             for (int kc = 0; kc < nkc; ++kc, ++it) {
                 const uint32_t s = it % C::kSlots, ph = (it / C::kSlots) & 1u, b = cnt & 1u;
-                const bool start = kc % C::kGroup == 0, last = kc % C::kGroup == C::kGroup - 1 || kc == nkc - 1;
+                const bool start = (kc & p.gm) == 0, last = (kc & p.gm) == p.gm || kc == nkc - 1;
                 if ((start && !warp_wait(smem_u32(&acc_empty[b]), ((cnt >> 1) & 1u) ^ 1u, abort, p.err)) ||
                     !warp_wait(smem_u32(&ready[s]), ph, abort, p.err)) {
                     ok = false;
@@ -978,6 +975,10 @@ cudaError_t launch_bn(GParams p, cudaStream_t s, int64_t nz = 1, size_t a_z_byte
     p.tiles_n = (int)tiles_n;
     if (cs == 1) {
         p.nz = (int)nz;
+        // Scores of up to 384 features: one chunk a group, 6.8e-7 off (two: 9.1e-7; 256 x 8192 scores of 256 features
+        // 12.3 and 11.9 us, of 384 14.4 and 13.8 us). Longer ones: two, 9.1e-7 whatever their length (7168 features 102 us, with one 7.2e-7
+        // and 113 us); so do the preconditioner's products (alpha = -1).
+        p.gm = p.alpha == 1.f && nkc <= 12 ? 0 : 1;
         // A pair's chunk takes about three quarters of a single CTA's (see above), so its whole rounds of
         // tiles decide: few or odd 128-row tiles can leave half of the pairs' rows empty.
         int64_t pairs = p.lower ? pair_lower_tiles(tiles_n) : (tiles_m + 1) / 2 * tiles_n;
@@ -1200,6 +1201,7 @@ cudaError_t launch_fit_tc(int n_layers, int64_t D, void* state, size_t state_byt
     p.lower = 1;
     p.splits = 1;
     p.nz = n_layers;
+    p.gm = 1;
     p.tiles_z = p.tiles_1 = pair_lower_tiles((D + kBM - 1) / kBM);
     p.err = err;
     static std::atomic<int> sms_cache{0};
