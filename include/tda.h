@@ -468,8 +468,8 @@ tda_status tda_mask_gather(const tda_layer_desc* L, tda_dtype dtype, const void*
  *         cores as three TF32 products per element pair (hi*hi + hi*lo + lo*hi
  *         of the split x = hi + lo), accurate to about fp32 rounding (1e-6
  *         relative at D = 7168): the tensor pipe's fp32 accumulators add with
- *         truncation, and every 64 features they are added to registers with
- *         round-to-nearest.
+ *         truncation, and every 32 or 64 features they are added to registers
+ *         with round-to-nearest.
  *   Phi   device fp32, n_t rows of D, row stride ld_phi.
  *   S     device fp32, row stride ld_S >= n_t. beta 0 overwrites (S may hold
  *         garbage); beta 1 accumulates layers.
