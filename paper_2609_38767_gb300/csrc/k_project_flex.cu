@@ -10,13 +10,13 @@
 // Accuracy: the tensor pipe adds 16 features at a time into its accumulators with truncation. Among values
 // of similar size it loses almost nothing (the terms are coarse against the sum's ulp), but every loss
 // points to zero, so that wide layers with a few large features drift (cubed normals, 49152 features: 5.3e-5
-// off in one sum; rounded fp32 chain 4.0e-6, bf16 1.9e-6). So an accumulator takes four chunks (256
-// features; bf16, whose rounded chain is almost exact, two), and the epilogue adds it to the token's row of
-// At or Bt with round-to-nearest (3.8e-7; bf16 3.9e-7). The accumulators form groups in two TMEM buffers:
-// one group is added beside the next one's MMAs, and bf16 has four accumulators a group, so that barriers and
-// commits are as rare as with fp32. At the end of a tile the epilogue contracts the rows, Phi += Bt^T At, in
-// fp32, as the other kernels do. One sum a side and one accumulator a group against this: fp32 2048 -> 2048,
-// k = 64, 64 x 512 tokens 133.8 and 129.7 us; bf16 4096 -> 4096, k = 64 x 48, 64 x 300 tokens 94.9 and 96.9 us.
+// off in one sum; rounded fp32 chain 4.0e-6, bf16 1.9e-6). So an accumulator takes four chunks (256 features; eight
+// where the streaming kernel's one sum is the alternative), and the epilogue adds it to the token's row of At or
+// Bt with round-to-nearest (3.8e-7; bf16 3.5e-7, in runs of eight 5.2e-7). The accumulators form groups in two TMEM buffers: one group is added beside the
+// next one's MMAs, and bf16 has four accumulators a group, so that barriers and commits are rare. At the end of
+// a tile the epilogue contracts the rows, Phi += Bt^T At, in fp32, as the other kernels do. One sum a side against
+// this: fp32 2048 -> 2048, k = 64, 64 x 512 tokens 134 and 128 us; bf16 4096 -> 4096, k = 64 x 48, 64 x 300 tokens 95 and
+// 95 us; at worst (narrow layers of many tokens, bound by the epilogue: 128 -> 1528, k = 64 x 32, 201 x 300) 77 and 84 us.
 //
 // The pieces go to TMEM, not to shared memory: the MMA takes its A operand from
 // TMEM (a lane per token, two bf16 features per column), the split warps read
@@ -72,8 +72,7 @@ struct Cfg {
     static constexpr uint32_t kTileBytes = (F32 ? 2 : 1) * kBoxBytes;
     static constexpr uint32_t kSignBytes = K * 128;
     static constexpr uint32_t kStageBytes = kTileBytes + kSignBytes;
-    static constexpr int kGroup = F32 ? 4 : 8;             // chunks accumulated in TMEM before they are drained
-    static constexpr int kAccs = F32 ? 2 : 4;              // their accumulators: h and m + l, or two chunks each
+    static constexpr int kAccs = F32 ? 2 : 4;              // accumulators of a group: h and m + l, or of one run of chunks each
     static constexpr int kBufCols = kAccs * K;
     static constexpr int kAOff = 2 * kBufCols;             // first column of the A pieces (fp32)
     static constexpr int kStageLd = K + 4;
@@ -100,6 +99,7 @@ struct Params {
     int pack;        // examples per tile, or 1
     int k_in, k_out, nk_in, nk_out;
     int cs;          // CTAs per cluster sharing one example's tiles
+    int run;         // log2 of the chunks that an accumulator takes before it is drained
 };
 
 #include "tc_ptx.cuh"
@@ -231,6 +231,7 @@ project_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     const uint32_t tmem = *tmem_slot;
     const uint32_t crank = cluster_rank(), cid = blockIdx.x / p.cs, ncl = gridDim.x / p.cs;
     const int nk_tot = p.nk_in + p.nk_out;
+    const int group = F32 ? 1 << p.run : C::kAccs << p.run;  // chunks of a group
     Units it{(int64_t)cid, (int)crank};
 
     if (warp == 0 && lane == 0) {
@@ -277,7 +278,7 @@ project_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             for (int k0 = 0; ok && k0 < nk_tot; ++grp) {  // groups end with a side
                 const uint32_t b = grp & 1u;
                 const int side_end = k0 < p.nk_in ? p.nk_in : nk_tot;
-                const int n = side_end - k0 < C::kGroup ? side_end - k0 : C::kGroup;
+                const int n = side_end - k0 < group ? side_end - k0 : group;
                 if (!warp_wait(smem_u32(&tempty[b]), ((grp >> 1) & 1u) ^ 1u, abort, p.err)) {
                     ok = false;
                     break;
@@ -293,9 +294,8 @@ project_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                     tc_fence_after();
                     const uint32_t st = smem_u32(smem + (size_t)s * C::kStageBytes);
                     const uint64_t bd = sw128_desc(st + C::kTileBytes);
-                    // bf16: two chunks an accumulator
-                    const uint32_t dh = tmem + b * C::kBufCols + (F32 ? 0 : c / 2 * K), dl = dh + K;
-                    const bool clear = F32 ? c == 0 : c % 2 == 0;
+                    const uint32_t dh = tmem + b * C::kBufCols + (F32 ? 0 : (c >> p.run) * K), dl = dh + K;
+                    const bool clear = (c & ((1 << p.run) - 1)) == 0;
                     if (elect_one()) {
 #pragma unroll
                         for (int k = 0; k < kChunkK / 16; ++k) {  // K = 16: 32 bytes of bf16, 8 columns of pieces
@@ -524,7 +524,7 @@ project_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 float sum[K];  // bf16
 #pragma unroll
                 for (int i = 0; i < K; ++i) sum[i] = 0.f;
-                for (int k0 = 0; k0 < nk; k0 += C::kGroup, ++grp) {
+                for (int k0 = 0; k0 < nk; k0 += group, ++grp) {
                     const uint32_t b = grp & 1u;
                     ok = warp_wait(smem_u32(&tfull[b]), (grp >> 1) & 1u, abort, p.err);
                     if (!ok) break;
@@ -545,7 +545,7 @@ project_flex_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                             }
                         }
                     } else if (active) {
-                        for (int a = 0; a < C::kAccs && k0 + 2 * a < nk; ++a) {
+                        for (int a = 0; a < C::kAccs && k0 + (a << p.run) < nk; ++a) {
                             float v[K];
                             tmem_ld<K>(tb + a * K, v);
 #pragma unroll
@@ -801,6 +801,9 @@ cudaError_t launch_k(const tda_layer_desc& L, const void* A, const void* B, int6
     p.nk_in = (int)((L.d_in + kChunkK - 1) / kChunkK);
     p.nk_out = (int)((L.d_out + kChunkK - 1) / kChunkK);
     p.cs = pl.cs;
+    // fp32 and other k: sums of 256 features. k_in = k_out of 16, 32 or 64, which the streaming kernel sums
+    // at once: 512, for half of the drains' time.
+    p.run = !F32 && L.k_in == L.k_out && L.k_in == K ? 3 : 2;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
     cluster_config<K, F32>(cfg, attr, pl.cs, s);
