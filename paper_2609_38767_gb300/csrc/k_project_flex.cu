@@ -10,13 +10,14 @@
 // Accuracy: the tensor pipe adds 16 features at a time into its accumulators with truncation. Among values
 // of similar size it loses almost nothing (the terms are coarse against the sum's ulp), but every loss
 // points to zero, so that wide layers with a few large features drift (cubed normals, 49152 features: 5.3e-5
-// off in one sum; rounded fp32 chain 4.0e-6, bf16 1.9e-6). So an accumulator takes four chunks (256 features; eight
-// where the streaming kernel's one sum is the alternative), and the epilogue adds it to the token's row of At or
-// Bt with round-to-nearest (3.8e-7; bf16 3.5e-7, in runs of eight 5.2e-7). The accumulators form groups in two TMEM buffers: one group is added beside the
-// next one's MMAs, and bf16 has four accumulators a group, so that barriers and commits are rare. At the end of
-// a tile the epilogue contracts the rows, Phi += Bt^T At, in fp32, as the other kernels do. One sum a side against
-// this: fp32 2048 -> 2048, k = 64, 64 x 512 tokens 134 and 128 us; bf16 4096 -> 4096, k = 64 x 48, 64 x 300 tokens 95 and
-// 95 us; at worst (narrow layers of many tokens, bound by the epilogue: 128 -> 1528, k = 64 x 32, 201 x 300) 77 and 84 us.
+// off in one sum; rounded fp32 chain 4.0e-6, bf16 1.9e-6). So an accumulator takes four chunks (256 features;
+// eight where the streaming kernel's one sum is the alternative), and the epilogue adds it to the token's row
+// of At or Bt with round-to-nearest (3.8e-7; bf16 3.5e-7, in runs of eight 5.2e-7). The accumulators form
+// groups in two TMEM buffers: one group is added beside the next one's MMAs, and bf16 has four accumulators a
+// group, so that barriers and commits are rare. At the end of a tile the epilogue contracts the rows, Phi +=
+// Bt^T At, in fp32, as the other kernels do. One sum a side against this: fp32 2048 -> 2048, k = 64, 64 x 512
+// tokens 134 and 128 us; bf16 4096 -> 4096, k = 64 x 48, 64 x 300 tokens 95 and 95 us; at worst (narrow
+// layers of many tokens, bound by the epilogue: 128 -> 1528, k = 64 x 32, 201 x 300) 77 and 84 us.
 //
 // The pieces go to TMEM, not to shared memory: the MMA takes its A operand from
 // TMEM (a lane per token, two bf16 features per column), the split warps read
